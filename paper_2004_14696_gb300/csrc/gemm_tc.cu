@@ -3,14 +3,19 @@
 // memory stages guarded by mbarriers, one thread issuing tcgen05.mma into a
 // TMEM accumulator, and four epilogue warps reading TMEM with tcgen05.ld.
 //
-//   C[M, N] = sum_k A[m, k] * B[n, k]      (both operands K-major, bf16; fp32 accumulation)
+//   C[M, N] = sum_k A(m, k) * B(n, k)      (bf16 operands, fp32 accumulation)
+//
+// Operands stay in the row-major layout their producer wrote.  One whose rows run along
+// K (activations and dZ as forward operands, W in the forward pass) is staged K-major:
+// 64-element K slices of the tile's rows.  One whose rows run along M or N (dZ and the
+// activations in the weight gradients, W in the input gradient) is staged MN-major:
+// groups of 64 columns, each group one row per K index; the UMMA descriptors say which
+// (tc_ptx.cuh).  Both use 128-byte rows with the 128-byte swizzle.
 //
 // CTA = 6 warps:  warp 0  TMA producer (one lane) and TMEM owner
 //                 warp 1  MMA issuer (one lane)
 //                 warps 2-5  epilogue: warp w reads TMEM lanes 32*(w%4) .. +31,
 //                            i.e. rows m0 + 32*(w%4) + lane of the 128-row tile.
-// Tile 128 x BN x BK; K-major operands staged with the 128B (BK = 64) or 64B
-// (BK = 32) swizzle that both TMA and the UMMA shared-memory descriptors use.
 //
 // Every wait on an mbarrier is bounded (2 s of %globaltimer).  A wait that runs
 // out sets bit 0 of *status, the producer drains the TMA loads it still has in
@@ -33,6 +38,16 @@ using namespace tcx;
 
 constexpr int BM = 128;
 constexpr int kThreads = 192;
+
+// Whether the rows of operand A / B of a GEMM kind run along M / N (MN-major staging).
+__host__ __device__ constexpr bool a_mn(int kind) { return kind == TC_GBAR || kind == TC_DW; }
+__host__ __device__ constexpr bool b_mn(int kind) { return kind == TC_GBAR || kind == TC_DW || kind == TC_DX; }
+
+// Descriptor of K step kk (16 elements) of an operand tile staged at ``base`` in BK-deep stages.
+template <bool MN, int BK>
+__device__ __forceinline__ uint64_t operand_desc(uint32_t base, int kk) {
+    return MN ? smem_desc_mn(base + kk * 2048, BK * 128) : smem_desc(base + kk * 32, 128);
+}
 
 // ------------------------------------------------------------------ epilogues
 // One thread: row ``row`` of the tile, 32 columns starting at ``nb`` (logits and the
@@ -74,19 +89,8 @@ __device__ __forceinline__ void epilogue_chunk(const TcEpi& e, int z, int row, i
 // step, the layer input for the ReLU mask) are issued one chunk ahead, so that
 // their latency overlaps the previous chunk's work.
 
-// Per epilogue warp: a 32 x 32 bf16 chunk, transposed ([column][row], rows padded to 40
-// elements), between TMEM and the transposed copy.
-constexpr int kStageLd = 40;
-constexpr int kStageBytes = 32 * kStageLd * 2;
-
-// bf16 activation chunk -> out (row-major) and, when asked, outT (transposed).  The
-// lanes of a warp hold 32 consecutive rows (row = row0 + lane; M is a multiple of 32,
-// so a warp's rows are all inside or all outside the matrix); the transposed copy goes
-// through the warp's staging chunk ``stg`` so that each global store writes 16 bytes
-// and four lanes cover 64 contiguous bytes of one transposed row.
-__device__ __forceinline__ void store_act_chunk(const TcEpi& e, int row, int nb, int N, const float (&x)[32],
-                                                __nv_bfloat16* stg) {
-    const int lane = threadIdx.x & 31;
+// bf16 activation chunk (32 columns of row ``row``) -> out.
+__device__ __forceinline__ void store_act_chunk(const TcEpi& e, int row, int nb, int N, const float (&x)[32]) {
     __nv_bfloat16* op = e.out + static_cast<int64_t>(row) * e.ldo + nb;
     if (nb + 32 <= N && ((reinterpret_cast<uintptr_t>(op) & 15u) == 0)) {
 #pragma unroll
@@ -103,39 +107,16 @@ __device__ __forceinline__ void store_act_chunk(const TcEpi& e, int row, int nb,
         for (int j = 0; j < 32; ++j)
             if (nb + j < N) op[j] = __float2bfloat16_rn(x[j]);
     }
-    if (e.outT) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) stg[j * kStageLd + lane] = __float2bfloat16_rn(x[j]);
-        __syncwarp();
-        const int row0 = row - lane;
-        const bool vec = ((reinterpret_cast<uintptr_t>(e.outT) & 15u) == 0) && e.ldT % 8 == 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int idx = i * 32 + lane;
-            const int j = idx >> 2, p = idx & 3;   // transposed row nb + j, rows row0 + 8p .. +7
-            if (nb + j < N) {
-                __nv_bfloat16* dst = e.outT + static_cast<int64_t>(nb + j) * e.ldT + row0 + 8 * p;
-                const __nv_bfloat16* src = stg + j * kStageLd + 8 * p;
-                if (vec) {
-                    *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(src);
-                } else {
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) dst[t] = src[t];
-                }
-            }
-        }
-        __syncwarp();
-    }
 }
 
 // TC_HIDDEN: A_l = ReLU(Z_l + b_l) in bf16.
-__device__ __forceinline__ void hidden_cols(const TcEpi& e, int row, int nb0, int M, int N, uint32_t taddr,
-                                            __nv_bfloat16* stg) {
+__device__ __forceinline__ void hidden_cols(const TcEpi& e, int row, int nb0, int M, int N, uint32_t taddr) {
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {
         const int nb = nb0 + 32 * c;
         if (nb >= N) break;
         uint32_t r[32];
+        __syncwarp();   // lanes past M skipped the previous chunk's stores
         tc_ld_32cols(taddr + 32 * c, r);
         tc_wait_ld();
         if (row >= M) continue;
@@ -145,14 +126,13 @@ __device__ __forceinline__ void hidden_cols(const TcEpi& e, int row, int nb0, in
             const float v = u2f(r[j]) + (nb + j < N ? __ldg(e.bias + nb + j) : 0.f);
             x[j] = v > 0.f ? v : 0.f;
         }
-        store_act_chunk(e, row, nb, N, x, stg);
+        store_act_chunk(e, row, nb, N, x);
     }
 }
 
 // TC_DX: dZ_{l-1} = (dZ_l W_l) * 1[A_{l-1} > 0] in bf16; ``avec``: the act rows allow
 // 16-byte loads.
-__device__ __forceinline__ void dx_cols(const TcEpi& e, int row, int nb0, int M, int N, uint32_t taddr, bool avec,
-                                        __nv_bfloat16* stg) {
+__device__ __forceinline__ void dx_cols(const TcEpi& e, int row, int nb0, int M, int N, uint32_t taddr, bool avec) {
     const bool rowok = row < M;
     const __nv_bfloat16* ap = e.act + static_cast<int64_t>(row) * e.ldact + nb0;
     uint4 nxt[4];
@@ -172,6 +152,7 @@ __device__ __forceinline__ void dx_cols(const TcEpi& e, int row, int nb0, int M,
         for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
         if (c + 1 < 4) fetch(c + 1);
         uint32_t r[32];
+        __syncwarp();   // lanes past M skipped the previous chunk's stores
         tc_ld_32cols(taddr + 32 * c, r);
         tc_wait_ld();
         if (!rowok) continue;
@@ -189,7 +170,7 @@ __device__ __forceinline__ void dx_cols(const TcEpi& e, int row, int nb0, int M,
             for (int j = 0; j < 32; ++j)
                 x[j] = (nb + j < N) ? u2f(r[j]) * (__bfloat162float(ap[32 * c + j]) > 0.f ? 1.f : 0.f) : 0.f;
         }
-        store_act_chunk(e, row, nb, N, x, stg);
+        store_act_chunk(e, row, nb, N, x);
     }
 }
 
@@ -220,6 +201,7 @@ __device__ __forceinline__ double gbar_cols(const TcEpi& e, int row, int nb0, in
         for (int j = 0; j < 8; ++j) cur[j] = nxt[j];
         if (c + 1 < 4) fetch(c + 1);
         uint32_t r[32];
+        __syncwarp();   // lanes past M skipped the previous chunk's stores
         tc_ld_32cols(taddr + 32 * c, r);
         tc_wait_ld();
         if (!rowok) continue;
@@ -262,7 +244,6 @@ struct TcCfg {
     static constexpr int A_BYTES = BM * BK * 2;
     static constexpr int B_BYTES = BN * BK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int SW = BK * 2;   // swizzle span in bytes: 128 (BK = 64) or 64 (BK = 32)
     static constexpr int BAR_BYTES = 256;
     static constexpr int SMEM = STAGES * STAGE_BYTES + BAR_BYTES + 1024;   // + alignment slack
     static_assert(BK == 64 || BK == 32, "BK must be 64 or 32");
@@ -272,7 +253,8 @@ struct TcCfg {
 template <int BN, int BK, int STAGES, int KIND, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N,
-                   int K, int64_t kz, TcEpi epi, int* status) {
+                   int K, TcEpi epi, int* status) {
+    static_assert(KIND == TC_DW, "the one-CTA-per-tile kernel serves the per-worker weight gradient");
     using Cfg = TcCfg<BN, BK, STAGES>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -287,7 +269,6 @@ __global__ void __launch_bounds__(kThreads, MINB)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN, z = blockIdx.z;
     const int nk = (K + BK - 1) / BK;
-    const int kbase = static_cast<int>(z * kz);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -320,8 +301,12 @@ __global__ void __launch_bounds__(kThreads, MINB)
             }
             if (*reinterpret_cast<volatile int*>(abort_flag)) break;
             mbar_expect_tx(smem_u32(full_bar + s), Cfg::STAGE_BYTES);
-            tma_load_2d(smem_u32(sA + s * Cfg::A_BYTES), &tmA, kbase + kb * BK, m0, smem_u32(full_bar + s));
-            tma_load_2d(smem_u32(sB + s * Cfg::B_BYTES), &tmB, kbase + kb * BK, n0, smem_u32(full_bar + s));
+            for (int c = 0; c < BM; c += 64)
+                tma_load_3d(smem_u32(sA + s * Cfg::A_BYTES + c * BK * 2), &tmA, m0 + c, kb * BK, z,
+                            smem_u32(full_bar + s));
+            for (int c = 0; c < BN; c += 64)
+                tma_load_3d(smem_u32(sB + s * Cfg::B_BYTES + c * BK * 2), &tmB, n0 + c, kb * BK, z,
+                            smem_u32(full_bar + s));
             issued = kb + 1;
         }
         if (*reinterpret_cast<volatile int*>(abort_flag)) {
@@ -331,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
         }
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer
-        constexpr uint32_t idesc = instr_desc_bf16(BM, BN);
+        constexpr uint32_t idesc = instr_desc_bf16(BM, BN, true, true);
         for (int kb = 0; kb < nk; ++kb) {
             const int s = kb % STAGES;
             const uint32_t ph = (kb / STAGES) & 1;
@@ -345,7 +330,8 @@ __global__ void __launch_bounds__(kThreads, MINB)
             const uint32_t b0 = smem_u32(sB + s * Cfg::B_BYTES);
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
-                tc_mma(tmem, smem_desc(a0 + kk * 32, Cfg::SW), smem_desc(b0 + kk * 32, Cfg::SW), idesc,
+                if (kb * BK + 16 * kk >= K) break;   // rows past K are zero
+                tc_mma(tmem, operand_desc<true, BK>(a0, kk), operand_desc<true, BK>(b0, kk), idesc,
                        (kb > 0 || kk > 0) ? 1u : 0u);
             }
             tc_commit(smem_u32(empty_bar + s));   // frees the stage once these MMAs have read it
@@ -364,6 +350,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
             for (int c = 0; c < BN / 32; ++c) {
                 if (n0 + c * 32 >= N) break;
                 uint32_t r[32];
+                __syncwarp();
                 tc_ld_32cols(tbase + c * 32, r);
                 tc_wait_ld();
                 epilogue_chunk<KIND>(epi, z, row, n0 + c * 32, M, N, r);
@@ -391,8 +378,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
 // One launch may carry two independent problems (nprob = 2, kinds KIND0 and
 // KIND1): their tiles form one list, those of problem 0 first, dealt to the pairs
 // in turn, so that the second problem fills the last partial wave of the first.
-// Shared memory: the ring of STAGES stages, 256 bytes of barriers, then a 32 x 32
-// bf16 transposing chunk per epilogue warp.
+// Shared memory: the ring of STAGES stages, then 256 bytes of barriers.
 //
 // Barriers (the same shared-memory offsets in both CTAs):
 //   full[s]    even CTA only: its producer arrives with the byte count of both
@@ -448,7 +434,7 @@ __device__ __forceinline__ PairShape pair_shape(const PairProblem& P) {
 // Epilogue of one tile for problem kind KIND (one thread: one row, 128 columns).
 template <int KIND>
 __device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairShape& S, long long t, int rank, int q,
-                                              int h, int lane, uint32_t taddr, __nv_bfloat16* stg) {
+                                              int h, int lane, uint32_t taddr) {
     constexpr int BN = 256;
     const TcEpi& epi = P.epi;
     const int nt = static_cast<int>(t % S.nt_n);
@@ -466,14 +452,15 @@ __device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairSh
         if (lane == 0 && msub < S.msub_n) epi.pieces[(static_cast<long long>(msub) * S.nt_n + nt) * 8 + h * 4 + q] = sq;
     } else if constexpr (KIND == TC_DX) {
         const bool avec = ((reinterpret_cast<uintptr_t>(epi.act) & 15u) == 0) && epi.ldact % 8 == 0;
-        dx_cols(epi, row, nb0, P.M, P.N, taddr, avec, stg);
+        dx_cols(epi, row, nb0, P.M, P.N, taddr, avec);
     } else if constexpr (KIND == TC_HIDDEN) {
-        hidden_cols(epi, row, nb0, P.M, P.N, taddr, stg);
+        hidden_cols(epi, row, nb0, P.M, P.N, taddr);
     } else {
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
             if (nb0 + c * 32 >= P.N) break;
             uint32_t r[32];
+            __syncwarp();
             tc_ld_32cols(taddr + c * 32, r);
             tc_wait_ld();
             epilogue_chunk<KIND>(epi, 0, row, nb0 + c * 32, P.M, P.N, r);
@@ -481,10 +468,39 @@ __device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairSh
     }
 }
 
+// One stage of this CTA's half tiles of problem kind KIND: 128 rows (or columns) of A from
+// ``ma``, 128 of B from ``nb``, K block kb.
+template <int KIND, int BK>
+__device__ __forceinline__ void pair_load(const PairProblem& P, uint8_t* dA, uint8_t* dB, int kb, int ma, int nb,
+                                          uint32_t bar) {
+    if constexpr (a_mn(KIND)) {
+        tma_load_2d_pair(smem_u32(dA), &P.tmA, ma, kb * BK, bar);
+        tma_load_2d_pair(smem_u32(dA + BK * 128), &P.tmA, ma + 64, kb * BK, bar);
+    } else {
+        tma_load_2d_pair(smem_u32(dA), &P.tmA, kb * BK, ma, bar);
+    }
+    if constexpr (b_mn(KIND)) {
+        tma_load_2d_pair(smem_u32(dB), &P.tmB, nb, kb * BK, bar);
+        tma_load_2d_pair(smem_u32(dB + BK * 128), &P.tmB, nb + 64, kb * BK, bar);
+    } else {
+        tma_load_2d_pair(smem_u32(dB), &P.tmB, kb * BK, nb, bar);
+    }
+}
+
+// The MMAs of one stage (even CTA).
+template <int KIND, int BK, int BN>
+__device__ __forceinline__ void pair_mma(uint32_t dcol, uint32_t a0, uint32_t b0, bool first) {
+    constexpr uint32_t idesc = instr_desc_bf16(2 * BM, BN, a_mn(KIND), b_mn(KIND));
+#pragma unroll
+    for (int kk = 0; kk < BK / 16; ++kk)
+        tc2_mma(dcol, operand_desc<a_mn(KIND), BK>(a0, kk), operand_desc<b_mn(KIND), BK>(b0, kk), idesc,
+                (!first || kk > 0) ? 1u : 0u);
+}
+
 template <int KIND0, int KIND1, int STAGES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     tc_gemm_pair_kernel(const __grid_constant__ PairArgs args) {
-    constexpr int BN = 256, BK = 64, SW = 128;
+    constexpr int BN = 256, BK = 64;
     constexpr int A_BYTES = BM * BK * 2;          // 128 rows of A
     constexpr int B_BYTES = (BN / 2) * BK * 2;    // this CTA's 128 rows of B
     constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
@@ -498,8 +514,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     uint64_t* tempty_bar = tfull_bar + 2;        // [2]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty_bar + 2);
     int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-    // epilogue warps' transposing chunks, after the 256 bytes of barriers
-    __nv_bfloat16* staging = reinterpret_cast<__nv_bfloat16*>(smem + STAGES * STAGE_BYTES + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
@@ -541,8 +555,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             const bool second = t >= S0.tiles;
             const long long u = second ? t - S0.tiles : t;
             const PairShape& S = second ? S1 : S0;
-            const CUtensorMap* tmA = second ? &args.p[1].tmA : &args.p[0].tmA;
-            const CUtensorMap* tmB = second ? &args.p[1].tmB : &args.p[0].tmB;
             const int ma = static_cast<int>(u / S.nt_n) * (2 * BM) + static_cast<int>(rank) * BM;
             const int nb = static_cast<int>(u % S.nt_n) * BN + static_cast<int>(rank) * (BN / 2);
             for (int kb = 0; kb < S.nk; ++kb, ++g) {
@@ -555,8 +567,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 }
                 if (rank == 0) mbar_expect_tx(smem_u32(full_bar + s), 2 * STAGE_BYTES);
                 const uint32_t bar = map_to_rank(smem_u32(full_bar + s), 0);
-                tma_load_2d_pair(smem_u32(sA + s * A_BYTES), tmA, kb * BK, ma, bar);
-                tma_load_2d_pair(smem_u32(sB + s * B_BYTES), tmB, kb * BK, nb, bar);
+                if (second)
+                    pair_load<KIND1, BK>(args.p[1], sA + s * A_BYTES, sB + s * B_BYTES, kb, ma, nb, bar);
+                else
+                    pair_load<KIND0, BK>(args.p[0], sA + s * A_BYTES, sB + s * B_BYTES, kb, ma, nb, bar);
             }
         }
         // the last use of every stage has been consumed: no load or commit is still
@@ -572,11 +586,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         }
     } else if (warp == 1 && lane == 0 && rank == 0) {
         // ---------------- MMA issuer (even CTA)
-        constexpr uint32_t idesc = instr_desc_bf16(2 * BM, BN);
         long long g = 0;
         int i = 0;
         for (long long t = pair; t < total && !*vabort; t += npairs, ++i) {
-            const int nk = t >= S0.tiles ? S1.nk : S0.nk;
+            const bool second = t >= S0.tiles;
+            const int nk = second ? S1.nk : S0.nk;
             const int acc = i & 1;
             const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
             if (!mbar_wait(smem_u32(tempty_bar + acc), aph ^ 1)) {
@@ -599,10 +613,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 tc_fence_after();
                 const uint32_t a0 = smem_u32(sA + s * A_BYTES);
                 const uint32_t b0 = smem_u32(sB + s * B_BYTES);
-#pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                    tc2_mma(dcol, smem_desc(a0 + kk * 32, SW), smem_desc(b0 + kk * 32, SW), idesc,
-                            (kb > 0 || kk > 0) ? 1u : 0u);
+                if (second)
+                    pair_mma<KIND1, BK, BN>(dcol, a0, b0, kb == 0);
+                else
+                    pair_mma<KIND0, BK, BN>(dcol, a0, b0, kb == 0);
                 tc2_commit_multicast(smem_u32(empty_bar + s), 0x3);
             }
             tc2_commit_multicast(smem_u32(tfull_bar + acc), 0x3);
@@ -611,7 +625,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     } else if (warp >= 2) {
         // ---------------- epilogue (both CTAs): 128-row sub-tile msub, lane quarter q, column half h
         const int q = warp & 3, h = (warp - 2) >> 2;
-        __nv_bfloat16* stg = staging + (warp - 2) * (kStageBytes / 2);
         int i = 0;
         for (long long t = pair; t < total; t += npairs, ++i) {
             const int acc = i & 1;
@@ -626,10 +639,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             const uint32_t taddr = tmem + static_cast<uint32_t>(acc * BN + h * (BN / 2)) +
                                    (static_cast<uint32_t>(q * 32) << 16);
             if (t < S0.tiles)
-                pair_epilogue<KIND0>(args.p[0], S0, t, static_cast<int>(rank), q, h, lane, taddr, stg);
+                pair_epilogue<KIND0>(args.p[0], S0, t, static_cast<int>(rank), q, h, lane, taddr);
             else
-                pair_epilogue<KIND1>(args.p[1], S1, t - S0.tiles, static_cast<int>(rank), q, h, lane, taddr,
-                                     stg);
+                pair_epilogue<KIND1>(args.p[1], S1, t - S0.tiles, static_cast<int>(rank), q, h, lane, taddr);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_remote(map_to_rank(smem_u32(tempty_bar + acc), 0));
@@ -653,8 +665,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 }
 
 // ------------------------------------------------------------------ persistent dW kernel
-// Per-worker weight gradient G[z*ldG + m*ldrow + n] = sum_{k < K} A[m, z*K + k] B[n, z*K + k]
-// (A = dZ^T [out, M], B = A_{l-1}^T [in, M], K = the worker's B samples).
+// Per-worker weight gradient G[z*ldG + m*ldrow + n] = sum_{k < K} A[z*K + k, m] B[z*K + k, n]
+// (A = dZ [M, out], B = A_{l-1} [M, in], K = the worker's B samples).  The tensor maps
+// are 3-D, (column, sample of the worker, worker), so that rows past a worker's K samples
+// read as zero whatever K is.
 //
 // The kernel is bound by writing G (K is small), so it is built around that
 // store.  A persistent grid (one CTA per SM) walks the tiles worker-major with n
@@ -676,7 +690,6 @@ struct DwCfg {
     static constexpr int A_BYTES = BM * BK * 2;
     static constexpr int B_BYTES = DW_BN * BK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int SW = BK * 2;
     static constexpr int STAGING = DW_EPI_WARPS * DW_STAGING_BYTES;
     static constexpr int BAR_BYTES = 256;
     static constexpr int SMEM = STAGES * STAGE_BYTES + STAGING + BAR_BYTES + 1024;
@@ -757,9 +770,14 @@ __global__ void __launch_bounds__(DW_THREADS, 1)
                 }
                 if (!(kTest && blockIdx.x == 0 && g == wt.skip_stage)) {
                     mbar_expect_tx(smem_u32(full_bar + s), Cfg::STAGE_BYTES);
-                    const int kx = z * K + kb * BK;
-                    tma_load_2d(smem_u32(sA + s * Cfg::A_BYTES), &tmA, kx, m0, smem_u32(full_bar + s));
-                    tma_load_2d(smem_u32(sB + s * Cfg::B_BYTES), &tmB, kx, n0, smem_u32(full_bar + s));
+#pragma unroll
+                    for (int c = 0; c < BM; c += 64)
+                        tma_load_3d(smem_u32(sA + s * Cfg::A_BYTES + c * BK * 2), &tmA, m0 + c, kb * BK, z,
+                                    smem_u32(full_bar + s));
+#pragma unroll
+                    for (int c = 0; c < DW_BN; c += 64)
+                        tma_load_3d(smem_u32(sB + s * Cfg::B_BYTES + c * BK * 2), &tmB, n0 + c, kb * BK, z,
+                                    smem_u32(full_bar + s));
                 }
                 issued = g + 1;
             }
@@ -772,7 +790,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1)
         }
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer
-        constexpr uint32_t idesc = instr_desc_bf16(BM, DW_BN);
+        constexpr uint32_t idesc = instr_desc_bf16(BM, DW_BN, true, true);
         long long g = 0;
         int i = 0;
         for (long long t = blockIdx.x; t < total && !*vabort; t += gridDim.x, ++i) {
@@ -799,9 +817,11 @@ __global__ void __launch_bounds__(DW_THREADS, 1)
                 const uint32_t a0 = smem_u32(sA + s * Cfg::A_BYTES);
                 const uint32_t b0 = smem_u32(sB + s * Cfg::B_BYTES);
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                    tc_mma(dcol, smem_desc(a0 + kk * 32, Cfg::SW), smem_desc(b0 + kk * 32, Cfg::SW), idesc,
+                for (int kk = 0; kk < BK / 16; ++kk) {
+                    if (kb * BK + 16 * kk >= K) break;   // rows past K are zero
+                    tc_mma(dcol, operand_desc<true, BK>(a0, kk), operand_desc<true, BK>(b0, kk), idesc,
                            (kb > 0 || kk > 0) ? 1u : 0u);
+                }
                 tc_commit(smem_u32(empty_bar + s));
             }
             tc_commit(smem_u32(tfull_bar + acc));
@@ -930,7 +950,7 @@ int pair_slots(Kern kern, int smem) {
 template <int KIND0, int KIND1>
 cudaError_t launch_pair(const PairArgs& args, cudaStream_t st) {
     constexpr int STAGES = DBW_PAIR_STAGES;
-    constexpr int SMEM = STAGES * (2 * BM * 64 * 2) + 256 + 8 * kStageBytes + 1024;
+    constexpr int SMEM = STAGES * (2 * BM * 64 * 2) + 256 + 1024;
     static_assert(SMEM <= 227 * 1024, "pair ring does not fit in shared memory");
     auto kern = tc_gemm_pair_kernel<KIND0, KIND1, STAGES>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
@@ -948,15 +968,15 @@ cudaError_t launch_pair(const PairArgs& args, cudaStream_t st) {
 }
 
 template <int BN, int BK, int STAGES, int KIND, int MINB>
-cudaError_t launch_cfg(const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, int batch, int64_t kz,
-                       const TcEpi& e, int* status, cudaStream_t st, int min_smem) {
+cudaError_t launch_cfg(const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, int batch, const TcEpi& e,
+                       int* status, cudaStream_t st, int min_smem) {
     using Cfg = TcCfg<BN, BK, STAGES>;
     auto kern = tc_gemm_kernel<BN, BK, STAGES, KIND, MINB>;
     const int smem = Cfg::SMEM > min_smem ? Cfg::SMEM : min_smem;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (err != cudaSuccess) return err;
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch);
-    kern<<<grid, kThreads, smem, st>>>(a, b, M, N, K, kz, e, status);
+    kern<<<grid, kThreads, smem, st>>>(a, b, M, N, K, e, status);
     return cudaGetLastError();
 }
 
@@ -986,16 +1006,31 @@ static EncodeTiledFn encode_fn() {
 }
 
 // 2-D tensor map of a row-major bf16 matrix [rows, cols] with row stride ld (elements).
-bool tc_make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_k, int box_rows) {
+bool tc_make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
     cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld * 2)};
-    cuuint32_t box[2] = {static_cast<cuuint32_t>(box_k), static_cast<cuuint32_t>(box_rows)};
+    cuuint32_t box[2] = {64u, static_cast<cuuint32_t>(box_rows)};
     cuuint32_t estr[2] = {1, 1};
-    const CUtensorMapSwizzle sw = box_k == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
     return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The same matrix as batch blocks of rows_z rows: dimensions (column, row of the block,
+// block), box 64 x box_rows x 1; rows past rows_z of a block read as zero.
+static bool make_batch_map(CUtensorMap* tm, const void* base, int64_t rows_z, int64_t batch, int64_t cols, int64_t ld,
+                           int box_rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows_z),
+                          static_cast<cuuint64_t>(batch)};
+    cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld * 2), static_cast<cuuint64_t>(rows_z * ld * 2)};
+    cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1013,25 +1048,23 @@ bool tc_make_map_f32(CUtensorMap* tm, const void* base, int64_t rows, int64_t co
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool tc_shape_ok(int64_t lda, int64_t ldb, int K, int64_t kz, const void* A, const void* B) {
-    if (!encode_fn()) return false;
-    if ((lda % 8) || (ldb % 8) || (kz % 8)) return false;
-    if ((reinterpret_cast<uintptr_t>(A) & 15u) || (reinterpret_cast<uintptr_t>(B) & 15u)) return false;
-    if (kz > 0 && K % 32) return false;   // a batch's K must be whole K blocks (it is the column offset step)
-    return K >= 1;
+static bool operands_ok(const TcOperands& o) {
+    return encode_fn() && o.lda % 8 == 0 && o.ldb % 8 == 0 && (reinterpret_cast<uintptr_t>(o.A) & 15u) == 0 &&
+           (reinterpret_cast<uintptr_t>(o.B) & 15u) == 0 && o.K >= 1;
 }
 
-// One problem of the pair kernel: 256 x 256 tiles, each CTA stages 128 rows of A
-// and 128 rows of B.
-static int pair_problem(PairProblem* P, const __nv_bfloat16* A, int64_t lda, int64_t rowsA, int64_t colsA,
-                        const __nv_bfloat16* B, int64_t ldb, int64_t rowsB, int64_t colsB, int M, int N, int K,
-                        const TcEpi& epi) {
-    if (!tc_shape_ok(lda, ldb, K, 0, A, B)) return fail(DBW_EALIGN, "tc_gemm: unsupported operand alignment");
-    if (!tc_make_map(&P->tmA, A, rowsA, colsA, lda, 64, BM) || !tc_make_map(&P->tmB, B, rowsB, colsB, ldb, 64, 128))
-        return fail(DBW_ECUDA, "tc_gemm: cuTensorMapEncodeTiled failed");
-    P->M = M;
-    P->N = N;
-    P->K = K;
+// One problem of the pair kernel: 256 x 256 tiles, each CTA stages 128 rows (or columns)
+// of A and 128 of B.
+static int pair_problem(PairProblem* P, int kind, const TcOperands& o, const TcEpi& epi) {
+    if (!operands_ok(o)) return fail(DBW_EALIGN, "tc_gemm: unsupported operand alignment");
+    const bool oka = a_mn(kind) ? tc_make_map(&P->tmA, o.A, o.K, o.M, o.lda, 64)
+                                : tc_make_map(&P->tmA, o.A, o.M, o.K, o.lda, BM);
+    const bool okb = b_mn(kind) ? tc_make_map(&P->tmB, o.B, o.K, o.N, o.ldb, 64)
+                                : tc_make_map(&P->tmB, o.B, o.N, o.K, o.ldb, 128);
+    if (!oka || !okb) return fail(DBW_ECUDA, "tc_gemm: cuTensorMapEncodeTiled failed");
+    P->M = o.M;
+    P->N = o.N;
+    P->K = o.K;
     P->epi = epi;
     return DBW_OK;
 }
@@ -1041,9 +1074,9 @@ int tc_gemm_mean_dx(const TcOperands& g, const TcEpi& ge, const TcOperands& x, c
     PairArgs args{};
     args.nprob = 2;
     args.status = status;
-    int rc = pair_problem(&args.p[0], g.A, g.lda, g.rowsA, g.colsA, g.B, g.ldb, g.rowsB, g.colsB, g.M, g.N, g.K, ge);
+    int rc = pair_problem(&args.p[0], TC_GBAR, g, ge);
     if (rc) return rc;
-    rc = pair_problem(&args.p[1], x.A, x.lda, x.rowsA, x.colsA, x.B, x.ldb, x.rowsB, x.colsB, x.M, x.N, x.K, xe);
+    rc = pair_problem(&args.p[1], TC_DX, x, xe);
     if (rc) return rc;
     void* prof = profile_begin(PROF_GEMM, st, 0.0);
     const cudaError_t e = launch_pair<TC_GBAR, TC_DX>(args, st);
@@ -1052,50 +1085,49 @@ int tc_gemm_mean_dx(const TcOperands& g, const TcEpi& ge, const TcOperands& x, c
     return DBW_OK;
 }
 
-int tc_gemm(int kind, const __nv_bfloat16* A, int64_t lda, int64_t rowsA, int64_t colsA, const __nv_bfloat16* B,
-            int64_t ldb, int64_t rowsB, int64_t colsB, int M, int N, int K, int batch, int64_t kz, const TcEpi& epi,
-            int* status, cudaStream_t st) {
-    cudaError_t e = cudaSuccess;
-    if (kind == TC_DW) {
-        if (!tc_shape_ok(lda, ldb, K, kz, A, B)) return fail(DBW_EALIGN, "tc_gemm: unsupported operand alignment");
-        CUtensorMap ta, tb;
-        // K = the per-worker sample count: 64-deep blocks when it allows, else 32
-        const int bk = (K % 64 == 0) ? 64 : 32;
-        // algorithmic bytes: G written once (fp32), both bf16 operands read once
-        const double dw_bytes = 4.0 * batch * double(M) * N + 2.0 * batch * double(K) * (double(M) + N);
-        if (!tc_make_map(&ta, A, rowsA, colsA, lda, bk, BM) || !tc_make_map(&tb, B, rowsB, colsB, ldb, bk, DW_BN))
-            return fail(DBW_ECUDA, "tc_gemm: cuTensorMapEncodeTiled failed");
-        float* gb = epi.G + epi.off;
-        const bool vec_ok = ((reinterpret_cast<uintptr_t>(gb) & 15u) == 0) && epi.ldrow % 4 == 0 && epi.ldG % 4 == 0;
+int tc_dw(const TcOperands& o, int batch, const TcEpi& epi, int* status, cudaStream_t st) {
+    if (!operands_ok(o)) return fail(DBW_EALIGN, "tc_dw: unsupported operand alignment");
+    // 64-deep K blocks unless the worker's samples fit in one 32-deep block
+    const int bk = o.K > 32 ? 64 : 32;
+    CUtensorMap ta, tb;
+    if (!make_batch_map(&ta, o.A, o.K, batch, o.M, o.lda, bk) || !make_batch_map(&tb, o.B, o.K, batch, o.N, o.ldb, bk))
+        return fail(DBW_ECUDA, "tc_dw: cuTensorMapEncodeTiled failed");
+    // algorithmic bytes: G written once (fp32), both bf16 operands read once
+    const double bytes = 4.0 * batch * double(o.M) * o.N + 2.0 * batch * double(o.K) * (double(o.M) + o.N);
+    float* gb = epi.G + epi.off;
+    const bool vec_ok = ((reinterpret_cast<uintptr_t>(gb) & 15u) == 0) && epi.ldrow % 4 == 0 && epi.ldG % 4 == 0;
+    cudaError_t e;
+    void* prof = profile_begin(PROF_DW, st, bytes);
+    if (!vec_ok) {
         // unaligned rows: the one-CTA-per-tile kernel (128-column tiles) with scalar stores
-        if (!vec_ok && !tc_make_map(&tb, B, rowsB, colsB, ldb, bk, 128))
-            return fail(DBW_ECUDA, "tc_gemm: cuTensorMapEncodeTiled failed");
-        void* prof = profile_begin(PROF_DW, st, dw_bytes);
-        if (!vec_ok) {
-            e = bk == 64 ? launch_cfg<128, 64, 2, TC_DW, 4>(ta, tb, M, N, K, batch, kz, epi, status, st, 48 * 1024)
-                         : launch_cfg<128, 32, 2, TC_DW, 4>(ta, tb, M, N, K, batch, kz, epi, status, st, 48 * 1024);
-        } else {
-            e = bk == 64 ? launch_dw<64, 2>(ta, tb, M, N, K, batch, status, gb, epi.ldrow, epi.ldG, st)
-                         : launch_dw<32, 4>(ta, tb, M, N, K, batch, status, gb, epi.ldrow, epi.ldG, st);
-        }
-        profile_end(prof, st);
+        e = bk == 64 ? launch_cfg<128, 64, 2, TC_DW, 4>(ta, tb, o.M, o.N, o.K, batch, epi, status, st, 48 * 1024)
+                     : launch_cfg<128, 32, 2, TC_DW, 4>(ta, tb, o.M, o.N, o.K, batch, epi, status, st, 48 * 1024);
     } else {
-        PairArgs args{};
-        args.nprob = 1;
-        args.status = status;
-        const int rc = pair_problem(&args.p[0], A, lda, rowsA, colsA, B, ldb, rowsB, colsB, M, N, K, epi);
-        if (rc) return rc;
-        void* prof = profile_begin(PROF_GEMM, st, 0.0);
-        if (kind == TC_HIDDEN)
-            e = launch_pair<TC_HIDDEN, TC_HIDDEN>(args, st);
-        else if (kind == TC_LOGITS)
-            e = launch_pair<TC_LOGITS, TC_LOGITS>(args, st);
-        else if (kind == TC_GBAR)
-            e = launch_pair<TC_GBAR, TC_GBAR>(args, st);
-        else
-            e = launch_pair<TC_DX, TC_DX>(args, st);
-        profile_end(prof, st);
+        e = bk == 64 ? launch_dw<64, 2>(ta, tb, o.M, o.N, o.K, batch, status, gb, epi.ldrow, epi.ldG, st)
+                     : launch_dw<32, 4>(ta, tb, o.M, o.N, o.K, batch, status, gb, epi.ldrow, epi.ldG, st);
     }
+    profile_end(prof, st);
+    if (e != cudaSuccess) return fail(DBW_ECUDA, "tc_dw launch: %s", cudaGetErrorString(e));
+    return DBW_OK;
+}
+
+int tc_gemm(int kind, const TcOperands& o, const TcEpi& epi, int* status, cudaStream_t st) {
+    PairArgs args{};
+    args.nprob = 1;
+    args.status = status;
+    const int rc = pair_problem(&args.p[0], kind, o, epi);
+    if (rc) return rc;
+    cudaError_t e;
+    void* prof = profile_begin(PROF_GEMM, st, 0.0);
+    if (kind == TC_HIDDEN)
+        e = launch_pair<TC_HIDDEN, TC_HIDDEN>(args, st);
+    else if (kind == TC_LOGITS)
+        e = launch_pair<TC_LOGITS, TC_LOGITS>(args, st);
+    else if (kind == TC_GBAR)
+        e = launch_pair<TC_GBAR, TC_GBAR>(args, st);
+    else
+        e = launch_pair<TC_DX, TC_DX>(args, st);
+    profile_end(prof, st);
     if (e != cudaSuccess) return fail(DBW_ECUDA, "tc_gemm launch: %s", cudaGetErrorString(e));
     return DBW_OK;
 }

@@ -17,8 +17,6 @@ struct TcEpi {
     const float* bias;            // HIDDEN, LOGITS: + bias[n]
     __nv_bfloat16* out;           // HIDDEN, DX: out[m * ldo + n] (bf16, row-major)
     int64_t ldo;
-    __nv_bfloat16* outT;          // HIDDEN, DX: outT[n * ldT + m] (bf16, transposed), nullable
-    int64_t ldT;
     float* outF;                  // LOGITS: outF[m * ldF + n] (fp32)
     int64_t ldF;
     const __nv_bfloat16* act;     // DX: ReLU mask 1[act[m * ldact + n] > 0]
@@ -40,37 +38,40 @@ struct TcEpi {
     int kmul;
 };
 
-// C[M, N] = sum_{k < K} A[m, z*kz + k] * B[n, z*kz + k] for z < batch, then the
-// epilogue ``kind``.  A is [rowsA >= M, lda] and B is [rowsB >= N, ldb], both
-// row-major bf16 with K contiguous (lda, ldb multiples of 8, bases 16-byte
-// aligned, z*kz a multiple of 8).  colsA / colsB: the logical column count of A
-// / B (reads past it are zero).  ``status`` (device int) gets bit 0 set if a
-// pipeline wait ever times out; it must be zeroed by the caller.
-int tc_gemm(int kind, const __nv_bfloat16* A, int64_t lda, int64_t rowsA, int64_t colsA, const __nv_bfloat16* B,
-            int64_t ldb, int64_t rowsB, int64_t colsB, int M, int N, int K, int batch, int64_t kz, const TcEpi& epi,
-            int* status, cudaStream_t st);
+// Operands of one GEMM, both row-major bf16 as their producers left them (ld multiples of
+// 8 elements, bases 16-byte aligned):
+//   HIDDEN, LOGITS  C[m, n] = sum_k A[m, k] B[n, k]   A [M, lda], B [N, ldb]
+//   DX              C[m, n] = sum_k A[m, k] B[k, n]   A [M, lda], B [K, ldb]
+//   GBAR            C[m, n] = sum_k A[k, m] B[k, n]   A [K, lda], B [K, ldb]
+// An operand whose K runs along its rows is read as an MN-major tile: no transposed copy
+// of the weights, the activations or dZ exists.
+struct TcOperands {
+    const __nv_bfloat16* A;
+    int64_t lda;
+    const __nv_bfloat16* B;
+    int64_t ldb;
+    int M, N, K;
+};
+
+// The GEMM and then the epilogue ``kind`` (HIDDEN, LOGITS, DX or GBAR).  ``status``
+// (device int) gets bit 0 set if a pipeline wait ever times out; it must be zeroed by
+// the caller.
+int tc_gemm(int kind, const TcOperands& o, const TcEpi& epi, int* status, cudaStream_t st);
+
+// Per-worker weight gradients: for z < batch, C_z[m, n] = sum_{r < B} A[z B + r, m] B_[z B + r, n]
+// (A = dZ, o.M = out; o.B = the layer input, o.N = in; o.K = B samples per worker, any
+// B >= 1: a worker's rows past B read as zero), stored by the TC_DW epilogue.
+int tc_dw(const TcOperands& o, int batch, const TcEpi& epi, int* status, cudaStream_t st);
 
 // 2-D TMA tensor map of a row-major bf16 matrix [rows, cols] with row stride ld
-// (elements), box box_k x box_rows, 128-byte (box_k = 64) or 64-byte (32) swizzle;
-// reads past the extents are zero.  False if the driver's encoder is unavailable
-// or rejects the arguments.
-bool tc_make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_k, int box_rows);
+// (elements), box 64 columns (128 bytes, 128-byte swizzle) x box_rows; reads past the
+// extents are zero.  False if the driver's encoder is unavailable or rejects the
+// arguments.
+bool tc_make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows);
 
 // The same for a row-major fp32 matrix: box 32 (128 bytes, 128-byte swizzle) x box_rows;
 // ld a multiple of 4 and base 16-byte aligned.
 bool tc_make_map_f32(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows);
-
-// True when tc_gemm can run this problem (alignment rules above).
-bool tc_shape_ok(int64_t lda, int64_t ldb, int K, int64_t kz, const void* A, const void* B);
-
-// Operands of one GEMM of tc_gemm_mean_dx (the same meaning as tc_gemm's arguments).
-struct TcOperands {
-    const __nv_bfloat16* A;
-    int64_t lda, rowsA, colsA;
-    const __nv_bfloat16* B;
-    int64_t ldb, rowsB, colsB;
-    int M, N, K;
-};
 
 // The mean-gradient GEMM (TC_GBAR, operands g, epilogue ge) and the input-gradient
 // GEMM (TC_DX, operands x, epilogue xe) of one layer in one launch: both read dZ_l

@@ -43,21 +43,16 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
 // leading dimension (ld*) a multiple of 8 elements.
 struct TcPlan {
     GradsPlan g;                       // shapes and parameter offsets
-    int64_t M8;                        // leading dimension of the transposed [width, M] buffers
     size_t off_status;                 // device int: bit 0 = a pipeline wait timed out
     size_t off_wb[DBW_LMAX];           // W_l bf16 [out, ldw]
     int64_t ldw[DBW_LMAX];
-    size_t off_wt[DBW_LMAX];           // W_l^T bf16 [in, ldwt]
-    int64_t ldwt[DBW_LMAX];
     size_t off_act[DBW_LMAX];          // layer-l input bf16 [M, ldact] (act[0] = X)
     int64_t ldact[DBW_LMAX];
-    size_t off_actT[DBW_LMAX];         // its transpose bf16 [width, M8]
     size_t off_logits;                 // fp32 [M, ldlog]
     int64_t ldlog;
     size_t off_sloss;                  // fp32 [M]
     size_t off_dz[2];                  // bf16 [M, ldz] ping-pong
     int64_t ldz;
-    size_t off_dzT;                    // bf16 [max width, M8]
     size_t ws_bytes;
 };
 
@@ -76,8 +71,6 @@ struct RxPlan {
     size_t off_pb[DBW_LMAX];           // fp64 [ceil(out_l / 256)]: pieces of ||g_t(b_l)||^2
     int npb[DBW_LMAX];
     size_t off_pg[DBW_LMAX];           // fp64 [(M / 32) * CT]: Gram pieces of ||g_j||^2
-    size_t off_dzT2;                   // bf16 [max width, M8]: second dZ^T buffer (the dX GEMM of a layer
-                                       // writes dZ_{l-1}^T while the mean-gradient GEMM reads dZ_l^T)
     size_t off_gpart;                  // fp32: partial Gram products of the K ranges (shared by the layers)
     size_t off_gcnt;                   // int32 [gram items]: per-item range counters, zeroed at the start of a call
     int ngcnt;

@@ -2,23 +2,25 @@
 //
 // Same computation as the SIMT pass in grads.cu (forward over the stacked
 // M = n B rows, softmax cross entropy, backward with a per-worker weight
-// gradient of depth K = B), laid out so that every GEMM has both operands
-// K-major, which is what the tcgen05 kernel of gemm_tc.cu consumes:
+// gradient of depth K = B) on the GEMMs of gemm_tc.cu:
 //
 //   forward   Z_l = A_{l-1} . W_l^T          A = act[l-1] [M, in],   B = W_l [out, in]
-//   dX        dZ_{l-1} = dZ_l . W_l          A = dZ_l [M, out],      B = W_l^T [in, out]
-//   dW        G_i = dZ_l[i]^T . A_{l-1}[i]   A = dZ_l^T [out, M],    B = A_{l-1}^T [in, M]
-//                                            (worker i: columns i*B .. i*B+B-1, K = B)
+//   dX        dZ_{l-1} = dZ_l . W_l          A = dZ_l [M, out],      B = W_l [out, in]
+//   dW        G_i = dZ_l[i]^T . A_{l-1}[i]   A = dZ_l [M, out],      B = act[l-1] [M, in]
+//                                            (worker i: rows i*B .. i*B+B-1, K = B)
 //
-// The transposed activations and dZ are written by the epilogue that produces
-// them (a store whose 32 lanes cover 32 consecutive samples, 64 contiguous
-// bytes), X^T and dZ_L^T by a tiled transpose, W^T by a tiled cast-transpose.
+// Every operand is the row-major bf16 buffer its producer wrote: the tensor cores read
+// dZ, the activations and (in dX) W as MN-major tiles, so no transposed copy is formed.
+// With transposed copies (written by the GEMM epilogues, the X and W casts and the
+// softmax) the 3072-1024-1024-10 pass of 128 x 128 samples took 827 us, and those copies
+// were a third of the casts' bytes and half of the epilogues' stores.
 // Leading dimensions are padded to multiples of 8 elements (16 bytes, the TMA
 // stride rule); padding is never read (tensor maps carry the logical extents).
 #include <math.h>
 
 #include "gemm_tc.cuh"
 #include "grads.cuh"
+#include "tc_ptx.cuh"
 
 namespace dbw {
 
@@ -26,120 +28,78 @@ namespace {
 
 inline int64_t rup(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
-// One pass over fp32 rows: out[m, :] = bf16(src[row(m), :]) and outT = its
-// transpose, for m < rows (cols logical columns; padding is never written).  A
-// CTA handles a 64 x 64 tile: the rows are read as float4 where aligned, the
-// bf16 tile is written row-major with 8-byte stores and, through a padded
-// shared-memory tile, column-major with 8-byte stores along m.  row(m) < 0 makes
-// row m zero.  Used for X (gathered minibatch rows) and for W_l (rows = out).
+// out[m, :] = bf16(src[row(m), :]) for one row of ``cols`` values, by one warp: a lane
+// takes groups of 8 columns (two 16-byte loads, one 16-byte store), four groups' loads in
+// flight.  src rows are 16-byte aligned when ``vec``; ldo is a multiple of 8.
+__device__ __forceinline__ void cast_row(const float* __restrict__ s, int cols, __nv_bfloat16* __restrict__ o,
+                                         bool vec) {
+    const int lane = threadIdx.x & 31;
+    const int groups = vec ? cols / 8 : 0;
+    for (int g0 = lane; g0 < groups; g0 += 128) {
+        float4 v[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int g = g0 + 32 * u;
+            if (g < groups) {
+                v[u][0] = __ldcs(reinterpret_cast<const float4*>(s) + 2 * g);
+                v[u][1] = __ldcs(reinterpret_cast<const float4*>(s) + 2 * g + 1);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int g = g0 + 32 * u;
+            if (g < groups) {
+                uint4 h;
+                h.x = tcx::pack_bf16(v[u][0].x, v[u][0].y);
+                h.y = tcx::pack_bf16(v[u][0].z, v[u][0].w);
+                h.z = tcx::pack_bf16(v[u][1].x, v[u][1].y);
+                h.w = tcx::pack_bf16(v[u][1].z, v[u][1].w);
+                reinterpret_cast<uint4*>(o)[g] = h;
+            }
+        }
+    }
+    for (int c = 8 * groups + lane; c < cols; c += 32) o[c] = __float2bfloat16_rn(s[c]);
+}
+
+// X: out[m, :] = bf16(src[rowmap(m), :]) for the live rows; rowmap(m) < 0 makes row m
+// zero.  A warp per row, grid-stride.  The pool's rows are 16-byte aligned (the width is
+// a multiple of 4 and the base aligned: checked by the caller).
 template <class RowMap>
-__device__ __forceinline__ void cast_transpose_tile(const float* __restrict__ src, int64_t lds, int rows, int cols,
-                                                    RowMap rowmap, __nv_bfloat16* __restrict__ out, int64_t ldo,
-                                                    __nv_bfloat16* __restrict__ outT, int64_t ldT, int c0, int m0) {
-    __shared__ __nv_bfloat16 tile[64][64 + 8];
+__global__ void __launch_bounds__(256) cast_rows_kernel(const float* __restrict__ src, int64_t lds, int rows, int cols,
+                                                        RowMap rowmap, __nv_bfloat16* __restrict__ out, int64_t ldo) {
     const int live = rowmap.live(rows);
-    if (m0 >= live) return;
-    const int t = threadIdx.x;
-    // all four rows' loads first, so that each thread has 64 bytes in flight
-    float v[4][4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int e = t + 256 * q;
-        const int r = e >> 4, c = c0 + 4 * (e & 15);
-        const int m = m0 + r;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[q][j] = 0.f;
-        if (m < live && c < cols) {
-            const int64_t sr = rowmap(m);
-            if (sr >= 0) {
-                const float* p = src + sr * lds + c;
-                if (c + 3 < cols && ((reinterpret_cast<uintptr_t>(p) & 15u) == 0)) {
-                    const float4 f = __ldcs(reinterpret_cast<const float4*>(p));
-                    v[q][0] = f.x, v[q][1] = f.y, v[q][2] = f.z, v[q][3] = f.w;
-                } else {
-                    for (int j = 0; j < 4 && c + j < cols; ++j) v[q][j] = p[j];
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int e = t + 256 * q;
-        const int r = e >> 4, c = c0 + 4 * (e & 15);
-        const int m = m0 + r;
-        __nv_bfloat16 h[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) h[j] = __float2bfloat16_rn(v[q][j]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) tile[r][4 * (e & 15) + j] = h[j];
-        if (m < live && c < cols) {
-            __nv_bfloat16* o = out + static_cast<int64_t>(m) * ldo + c;
-            if (c + 3 < cols && ((reinterpret_cast<uintptr_t>(o) & 7u) == 0)) {
-                uint2 pk;
-                pk.x = static_cast<uint32_t>(__bfloat16_as_ushort(h[0])) |
-                       (static_cast<uint32_t>(__bfloat16_as_ushort(h[1])) << 16);
-                pk.y = static_cast<uint32_t>(__bfloat16_as_ushort(h[2])) |
-                       (static_cast<uint32_t>(__bfloat16_as_ushort(h[3])) << 16);
-                *reinterpret_cast<uint2*>(o) = pk;
-            } else {
-                for (int j = 0; j < 4 && c + j < cols; ++j) o[j] = h[j];
-            }
-        }
-    }
-    __syncthreads();
-    if (!outT) return;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int e = t + 256 * q;
-        const int cc = e >> 4, r = 4 * (e & 15);
-        const int c = c0 + cc, m = m0 + r;
-        if (c >= cols || m >= live) continue;
-        __nv_bfloat16* o = outT + static_cast<int64_t>(c) * ldT + m;
-        if (m + 3 < live && ((reinterpret_cast<uintptr_t>(o) & 7u) == 0)) {
-            uint2 pk;
-            pk.x = static_cast<uint32_t>(__bfloat16_as_ushort(tile[r][cc])) |
-                   (static_cast<uint32_t>(__bfloat16_as_ushort(tile[r + 1][cc])) << 16);
-            pk.y = static_cast<uint32_t>(__bfloat16_as_ushort(tile[r + 2][cc])) |
-                   (static_cast<uint32_t>(__bfloat16_as_ushort(tile[r + 3][cc])) << 16);
-            *reinterpret_cast<uint2*>(o) = pk;
+    const int warps = gridDim.x * (blockDim.x >> 5);
+    for (int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < live; m += warps) {
+        const int64_t sr = rowmap(m);
+        __nv_bfloat16* o = out + static_cast<int64_t>(m) * ldo;
+        if (sr >= 0) {
+            cast_row(src + sr * lds, cols, o, true);
         } else {
-            for (int j = 0; j < 4 && m + j < live; ++j) o[j] = tile[r + j][cc];
+            for (int c = threadIdx.x & 31; c < cols; c += 32) o[c] = __float2bfloat16_rn(0.f);
         }
     }
 }
 
-template <class RowMap>
-__global__ void __launch_bounds__(256) cast_transpose_tile_kernel(const float* __restrict__ src, int64_t lds,
-                                                                  int rows, int cols, RowMap rowmap,
-                                                                  __nv_bfloat16* __restrict__ out, int64_t ldo,
-                                                                  __nv_bfloat16* __restrict__ outT, int64_t ldT) {
-    cast_transpose_tile(src, lds, rows, cols, rowmap, out, ldo, outT, ldT, blockIdx.x * 64, blockIdx.y * 64);
-}
-
-// Row maps of cast_transpose_tile_kernel.
-struct IdentityRows {   // W_l: row o of the matrix
-    __device__ int live(int rows) const { return rows; }
-    __device__ int64_t operator()(int m) const { return m; }
-};
-// Every layer's W_l -> bf16 W_l and W_l^T in one launch: the layers' 64 x 64 tiles one
-// after the other in x (t0: first tile of layer l; tx: its tiles per row of tiles).
+// Every layer's W_l -> bf16 in one launch: a warp per row, the layers' rows one after the
+// other (r0: first row of layer l).
 struct WeightCasts {
     int L;
     const float* w[DBW_LMAX];
-    int fin[DBW_LMAX], fout[DBW_LMAX], tx[DBW_LMAX];
-    int t0[DBW_LMAX + 1];
+    int fin[DBW_LMAX];
+    int r0[DBW_LMAX + 1];
+    bool vec[DBW_LMAX];       // rows of W_l 16-byte aligned
     __nv_bfloat16* wb[DBW_LMAX];
     int64_t ldw[DBW_LMAX];
-    __nv_bfloat16* wt[DBW_LMAX];
-    int64_t ldwt[DBW_LMAX];
 };
 
-__global__ void __launch_bounds__(256) cast_transpose_weights_kernel(WeightCasts a) {
-    int l = 0;
-    while (l + 1 < a.L && static_cast<int>(blockIdx.x) >= a.t0[l + 1]) ++l;
-    const int t = blockIdx.x - a.t0[l];
-    cast_transpose_tile(a.w[l], a.fin[l], a.fout[l], a.fin[l], IdentityRows{}, a.wb[l], a.ldw[l], a.wt[l], a.ldwt[l],
-                        (t % a.tx[l]) * 64, (t / a.tx[l]) * 64);
+__global__ void __launch_bounds__(256) cast_weights_kernel(WeightCasts a) {
+    const int warps = gridDim.x * (blockDim.x >> 5);
+    for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < a.r0[a.L]; r += warps) {
+        int l = 0;
+        while (l + 1 < a.L && r >= a.r0[l + 1]) ++l;
+        const int64_t o = r - a.r0[l];
+        cast_row(a.w[l] + o * a.fin[l], a.fin[l], a.wb[l] + o * a.ldw[l], a.vec[l]);
+    }
 }
 
 struct GatherRows {     // X of the per-worker pass: pool row idx[m]; an index outside [0, S) reads row 0
@@ -179,47 +139,9 @@ struct ReceivedRows {
     }
 };
 
-// dst [cols, ldd] = src [rows, lds]^T  (bf16), rows x cols logical; with kdev, only
-// the live rows (live_rows) are transposed.
-__global__ void transpose_bf16_kernel(const __nv_bfloat16* __restrict__ src, int rows, int cols, int64_t lds,
-                                      __nv_bfloat16* __restrict__ dst, int64_t ldd, const int* kdev = nullptr,
-                                      int B = 0) {
-    __shared__ __nv_bfloat16 tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    rows = live_rows(kdev, B, rows);
-    if (r0 >= rows) return;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    for (int r = ty; r < 32; r += 8) {
-        const int rr = r0 + r, cc = c0 + tx;
-        tile[r][tx] = (rr < rows && cc < cols) ? src[static_cast<int64_t>(rr) * lds + cc] : __float2bfloat16_rn(0.f);
-    }
-    __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
-        const int cc = c0 + r, rr = r0 + tx;
-        if (cc < cols && rr < rows) dst[static_cast<int64_t>(cc) * ldd + rr] = tile[tx][r];
-    }
-}
-
 // With ``sel`` (received-workers pass): CTA s handles slot s, i.e. worker sel[s]
 // (stacked rows s B .., samples idx[sel[s] B + r], loss[sel[s]]); slots s >= k
 // zero their dZ rows up to the live row count and stop.
-// With ``dZT`` the CTA also writes its rows of the transposed copy dZT [C, ldT]
-// (columns i B .. i B + B - 1): the bf16 values go through a [B, C + 8] shared tile
-// (dynamic shared memory) and leave as 16-byte pieces of 8 rows.
-__device__ __forceinline__ void write_dzT(const __nv_bfloat16* tile, int C, int B, int64_t col0, int rows_live,
-                                          __nv_bfloat16* __restrict__ dZT, int64_t ldT) {
-    const int groups = B / 8;   // B % 32 == 0 on the tcgen05 path
-    for (int q = threadIdx.x; q < C * groups; q += blockDim.x) {
-        const int c = q / groups, g8 = q % groups;
-        if (8 * g8 >= rows_live) continue;
-        uint4 v;
-        __nv_bfloat16* h = reinterpret_cast<__nv_bfloat16*>(&v);
-#pragma unroll
-        for (int t = 0; t < 8; ++t) h[t] = tile ? tile[(8 * g8 + t) * (C + 8) + c] : __float2bfloat16_rn(0.f);
-        *reinterpret_cast<uint4*>(dZT + static_cast<int64_t>(c) * ldT + col0 + 8 * g8) = v;
-    }
-}
-
 __global__ void __launch_bounds__(256) softmax_xent_ld_kernel(const float* __restrict__ logits, int64_t ldl, int C,
                                                               int B, const int32_t* __restrict__ idx, int64_t S,
                                                               const int32_t* __restrict__ labels,
@@ -227,10 +149,7 @@ __global__ void __launch_bounds__(256) softmax_xent_ld_kernel(const float* __res
                                                               __nv_bfloat16* __restrict__ dZ, int64_t ldz,
                                                               float* __restrict__ loss,
                                                               const int32_t* __restrict__ sel = nullptr,
-                                                              const int* __restrict__ kdev = nullptr,
-                                                              __nv_bfloat16* __restrict__ dZT = nullptr,
-                                                              int64_t ldT = 0) {
-    extern __shared__ __nv_bfloat16 tileT[];   // [B][C + 8] when dZT is given
+                                                              const int* __restrict__ kdev = nullptr) {
     const int i = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     int worker = i;
@@ -240,7 +159,6 @@ __global__ void __launch_bounds__(256) softmax_xent_ld_kernel(const float* __res
             for (int r = warp; r < B && i * B + r < live; r += nw)
                 for (int c = lane; c < C; c += 32)
                     dZ[(static_cast<int64_t>(i) * B + r) * ldz + c] = __float2bfloat16_rn(0.f);
-            if (dZT) write_dzT(nullptr, C, B, static_cast<int64_t>(i) * B, live - i * B, dZT, ldT);
             return;
         }
         worker = sel[i];
@@ -285,9 +203,7 @@ __global__ void __launch_bounds__(256) softmax_xent_ld_kernel(const float* __res
                 if (c < C) {
                     float g = v[j] * inv_se;
                     if (c == y) g -= 1.0f;
-                    const __nv_bfloat16 h = __float2bfloat16_rn(bad ? NAN : g * invB);
-                    dZ[row * ldz + c] = h;
-                    if (dZT) tileT[r * (C + 8) + c] = h;
+                    dZ[row * ldz + c] = __float2bfloat16_rn(bad ? NAN : g * invB);
                 }
             }
         } else {
@@ -301,9 +217,7 @@ __global__ void __launch_bounds__(256) softmax_xent_ld_kernel(const float* __res
             for (int c = lane; c < C; c += 32) {
                 float g = expf(z[c] - mx) * inv_se;
                 if (c == y) g -= 1.0f;
-                const __nv_bfloat16 h = __float2bfloat16_rn(bad ? NAN : g * invB);
-                dZ[row * ldz + c] = h;
-                if (dZT) tileT[r * (C + 8) + c] = h;
+                dZ[row * ldz + c] = __float2bfloat16_rn(bad ? NAN : g * invB);
             }
         }
         if (lane == 0) {
@@ -320,14 +234,6 @@ __global__ void __launch_bounds__(256) softmax_xent_ld_kernel(const float* __res
         for (int r = 0; r < B; ++r) acc += r < kShared ? ls[r] : sample_loss[static_cast<int64_t>(i) * B + r];
         loss[worker] = bad_s ? NAN : acc * invB;
     }
-    if (dZT) write_dzT(tileT, C, B, static_cast<int64_t>(i) * B, B, dZT, ldT);
-}
-
-// Shared memory of softmax_xent_ld_kernel's transposing tile, or 0 when it does not
-// fit (the transpose then runs as transpose_bf16_kernel).
-inline int softmax_tile_bytes(int B, int C) {
-    const long long bytes = static_cast<long long>(B) * (C + 8) * 2;
-    return bytes <= 160 * 1024 ? static_cast<int>(bytes) : 0;
 }
 
 // G[i, offb + o] = sum_{r < B} dZ[i*B + r, o] (rows in order).
@@ -535,26 +441,27 @@ __global__ void __launch_bounds__(kFinishThreads) finish_received_kernel(FinishA
 
 bool tc_eligible(int prec, int B) { return prec == DBW_PREC_BF16 && B % 32 == 0; }
 
-// bf16 W_l and W_l^T of every layer (one launch).
+// CTAs of a warp-per-row kernel over ``rows`` rows (8 warps each, at most 8 per SM).
+static int row_ctas(int64_t rows) {
+    const int64_t want = (rows + 7) / 8, most = 8 * sm_count();
+    return static_cast<int>(want < most ? want : most);
+}
+
+// bf16 W_l of every layer (one launch).
 static void launch_weight_casts(const TcPlan& P, const float* w, char* ws, cudaStream_t st) {
     const GradsPlan& g = P.g;
     WeightCasts a{};
     a.L = g.L;
-    a.t0[0] = 0;
+    a.r0[0] = 0;
     for (int l = 0; l < g.L; ++l) {
-        const int fin = g.widths[l], fout = g.widths[l + 1];
         a.w[l] = w + g.offW[l];
-        a.fin[l] = fin;
-        a.fout[l] = fout;
-        a.tx[l] = (fin + 63) / 64;
-        a.t0[l + 1] = a.t0[l] + a.tx[l] * ((fout + 63) / 64);
+        a.fin[l] = g.widths[l];
+        a.r0[l + 1] = a.r0[l] + g.widths[l + 1];
+        a.vec[l] = aligned16(a.w[l]) && g.widths[l] % 4 == 0;
         a.wb[l] = reinterpret_cast<__nv_bfloat16*>(ws + P.off_wb[l]);
         a.ldw[l] = P.ldw[l];
-        // no input gradient is formed for the first layer: W_0^T is never read
-        a.wt[l] = l == 0 ? nullptr : reinterpret_cast<__nv_bfloat16*>(ws + P.off_wt[l]);
-        a.ldwt[l] = P.ldwt[l];
     }
-    cast_transpose_weights_kernel<<<a.t0[g.L], 256, 0, st>>>(a);
+    cast_weights_kernel<<<row_ctas(a.r0[g.L]), 256, 0, st>>>(a);
 }
 
 bool make_tc_plan(int L, const int32_t* widths, int n, int B, TcPlan* P) {
@@ -562,7 +469,6 @@ bool make_tc_plan(int L, const int32_t* widths, int n, int B, TcPlan* P) {
     if (!make_grads_plan(L, widths, n, B, DBW_PREC_BF16, &g)) return false;
     P->g = g;
     const int64_t M = static_cast<int64_t>(n) * B;
-    P->M8 = rup(M, 8);
     int maxw = 0;
     for (int l = 0; l <= L; ++l) maxw = widths[l] > maxw ? widths[l] : maxw;
     size_t cur = 0;
@@ -573,16 +479,12 @@ bool make_tc_plan(int L, const int32_t* widths, int n, int B, TcPlan* P) {
     };
     P->off_status = take(256);
     for (int l = 0; l < L; ++l) {
-        const int fin = widths[l], fout = widths[l + 1];
-        P->ldw[l] = rup(fin, 8);
-        P->ldwt[l] = rup(fout, 8);
-        P->off_wb[l] = take(static_cast<size_t>(fout) * P->ldw[l] * 2);
-        P->off_wt[l] = take(static_cast<size_t>(fin) * P->ldwt[l] * 2);
+        P->ldw[l] = rup(widths[l], 8);
+        P->off_wb[l] = take(static_cast<size_t>(widths[l + 1]) * P->ldw[l] * 2);
     }
     for (int l = 0; l < L; ++l) {   // act[0] = X
         P->ldact[l] = rup(widths[l], 8);
         P->off_act[l] = take(static_cast<size_t>(M) * P->ldact[l] * 2);
-        P->off_actT[l] = take(static_cast<size_t>(widths[l]) * P->M8 * 2);
     }
     P->ldlog = rup(widths[L], 4);
     P->off_logits = take(static_cast<size_t>(M) * P->ldlog * 4);
@@ -590,7 +492,6 @@ bool make_tc_plan(int L, const int32_t* widths, int n, int B, TcPlan* P) {
     P->ldz = rup(maxw, 8);
     P->off_dz[0] = take(static_cast<size_t>(M) * P->ldz * 2);
     P->off_dz[1] = take(static_cast<size_t>(M) * P->ldz * 2);
-    P->off_dzT = take(static_cast<size_t>(maxw) * P->M8 * 2);
     P->ws_bytes = cur;
     return true;
 }
@@ -604,55 +505,36 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
     cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
 
-    // bf16 weights and their transposes
     launch_weight_casts(P, w, ws, st);
-    // X and X^T
-    {
-        const int in = g.widths[0];
-        dim3 grid((in + 63) / 64, (M + 63) / 64);
-        cast_transpose_tile_kernel<<<grid, 256, 0, st>>>(pool, in, M, in, GatherRows{idx, S}, bf(P.off_act[0]),
-                                                         P.ldact[0], bf(P.off_actT[0]), P.M8);
-    }
+    cast_rows_kernel<<<row_ctas(M), 256, 0, st>>>(pool, g.widths[0], M, g.widths[0], GatherRows{idx, S},
+                                                  bf(P.off_act[0]), P.ldact[0]);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
 
     // forward
     float* logits = reinterpret_cast<float*>(ws + P.off_logits);
     for (int l = 0; l < L; ++l) {
-        const int fin = g.widths[l], fout = g.widths[l + 1];
+        const TcOperands fo{bf(P.off_act[l]), P.ldact[l], bf(P.off_wb[l]), P.ldw[l], M, g.widths[l + 1], g.widths[l]};
         TcEpi ep{};
         ep.bias = w + g.offb[l];
         int rc;
         if (l < L - 1) {
             ep.out = bf(P.off_act[l + 1]);
             ep.ldo = P.ldact[l + 1];
-            ep.outT = bf(P.off_actT[l + 1]);
-            ep.ldT = P.M8;
-            rc = tc_gemm(TC_HIDDEN, bf(P.off_act[l]), P.ldact[l], M, fin, bf(P.off_wb[l]), P.ldw[l], fout, fin, M,
-                         fout, fin, 1, 0, ep, status, st);
+            rc = tc_gemm(TC_HIDDEN, fo, ep, status, st);
         } else {
             ep.outF = logits;
             ep.ldF = P.ldlog;
-            rc = tc_gemm(TC_LOGITS, bf(P.off_act[l]), P.ldact[l], M, fin, bf(P.off_wb[l]), P.ldw[l], fout, fin, M,
-                         fout, fin, 1, 0, ep, status, st);
+            rc = tc_gemm(TC_LOGITS, fo, ep, status, st);
         }
         if (rc) return rc;
     }
-    // loss, dZ_L and its transpose
+    // loss and dZ_L
     const int C = g.widths[L];
     float* sloss = reinterpret_cast<float*>(ws + P.off_sloss);
     int cur = 0;
-    if (const int tb = softmax_tile_bytes(B, C)) {
-        e = cudaFuncSetAttribute(softmax_xent_ld_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tb);
-        if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
-        softmax_xent_ld_kernel<<<n, 256, tb, st>>>(logits, P.ldlog, C, B, idx, S, labels, sloss, bf(P.off_dz[0]),
-                                                   P.ldz, loss, nullptr, nullptr, bf(P.off_dzT), P.M8);
-    } else {
-        softmax_xent_ld_kernel<<<n, 256, 0, st>>>(logits, P.ldlog, C, B, idx, S, labels, sloss, bf(P.off_dz[0]),
-                                                  P.ldz, loss);
-        dim3 tg((C + 31) / 32, (M + 31) / 32);
-        transpose_bf16_kernel<<<tg, dim3(32, 8), 0, st>>>(bf(P.off_dz[0]), M, C, P.ldz, bf(P.off_dzT), P.M8);
-    }
+    softmax_xent_ld_kernel<<<n, 256, 0, st>>>(logits, P.ldlog, C, B, idx, S, labels, sloss, bf(P.off_dz[0]), P.ldz,
+                                              loss);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
 
@@ -664,8 +546,7 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
         ep.ldG = ld;
         ep.off = g.offW[l];
         ep.ldrow = fin;
-        int rc = tc_gemm(TC_DW, bf(P.off_dzT), P.M8, fout, M, bf(P.off_actT[l]), P.M8, fin, M, fout, fin, B, n, B,
-                         ep, status, st);
+        int rc = tc_dw({bf(P.off_dz[cur]), P.ldz, bf(P.off_act[l]), P.ldact[l], fout, fin, B}, n, ep, status, st);
         if (rc) return rc;
         bias_grad_ld_kernel<<<dim3((fout + 127) / 128, n), 128, 0, st>>>(bf(P.off_dz[cur]), P.ldz, fout, B, G, ld,
                                                                           g.offb[l]);
@@ -677,10 +558,7 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
             ex.ldact = P.ldact[l];
             ex.out = bf(P.off_dz[cur ^ 1]);
             ex.ldo = P.ldz;
-            ex.outT = bf(P.off_dzT);
-            ex.ldT = P.M8;
-            rc = tc_gemm(TC_DX, bf(P.off_dz[cur]), P.ldz, M, fout, bf(P.off_wt[l]), P.ldwt[l], fin, fout, M, fin,
-                         fout, 1, 0, ex, status, st);
+            rc = tc_gemm(TC_DX, {bf(P.off_dz[cur]), P.ldz, bf(P.off_wb[l]), P.ldw[l], M, fin, fout}, ex, status, st);
             if (rc) return rc;
             cur ^= 1;
         }
@@ -711,8 +589,6 @@ bool make_rx_plan(int L, const int32_t* widths, int n, int B, RxPlan* P) {
     };
     P->off_sel = take(static_cast<size_t>(n) * 4);
     P->off_k = take(4);
-    int maxout = 0;
-    for (int l = 0; l < L; ++l) maxout = g.widths[l + 1] > maxout ? g.widths[l + 1] : maxout;
     for (int l = 0; l < L; ++l)   // bias column sums per 256-row chunk, per layer
         P->off_bpart[l] = take(static_cast<size_t>((g.M + 255) / 256) * g.widths[l + 1] * 4);
     // dZ_l of every layer stays until the bias sums and the Gram norms of all layers run
@@ -729,7 +605,6 @@ bool make_rx_plan(int L, const int32_t* widths, int n, int B, RxPlan* P) {
         P->off_pb[l] = take(static_cast<size_t>(P->npb[l]) * 8);
         P->off_pg[l] = take(static_cast<size_t>(g.M / 32) * P->CT * 8);
     }
-    P->off_dzT2 = take(static_cast<size_t>(maxout > g.widths[0] ? maxout : g.widths[0]) * P->t.M8 * 2);
     P->off_gpart = take(tc_gram_partial_floats(g.M, B, L) * 4);
     P->ngcnt = static_cast<int>(tc_gram_items(g.M, B, L));
     P->off_gcnt = take(static_cast<size_t>(P->ngcnt) * 4);
@@ -756,19 +631,15 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
     float* gpart = reinterpret_cast<float*>(ws + P.off_gpart);
     compact_received_kernel<<<1, 1024, 0, st>>>(mask, n, sel, kdev, loss, gcnt, P.ngcnt);
     launch_weight_casts(T, w, ws, st);
-    {
-        const int in = g.widths[0];
-        dim3 grid((in + 63) / 64, (M + 63) / 64);
-        cast_transpose_tile_kernel<<<grid, 256, 0, st>>>(pool, in, M, in, ReceivedRows{idx, sel, kdev, B, S},
-                                                         bf(T.off_act[0]), T.ldact[0], bf(T.off_actT[0]), T.M8);
-    }
+    cast_rows_kernel<<<row_ctas(M), 256, 0, st>>>(pool, g.widths[0], M, g.widths[0], ReceivedRows{idx, sel, kdev, B, S},
+                                                  bf(T.off_act[0]), T.ldact[0]);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 
     // forward over the live rows
     float* logits = reinterpret_cast<float*>(ws + T.off_logits);
     for (int l = 0; l < L; ++l) {
-        const int fin = g.widths[l], fout = g.widths[l + 1];
+        const TcOperands fo{bf(T.off_act[l]), T.ldact[l], bf(T.off_wb[l]), T.ldw[l], M, g.widths[l + 1], g.widths[l]};
         TcEpi ep{};
         ep.bias = w + g.offb[l];
         ep.kdev = kdev;
@@ -777,41 +648,23 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
         if (l < L - 1) {
             ep.out = bf(T.off_act[l + 1]);
             ep.ldo = T.ldact[l + 1];
-            ep.outT = bf(T.off_actT[l + 1]);
-            ep.ldT = T.M8;
-            rc = tc_gemm(TC_HIDDEN, bf(T.off_act[l]), T.ldact[l], M, fin, bf(T.off_wb[l]), T.ldw[l], fout, fin, M,
-                         fout, fin, 1, 0, ep, status, st);
+            rc = tc_gemm(TC_HIDDEN, fo, ep, status, st);
         } else {
             ep.outF = logits;
             ep.ldF = T.ldlog;
-            rc = tc_gemm(TC_LOGITS, bf(T.off_act[l]), T.ldact[l], M, fin, bf(T.off_wb[l]), T.ldw[l], fout, fin, M,
-                         fout, fin, 1, 0, ep, status, st);
+            rc = tc_gemm(TC_LOGITS, fo, ep, status, st);
         }
         if (rc) return rc;
     }
     const int C = g.widths[L];
     float* sloss = reinterpret_cast<float*>(ws + T.off_sloss);
-    if (const int tb = softmax_tile_bytes(B, C)) {
-        e = cudaFuncSetAttribute(softmax_xent_ld_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tb);
-        if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
-        softmax_xent_ld_kernel<<<n, 256, tb, st>>>(logits, T.ldlog, C, B, idx, S, labels, sloss,
-                                                   bf(P.off_dzl[L - 1]), T.ldz, loss, sel, kdev, bf(T.off_dzT), T.M8);
-    } else {
-        softmax_xent_ld_kernel<<<n, 256, 0, st>>>(logits, T.ldlog, C, B, idx, S, labels, sloss, bf(P.off_dzl[L - 1]),
-                                                  T.ldz, loss, sel, kdev);
-        dim3 tg((C + 31) / 32, (M + 31) / 32);
-        transpose_bf16_kernel<<<tg, dim3(32, 8), 0, st>>>(bf(P.off_dzl[L - 1]), M, C, T.ldz, bf(T.off_dzT), T.M8, kdev,
-                                                          B);
-    }
+    softmax_xent_ld_kernel<<<n, 256, 0, st>>>(logits, T.ldlog, C, B, idx, S, labels, sloss, bf(P.off_dzl[L - 1]),
+                                              T.ldz, loss, sel, kdev);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 
     // backward: per layer the mean gradient with the SGD step and dZ of the layer below in
-    // one launch.  dZ_l^T alternates between two buffers: the dX GEMM writes dZ_{l-1}^T
-    // into one while the mean-gradient GEMM reads dZ_l^T from the other.  dZ_l itself
-    // (row-major) is kept for every layer.
-    __nv_bfloat16* dzT[2] = {bf(T.off_dzT), bf(P.off_dzT2)};
-    int curT = 0;
+    // one launch: both read dZ_l, and dZ of every layer is kept in its own buffer.
     for (int l = L - 1; l >= 0; --l) {
         const int fin = g.widths[l], fout = g.widths[l + 1];
         TcEpi gb{};
@@ -823,7 +676,7 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
         gb.pieces = f64(P.off_pw[l]);
         gb.kdev = kdev;
         gb.kmul = B;
-        const TcOperands go{dzT[curT], T.M8, fout, M, bf(T.off_actT[l]), T.M8, fin, M, fout, fin, M};
+        const TcOperands go{bf(P.off_dzl[l]), T.ldz, bf(T.off_act[l]), T.ldact[l], fout, fin, M};
         int rc;
         if (l > 0) {
             TcEpi ex{};
@@ -831,18 +684,14 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
             ex.ldact = T.ldact[l];
             ex.out = bf(P.off_dzl[l - 1]);
             ex.ldo = T.ldz;
-            ex.outT = dzT[curT ^ 1];
-            ex.ldT = T.M8;
             ex.kdev = kdev;
             ex.kmul = B;
-            const TcOperands xo{bf(P.off_dzl[l]), T.ldz, M, fout, bf(T.off_wt[l]), T.ldwt[l], fin, fout, M, fin, fout};
+            const TcOperands xo{bf(P.off_dzl[l]), T.ldz, bf(T.off_wb[l]), T.ldw[l], M, fin, fout};
             rc = tc_gemm_mean_dx(go, gb, xo, ex, status, st);
         } else {
-            rc = tc_gemm(TC_GBAR, go.A, go.lda, go.rowsA, go.colsA, go.B, go.ldb, go.rowsB, go.colsB, go.M, go.N, go.K,
-                         1, 0, gb, status, st);
+            rc = tc_gemm(TC_GBAR, go, gb, status, st);
         }
         if (rc) return rc;
-        curT ^= 1;
     }
     // bias part of g_t and its step, every layer in two launches
     {

@@ -287,8 +287,8 @@ int tc_gram(int L, const __nv_bfloat16* const* act, const int64_t* ldA, const in
         if ((ldA[l] % 8) || (ldD % 8) || (reinterpret_cast<uintptr_t>(act[l]) & 15u) ||
             (reinterpret_cast<uintptr_t>(dz[l]) & 15u))
             return fail(DBW_EALIGN, "tc_gram: unsupported operand alignment");
-        if (!tc_make_map(&G.tmA[l], act[l], rows, colsA[l], ldA[l], GBK, GBM) ||
-            !tc_make_map(&G.tmD[l], dz[l], rows, colsD[l], ldD, GBK, GBM))
+        if (!tc_make_map(&G.tmA[l], act[l], rows, colsA[l], ldA[l], GBM) ||
+            !tc_make_map(&G.tmD[l], dz[l], rows, colsD[l], ldD, GBM))
             return fail(DBW_ECUDA, "tc_gram: cuTensorMapEncodeTiled failed");
         G.colsA[l] = colsA[l];
         G.colsD[l] = colsD[l];
