@@ -1,21 +1,20 @@
-// Eq. (2) for all n workers at once: g_i = (1/B) sum_{x in B_i} grad f(x, w).
+// Eq. (2) for all n workers at once, fp32 workloads: g_i = (1/B) sum_{x in B_i} grad f(x, w).
 //
 // The n workers share w, so their minibatches are stacked into one batch of
 // M = n * B rows and every forward and input-gradient GEMM is a single GEMM over
 // M rows.  Only the weight gradient is per worker: G[i, W_l] = dZ_l[i]^T A_{l-1}[i]
 // with K = B, a batched GEMM over the n workers that writes G directly.
 //
-//   gather     X = pool[idx]                                (fp32 or bf16)
+//   gather     X = pool[idx]
 //   forward    Z_l = A_{l-1} W_l^T + b_l, A_l = ReLU(Z_l)   (last layer: fp32 logits)
 //   loss       per-sample cross entropy, loss_i = mean over worker i's B samples,
 //              dZ_L = (softmax - onehot) / B
 //   backward   G[i, W_l] = dZ_l[i]^T A_{l-1}[i],  G[i, b_l] = sum_rows dZ_l[i],
 //              dZ_{l-1} = (dZ_l W_l) * 1[A_{l-1} > 0]      (ReLU'(0) = 0)
 //
-// GEMMs here are the SIMT path (fp32 FFMA on fp32 or bf16 operands), used for the
-// fp32 workloads and for bf16 shapes the tcgen05 pass (grads_tc.cu) does not take;
-// the fp32 workloads' large forward GEMMs run on the tensor cores in three tf32
-// passes instead (gemm_tf32.cuh), which keeps fp32 accuracy.
+// The large forward and weight-gradient GEMMs run on the tensor cores in three tf32
+// passes (gemm_tf32.cuh), which keeps fp32 accuracy; the others are fp32 FFMA kernels.
+// The bf16 workloads run in grads_tc.cu.
 #include <math.h>
 
 #include "common.cuh"
@@ -96,48 +95,17 @@ __global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols
 
 namespace {
 
-template <typename T> __device__ __forceinline__ float to_f(T v);
-template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <typename T> __device__ __forceinline__ T from_f(float v);
-template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-
 // ------------------------------------------------------------------ gather
-// X[m, :] = pool[idx[m], :].  An index outside [0, S) reads row 0; the loss
-// kernel poisons that worker.  With hi != nullptr (fp32 pass, first forward GEMM in
-// three tf32 passes) the row's tf32 parts go to hi / lo [M, ldo] as well (ldo % 4 == 0).
-template <typename T>
+// X[m, :] = pool[idx[m], :], 16 bytes a lane (in % 4 == 0).  An index outside [0, S)
+// reads row 0; the loss kernel poisons that worker.
 __global__ void gather_kernel(const float* __restrict__ pool, int64_t S, int in, const int32_t* __restrict__ idx,
-                              int M, T* __restrict__ X, float* __restrict__ hi, float* __restrict__ lo, int64_t ldo) {
+                              int M, float* __restrict__ X) {
     for (int m = blockIdx.y; m < M; m += gridDim.y) {
         int64_t r = idx[m];
         if (r < 0 || r >= S) r = 0;
-        const float* src = pool + r * in;
-        T* dst = X + (int64_t)m * in;
-        for (int c = (blockIdx.x * blockDim.x + threadIdx.x) * 4; c < in; c += gridDim.x * blockDim.x * 4) {
-            if (c + 3 < in) {
-                const float4 v = *reinterpret_cast<const float4*>(src + c);
-                dst[c] = from_f<T>(v.x);
-                dst[c + 1] = from_f<T>(v.y);
-                dst[c + 2] = from_f<T>(v.z);
-                dst[c + 3] = from_f<T>(v.w);
-                if (hi) {
-                    float4 h, l;
-                    tf32::split_value(v.x, h.x, l.x);
-                    tf32::split_value(v.y, h.y, l.y);
-                    tf32::split_value(v.z, h.z, l.z);
-                    tf32::split_value(v.w, h.w, l.w);
-                    *reinterpret_cast<float4*>(hi + (int64_t)m * ldo + c) = h;
-                    *reinterpret_cast<float4*>(lo + (int64_t)m * ldo + c) = l;
-                }
-            } else {
-                for (int e = c; e < in; ++e) {
-                    dst[e] = from_f<T>(src[e]);
-                    if (hi) tf32::split_value(src[e], hi[(int64_t)m * ldo + e], lo[(int64_t)m * ldo + e]);
-                }
-            }
-        }
+        const float4* src = reinterpret_cast<const float4*>(pool + r * in);
+        float4* dst = reinterpret_cast<float4*>(X + (int64_t)m * in);
+        for (int c = blockIdx.x * blockDim.x + threadIdx.x; 4 * c < in; c += gridDim.x * blockDim.x) dst[c] = src[c];
     }
 }
 
@@ -192,12 +160,6 @@ __global__ void gather_parts_kernel(const float* __restrict__ pool, int64_t S, i
     }
 }
 
-// bf16 copy of the weight matrices (same flat layout as w; bias slots unused).
-__global__ void cast_bf16_kernel(const float* __restrict__ w, int64_t d, __nv_bfloat16* __restrict__ wb) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
-        wb[i] = __float2bfloat16_rn(w[i]);
-}
-
 // ------------------------------------------------------------------ SIMT GEMM
 // C[m, n] = sum_k A(m, k) B(k, n) over a 128 x 128 tile per CTA, 16-deep K
 // slices staged in shared memory as fp32, 8 x 8 outputs per thread.  Two shared
@@ -213,9 +175,9 @@ constexpr int BM = 128, BN = 128, BK = 16;
 // instead of a batch index; split z covers k in [z * kps, (z + 1) * kps) and
 // writes its partial tile to part[z][M][N], which splitk_reduce_kernel sums in
 // split order before the epilogue.
-template <typename T, bool A_K, bool B_K, class Epi, bool SPLIT>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, const T* __restrict__ A, int64_t lda,
-                                                        int64_t batchA, const T* __restrict__ B, int64_t ldb,
+template <bool A_K, bool B_K, class Epi, bool SPLIT>
+__global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
+                                                        int64_t batchA, const float* __restrict__ B, int64_t ldb,
                                                         int64_t batchB, Epi epi, int kps, float* __restrict__ part) {
     __shared__ __align__(16) float As[2][BK][BM];
     __shared__ __align__(16) float Bs[2][BK][BN];
@@ -244,7 +206,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, con
             int mm, kk;
             if (A_K) { mm = e / BK; kk = e % BK; } else { kk = e / BM; mm = e % BM; }
             const int gm = m0 + mm, gk = k0 + kk;
-            ra[q] = (gm < M && gk < kend) ? to_f<T>(A_K ? A[(int64_t)gm * lda + gk] : A[(int64_t)gk * lda + gm]) : 0.f;
+            ra[q] = (gm < M && gk < kend) ? (A_K ? A[(int64_t)gm * lda + gk] : A[(int64_t)gk * lda + gm]) : 0.f;
         }
 #pragma unroll
         for (int q = 0; q < LB; ++q) {
@@ -252,7 +214,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, con
             int nn, kk;
             if (B_K) { nn = e / BK; kk = e % BK; } else { kk = e / BN; nn = e % BN; }
             const int gn = n0 + nn, gk = k0 + kk;
-            rb[q] = (gn < N && gk < kend) ? to_f<T>(B_K ? B[(int64_t)gn * ldb + gk] : B[(int64_t)gk * ldb + gn]) : 0.f;
+            rb[q] = (gn < N && gk < kend) ? (B_K ? B[(int64_t)gn * ldb + gk] : B[(int64_t)gk * ldb + gn]) : 0.f;
         }
     };
     // registers -> shared buffer ``buf``
@@ -324,14 +286,13 @@ __global__ void splitk_reduce_kernel(int M, int N, int splits, const float* __re
 }
 
 // forward hidden layer: A_l = ReLU(C + b)
-template <typename T>
 struct EpiHidden {
     const float* bias;
-    T* out;
+    float* out;
     int ldo;
     __device__ __forceinline__ void operator()(int, int m, int n, float v) const {
         v += bias[n];
-        out[(int64_t)m * ldo + n] = from_f<T>(v > 0.f ? v : 0.f);
+        out[(int64_t)m * ldo + n] = (v > 0.f ? v : 0.f);
     }
     // 32 consecutive outputs of row m from column n0 (those below N): the biases are
     // loaded before any store
@@ -342,7 +303,7 @@ struct EpiHidden {
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
             const float x = v[j] + b[j];
-            if (n0 + j < N) out[(int64_t)m * ldo + n0 + j] = from_f<T>(x > 0.f ? x : 0.f);
+            if (n0 + j < N) out[(int64_t)m * ldo + n0 + j] = (x > 0.f ? x : 0.f);
         }
     }
 };
@@ -364,14 +325,13 @@ struct EpiLogits {
     }
 };
 // input gradient: dZ_{l-1} = C * 1[A_{l-1} > 0]  (a product, so a NaN-poisoned row stays NaN)
-template <typename T>
 struct EpiDx {
-    const T* act;
-    T* out;
+    const float* act;
+    float* out;
     int ldo;
     __device__ __forceinline__ void operator()(int, int m, int n, float v) const {
-        const float a = to_f<T>(act[(int64_t)m * ldo + n]);
-        out[(int64_t)m * ldo + n] = from_f<T>(v * (a > 0.f ? 1.f : 0.f));
+        const float a = (act[(int64_t)m * ldo + n]);
+        out[(int64_t)m * ldo + n] = (v * (a > 0.f ? 1.f : 0.f));
     }
 };
 // weight gradient of worker z: G[z, off + o * in + c]
@@ -390,11 +350,10 @@ struct EpiDW {
 // dZ = (softmax - onehot) / B.  The worker's loss is the mean of its B sample
 // losses, summed in sample order.  A sample index outside [0, S) or a label
 // outside [0, C) makes the worker's loss and dZ rows NaN.
-template <typename T>
 __global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restrict__ logits, int C, int B,
                                                            const int32_t* __restrict__ idx, int64_t S,
                                                            const int32_t* __restrict__ labels,
-                                                           float* __restrict__ sample_loss, T* __restrict__ dZ,
+                                                           float* __restrict__ sample_loss, float* __restrict__ dZ,
                                                            float* __restrict__ loss) {
     const int i = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -440,7 +399,7 @@ __global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restri
                 if (lane < C) {
                     float g = ex * inv_se;
                     if (lane == y) g -= 1.0f;
-                    dZ[row * C + lane] = from_f<T>(bad ? NAN : g * invB);
+                    dZ[row * C + lane] = (bad ? NAN : g * invB);
                 }
                 const float zy = __shfl_sync(0xffffffffu, zv[j], bad ? 0 : y);
                 if (lane == 0) {
@@ -471,7 +430,7 @@ __global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restri
         for (int c = lane; c < C; c += 32) {
             float g = expf(z[c] - mx) * inv_se;
             if (c == y) g -= 1.0f;
-            dZ[row * C + c] = from_f<T>(bad ? NAN : g * invB);
+            dZ[row * C + c] = (bad ? NAN : g * invB);
         }
         if (lane == 0) {
             const float l = bad ? NAN : (mx + logf(se)) - z[y];
@@ -490,16 +449,15 @@ __global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restri
 
 // ------------------------------------------------------------------ bias gradient
 // G[i, offb + o] = sum_{r < B} dZ[i*B + r, o], summed in row order.
-template <typename T>
-__global__ void bias_grad_kernel(const T* __restrict__ dZ, int out, int B, float* __restrict__ G, int64_t ldG,
+__global__ void bias_grad_kernel(const float* __restrict__ dZ, int out, int B, float* __restrict__ G, int64_t ldG,
                                  int64_t offb) {
     const int i = blockIdx.y;
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= out) return;
-    const T* p = dZ + (int64_t)i * B * out + o;
+    const float* p = dZ + (int64_t)i * B * out + o;
     float acc = 0.f;
 #pragma unroll 16
-    for (int r = 0; r < B; ++r) acc += to_f<T>(p[(int64_t)r * out]);
+    for (int r = 0; r < B; ++r) acc += (p[(int64_t)r * out]);
     G[(int64_t)i * ldG + offb + o] = acc;
 }
 
@@ -542,11 +500,11 @@ constexpr int kSkinnyN = 16;
 constexpr int kSkinnyK = 32;
 constexpr size_t kSkinnySmem = 48 * 1024;
 
-template <typename T, class Epi>
-__global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, const T* __restrict__ A, int64_t lda,
-                                                       const T* __restrict__ W, int64_t ldw, Epi epi) {
+template <class Epi>
+__global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
+                                                       const float* __restrict__ W, int64_t ldw, Epi epi) {
     extern __shared__ float wsh[];   // W as [N, K] fp32
-    fill_shared(wsh, N * K, [&](int e) { return to_f<T>(W[(int64_t)(e / K) * ldw + e % K]); });
+    fill_shared(wsh, N * K, [&](int e) { return (W[(int64_t)(e / K) * ldw + e % K]); });
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -554,12 +512,12 @@ __global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, cons
         float acc[kSkinnyN];
 #pragma unroll
         for (int n = 0; n < kSkinnyN; ++n) acc[n] = 0.f;
-        const T* a = A + (int64_t)m * lda;
+        const float* a = A + (int64_t)m * lda;
         // 8 of the lane's elements loaded at a time, then multiplied
         for (int k0 = lane; k0 < K; k0 += 8 * 32) {
             float av[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) av[u] = k0 + 32 * u < K ? to_f<T>(a[k0 + 32 * u]) : 0.f;
+            for (int u = 0; u < 8; ++u) av[u] = k0 + 32 * u < K ? (a[k0 + 32 * u]) : 0.f;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int k = k0 + 32 * u;
@@ -670,18 +628,17 @@ __global__ void __launch_bounds__(128) skinny_n4_kernel(int M, int N, int K, con
 // added in increasing o (EpiDx's arithmetic, with the 16 masks loaded before any
 // store).  W and the CTA's 16 rows of dZ_l sit in shared memory; a thread per column
 // computes the 16 rows' outputs.
-template <typename T>
-__global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, const T* __restrict__ dZ, int64_t ldz,
-                                                          const T* __restrict__ W, int64_t ldw, EpiDx<T> epi) {
+__global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, const float* __restrict__ dZ, int64_t ldz,
+                                                          const float* __restrict__ W, int64_t ldw, EpiDx epi) {
     constexpr int R = 16;                               // rows per CTA
     extern __shared__ float wsh[];                      // W as [K, N] fp32, then the CTA's dZ rows [R, K]
     float* zsh = wsh + N * K;
-    fill_shared(wsh, N * K, [&](int e) { return to_f<T>(W[(int64_t)(e / N) * ldw + e % N]); });
+    fill_shared(wsh, N * K, [&](int e) { return (W[(int64_t)(e / N) * ldw + e % N]); });
     for (int m0 = blockIdx.y * R; m0 < M; m0 += gridDim.y * R) {
         __syncthreads();   // the previous rows' reads of zsh are done
         fill_shared(zsh, R * K, [&](int e) {
             const int m = m0 + e / K;
-            return m < M ? to_f<T>(dZ[(int64_t)m * ldz + e % K]) : 0.f;
+            return m < M ? (dZ[(int64_t)m * ldz + e % K]) : 0.f;
         });
         __syncthreads();
         for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
@@ -696,10 +653,10 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
             // the ReLU masks of the R rows, all loaded before the first store
             float a[R];
 #pragma unroll
-            for (int j = 0; j < R; ++j) a[j] = m0 + j < M ? to_f<T>(epi.act[(int64_t)(m0 + j) * epi.ldo + c]) : 0.f;
+            for (int j = 0; j < R; ++j) a[j] = m0 + j < M ? (epi.act[(int64_t)(m0 + j) * epi.ldo + c]) : 0.f;
 #pragma unroll
             for (int j = 0; j < R; ++j)
-                if (m0 + j < M) epi.out[(int64_t)(m0 + j) * epi.ldo + c] = from_f<T>(v[j] * (a[j] > 0.f ? 1.f : 0.f));
+                if (m0 + j < M) epi.out[(int64_t)(m0 + j) * epi.ldo + c] = (v[j] * (a[j] > 0.f ? 1.f : 0.f));
         }
     }
 }
@@ -707,8 +664,8 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
 inline bool skinny_n_ok(int N, int K) { return N <= kSkinnyN && (size_t)N * K * 4 <= kSkinnySmem; }
 inline bool skinny_k_ok(int N, int K) { return K <= kSkinnyK && ((size_t)N + 16) * K * 4 <= kSkinnySmem; }
 
-template <typename T, bool A_K, bool B_K, class Epi>
-cudaError_t run_gemm(int M, int N, int K, const T* A, int64_t lda, int64_t batchA, const T* B, int64_t ldb,
+template <bool A_K, bool B_K, class Epi>
+cudaError_t run_gemm(int M, int N, int K, const float* A, int64_t lda, int64_t batchA, const float* B, int64_t ldb,
                      int64_t batchB, int batch, Epi epi, cudaStream_t st, float* split_ws = nullptr,
                      size_t split_floats = 0) {
     int splits = split_ws ? splitk_count(M, N, K, batch) : 1;
@@ -717,7 +674,7 @@ cudaError_t run_gemm(int M, int N, int K, const T* A, int64_t lda, int64_t batch
         const int kps = ((K + splits - 1) / splits + BK - 1) / BK * BK;
         splits = (K + kps - 1) / kps;
         dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, splits);
-        gemm_simt_kernel<T, A_K, B_K, Epi, true><<<grid, 256, 0, st>>>(M, N, K, A, lda, 0, B, ldb, 0, epi, kps,
+        gemm_simt_kernel<A_K, B_K, Epi, true><<<grid, 256, 0, st>>>(M, N, K, A, lda, 0, B, ldb, 0, epi, kps,
                                                                        split_ws);
         const int64_t total = (int64_t)M * N;
         const int blocks = static_cast<int>((total + 255) / 256 < 4 * sm_count() ? (total + 255) / 256 : 4 * sm_count());
@@ -725,60 +682,50 @@ cudaError_t run_gemm(int M, int N, int K, const T* A, int64_t lda, int64_t batch
         return cudaGetLastError();
     }
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch);
-    gemm_simt_kernel<T, A_K, B_K, Epi, false><<<grid, 256, 0, st>>>(M, N, K, A, lda, batchA, B, ldb, batchB, epi, K,
+    gemm_simt_kernel<A_K, B_K, Epi, false><<<grid, 256, 0, st>>>(M, N, K, A, lda, batchA, B, ldb, batchB, epi, K,
                                                                     nullptr);
     return cudaGetLastError();
 }
 
-template <typename T>
-int worker_grads_impl(const GradsPlan& P, const float* w, const float* pool, int64_t S, const int32_t* labels,
+int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int64_t S, const int32_t* labels,
                       const int32_t* idx, float* G, int64_t ld, float* loss, char* ws, cudaStream_t st) {
     const int L = P.L;
     const int M = P.M;
     const int B = P.B;
-    T* X = reinterpret_cast<T*>(ws + P.off_x);
+    float* X = reinterpret_cast<float*>(ws + P.off_x);
     float* logits = reinterpret_cast<float*>(ws + P.off_logits);
     float* sloss = reinterpret_cast<float*>(ws + P.off_sloss);
-    T* dz[2] = {reinterpret_cast<T*>(ws + P.off_dz[0]), reinterpret_cast<T*>(ws + P.off_dz[1])};
+    float* dz[2] = {reinterpret_cast<float*>(ws + P.off_dz[0]), reinterpret_cast<float*>(ws + P.off_dz[1])};
     float* split_ws = P.split_floats ? reinterpret_cast<float*>(ws + P.off_split) : nullptr;
     cudaError_t e0 = cudaMemsetAsync(ws, 0, sizeof(int), st);
     if (e0 != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e0));
-    const T* wop;
-    if (sizeof(T) == 2) {
-        __nv_bfloat16* wb = reinterpret_cast<__nv_bfloat16*>(ws + P.off_wb);
-        cast_bf16_kernel<<<4 * sm_count(), 256, 0, st>>>(w, P.d, wb);
-        wop = reinterpret_cast<const T*>(wb);
-    } else {
-        wop = reinterpret_cast<const T*>(w);
-    }
     {
         const int in = P.widths[0];
-        dim3 grid((in + 1023) / 1024, M < 65535 ? M : 65535);
-        if (sizeof(T) == 4 && (P.tf32[0] || P.tf32_dw[0])) {
+        if (P.tf32[0] || P.tf32_dw[0]) {
             // the first layer's GEMMs in three tf32 passes take their X parts from the gather;
             // X itself only when one of them stays on SIMT
             const int ty = (M + 31) / 32;
             const bool need_x = !(P.tf32[0] && P.tf32_dw[0]);
             gather_parts_kernel<<<dim3((in + 127) / 128, ty < 65535 ? ty : 65535), dim3(32, 8), 0, st>>>(
-                pool, S, in, idx, M, need_x ? reinterpret_cast<float*>(X) : nullptr,
+                pool, S, in, idx, M, need_x ? X : nullptr,
                 P.tf32[0] ? reinterpret_cast<float*>(ws + P.off_ahi) : nullptr,
                 P.tf32[0] ? reinterpret_cast<float*>(ws + P.off_alo) : nullptr, (in + 3) / 4 * 4,
                 P.tf32_dw[0] ? reinterpret_cast<float*>(ws + P.off_xthi) : nullptr,
                 P.tf32_dw[0] ? reinterpret_cast<float*>(ws + P.off_xtlo) : nullptr, M);
         } else {
-            gather_kernel<T><<<grid, 256, 0, st>>>(pool, S, in, idx, M, X, nullptr, nullptr, 0);
+            gather_kernel<<<dim3((in + 1023) / 1024, M < 65535 ? M : 65535), 256, 0, st>>>(pool, S, in, idx, M, X);
         }
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "gather launch: %s", cudaGetErrorString(e));
 
     // forward
-    const T* Ain = X;
+    const float* Ain = X;
     for (int l = 0; l < L; ++l) {
         const int fin = P.widths[l], fout = P.widths[l + 1];
-        const T* W = wop + P.offW[l];
+        const float* W = w + P.offW[l];
         const float* bias = w + P.offb[l];
-        const bool tc = sizeof(T) == 4 && P.tf32[l];
+        const bool tc = P.tf32[l];
         float* part[4] = {nullptr, nullptr, nullptr, nullptr};
         if (tc) {
             part[0] = reinterpret_cast<float*>(ws + P.off_ahi);
@@ -788,36 +735,30 @@ int worker_grads_impl(const GradsPlan& P, const float* w, const float* pool, int
         }
         int* status = reinterpret_cast<int*>(ws);
         auto fwd = [&](auto epi) {
-            if constexpr (sizeof(T) == 4) {
-                if (tc)
-                    return tf32::run(M, fout, fin, Ain, fin, W, fin, part[0], part[1], part[2], part[3], epi, status,
-                                     st, /*a_parts_ready=*/l == 0);
-            }
-            if constexpr (sizeof(T) == 4) {
-                if (fout <= kSkinnyN && fin % 4 == 0 && aligned16(Ain) && aligned16(W)) {
-                    const int want = (M + 3) / 4;   // 4 rows (warps) per CTA
-                    const int grid = want < 8 * sm_count() ? want : 8 * sm_count();
-                    if (fin > 256)
-                        skinny_n4_kernel<true><<<grid, 128, 0, st>>>(M, fout, fin, reinterpret_cast<const float*>(Ain),
-                                                                     fin, reinterpret_cast<const float*>(W), fin, epi);
-                    else
-                        skinny_n4_kernel<false><<<grid, 128, 0, st>>>(M, fout, fin, reinterpret_cast<const float*>(Ain),
-                                                                      fin, reinterpret_cast<const float*>(W), fin, epi);
-                    return cudaGetLastError();
-                }
+            if (tc)
+                return tf32::run(M, fout, fin, Ain, fin, W, fin, part[0], part[1], part[2], part[3], epi, status, st,
+                                 /*a_parts_ready=*/l == 0);
+            if (fout <= kSkinnyN && fin % 4 == 0 && aligned16(Ain) && aligned16(W)) {
+                const int want = (M + 3) / 4;   // 4 rows (warps) per CTA
+                const int grid = want < 8 * sm_count() ? want : 8 * sm_count();
+                if (fin > 256)
+                    skinny_n4_kernel<true><<<grid, 128, 0, st>>>(M, fout, fin, Ain, fin, W, fin, epi);
+                else
+                    skinny_n4_kernel<false><<<grid, 128, 0, st>>>(M, fout, fin, Ain, fin, W, fin, epi);
+                return cudaGetLastError();
             }
             if (skinny_n_ok(fout, fin)) {
                 const int rows_per_cta = 8;
                 const int want = (M + rows_per_cta - 1) / rows_per_cta;
                 const int grid = want < 2 * sm_count() ? want : 2 * sm_count();
-                skinny_n_kernel<T><<<grid, 256, (size_t)fout * fin * 4, st>>>(M, fout, fin, Ain, fin, W, fin, epi);
+                skinny_n_kernel<<<grid, 256, (size_t)fout * fin * 4, st>>>(M, fout, fin, Ain, fin, W, fin, epi);
                 return cudaGetLastError();
             }
-            return run_gemm<T, true, true>(M, fout, fin, Ain, fin, 0, W, fin, 0, 1, epi, st, split_ws, P.split_floats);
+            return run_gemm<true, true>(M, fout, fin, Ain, fin, 0, W, fin, 0, 1, epi, st, split_ws, P.split_floats);
         };
         if (l < L - 1) {
-            T* Aout = reinterpret_cast<T*>(ws + P.off_act[l + 1]);
-            e = fwd(EpiHidden<T>{bias, Aout, fout});
+            float* Aout = reinterpret_cast<float*>(ws + P.off_act[l + 1]);
+            e = fwd(EpiHidden{bias, Aout, fout});
             Ain = Aout;
         } else {
             e = fwd(EpiLogits{bias, logits, fout});
@@ -825,7 +766,7 @@ int worker_grads_impl(const GradsPlan& P, const float* w, const float* pool, int
         if (e != cudaSuccess) return fail(DBW_ECUDA, "forward GEMM %d: %s", l, cudaGetErrorString(e));
     }
     const int C = P.widths[L];
-    softmax_xent_kernel<T><<<P.n, 256, 0, st>>>(logits, C, B, idx, S, labels, sloss, dz[0], loss);
+    softmax_xent_kernel<<<P.n, 256, 0, st>>>(logits, C, B, idx, S, labels, sloss, dz[0], loss);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "loss launch: %s", cudaGetErrorString(e));
 
@@ -833,40 +774,36 @@ int worker_grads_impl(const GradsPlan& P, const float* w, const float* pool, int
     int cur = 0;
     for (int l = L - 1; l >= 0; --l) {
         const int fin = P.widths[l], fout = P.widths[l + 1];
-        const T* Aprev = (l == 0) ? X : reinterpret_cast<const T*>(ws + P.off_act[l]);
-        const T* dZl = dz[cur];
+        const float* Aprev = (l == 0) ? X : reinterpret_cast<const float*>(ws + P.off_act[l]);
+        const float* dZl = dz[cur];
         // per-worker weight gradient: M' = fout, N' = fin, K = B; A(o, r) = dZ[r*fout + o], B(r, c) = A[r*fin + c]
-        bool dw_done = false;
-        if constexpr (sizeof(T) == 4) {
-            if (P.tf32_dw[l]) {
-                const size_t ath = l == 0 ? P.off_xthi : P.off_athi, atl = l == 0 ? P.off_xtlo : P.off_atlo;
-                e = tf32::run_dw(fout, fin, B, P.n, dZl, fout, Aprev, fin, reinterpret_cast<float*>(ws + P.off_zthi),
-                                 reinterpret_cast<float*>(ws + P.off_ztlo), reinterpret_cast<float*>(ws + ath),
-                                 reinterpret_cast<float*>(ws + atl), G + P.offW[l], fin, ld,
-                                 reinterpret_cast<int*>(ws), st, /*act_parts_ready=*/l == 0);
-                dw_done = true;
-            }
+        if (P.tf32_dw[l]) {
+            const size_t ath = l == 0 ? P.off_xthi : P.off_athi, atl = l == 0 ? P.off_xtlo : P.off_atlo;
+            e = tf32::run_dw(fout, fin, B, P.n, dZl, fout, Aprev, fin, reinterpret_cast<float*>(ws + P.off_zthi),
+                             reinterpret_cast<float*>(ws + P.off_ztlo), reinterpret_cast<float*>(ws + ath),
+                             reinterpret_cast<float*>(ws + atl), G + P.offW[l], fin, ld, reinterpret_cast<int*>(ws),
+                             st, /*act_parts_ready=*/l == 0);
+        } else {
+            e = run_gemm<false, false>(fout, fin, B, dZl, fout, (int64_t)B * fout, Aprev, fin, (int64_t)B * fin, P.n,
+                                       EpiDW{G, ld, P.offW[l], fin}, st);
         }
-        if (!dw_done)
-            e = run_gemm<T, false, false>(fout, fin, B, dZl, fout, (int64_t)B * fout, Aprev, fin, (int64_t)B * fin,
-                                          P.n, EpiDW{G, ld, P.offW[l], fin}, st);
         if (e != cudaSuccess) return fail(DBW_ECUDA, "dW GEMM %d: %s", l, cudaGetErrorString(e));
-        bias_grad_kernel<T><<<dim3((fout + 127) / 128, P.n), 128, 0, st>>>(dZl, fout, B, G, ld, P.offb[l]);
+        bias_grad_kernel<<<dim3((fout + 127) / 128, P.n), 128, 0, st>>>(dZl, fout, B, G, ld, P.offb[l]);
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail(DBW_ECUDA, "bias grad %d: %s", l, cudaGetErrorString(e));
         if (l > 0) {
             // dZ_{l-1}[m, c] = sum_o dZ_l[m, o] W_l[o, c]: A(m, o) = dZ[m*fout + o], B(o, c) = W[o*fin + c]
-            T* dnext = dz[cur ^ 1];
+            float* dnext = dz[cur ^ 1];
             if (skinny_k_ok(fin, fout)) {
                 const int ry = (M + 15) / 16;
                 dim3 grid((fin + 255) / 256, ry < 65535 ? ry : 65535);
-                skinny_k_dx_kernel<T><<<grid, 256, ((size_t)fin + 16) * fout * 4, st>>>(M, fin, fout, dZl, fout,
-                                                                                  wop + P.offW[l], fin,
-                                                                                  EpiDx<T>{Aprev, dnext, fin});
+                skinny_k_dx_kernel<<<grid, 256, ((size_t)fin + 16) * fout * 4, st>>>(M, fin, fout, dZl, fout,
+                                                                                  w + P.offW[l], fin,
+                                                                                  EpiDx{Aprev, dnext, fin});
                 e = cudaGetLastError();
             } else {
-                e = run_gemm<T, true, false>(M, fin, fout, dZl, fout, 0, wop + P.offW[l], fin, 0, 1,
-                                             EpiDx<T>{Aprev, dnext, fin}, st, split_ws, P.split_floats);
+                e = run_gemm<true, false>(M, fin, fout, dZl, fout, 0, w + P.offW[l], fin, 0, 1,
+                                             EpiDx{Aprev, dnext, fin}, st, split_ws, P.split_floats);
             }
             if (e != cudaSuccess) return fail(DBW_ECUDA, "dX GEMM %d: %s", l, cudaGetErrorString(e));
             cur ^= 1;
@@ -902,7 +839,6 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
         off += widths[l + 1];
     }
     P->d = off;
-    const size_t es = prec == DBW_PREC_BF16 ? 2 : 4;
     size_t cur = 0;
     auto take = [&](size_t bytes) {
         const size_t at = cur;
@@ -910,14 +846,13 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
         return at;
     };
     take(256);   // status word (int32 at offset 0), as in the tcgen05 plan
-    P->off_x = take((size_t)M * widths[0] * es);
+    P->off_x = take((size_t)M * widths[0] * 4);
     P->off_act[0] = P->off_x;
-    for (int l = 1; l < L; ++l) P->off_act[l] = take((size_t)M * widths[l] * es);
+    for (int l = 1; l < L; ++l) P->off_act[l] = take((size_t)M * widths[l] * 4);
     P->off_logits = take((size_t)M * widths[L] * 4);
     P->off_sloss = take((size_t)M * 4);
-    P->off_dz[0] = take((size_t)M * maxw * es);
-    P->off_dz[1] = take((size_t)M * maxw * es);
-    P->off_wb = prec == DBW_PREC_BF16 ? take((size_t)P->d * 2) : 0;
+    P->off_dz[0] = take((size_t)M * maxw * 4);
+    P->off_dz[1] = take((size_t)M * maxw * 4);
     // split-K scratch of the forward and input-gradient GEMMs (the largest splits x M x N)
     size_t split = 0;
     for (int l = 0; l < L; ++l) {
@@ -969,7 +904,7 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
 int grads_activations(int L, const int32_t* widths, int n, int B, int prec, int layer, size_t* offset, int64_t* ld,
                       int* elem_bytes) {
     if (layer < 1 || layer >= L) return fail(DBW_EINVAL, "dbw_worker_grads_activations: layer must be in [1, L-1]");
-    if (tc_eligible(prec, B)) {
+    if (prec == DBW_PREC_BF16) {
         TcPlan T;
         if (!make_tc_plan(L, widths, n, B, &T)) return fail(DBW_EINVAL, "dbw_worker_grads_activations: invalid shape");
         *offset = T.off_act[layer];
@@ -981,12 +916,12 @@ int grads_activations(int L, const int32_t* widths, int n, int B, int prec, int 
     if (!make_grads_plan(L, widths, n, B, prec, &P)) return fail(DBW_EINVAL, "dbw_worker_grads_activations: invalid shape");
     *offset = P.off_act[layer];
     *ld = widths[layer];
-    *elem_bytes = prec == DBW_PREC_BF16 ? 2 : 4;
+    *elem_bytes = 4;
     return DBW_OK;
 }
 
 size_t grads_workspace_bytes(int L, const int32_t* widths, int n, int B, int prec) {
-    if (tc_eligible(prec, B)) {
+    if (prec == DBW_PREC_BF16) {
         TcPlan T;
         if (!make_tc_plan(L, widths, n, B, &T)) return 0;
         return T.ws_bytes;
@@ -1003,18 +938,16 @@ int launch_worker_grads(int L, const int32_t* widths, int prec, const float* w, 
     if (!make_grads_plan(L, widths, n, B, prec, &P)) return fail(DBW_EINVAL, "dbw_worker_grads: invalid model shape");
     if (P.d != d) return fail(DBW_EINVAL, "dbw_worker_grads: d = %lld but the widths give %lld", (long long)d,
                               (long long)P.d);
-    if (!tc_eligible(prec, B) && ws_bytes < P.ws_bytes)
-        return fail(DBW_EINVAL, "dbw_worker_grads: workspace %zu bytes < %zu needed", ws_bytes, P.ws_bytes);
-    if (tc_eligible(prec, B)) {
+    if (prec == DBW_PREC_BF16) {
         TcPlan T;
         if (!make_tc_plan(L, widths, n, B, &T)) return fail(DBW_EINVAL, "dbw_worker_grads: invalid model shape");
         if (ws_bytes < T.ws_bytes)
             return fail(DBW_EINVAL, "dbw_worker_grads: workspace %zu bytes < %zu needed", ws_bytes, T.ws_bytes);
         return worker_grads_tc(T, w, pool, S, labels, idx, G, ld, loss, static_cast<char*>(ws), st);
     }
-    if (prec == DBW_PREC_BF16)
-        return worker_grads_impl<__nv_bfloat16>(P, w, pool, S, labels, idx, G, ld, loss, static_cast<char*>(ws), st);
-    return worker_grads_impl<float>(P, w, pool, S, labels, idx, G, ld, loss, static_cast<char*>(ws), st);
+    if (ws_bytes < P.ws_bytes)
+        return fail(DBW_EINVAL, "dbw_worker_grads: workspace %zu bytes < %zu needed", ws_bytes, P.ws_bytes);
+    return worker_grads_fp32(P, w, pool, S, labels, idx, G, ld, loss, static_cast<char*>(ws), st);
 }
 
 }  // namespace dbw

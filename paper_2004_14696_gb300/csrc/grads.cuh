@@ -1,4 +1,5 @@
-// Internal plan of the worker-gradient pass: layer offsets and workspace layout.
+// Internal plans of the worker-gradient passes: layer offsets (both precisions) and
+// workspace layout (GradsPlan's is the fp32 pass's, TcPlan's the bf16 pass's).
 #pragma once
 
 #include <stddef.h>
@@ -16,12 +17,11 @@ struct GradsPlan {
     int64_t offW[DBW_LMAX], offb[DBW_LMAX];   // offsets of W_l and b_l in w / in a row of G
     int64_t d;
     // workspace byte offsets (256-byte aligned)
-    size_t off_x;                   // X = gathered inputs [M, widths[0]] (operand type)
-    size_t off_act[DBW_LMAX];       // A_l [M, widths[l]] for l = 1..L-1 (off_act[0] = off_x)
+    size_t off_x;                   // X = gathered inputs [M, widths[0]] fp32
+    size_t off_act[DBW_LMAX];       // A_l [M, widths[l]] fp32 for l = 1..L-1 (off_act[0] = off_x)
     size_t off_logits;              // [M, C] fp32
     size_t off_sloss;               // [M] fp32 per-sample loss
-    size_t off_dz[2];               // ping-pong dZ [M, max width] (operand type)
-    size_t off_wb;                  // bf16 weights [d] (bf16 only)
+    size_t off_dz[2];               // ping-pong dZ [M, max width] fp32
     size_t off_split;               // split-K partial tiles of the SIMT GEMMs
     size_t split_floats;
     // fp32 forward GEMMs on the tensor cores in three tf32 passes (gemm_tf32.cuh):
@@ -77,16 +77,14 @@ struct RxPlan {
     size_t ws_bytes;
 };
 
-// The received-workers pass needs the tcgen05 path and a Gram tile layout: B % 32 == 0
-// and either 128 % B == 0 or B % 128 == 0.
+// The received-workers pass needs bf16 and a Gram tile layout: B % 32 == 0 and either
+// 128 % B == 0 or B % 128 == 0.
 bool rx_eligible(int prec, int B);
 bool make_rx_plan(int L, const int32_t* widths, int n, int B, RxPlan* P);
 int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, const int32_t* labels,
                       const int32_t* idx, const uint8_t* mask, float lr, float* gbar, float* loss, double* partials,
                       char* ws, cudaStream_t st);
 
-// The bf16 pass runs on tcgen05 when each worker's sample count is whole 32-deep K blocks.
-bool tc_eligible(int prec, int B);
 bool make_tc_plan(int L, const int32_t* widths, int n, int B, TcPlan* P);
 int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t S, const int32_t* labels,
                     const int32_t* idx, float* G, int64_t ld, float* loss, char* ws, cudaStream_t st);

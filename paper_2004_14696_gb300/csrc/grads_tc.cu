@@ -1,6 +1,6 @@
 // Eq. (2) for all n workers with bf16 GEMM operands on the tcgen05 tensor cores.
 //
-// Same computation as the SIMT pass in grads.cu (forward over the stacked
+// Same computation as the fp32 pass in grads.cu (forward over the stacked
 // M = n B rows, softmax cross entropy, backward with a per-worker weight
 // gradient of depth K = B) on the GEMMs of gemm_tc.cu:
 //
@@ -9,11 +9,16 @@
 //   dW        G_i = dZ_l[i]^T . A_{l-1}[i]   A = dZ_l [M, out],      B = act[l-1] [M, in]
 //                                            (worker i: rows i*B .. i*B+B-1, K = B)
 //
+// Every B runs here: a worker's rows are read through a 3-D tensor map (column, sample,
+// worker), so the last K block of a B that is not whole K blocks reads zeros past the
+// worker's samples.  (16 workers of 500 samples, 3072-1024-1024-10: 5,440 us on fp32 FFMA
+// tiles, which served B % 32 != 0 before.)
+//
 // Every operand is the row-major bf16 buffer its producer wrote: the tensor cores read
 // dZ, the activations and (in dX) W as MN-major tiles, so no transposed copy is formed.
 // With transposed copies (written by the GEMM epilogues, the X and W casts and the
-// softmax) the 3072-1024-1024-10 pass of 128 x 128 samples took 827 us, and those copies
-// were a third of the casts' bytes and half of the epilogues' stores.
+// softmax; a third of the casts' bytes and half of the epilogues' stores) the
+// 3072-1024-1024-10 pass of 128 x 128 samples took 822 us, without them 734.
 // Leading dimensions are padded to multiples of 8 elements (16 bytes, the TMA
 // stride rule); padding is never read (tensor maps carry the logical extents).
 #include <math.h>
@@ -439,8 +444,6 @@ __global__ void __launch_bounds__(kFinishThreads) finish_received_kernel(FinishA
 
 }  // namespace
 
-bool tc_eligible(int prec, int B) { return prec == DBW_PREC_BF16 && B % 32 == 0; }
-
 // CTAs of a warp-per-row kernel over ``rows`` rows (8 warps each, at most 8 per SM).
 static int row_ctas(int64_t rows) {
     const int64_t want = (rows + 7) / 8, most = 8 * sm_count();
@@ -575,7 +578,9 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
 // per-worker squared norms come from B x B Gram matrices (tc_gram).  The number
 // of received workers k is read on the device from ``mask``.
 
-bool rx_eligible(int prec, int B) { return tc_eligible(prec, B) && (128 % B == 0 || B % 128 == 0); }
+bool rx_eligible(int prec, int B) {
+    return prec == DBW_PREC_BF16 && B % 32 == 0 && (128 % B == 0 || B % 128 == 0);
+}
 
 bool make_rx_plan(int L, const int32_t* widths, int n, int B, RxPlan* P) {
     if (!make_tc_plan(L, widths, n, B, &P->t)) return false;

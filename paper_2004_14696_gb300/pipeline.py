@@ -200,19 +200,17 @@ class Iteration:
             # launch when l > 0); bias row sums and bias mean of all layers (2), Gram norms of all
             # layers (1), finish; grad_stats (2)
             return choose + 1 + (1 + 1 + 1 + L + 1 + L + 2 + 1 + 1) + 2
-        if self.wl.prec == dbw.PREC_BF16 and self.wl.B % 32 == 0:
+        if self.wl.prec == dbw.PREC_BF16:
             # tcgen05 pass: the weight casts of all layers (1), X, L forward GEMMs, loss + dZ_L,
             # L dW GEMMs, L bias gradients, L-1 dX GEMMs
             grads = 1 + 1 + L + 1 + L + L + (L - 1)
         else:
-            grads = 1 + L + 1 + L + L + (L - 1)    # gather, forward, loss, dW, bias, dX
-            if self.wl.prec == dbw.PREC_BF16:
-                grads += 1                          # bf16 weight cast
-            grads += self._simt_extra_launches()
+            # gather, forward, loss, dW, bias, dX
+            grads = 1 + L + 1 + L + L + (L - 1) + self._fp32_extra_launches()
         return choose + grads + 1 + 1 + 2
 
-    def _simt_extra_launches(self):
-        """Launches beyond one per GEMM on the SIMT pass: a GEMM in three tf32 passes splits
+    def _fp32_extra_launches(self):
+        """Launches beyond one per GEMM on the fp32 pass: a GEMM in three tf32 passes splits
         its two operands first (2), a split-K GEMM sums its splits (1); the skinny kernels
         are one launch.  Mirrors the plan's rules in csrc/grads.cu."""
         wd, M = self.wl.widths, self.wl.n * self.wl.B
@@ -227,8 +225,7 @@ class Iteration:
             return 1 if -(-k // kps) > 1 else 0
 
         def skinny_n(n, k, off):     # the forward GEMM with few outputs (W_l at offset off of w)
-            vec = self.wl.prec == dbw.PREC_FP32 and k % 4 == 0 and off % 4 == 0
-            return n <= 16 and (vec or n * k * 4 <= 48 * 1024)
+            return n <= 16 and ((k % 4 == 0 and off % 4 == 0) or n * k * 4 <= 48 * 1024)
 
         def skinny_k(n, k):     # the input-gradient GEMM with a short inner dimension
             return k <= 32 and (n + 16) * k * 4 <= 48 * 1024
@@ -237,10 +234,10 @@ class Iteration:
         extra = 0
         for l in range(len(wd) - 1):
             fin, fout = wd[l], wd[l + 1]
-            if (self.wl.prec == dbw.PREC_FP32 and B % 32 == 0 and B <= 256 and fin % 4 == 0 and off % 4 == 0
+            if (B % 32 == 0 and B <= 256 and fin % 4 == 0 and off % 4 == 0
                     and fout >= 32 and n * fout * fin * B >= 1 << 25):
                 extra += 1 if l == 0 else 2     # transposed parts of dZ_l (and of the input above layer 1)
-            if self.wl.prec == dbw.PREC_FP32 and fout >= 32 and M * fout * fin >= 1 << 27:
+            if fout >= 32 and M * fout * fin >= 1 << 27:
                 extra += 1 if l == 0 else 2     # the gather writes the first layer's input parts
             elif not skinny_n(fout, fin, off):
                 extra += split_launch(M, fout, fin)
