@@ -198,8 +198,8 @@ class Iteration:
             # select; compaction, the weight casts of all layers (1), X, L forward
             # GEMMs, loss + dZ_L, per layer the mean-gradient GEMM (with the dX GEMM in the same
             # launch when l > 0); bias row sums and bias mean of all layers (2), Gram norms of all
-            # layers (1), finish; grad_stats (2)
-            return choose + 1 + (1 + 1 + 1 + L + 1 + L + 2 + 1 + 1) + 2
+            # layers (1), finish; grad_stats
+            return choose + 1 + (1 + 1 + 1 + L + 1 + L + 2 + 1 + 1) + 1
         if self.wl.prec == dbw.PREC_BF16:
             # tcgen05 pass: the weight casts of all layers (1), X, L forward GEMMs, loss + dZ_L,
             # L dW GEMMs, L bias gradients, L-1 dX GEMMs
@@ -207,7 +207,7 @@ class Iteration:
         else:
             # gather, forward, loss, dW, bias, dX
             grads = 1 + L + 1 + L + L + (L - 1) + self._fp32_extra_launches()
-        return choose + grads + 1 + 1 + 2
+        return choose + grads + 1 + 1 + 1
 
     def _fp32_extra_launches(self):
         """Launches beyond one per GEMM on the fp32 pass: a GEMM in three tf32 passes splits
