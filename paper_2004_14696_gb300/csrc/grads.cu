@@ -20,6 +20,7 @@
 #include "common.cuh"
 #include "gemm_tf32.cuh"
 #include "grads.cuh"
+#include "loss_bias.cuh"
 
 namespace dbw {
 
@@ -345,122 +346,6 @@ struct EpiDW {
     }
 };
 
-// ------------------------------------------------------------------ loss
-// One CTA per worker.  Per sample: stable log-softmax cross entropy, and
-// dZ = (softmax - onehot) / B.  The worker's loss is the mean of its B sample
-// losses, summed in sample order.  A sample index outside [0, S) or a label
-// outside [0, C) makes the worker's loss and dZ rows NaN.
-__global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restrict__ logits, int C, int B,
-                                                           const int32_t* __restrict__ idx, int64_t S,
-                                                           const int32_t* __restrict__ labels,
-                                                           float* __restrict__ sample_loss, float* __restrict__ dZ,
-                                                           float* __restrict__ loss) {
-    const int i = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    constexpr int kShared = 2048;   // sample losses kept in shared memory up to this B
-    __shared__ float ls[kShared];
-    __shared__ int bad_s;
-    if (threadIdx.x == 0) bad_s = 0;
-    __syncthreads();
-    const float invB = 1.0f / (float)B;
-    if (C <= 32) {
-        // lane c holds class c; a warp's rows go in batches of 8 whose logits, sample
-        // indices and labels are all loaded before the first is reduced
-        for (int r0 = warp; r0 < B; r0 += 8 * nw) {
-            float zv[8];
-            int yv[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int r = r0 + j * nw;
-                zv[j] = -INFINITY;
-                yv[j] = -1;
-                if (r < B) {
-                    const int64_t row = (int64_t)i * B + r;
-                    if (lane < C) zv[j] = logits[row * C + lane];
-                    const int64_t sidx = idx[row];
-                    if (sidx >= 0 && sidx < S) yv[j] = labels[sidx];
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int r = r0 + j * nw;
-                if (r >= B) break;
-                const int64_t row = (int64_t)i * B + r;
-                const int y = yv[j];
-                const bool bad = (y < 0 || y >= C);
-                float mx = zv[j];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                const float ex = lane < C ? expf(zv[j] - mx) : 0.f;
-                float se = ex;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-                const float inv_se = 1.0f / se;
-                if (lane < C) {
-                    float g = ex * inv_se;
-                    if (lane == y) g -= 1.0f;
-                    dZ[row * C + lane] = (bad ? NAN : g * invB);
-                }
-                const float zy = __shfl_sync(0xffffffffu, zv[j], bad ? 0 : y);
-                if (lane == 0) {
-                    const float l = bad ? NAN : (mx + logf(se)) - zy;
-                    sample_loss[row] = l;
-                    if (r < kShared) ls[r] = l;
-                    if (bad) bad_s = 1;
-                }
-            }
-        }
-    }
-    for (int r = C <= 32 ? B : warp; r < B; r += nw) {
-        const int64_t row = (int64_t)i * B + r;
-        const int64_t sidx = idx[row];
-        int y = -1;
-        if (sidx >= 0 && sidx < S) y = labels[sidx];
-        const bool bad = (y < 0 || y >= C);
-        const float* z = logits + row * C;
-        float mx = -INFINITY;
-        for (int c = lane; c < C; c += 32) mx = fmaxf(mx, z[c]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        float se = 0.f;
-        for (int c = lane; c < C; c += 32) se += expf(z[c] - mx);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-        const float inv_se = 1.0f / se;
-        for (int c = lane; c < C; c += 32) {
-            float g = expf(z[c] - mx) * inv_se;
-            if (c == y) g -= 1.0f;
-            dZ[row * C + c] = (bad ? NAN : g * invB);
-        }
-        if (lane == 0) {
-            const float l = bad ? NAN : (mx + logf(se)) - z[y];
-            sample_loss[row] = l;
-            if (r < kShared) ls[r] = l;
-            if (bad) bad_s = 1;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float acc = 0.f;
-        for (int r = 0; r < B; ++r) acc += r < kShared ? ls[r] : sample_loss[(int64_t)i * B + r];
-        loss[i] = bad_s ? NAN : acc * invB;
-    }
-}
-
-// ------------------------------------------------------------------ bias gradient
-// G[i, offb + o] = sum_{r < B} dZ[i*B + r, o], summed in row order.
-__global__ void bias_grad_kernel(const float* __restrict__ dZ, int out, int B, float* __restrict__ G, int64_t ldG,
-                                 int64_t offb) {
-    const int i = blockIdx.y;
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= out) return;
-    const float* p = dZ + (int64_t)i * B * out + o;
-    float acc = 0.f;
-#pragma unroll 16
-    for (int r = 0; r < B; ++r) acc += (p[(int64_t)r * out]);
-    G[(int64_t)i * ldG + offb + o] = acc;
-}
-
 // Splits of K for an unbatched GEMM with few output tiles: enough CTAs for about
 // two per SM, each split at least 4 K blocks deep; 1 = no split.
 int splitk_count(int M, int N, int K, int batch) {
@@ -697,7 +582,8 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
     float* sloss = reinterpret_cast<float*>(ws + P.off_sloss);
     float* dz[2] = {reinterpret_cast<float*>(ws + P.off_dz[0]), reinterpret_cast<float*>(ws + P.off_dz[1])};
     float* split_ws = P.split_floats ? reinterpret_cast<float*>(ws + P.off_split) : nullptr;
-    cudaError_t e0 = cudaMemsetAsync(ws, 0, sizeof(int), st);
+    // the status word and the workers' loss counters
+    cudaError_t e0 = cudaMemsetAsync(ws, 0, P.off_cnt + P.n * sizeof(int), st);
     if (e0 != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e0));
     {
         const int in = P.widths[0];
@@ -766,8 +652,8 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
         if (e != cudaSuccess) return fail(DBW_ECUDA, "forward GEMM %d: %s", l, cudaGetErrorString(e));
     }
     const int C = P.widths[L];
-    softmax_xent_kernel<<<P.n, 256, 0, st>>>(logits, C, B, idx, S, labels, sloss, dz[0], loss);
-    e = cudaGetLastError();
+    e = launch_softmax(logits, C, C, P.n, B, idx, S, labels, sloss, dz[0], C, loss, reinterpret_cast<int*>(ws + P.off_cnt),
+                       st);
     if (e != cudaSuccess) return fail(DBW_ECUDA, "loss launch: %s", cudaGetErrorString(e));
 
     // backward
@@ -788,8 +674,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
                                        EpiDW{G, ld, P.offW[l], fin}, st);
         }
         if (e != cudaSuccess) return fail(DBW_ECUDA, "dW GEMM %d: %s", l, cudaGetErrorString(e));
-        bias_grad_kernel<<<dim3((fout + 127) / 128, P.n), 128, 0, st>>>(dZl, fout, B, G, ld, P.offb[l]);
-        e = cudaGetLastError();
+        e = launch_bias_grad(dZl, fout, fout, P.n, B, G, ld, P.offb[l], st);
         if (e != cudaSuccess) return fail(DBW_ECUDA, "bias grad %d: %s", l, cudaGetErrorString(e));
         if (l > 0) {
             // dZ_{l-1}[m, c] = sum_o dZ_l[m, o] W_l[o, c]: A(m, o) = dZ[m*fout + o], B(o, c) = W[o*fin + c]
@@ -829,7 +714,7 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
     for (int l = 0; l <= L; ++l) {
         if (widths[l] < 1 || widths[l] > (1 << 20)) return false;
         P->widths[l] = widths[l];
-        if (widths[l] > maxw) maxw = widths[l];
+        if (l > 0 && widths[l] > maxw) maxw = widths[l];   // of the layers dZ is formed for
     }
     if (widths[L] < 2) return false;
     for (int l = 0; l < L; ++l) {
@@ -846,6 +731,7 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
         return at;
     };
     take(256);   // status word (int32 at offset 0), as in the tcgen05 plan
+    P->off_cnt = take((size_t)n * 4);
     P->off_x = take((size_t)M * widths[0] * 4);
     P->off_act[0] = P->off_x;
     for (int l = 1; l < L; ++l) P->off_act[l] = take((size_t)M * widths[l] * 4);

@@ -17,6 +17,7 @@ struct GradsPlan {
     int64_t offW[DBW_LMAX], offb[DBW_LMAX];   // offsets of W_l and b_l in w / in a row of G
     int64_t d;
     // workspace byte offsets (256-byte aligned)
+    size_t off_cnt;                 // int32 [n]: loss counters of the workers, right after the status word
     size_t off_x;                   // X = gathered inputs [M, widths[0]] fp32
     size_t off_act[DBW_LMAX];       // A_l [M, widths[l]] fp32 for l = 1..L-1 (off_act[0] = off_x)
     size_t off_logits;              // [M, C] fp32
@@ -44,6 +45,7 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
 struct TcPlan {
     GradsPlan g;                       // shapes and parameter offsets
     size_t off_status;                 // device int: bit 0 = a pipeline wait timed out
+    size_t off_cnt;                    // int32 [n]: loss counters of the workers, right after the status word
     size_t off_wb[DBW_LMAX];           // W_l bf16 [out, ldw]
     int64_t ldw[DBW_LMAX];
     size_t off_act[DBW_LMAX];          // layer-l input bf16 [M, ldact] (act[0] = X)

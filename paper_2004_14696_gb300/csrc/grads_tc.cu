@@ -25,6 +25,7 @@
 
 #include "gemm_tc.cuh"
 #include "grads.cuh"
+#include "loss_bias.cuh"
 #include "tc_ptx.cuh"
 
 namespace dbw {
@@ -117,15 +118,6 @@ struct GatherRows {     // X of the per-worker pass: pool row idx[m]; an index o
     }
 };
 
-// Rows of the stacked buffers that a received-workers pass computes: the k B
-// received rows rounded up to the 128-row GEMM tile (all M when kdev is null).
-__device__ __forceinline__ int live_rows(const int* kdev, int B, int M) {
-    if (!kdev) return M;
-    const int k = *kdev;
-    const long long r = (static_cast<long long>(k > 0 ? k : 0) * B + 127) / 128 * 128;
-    return r < M ? static_cast<int>(r) : M;
-}
-
 // X of the received-workers pass: row m of slot s = m / B < k is pool row
 // idx[sel[s] B + m % B] (an index outside [0, S) reads row 0); rows from k B up to
 // the live row count are zero; later rows are not written.
@@ -143,115 +135,6 @@ struct ReceivedRows {
         return (r < 0 || r >= S) ? 0 : r;
     }
 };
-
-// With ``sel`` (received-workers pass): CTA s handles slot s, i.e. worker sel[s]
-// (stacked rows s B .., samples idx[sel[s] B + r], loss[sel[s]]); slots s >= k
-// zero their dZ rows up to the live row count and stop.
-__global__ void __launch_bounds__(256) softmax_xent_ld_kernel(const float* __restrict__ logits, int64_t ldl, int C,
-                                                              int B, const int32_t* __restrict__ idx, int64_t S,
-                                                              const int32_t* __restrict__ labels,
-                                                              float* __restrict__ sample_loss,
-                                                              __nv_bfloat16* __restrict__ dZ, int64_t ldz,
-                                                              float* __restrict__ loss,
-                                                              const int32_t* __restrict__ sel = nullptr,
-                                                              const int* __restrict__ kdev = nullptr) {
-    const int i = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int worker = i;
-    if (sel) {
-        if (i >= *kdev) {
-            const int live = live_rows(kdev, B, gridDim.x * B);
-            for (int r = warp; r < B && i * B + r < live; r += nw)
-                for (int c = lane; c < C; c += 32)
-                    dZ[(static_cast<int64_t>(i) * B + r) * ldz + c] = __float2bfloat16_rn(0.f);
-            return;
-        }
-        worker = sel[i];
-    }
-    __shared__ int bad_s;
-    constexpr int kShared = 1024;   // sample losses kept in shared memory up to this B
-    __shared__ float ls[kShared];
-    if (threadIdx.x == 0) bad_s = 0;
-    __syncthreads();
-    const float invB = 1.0f / static_cast<float>(B);
-    constexpr int kRegs = 32;   // logits a lane keeps in registers: rows of up to 1024 classes in one read
-    for (int r = warp; r < B; r += nw) {
-        const int64_t row = static_cast<int64_t>(i) * B + r;
-        const int64_t sidx = idx[static_cast<int64_t>(worker) * B + r];
-        int y = -1;
-        if (sidx >= 0 && sidx < S) y = labels[sidx];
-        const bool bad = (y < 0 || y >= C);
-        const float* z = logits + row * ldl;
-        float mx = -INFINITY, se = 0.f;
-        if (C <= 32 * kRegs) {
-            // the row is read once: max, sum of exponentials and dZ from registers
-            float v[kRegs];
-#pragma unroll
-            for (int j = 0; j < kRegs; ++j) {
-                const int c = lane + 32 * j;
-                v[j] = c < C ? z[c] : -INFINITY;
-                mx = fmaxf(mx, v[j]);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-#pragma unroll
-            for (int j = 0; j < kRegs; ++j) {
-                v[j] = lane + 32 * j < C ? expf(v[j] - mx) : 0.f;
-                se += v[j];
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-            const float inv_se = 1.0f / se;
-#pragma unroll
-            for (int j = 0; j < kRegs; ++j) {
-                const int c = lane + 32 * j;
-                if (c < C) {
-                    float g = v[j] * inv_se;
-                    if (c == y) g -= 1.0f;
-                    dZ[row * ldz + c] = __float2bfloat16_rn(bad ? NAN : g * invB);
-                }
-            }
-        } else {
-            for (int c = lane; c < C; c += 32) mx = fmaxf(mx, z[c]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            for (int c = lane; c < C; c += 32) se += expf(z[c] - mx);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-            const float inv_se = 1.0f / se;
-            for (int c = lane; c < C; c += 32) {
-                float g = expf(z[c] - mx) * inv_se;
-                if (c == y) g -= 1.0f;
-                dZ[row * ldz + c] = __float2bfloat16_rn(bad ? NAN : g * invB);
-            }
-        }
-        if (lane == 0) {
-            const float l = bad ? NAN : (mx + logf(se)) - z[y];
-            sample_loss[row] = l;
-            if (r < kShared) ls[r] = l;
-            if (bad) bad_s = 1;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // in sample order, from shared memory
-        float acc = 0.f;
-        for (int r = 0; r < B; ++r) acc += r < kShared ? ls[r] : sample_loss[static_cast<int64_t>(i) * B + r];
-        loss[worker] = bad_s ? NAN : acc * invB;
-    }
-}
-
-// G[i, offb + o] = sum_{r < B} dZ[i*B + r, o] (rows in order).
-__global__ void bias_grad_ld_kernel(const __nv_bfloat16* __restrict__ dZ, int64_t ldz, int out, int B,
-                                    float* __restrict__ G, int64_t ldG, int64_t offb) {
-    const int i = blockIdx.y;
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= out) return;
-    const __nv_bfloat16* p = dZ + static_cast<int64_t>(i) * B * ldz + o;
-    float acc = 0.f;
-    for (int r = 0; r < B; ++r) acc += __bfloat162float(p[static_cast<int64_t>(r) * ldz]);
-    G[static_cast<int64_t>(i) * ldG + offb + o] = acc;
-}
 
 // ------------------------------------------------------------------ received-workers pass
 // sel[0..k) = the workers with mask[j] != 0 in increasing order, *kout = k, and
@@ -319,7 +202,7 @@ __global__ void __launch_bounds__(256) bias_rows_kernel(BiasLayers a, int B, con
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     const int rend = r0 + 256 < rows ? r0 + 256 : rows;
     if (c + 7 < out) {
-#pragma unroll 4
+#pragma unroll 8
         for (int r = r0 + y; r < rend; r += 8) {
             const uint4 raw = *reinterpret_cast<const uint4*>(dZ + static_cast<int64_t>(r) * ldz + c);
             const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&raw);
@@ -355,6 +238,7 @@ __global__ void __launch_bounds__(256) bias_mean_update_kernel(BiasLayers a, int
     double sq = 0.0;
     if (o < out && k > 0) {
         float t = 0.f;
+#pragma unroll 16
         for (int q = 0; q < chunks; ++q) t += a.part[l][static_cast<int64_t>(q) * out + o];
         const float g = t * (1.0f / static_cast<float>(k));
         a.wb[l][o] = fmaf(-lr, g, a.wb[l][o]);
@@ -393,8 +277,8 @@ constexpr int kFinishThreads = 1024;
 __global__ void __launch_bounds__(kFinishThreads) finish_received_kernel(FinishArgs a, const int32_t* __restrict__ sel,
                                                                          const int* __restrict__ kdev,
                                                                          double* __restrict__ partials) {
-    __shared__ double red[2][kFinishThreads];
-    const int t = threadIdx.x, n = a.n;
+    __shared__ double red[2][32];
+    const int t = threadIdx.x, n = a.n, lane = t & 31, warp = t >> 5;
     const int k = *kdev;
     int64_t* hdr = reinterpret_cast<int64_t*>(partials);
     double* vals = partials + kPartialsHeader + (n + 2);
@@ -407,34 +291,44 @@ __global__ void __launch_bounds__(kFinishThreads) finish_received_kernel(FinishA
     for (int j = t; j < n; j += kFinishThreads) vals[j] = 0.0;
     double g2 = 0.0, rs = 0.0;
     for (int l = 0; l < a.L; ++l) {
+#pragma unroll 8
         for (int64_t i = t; i < a.npw[l]; i += kFinishThreads) g2 += a.pw[l][i];
         for (int i = t; i < a.npb[l]; i += kFinishThreads) g2 += a.pb[l][i];
     }
     __syncthreads();   // zeros above land before the received rows below
-    const int groups = a.B / 32;   // 32-row groups per worker
+    const int per = a.B / 32 * a.CT;   // pieces of a worker and layer: 32-row groups x column tiles
     for (int s = t; s < k; s += kFinishThreads) {
         double v = 0.0;
         for (int l = 0; l < a.L; ++l) {
-            const double* pg = a.pg[l] + static_cast<int64_t>(s) * groups * a.CT;
-            for (int i = 0; i < groups * a.CT; ++i) v += pg[i];
+            const double* pg = a.pg[l] + static_cast<int64_t>(s) * per;
+#pragma unroll 8
+            for (int i = 0; i < per; ++i) v += pg[i];
         }
         vals[sel[s]] = v;
         rs += v;
     }
-    red[0][t] = g2;
-    red[1][t] = rs;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        g2 += __shfl_xor_sync(0xffffffffu, g2, o);
+        rs += __shfl_xor_sync(0xffffffffu, rs, o);
+    }
+    if (lane == 0) {
+        red[0][warp] = g2;
+        red[1][warp] = rs;
+    }
     __syncthreads();
-    for (int h = kFinishThreads / 2; h > 0; h >>= 1) {
-        if (t < h) {
-            red[0][t] += red[0][t + h];
-            red[1][t] += red[1][t + h];
-        }
-        __syncthreads();
+    if (t >= 32) return;
+    g2 = red[0][lane];
+    rs = red[1][lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        g2 += __shfl_xor_sync(0xffffffffu, g2, o);
+        rs += __shfl_xor_sync(0xffffffffu, rs, o);
     }
     if (t == 0) {
         if (k > 0) {
-            vals[n + 1] = red[0][0];
-            vals[n] = red[1][0] - static_cast<double>(k) * red[0][0];
+            vals[n + 1] = g2;
+            vals[n] = rs - static_cast<double>(k) * g2;
         } else {
             vals[n + 1] = NAN;
             vals[n] = NAN;
@@ -472,8 +366,8 @@ bool make_tc_plan(int L, const int32_t* widths, int n, int B, TcPlan* P) {
     if (!make_grads_plan(L, widths, n, B, DBW_PREC_BF16, &g)) return false;
     P->g = g;
     const int64_t M = static_cast<int64_t>(n) * B;
-    int maxw = 0;
-    for (int l = 0; l <= L; ++l) maxw = widths[l] > maxw ? widths[l] : maxw;
+    int maxw = 0;   // of the layers dZ is formed for
+    for (int l = 1; l <= L; ++l) maxw = widths[l] > maxw ? widths[l] : maxw;
     size_t cur = 0;
     auto take = [&](size_t bytes) {
         const size_t at = cur;
@@ -481,6 +375,7 @@ bool make_tc_plan(int L, const int32_t* widths, int n, int B, TcPlan* P) {
         return at;
     };
     P->off_status = take(256);
+    P->off_cnt = take(static_cast<size_t>(n) * 4);
     for (int l = 0; l < L; ++l) {
         P->ldw[l] = rup(widths[l], 8);
         P->off_wb[l] = take(static_cast<size_t>(widths[l + 1]) * P->ldw[l] * 2);
@@ -505,7 +400,8 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
     const int L = g.L, M = g.M, B = g.B, n = g.n;
     int* status = reinterpret_cast<int*>(ws + P.off_status);
     auto bf = [&](size_t off) { return reinterpret_cast<__nv_bfloat16*>(ws + off); };
-    cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
+    int* cnt = reinterpret_cast<int*>(ws + P.off_cnt);
+    cudaError_t e = cudaMemsetAsync(status, 0, P.off_cnt - P.off_status + n * sizeof(int), st);   // and the counters
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
 
     launch_weight_casts(P, w, ws, st);
@@ -536,9 +432,7 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
     const int C = g.widths[L];
     float* sloss = reinterpret_cast<float*>(ws + P.off_sloss);
     int cur = 0;
-    softmax_xent_ld_kernel<<<n, 256, 0, st>>>(logits, P.ldlog, C, B, idx, S, labels, sloss, bf(P.off_dz[0]), P.ldz,
-                                              loss);
-    e = cudaGetLastError();
+    e = launch_softmax(logits, P.ldlog, C, n, B, idx, S, labels, sloss, bf(P.off_dz[0]), P.ldz, loss, cnt, st);
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
 
     // backward
@@ -551,9 +445,7 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
         ep.ldrow = fin;
         int rc = tc_dw({bf(P.off_dz[cur]), P.ldz, bf(P.off_act[l]), P.ldact[l], fout, fin, B}, n, ep, status, st);
         if (rc) return rc;
-        bias_grad_ld_kernel<<<dim3((fout + 127) / 128, n), 128, 0, st>>>(bf(P.off_dz[cur]), P.ldz, fout, B, G, ld,
-                                                                          g.offb[l]);
-        e = cudaGetLastError();
+        e = launch_bias_grad(bf(P.off_dz[cur]), P.ldz, fout, n, B, G, ld, g.offb[l], st);
         if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
         if (l > 0) {
             TcEpi ex{};
@@ -629,7 +521,8 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
     auto bf = [&](size_t off) { return reinterpret_cast<__nv_bfloat16*>(ws + off); };
     auto f64 = [&](size_t off) { return reinterpret_cast<double*>(ws + off); };
     const char* what = "dbw_received_grads_update";
-    cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
+    int* cnt = reinterpret_cast<int*>(ws + T.off_cnt);
+    cudaError_t e = cudaMemsetAsync(status, 0, T.off_cnt - T.off_status + n * sizeof(int), st);   // and the counters
     if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 
     int* gcnt = reinterpret_cast<int*>(ws + P.off_gcnt);
@@ -663,9 +556,8 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
     }
     const int C = g.widths[L];
     float* sloss = reinterpret_cast<float*>(ws + T.off_sloss);
-    softmax_xent_ld_kernel<<<n, 256, 0, st>>>(logits, T.ldlog, C, B, idx, S, labels, sloss, bf(P.off_dzl[L - 1]),
-                                              T.ldz, loss, sel, kdev);
-    e = cudaGetLastError();
+    e = launch_softmax(logits, T.ldlog, C, n, B, idx, S, labels, sloss, bf(P.off_dzl[L - 1]), T.ldz, loss, cnt, st, sel,
+                       kdev);
     if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 
     // backward: per layer the mean gradient with the SGD step and dZ of the layer below in
