@@ -504,7 +504,16 @@ bool make_rx_plan(int L, const int32_t* widths, int n, int B, RxPlan* P) {
     }
     P->off_gpart = take(tc_gram_partial_floats(g.M, B, L) * 4);
     P->ngcnt = static_cast<int>(tc_gram_items(g.M, B, L));
-    P->off_gcnt = take(static_cast<size_t>(P->ngcnt) * 4);
+    size_t part = 0, pcnt = 0;
+    for (int l = 0; l < L; ++l) {
+        const size_t f = tc_split_floats(g.widths[l + 1], g.widths[l]), c = tc_split_counters(g.widths[l + 1], g.widths[l]);
+        part = f > part ? f : part;
+        pcnt = c > pcnt ? c : pcnt;
+    }
+    P->npcnt = static_cast<int>(pcnt);
+    P->off_gcnt = take((static_cast<size_t>(P->ngcnt) + pcnt) * 4);
+    P->off_pcnt = P->off_gcnt + static_cast<size_t>(P->ngcnt) * 4;
+    P->off_part = take(part * 4);
     P->ws_bytes = cur;
     return true;
 }
@@ -527,7 +536,7 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
 
     int* gcnt = reinterpret_cast<int*>(ws + P.off_gcnt);
     float* gpart = reinterpret_cast<float*>(ws + P.off_gpart);
-    compact_received_kernel<<<1, 1024, 0, st>>>(mask, n, sel, kdev, loss, gcnt, P.ngcnt);
+    compact_received_kernel<<<1, 1024, 0, st>>>(mask, n, sel, kdev, loss, gcnt, P.ngcnt + P.npcnt);
     launch_weight_casts(T, w, ws, st);
     cast_rows_kernel<<<row_ctas(M), 256, 0, st>>>(pool, g.widths[0], M, g.widths[0], ReceivedRows{idx, sel, kdev, B, S},
                                                   bf(T.off_act[0]), T.ldact[0]);
@@ -571,6 +580,8 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
         gb.off = g.offW[l];
         gb.ldrow = fin;
         gb.pieces = f64(P.off_pw[l]);
+        gb.part = reinterpret_cast<float*>(ws + P.off_part);
+        gb.part_cnt = reinterpret_cast<int*>(ws + P.off_pcnt);
         gb.kdev = kdev;
         gb.kmul = B;
         const TcOperands go{bf(P.off_dzl[l]), T.ldz, bf(T.off_act[l]), T.ldact[l], fout, fin, M};
