@@ -1231,6 +1231,20 @@ bool tc_make_map_f32(CUtensorMap* tm, const void* base, int64_t rows, int64_t co
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool tc_make_batch_map_f32(CUtensorMap* tm, const void* base, int64_t rows, int64_t batch, int64_t cols_z, int64_t ld_z,
+                           int box_rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols_z), static_cast<cuuint64_t>(batch),
+                          static_cast<cuuint64_t>(rows)};
+    cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld_z * 4), static_cast<cuuint64_t>(batch * ld_z * 4)};
+    cuuint32_t box[3] = {32u, 1u, static_cast<cuuint32_t>(box_rows)};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 static bool operands_ok(const TcOperands& o) {
     return encode_fn() && o.lda % 8 == 0 && o.ldb % 8 == 0 && (reinterpret_cast<uintptr_t>(o.A) & 15u) == 0 &&
            (reinterpret_cast<uintptr_t>(o.B) & 15u) == 0 && o.K >= 1;

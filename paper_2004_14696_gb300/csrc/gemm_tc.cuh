@@ -82,6 +82,11 @@ bool tc_make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, 
 // The same for a row-major fp32 matrix: box 32 (128 bytes, 128-byte swizzle) x box_rows;
 // ld a multiple of 4 and base 16-byte aligned.
 bool tc_make_map_f32(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows);
+// Row-major fp32 [rows, batch blocks of ld_z columns, the first cols_z of them used]:
+// dimensions (column of the block, block, row), box 32 x 1 x box_rows; columns past cols_z
+// of a block read as zero.  ld_z a multiple of 4.
+bool tc_make_batch_map_f32(CUtensorMap* tm, const void* base, int64_t rows, int64_t batch, int64_t cols_z, int64_t ld_z,
+                           int box_rows);
 
 // The mean-gradient GEMM (TC_GBAR, operands g, epilogue ge) and the input-gradient
 // GEMM (TC_DX, operands x, epilogue xe) of one layer in one launch: both read dZ_l

@@ -93,9 +93,10 @@ __global__ void split4_kernel(const float* __restrict__ src, int rows, int cols,
                               float* __restrict__ hi, float* __restrict__ lo, int64_t ldo);
 // Launches split4_kernel where its alignment holds, else split_kernel.
 void split(const float* src, int rows, int cols, int64_t lds, float* hi, float* lo, int64_t ldo, cudaStream_t st);
-// The same, transposed: hiT[c * ldt + r], loT[c * ldt + r] for r < rows, c < cols
-// (32 x 32 tiles through shared memory; blocks of 32 x 8 threads).
-__global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols, int64_t lds,
+// The same, transposed: hiT[c * ldt + t], loT[c * ldt + t] with t = r + (r / B) pad for r <
+// rows, c < cols: the workers' B samples in blocks of B + pad columns (32 x 32 tiles through
+// shared memory; blocks of 32 x 8 threads).
+__global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols, int64_t lds, int B, int pad,
                                float* __restrict__ hiT, float* __restrict__ loT, int64_t ldt);
 
 template <int BN, int STAGES, int NMAIN, class Epi>
@@ -267,13 +268,18 @@ cudaError_t run(int M, int N, int K, const float* A, int64_t lda, const float* B
 
 // ------------------------------------------------------------------ per-worker weight gradient
 // G[z, off + o ldrow + c] = sum_{r < K} dZ[z K + r, o] act[z K + r, c] for every worker z,
-// in three tf32 passes: A = the hi / lo parts of dZ^T [Mr = out rows, z K + r], B = those
-// of act^T [Nr = in rows, z K + r], both K-major (the transposed parts are written by
-// split_t_kernel).  A persistent grid walks 128 x 128 tiles (out x in) worker-major with
+// in three tf32 passes: A = the hi / lo parts of dZ^T [Mr = out rows, z Kp + r], B = those
+// of act^T [Nr = in rows, z Kp + r], both K-major (the transposed parts are written by
+// split_t_kernel; Kp = K rounded up to 4 for the 16-byte strides, and the 3-D tensor maps
+// read zeros past a worker's K samples, so any K runs here).  A persistent grid walks 128 x 128 tiles (out x in) worker-major with
 // the in-tiles fastest; each tile has a hi.hi accumulator and a correction accumulator
 // (256 TMEM columns), two tiles in flight (512 columns), so that the MMAs of tile i + 1
-// run while the epilogue drains tile i.  With K = B <= 256 the hi.hi accumulator takes at
-// most 32 MMA additions.  Eight epilogue warps, two per TMEM lane quarter (32 G rows),
+// run while the epilogue drains tile i.  A K above 256 goes in chunks of 256 samples, each
+// into the next accumulator pair, which the epilogue warps add up in registers (rounding to
+// nearest), so a hi.hi accumulator takes at most 32 MMA additions.  (784-256-10, 16 workers
+// of 500 samples: both layers' weight gradients took 175 us on fp32 FFMA tiles, which
+// served B % 32 != 0 and B > 256; now 42 here, 7 for the parts of dZ, and 14 in the
+// few-output kernel.)  Eight epilogue warps, two per TMEM lane quarter (32 G rows),
 // each copy their 32 x 64 block TMEM -> registers (hi.hi + corrections, rounded to
 // nearest; its four TMEM loads in flight together) -> shared memory (16-byte pieces
 // XOR-swizzled by row) and then store it, 256 contiguous bytes of each of two G rows per
@@ -296,9 +302,32 @@ static_assert(WARP_COLS % 32 == 0 && EPI_WARPS % 4 == 0, "whole 32-column segmen
 constexpr int SMEM = STAGES * STAGE_BYTES + EPI_WARPS * WARP_STAGING + 256 + 1024;
 constexpr int TILE_COLS = 2 * BN;                         // hi.hi, then the corrections
 constexpr int TMEM_COLS = 2 * TILE_COLS;
-constexpr int kMaxK = 256;
+constexpr int CHUNK = 8;   // 32-deep K blocks of a chunk
 }  // namespace dw
 
+// v = (or +=) main + corrections, 32 columns of one row.
+static __device__ __forceinline__ void add_parts(float4 (&v)[8], const uint32_t (&rm)[32], const uint32_t (&rc)[32],
+                                                 bool first) {
+    using tcx::u2f;
+#pragma unroll
+    for (int pc = 0; pc < 8; ++pc) {
+        float4 x;
+        x.x = u2f(rm[4 * pc]) + u2f(rc[4 * pc]);
+        x.y = u2f(rm[4 * pc + 1]) + u2f(rc[4 * pc + 1]);
+        x.z = u2f(rm[4 * pc + 2]) + u2f(rc[4 * pc + 2]);
+        x.w = u2f(rm[4 * pc + 3]) + u2f(rc[4 * pc + 3]);
+        if (!first) {
+            x.x += v[pc].x;
+            x.y += v[pc].y;
+            x.z += v[pc].z;
+            x.w += v[pc].w;
+        }
+        v[pc] = x;
+    }
+}
+
+// kChunks: K spans several chunks.
+template <bool kChunks>
 static __global__ void __launch_bounds__(dw::THREADS, 1)
     dw_kernel(const __grid_constant__ Operands op, int Mr, int Nr, int K, int batch, int* status,
               float* __restrict__ Gbase, int64_t ldrow, int64_t ldG) {
@@ -362,11 +391,10 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
                 }
                 const uint32_t fb = smem_u32(full_bar + s);
                 mbar_expect_tx(fb, dw::STAGE_BYTES);
-                const int kx = z * K + kb * BK;
-                tma_load_2d(smem_u32(part(s, 0)), &op.a_hi, kx, m0, fb);
-                tma_load_2d(smem_u32(part(s, 1)), &op.a_lo, kx, m0, fb);
-                tma_load_2d(smem_u32(part(s, 2)), &op.b_hi, kx, n0, fb);
-                tma_load_2d(smem_u32(part(s, 3)), &op.b_lo, kx, n0, fb);
+                tma_load_3d(smem_u32(part(s, 0)), &op.a_hi, kb * BK, z, m0, fb);
+                tma_load_3d(smem_u32(part(s, 1)), &op.a_lo, kb * BK, z, m0, fb);
+                tma_load_3d(smem_u32(part(s, 2)), &op.b_hi, kb * BK, z, n0, fb);
+                tma_load_3d(smem_u32(part(s, 3)), &op.b_lo, kb * BK, z, n0, fb);
                 issued = g + 1;
             }
         }
@@ -378,90 +406,114 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
         // ---------------- MMA issuer
         constexpr uint32_t idesc = instr_desc_tf32(BM, dw::BN);
         long long g = 0;
-        int i = 0;
-        for (long long t = blockIdx.x; t < total && !*vabort; t += gridDim.x, ++i) {
-            const int acc = i & 1;
-            const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
-            if (!mbar_wait(smem_u32(tempty_bar + acc), aph ^ 1)) {
-                atomicOr(status, 1);
-                *vabort = 1;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t dmain = tmem + static_cast<uint32_t>(acc * dw::TILE_COLS);
-            const uint32_t dcorr = dmain + dw::BN;
-            bool ok = true;
-            for (int kb = 0; kb < nk; ++kb, ++g) {
-                const int s = static_cast<int>(g % dw::STAGES);
-                const uint32_t ph = static_cast<uint32_t>((g / dw::STAGES) & 1);
-                if (!mbar_wait(smem_u32(full_bar + s), ph)) {
+        int i = 0;   // chunks so far
+        bool ok = true;
+        for (long long t = blockIdx.x; t < total && ok && !*vabort; t += gridDim.x) {
+            for (int k0 = 0; k0 < nk && ok; k0 += dw::CHUNK, ++i) {
+                const int acc = i & 1;
+                const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
+                if (!mbar_wait(smem_u32(tempty_bar + acc), aph ^ 1)) {
                     atomicOr(status, 1);
                     *vabort = 1;
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t ah = smem_u32(part(s, 0)), al = smem_u32(part(s, 1));
-                const uint32_t bh = smem_u32(part(s, 2)), bl = smem_u32(part(s, 3));
+                const uint32_t dmain = tmem + static_cast<uint32_t>(acc * dw::TILE_COLS);
+                const uint32_t dcorr = dmain + dw::BN;
+                const int k1 = k0 + dw::CHUNK < nk ? k0 + dw::CHUNK : nk;
+                for (int kb = k0; kb < k1; ++kb, ++g) {
+                    const int s = static_cast<int>(g % dw::STAGES);
+                    const uint32_t ph = static_cast<uint32_t>((g / dw::STAGES) & 1);
+                    if (!mbar_wait(smem_u32(full_bar + s), ph)) {
+                        atomicOr(status, 1);
+                        *vabort = 1;
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t ah = smem_u32(part(s, 0)), al = smem_u32(part(s, 1));
+                    const uint32_t bh = smem_u32(part(s, 2)), bl = smem_u32(part(s, 3));
 #pragma unroll
-                for (int kk = 0; kk < BK / 8; ++kk) {
-                    const uint32_t o = kk * 32;
-                    const uint32_t accum = (kb > 0 || kk > 0) ? 1u : 0u;
-                    tc_mma_tf32(dmain, smem_desc(ah + o, 128), smem_desc(bh + o, 128), idesc, accum);
-                    tc_mma_tf32(dcorr, smem_desc(ah + o, 128), smem_desc(bl + o, 128), idesc, accum);
-                    tc_mma_tf32(dcorr, smem_desc(al + o, 128), smem_desc(bh + o, 128), idesc, 1u);
+                    for (int kk = 0; kk < BK / 8; ++kk) {
+                        if (kb * BK + 8 * kk >= K) break;   // samples past K are zero
+                        const uint32_t o = kk * 32;
+                        const uint32_t accum = (kb > k0 || kk > 0) ? 1u : 0u;
+                        tc_mma_tf32(dmain, smem_desc(ah + o, 128), smem_desc(bh + o, 128), idesc, accum);
+                        tc_mma_tf32(dcorr, smem_desc(ah + o, 128), smem_desc(bl + o, 128), idesc, accum);
+                        tc_mma_tf32(dcorr, smem_desc(al + o, 128), smem_desc(bh + o, 128), idesc, 1u);
+                    }
+                    tc_commit(smem_u32(empty_bar + s));
                 }
-                tc_commit(smem_u32(empty_bar + s));
+                tc_commit(smem_u32(tfull_bar + acc));
             }
-            tc_commit(smem_u32(tfull_bar + acc));
-            if (!ok) break;
         }
     } else if (warp >= 2) {
         // ---------------- epilogue
         const int q = warp & 3;          // TMEM lanes 32 q .. 32 q + 31 = G rows m0 + 32 q ..
         const int h = (warp - 2) >> 2;   // columns [WARP_COLS h, WARP_COLS (h + 1)) of the tile
         uint8_t* buf = staging + (warp - 2) * dw::WARP_STAGING;
-        int i = 0;
-        for (long long t = blockIdx.x; t < total; t += gridDim.x, ++i) {
-            const int acc = i & 1;
-            const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
-            if (!mbar_wait(smem_u32(tfull_bar + acc), aph)) {
-                atomicOr(status, 1);
-                *vabort = 1;
-                break;
-            }
-            if (*vabort) break;
-            tc_fence_after();
+        int i = 0;   // chunks so far
+        bool ok = true;
+        for (long long t = blockIdx.x; t < total && ok; t += gridDim.x) {
             const int z = static_cast<int>(t / tiles_per_z);
             const int rem = static_cast<int>(t % tiles_per_z);
             const int m0 = (rem / nt_n) * BM, n0 = (rem % nt_n) * dw::BN;
-            const uint32_t tbase =
-                tmem + static_cast<uint32_t>(acc * dw::TILE_COLS) + (static_cast<uint32_t>(q * 32) << 16);
             const int row0 = m0 + q * 32;
             const int c0 = h * dw::WARP_COLS;   // this warp's first column of the tile
-            if (row0 < Mr && n0 + c0 < Nr) {
-                // TMEM -> smem, every segment's loads in flight together: lane = row; piece p of
-                // 128-byte segment s of row r at r * ROW_BYTES + s * 128 + ((p ^ (r & 7)) * 16)
-                uint32_t rm[dw::NSEG][32], rc[dw::NSEG][32];
-#pragma unroll
-                for (int sg = 0; sg < dw::NSEG; ++sg) {
-                    tc_ld_32cols(tbase + c0 + 32 * sg, rm[sg]);
-                    tc_ld_32cols(tbase + dw::BN + c0 + 32 * sg, rc[sg]);
+            const bool live = row0 < Mr && n0 + c0 < Nr;
+            float4 v[dw::NSEG][8];   // this lane's row of the warp's block
+            for (int k0 = 0; k0 < nk; k0 += dw::CHUNK, ++i) {
+                const int acc = i & 1;
+                const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
+                if (!mbar_wait(smem_u32(tfull_bar + acc), aph)) {
+                    atomicOr(status, 1);
+                    *vabort = 1;
+                    ok = false;
+                    break;
                 }
-                tc_wait_ld();
+                if (*vabort) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t tbase =
+                    tmem + static_cast<uint32_t>(acc * dw::TILE_COLS) + (static_cast<uint32_t>(q * 32) << 16);
+                if (live) {
+                    if constexpr (!kChunks) {   // every segment's TMEM loads in flight together
+                        uint32_t rm[dw::NSEG][32], rc[dw::NSEG][32];
 #pragma unroll
-                for (int sg = 0; sg < dw::NSEG; ++sg) {
+                        for (int sg = 0; sg < dw::NSEG; ++sg) {
+                            tc_ld_32cols(tbase + c0 + 32 * sg, rm[sg]);
+                            tc_ld_32cols(tbase + dw::BN + c0 + 32 * sg, rc[sg]);
+                        }
+                        tc_wait_ld();
 #pragma unroll
-                    for (int pc = 0; pc < 8; ++pc) {
-                        float4 v;
-                        v.x = u2f(rm[sg][4 * pc]) + u2f(rc[sg][4 * pc]);
-                        v.y = u2f(rm[sg][4 * pc + 1]) + u2f(rc[sg][4 * pc + 1]);
-                        v.z = u2f(rm[sg][4 * pc + 2]) + u2f(rc[sg][4 * pc + 2]);
-                        v.w = u2f(rm[sg][4 * pc + 3]) + u2f(rc[sg][4 * pc + 3]);
-                        *reinterpret_cast<float4*>(buf + lane * dw::ROW_BYTES + sg * 128 + ((pc ^ (lane & 7)) << 4)) =
-                            v;
+                        for (int sg = 0; sg < dw::NSEG; ++sg) add_parts(v[sg], rm[sg], rc[sg], true);
+                    } else {
+#pragma unroll
+                        for (int sg = 0; sg < dw::NSEG; ++sg) {
+                            uint32_t rm[32], rc[32];
+                            tc_ld_32cols(tbase + c0 + 32 * sg, rm);
+                            tc_ld_32cols(tbase + dw::BN + c0 + 32 * sg, rc);
+                            tc_wait_ld();
+                            add_parts(v[sg], rm, rc, k0 == 0);
+                        }
                     }
                 }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(tempty_bar + acc));
+            }
+            if (ok && live) {
+                // registers -> smem: lane = row; piece p of 128-byte segment s of row r at
+                // r * ROW_BYTES + s * 128 + ((p ^ (r & 7)) * 16)
+#pragma unroll
+                for (int sg = 0; sg < dw::NSEG; ++sg)
+#pragma unroll
+                    for (int pc = 0; pc < 8; ++pc)
+                        *reinterpret_cast<float4*>(buf + lane * dw::ROW_BYTES + sg * 128 + ((pc ^ (lane & 7)) << 4)) =
+                            v[sg][pc];
                 __syncwarp();
                 // smem -> G, ROWS_PER_STORE rows per instruction: a lane writes columns
                 // n0 + c0 + 4 piece .. + 3 of row rr + ro (ROW_BYTES contiguous bytes of each row)
@@ -480,9 +532,6 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
                 }
                 __syncwarp();
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(tempty_bar + acc));
         }
     }
     tc_fence_before();
@@ -493,35 +542,43 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
     }
 }
 
+// Samples of a worker's block in the transposed parts (16-byte strides).
+__host__ __device__ inline int64_t padded_samples(int64_t B) { return (B + 3) / 4 * 4; }
+
 // Per-worker weight gradient of one layer: dz [batch K, Mr] and act [batch K, Nr]
 // (row-major fp32, row strides ldz / lda) -> G[z ldG + o ldrow + c] (Gbase = G + the
-// layer's offset).  Needs K % 32 == 0, K <= 256, Nr % 4 == 0, ldrow % 4 == 0, ldG % 4 == 0
-// and Gbase 16-byte aligned (the caller checks).  zt_hi / zt_lo: [Mr, batch K] scratch,
-// at_hi / at_lo: [Nr, batch K] scratch.
+// layer's offset).  Needs Nr % 4 == 0, ldrow % 4 == 0, ldG % 4 == 0 and Gbase 16-byte
+// aligned (the caller checks).  zt_hi / zt_lo: [Mr, batch Kp] scratch, at_hi / at_lo: [Nr,
+// batch Kp] scratch, Kp = padded_samples(K).
 // act_parts_ready: at_hi / at_lo already hold act's transposed parts (act is not read).
 inline cudaError_t run_dw(int Mr, int Nr, int K, int batch, const float* dz, int64_t ldz, const float* act,
                           int64_t lda, float* zt_hi, float* zt_lo, float* at_hi, float* at_lo, float* Gbase,
                           int64_t ldrow, int64_t ldG, int* status, cudaStream_t st, bool act_parts_ready = false) {
-    const int64_t Mt = static_cast<int64_t>(batch) * K;   // rows of dz / act = columns of the transposes
+    const int64_t rows = static_cast<int64_t>(batch) * K;   // rows of dz / act
+    const int64_t Kp = padded_samples(K), Mt = batch * Kp;  // columns of the transposes
+    const int pad = static_cast<int>(Kp - K);
     const dim3 blk(32, 8);
     {
-        const int64_t ry = (Mt + 31) / 32;
+        const int64_t ry = (rows + 31) / 32;
         dim3 g((Mr + 31) / 32, ry < 65535 ? static_cast<unsigned>(ry) : 65535u);
-        split_t_kernel<<<g, blk, 0, st>>>(dz, static_cast<int>(Mt), Mr, ldz, zt_hi, zt_lo, Mt);
+        split_t_kernel<<<g, blk, 0, st>>>(dz, static_cast<int>(rows), Mr, ldz, K, pad, zt_hi, zt_lo, Mt);
         if (!act_parts_ready) {
             dim3 g2((Nr + 31) / 32, g.y);
-            split_t_kernel<<<g2, blk, 0, st>>>(act, static_cast<int>(Mt), Nr, lda, at_hi, at_lo, Mt);
+            split_t_kernel<<<g2, blk, 0, st>>>(act, static_cast<int>(rows), Nr, lda, K, pad, at_hi, at_lo, Mt);
         }
     }
     Operands op;
-    if (!tc_make_map_f32(&op.a_hi, zt_hi, Mr, Mt, Mt, BM) || !tc_make_map_f32(&op.a_lo, zt_lo, Mr, Mt, Mt, BM) ||
-        !tc_make_map_f32(&op.b_hi, at_hi, Nr, Mt, Mt, dw::BN) || !tc_make_map_f32(&op.b_lo, at_lo, Nr, Mt, Mt, dw::BN))
+    if (!tc_make_batch_map_f32(&op.a_hi, zt_hi, Mr, batch, K, Kp, BM) ||
+        !tc_make_batch_map_f32(&op.a_lo, zt_lo, Mr, batch, K, Kp, BM) ||
+        !tc_make_batch_map_f32(&op.b_hi, at_hi, Nr, batch, K, Kp, dw::BN) ||
+        !tc_make_batch_map_f32(&op.b_lo, at_lo, Nr, batch, K, Kp, dw::BN))
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dw::SMEM);
+    auto kern = K > BK * dw::CHUNK ? dw_kernel<true> : dw_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dw::SMEM);
     if (e != cudaSuccess) return e;
     const long long tiles = static_cast<long long>((Mr + BM - 1) / BM) * ((Nr + dw::BN - 1) / dw::BN) * batch;
     const int grid = static_cast<int>(tiles < sm_count() ? tiles : sm_count());
-    dw_kernel<<<grid, dw::THREADS, dw::SMEM, st>>>(op, Mr, Nr, K, batch, status, Gbase, ldrow, ldG);
+    kern<<<grid, dw::THREADS, dw::SMEM, st>>>(op, Mr, Nr, K, batch, status, Gbase, ldrow, ldG);
     return cudaGetLastError();
 }
 

@@ -67,7 +67,7 @@ void split(const float* src, int rows, int cols, int64_t lds, float* hi, float* 
     }
 }
 
-__global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols, int64_t lds,
+__global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols, int64_t lds, int B, int pad,
                                float* __restrict__ hiT, float* __restrict__ loT, int64_t ldt) {
     __shared__ float tile[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
@@ -79,14 +79,15 @@ __global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols
             tile[j][tx] = (r < rows && c < cols) ? src[r * lds + c] : 0.f;
         }
         __syncthreads();
+        const int64_t r = r0 + tx;
+        const int64_t t = pad ? r + static_cast<int>(r) / B * pad : r;
         for (int j = ty; j < 32; j += 8) {
             const int c = c0 + j;
-            const int64_t r = r0 + tx;
             if (c < cols && r < rows) {
                 float h, l;
                 split_value(tile[tx][j], h, l);
-                hiT[(int64_t)c * ldt + r] = h;
-                loT[(int64_t)c * ldt + r] = l;
+                hiT[(int64_t)c * ldt + t] = h;
+                loT[(int64_t)c * ldt + t] = l;
             }
         }
         __syncthreads();
@@ -112,14 +113,15 @@ __global__ void gather_kernel(const float* __restrict__ pool, int64_t S, int in,
 
 // The gather of the fp32 pass when its first layer runs in three tf32 passes: the
 // gathered rows' tf32 parts row-major (hi / lo [M, ldo], when hi != nullptr) and
-// transposed (hiT / loT [in, ldt], when hiT != nullptr), and X itself when X != nullptr.
+// transposed (hiT / loT [in, ldt], when hiT != nullptr: the workers' B samples in blocks of
+// B + pad columns), and X itself when X != nullptr.
 // Tiles of 32 rows x 128 columns through shared memory, blocks of 32 x 8 threads: a lane
 // moves 16 bytes of a row (in, ldo multiples of 4), then 4-byte pieces of the transposed
 // rows, 128 contiguous bytes a warp.
 __global__ void gather_parts_kernel(const float* __restrict__ pool, int64_t S, int in,
                                     const int32_t* __restrict__ idx, int M, float* __restrict__ X,
                                     float* __restrict__ hi, float* __restrict__ lo, int64_t ldo,
-                                    float* __restrict__ hiT, float* __restrict__ loT, int64_t ldt) {
+                                    float* __restrict__ hiT, float* __restrict__ loT, int64_t ldt, int B, int pad) {
     __shared__ float tile[32][129];   // [row][column], padded: the transposed reads are conflict-free
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int c0 = blockIdx.x * 128;
@@ -150,11 +152,12 @@ __global__ void gather_parts_kernel(const float* __restrict__ pool, int64_t S, i
         }
         if (hiT) {
             __syncthreads();
+            const int64_t m = m0 + tx;
+            const int64_t t = pad ? m + static_cast<int>(m) / B * pad : m;
             for (int cc = ty; cc < 128; cc += 8) {
                 const int c = c0 + cc;
-                const int64_t m = m0 + tx;
                 if (c < in && m < M)
-                    tf32::split_value(tile[tx][cc], hiT[(int64_t)c * ldt + m], loT[(int64_t)c * ldt + m]);
+                    tf32::split_value(tile[tx][cc], hiT[(int64_t)c * ldt + t], loT[(int64_t)c * ldt + t]);
             }
             __syncthreads();
         }
@@ -546,6 +549,94 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
     }
 }
 
+// Weight gradient of a layer with few outputs (out <= kSkinnyN, the logits layer):
+// G[i, offW + o in + c] = sum_{r < B} dZ[i B + r, o] A[i B + r, c], and the bias part, its sum
+// over the rows of dZ alone.  CTA = 32 columns of one worker: the dZ rows sit in shared
+// memory kDwRows at a time (padded to 4 NO4 outputs), warp w takes rows w, w + 8, .. with its
+// 8 next activations loaded at a time, and the warps' sums are added in warp order; the first
+// column block also adds the bias part.  (On 128 x 128 FFMA tiles 118 of 128 rows were padding
+// and a CTA ran all B rows alone: 9.8 us for 64 workers of 64 samples, 256 x 10, and 5.4 for 16
+// of 32, 784 x 10, beside bias launches of 3.6 and 1.8; here 4.9 and under 3 with the bias.)
+constexpr int kDwRows = 128;
+template <int NO4>
+__global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict__ dZ, const float* __restrict__ A,
+                                                        int out, int in, int B, float* __restrict__ G, int64_t ldG,
+                                                        int64_t offW, int64_t offb) {
+    constexpr int NO = 4 * NO4;
+    __shared__ __align__(16) float zs[kDwRows][NO];
+    __shared__ float red[8][NO][33];
+    const int i = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = blockIdx.x * 32 + lane;
+    const float* z = dZ + (int64_t)i * B * out;
+    const float* a = A + (int64_t)i * B * in + c;
+    float acc[NO];
+#pragma unroll
+    for (int o = 0; o < NO; ++o) acc[o] = 0.f;
+    float bsum = 0.f;   // bias: output threadIdx.x % NO, rows threadIdx.x / NO, + 256 / NO, ..
+    for (int r0 = 0; r0 < B; r0 += kDwRows) {
+        const int rows = B - r0 < kDwRows ? B - r0 : kDwRows;
+        __syncthreads();   // the previous rows' reads of zs are done
+        for (int e = threadIdx.x; e < rows * NO; e += 256) {
+            const int r = e / NO, o = e % NO;
+            zs[r][o] = o < out ? z[(int64_t)(r0 + r) * out + o] : 0.f;
+        }
+        __syncthreads();
+        for (int q0 = warp; q0 < rows; q0 += 64) {
+            float av[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int r = q0 + 8 * u;
+                av[u] = r < rows && c < in ? a[(int64_t)(r0 + r) * in] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int r = q0 + 8 * u;
+                if (r >= rows) break;
+#pragma unroll
+                for (int g = 0; g < NO4; ++g) {
+                    const float4 zv = *reinterpret_cast<const float4*>(&zs[r][4 * g]);
+                    acc[4 * g] = fmaf(zv.x, av[u], acc[4 * g]);
+                    acc[4 * g + 1] = fmaf(zv.y, av[u], acc[4 * g + 1]);
+                    acc[4 * g + 2] = fmaf(zv.z, av[u], acc[4 * g + 2]);
+                    acc[4 * g + 3] = fmaf(zv.w, av[u], acc[4 * g + 3]);
+                }
+            }
+        }
+        if (blockIdx.x == 0)
+            for (int r = threadIdx.x / NO; r < rows; r += 256 / NO) bsum += zs[r][threadIdx.x % NO];
+    }
+#pragma unroll
+    for (int o = 0; o < NO; ++o) red[warp][o][lane] = acc[o];
+    __syncthreads();
+    float* g = G + (int64_t)i * ldG;
+    for (int e = threadIdx.x; e < out * 32; e += 256) {
+        const int o = e >> 5;
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += red[w][o][lane];
+        if (c < in) g[offW + (int64_t)o * in + c] = t;
+    }
+    if (blockIdx.x == 0) {
+        float* bs = &zs[0][0];   // 256 partial sums (zs holds at least 512 floats)
+        __syncthreads();
+        bs[threadIdx.x] = bsum;
+        __syncthreads();
+        if (threadIdx.x < out) {
+            float t = 0.f;
+            for (int q = 0; q < 256 / NO; ++q) t += bs[q * NO + threadIdx.x];
+            g[offb + threadIdx.x] = t;
+        }
+    }
+}
+
+cudaError_t launch_skinny_dw(const float* dZ, const float* A, int out, int in, int n, int B, float* G, int64_t ldG,
+                             int64_t offW, int64_t offb, cudaStream_t st) {
+    const dim3 grid((in + 31) / 32, n);
+    auto kern = out <= 4 ? skinny_dw_kernel<1> : out <= 8 ? skinny_dw_kernel<2> : skinny_dw_kernel<4>;
+    kern<<<grid, 256, 0, st>>>(dZ, A, out, in, B, G, ldG, offW, offb);
+    return cudaGetLastError();
+}
+
 inline bool skinny_n_ok(int N, int K) { return N <= kSkinnyN && (size_t)N * K * 4 <= kSkinnySmem; }
 inline bool skinny_k_ok(int N, int K) { return K <= kSkinnyK && ((size_t)N + 16) * K * 4 <= kSkinnySmem; }
 
@@ -597,7 +688,8 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
                 P.tf32[0] ? reinterpret_cast<float*>(ws + P.off_ahi) : nullptr,
                 P.tf32[0] ? reinterpret_cast<float*>(ws + P.off_alo) : nullptr, (in + 3) / 4 * 4,
                 P.tf32_dw[0] ? reinterpret_cast<float*>(ws + P.off_xthi) : nullptr,
-                P.tf32_dw[0] ? reinterpret_cast<float*>(ws + P.off_xtlo) : nullptr, M);
+                P.tf32_dw[0] ? reinterpret_cast<float*>(ws + P.off_xtlo) : nullptr, P.n * tf32::padded_samples(B), B,
+                static_cast<int>(tf32::padded_samples(B) - B));
         } else {
             gather_kernel<<<dim3((in + 1023) / 1024, M < 65535 ? M : 65535), 256, 0, st>>>(pool, S, in, idx, M, X);
         }
@@ -663,7 +755,9 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
         const float* Aprev = (l == 0) ? X : reinterpret_cast<const float*>(ws + P.off_act[l]);
         const float* dZl = dz[cur];
         // per-worker weight gradient: M' = fout, N' = fin, K = B; A(o, r) = dZ[r*fout + o], B(r, c) = A[r*fin + c]
-        if (P.tf32_dw[l]) {
+        if (fout <= kSkinnyN) {
+            e = launch_skinny_dw(dZl, Aprev, fout, fin, P.n, B, G, ld, P.offW[l], P.offb[l], st);
+        } else if (P.tf32_dw[l]) {
             const size_t ath = l == 0 ? P.off_xthi : P.off_athi, atl = l == 0 ? P.off_xtlo : P.off_atlo;
             e = tf32::run_dw(fout, fin, B, P.n, dZl, fout, Aprev, fin, reinterpret_cast<float*>(ws + P.off_zthi),
                              reinterpret_cast<float*>(ws + P.off_ztlo), reinterpret_cast<float*>(ws + ath),
@@ -674,7 +768,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
                                        EpiDW{G, ld, P.offW[l], fin}, st);
         }
         if (e != cudaSuccess) return fail(DBW_ECUDA, "dW GEMM %d: %s", l, cudaGetErrorString(e));
-        e = launch_bias_grad(dZl, fout, fout, P.n, B, G, ld, P.offb[l], st);
+        if (fout > kSkinnyN) e = launch_bias_grad(dZl, fout, fout, P.n, B, G, ld, P.offb[l], st);
         if (e != cudaSuccess) return fail(DBW_ECUDA, "bias grad %d: %s", l, cudaGetErrorString(e));
         if (l > 0) {
             // dZ_{l-1}[m, c] = sum_o dZ_l[m, o] W_l[o, c]: A(m, o) = dZ[m*fout + o], B(o, c) = W[o*fin + c]
@@ -764,23 +858,23 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
     P->off_alo = a_parts ? take(a_parts * 4) : 0;
     P->off_whi = w_parts ? take(w_parts * 4) : 0;
     P->off_wlo = w_parts ? take(w_parts * 4) : 0;
-    // weight gradients with at least 2^25 multiply-adds run in three tf32 passes when each
-    // worker's samples are whole 32-deep K blocks (at most 256) and the G rows of the layer
-    // take 16-byte stores
+    // weight gradients with at least 2^25 multiply-adds run in three tf32 passes when the G
+    // rows of the layer take 16-byte stores
+    const size_t Mt = (size_t)n * tf32::padded_samples(B);   // columns of the transposed parts
     size_t zt = 0, at = 0;
     for (int l = 0; l < L; ++l) {
         const int fin = widths[l], fout = widths[l + 1];
-        P->tf32_dw[l] = prec == DBW_PREC_FP32 && B % 32 == 0 && B <= tf32::dw::kMaxK && fin % 4 == 0 &&
-                        P->offW[l] % 4 == 0 && fout >= 32 && (int64_t)n * fout * fin * B >= (int64_t(1) << 25);
+        P->tf32_dw[l] = prec == DBW_PREC_FP32 && fin % 4 == 0 && P->offW[l] % 4 == 0 && fout >= 32 &&
+                        (int64_t)n * fout * fin * B >= (int64_t(1) << 25);
         if (!P->tf32_dw[l]) continue;
-        zt = (size_t)fout * P->M > zt ? (size_t)fout * P->M : zt;
-        if (l > 0) at = (size_t)fin * P->M > at ? (size_t)fin * P->M : at;
+        zt = (size_t)fout * Mt > zt ? (size_t)fout * Mt : zt;
+        if (l > 0) at = (size_t)fin * Mt > at ? (size_t)fin * Mt : at;
     }
     P->off_zthi = zt ? take(zt * 4) : 0;
     P->off_ztlo = zt ? take(zt * 4) : 0;
     P->off_athi = at ? take(at * 4) : 0;
     P->off_atlo = at ? take(at * 4) : 0;
-    const size_t xt = P->tf32_dw[0] ? (size_t)widths[0] * P->M : 0;
+    const size_t xt = P->tf32_dw[0] ? (size_t)widths[0] * Mt : 0;
     P->off_xthi = xt ? take(xt * 4) : 0;
     P->off_xtlo = xt ? take(xt * 4) : 0;
     P->ws_bytes = cur;

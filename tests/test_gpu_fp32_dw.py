@@ -1,0 +1,44 @@
+"""GPU parity of the fp32 weight gradients at minibatches off the 32-sample blocks and the
+256-sample chunks of the three-tf32-pass kernel (a worker's samples past B must read as
+zero, and the chunks add up), and of the few-output kernel around its row blocks and
+output groups: every worker's row against the oracle."""
+import pytest
+import torch
+
+from paper_2004_14696_gb300 import dbw, workloads
+from paper_2004_14696_gb300.pipeline import Iteration
+from gpu_util import RTOL_FP32, assert_worker_grads_match, gpu_active_sets
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+    torch.cuda.set_device(0)
+
+
+# n out in B >= 2^25 in the first layer: three tf32 passes there; the last layers have few outputs
+CASES = [((1028, 256, 10), n, B) for n, B in ((128, 1), (64, 3), (43, 7), (9, 31), (5, 33), (3, 255), (2, 257), (1, 513),
+                                              (2, 500))]
+CASES += [((516, 200, 136, 12), 21, 90), ((40, 4), 3, 127), ((40, 5), 3, 128), ((33 * 4, 8), 2, 129),
+          ((40, 16), 2, 300), ((64, 17), 2, 65), ((784, 10), 2, 1), ((24, 9, 3), 1, 1)]
+
+
+@pytest.mark.parametrize("widths,n,B", CASES, ids=lambda v: "-".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_fp32_gradients_at_any_batch(widths, n, B):
+    wl = workloads.Workload(key="fp32_dw", widths=widths, n=n, B=B, prec=workloads.PREC_FP32, S=300,
+                            feature_dist="normal", time_model="shifted_exp",
+                            time_params={"shift": 1.0, "rate": 1.0}, lr=0.01, seed_offset=112)
+    it = Iteration(wl, static_b=0)
+    idx, _ = it.host_inputs(0)
+    it.load_inputs(0)
+    it.G.fill_(float("nan"))
+    it.ws.fill_(255)   # NaN everywhere: nothing may be read that this call did not write
+    dbw.dbw_worker_grads(wl.widths, wl.prec, it.w, it.pool, it.labels, it.idx, n, B, it.G, it.loss, it.ws)
+    torch.cuda.synchronize()
+    assert int(it.ws[:4].view(torch.int32).item()) == 0, "device status word set"
+    pool, labels, w = it.pool.cpu().numpy(), it.labels.cpu().numpy(), it.w.cpu().numpy()
+    assert_worker_grads_match(it.G.cpu().numpy()[:, :wl.d], it.loss.cpu().numpy(), widths, w, pool[idx], labels[idx],
+                              B, False, range(n), RTOL_FP32, gpu_active_sets(it.ws, widths, n, B, wl.prec))
