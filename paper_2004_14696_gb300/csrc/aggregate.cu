@@ -351,6 +351,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) aggregate_kernel(
     const float* __restrict__ G, int64_t ld, int n, int64_t d, const uint8_t* __restrict__ mask,
     float lr, float* __restrict__ w, float* __restrict__ gbar, double* __restrict__ partials,
     int nblocks) {
+    grid_begin();
     extern __shared__ __align__(16) double smem_d[];
     float* rings = reinterpret_cast<float*>(smem_d);   // [kWarps][R] ring slots
     double* rowacc = smem_d + kRingBytes / 8;          // [kWarps][n] fp64 row-norm pieces
@@ -404,6 +405,7 @@ __global__ void __launch_bounds__(kWideThreads, 3) aggregate_wide_kernel(
     const float* __restrict__ G, int64_t ld, int n, int64_t d, const uint8_t* __restrict__ mask,
     float lr, float* __restrict__ w, float* __restrict__ gbar, double* __restrict__ partials,
     int nblocks) {
+    grid_begin();
     using namespace tcx;
     extern __shared__ __align__(128) double smem_w[];
     float* ring = reinterpret_cast<float*>(smem_w);
@@ -566,7 +568,10 @@ cudaError_t launch_aggregate_t(const float* G, int64_t ld, int n, int64_t d, con
     auto kern = wide ? aggregate_wide_kernel<kAllRows> : aggregate_kernel<kAllRows>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<g.blocks, wide ? kWideThreads : kThreads, smem, st>>>(G, ld, n, d, mask, lr, w, gbar, partials, g.blocks);
+    // A grid of several CTAs per SM must not be set up early: CTAs placed while other kernels
+    // still hold an SM find its shared memory configured for those, fewer fit, and the rest of
+    // this grid becomes a second round (n = 64, d = 1e7 in a row: 395 us, early 523).
+    launch_when(g.blocks <= sm_count(), kern, g.blocks, wide ? kWideThreads : kThreads, smem, st, G, ld, n, d, mask, lr, w, gbar, partials, g.blocks);
     return cudaGetLastError();
 }
 }  // namespace

@@ -69,6 +69,7 @@ int scratch_address(void** out) {
 constexpr int kRed = 256;
 __global__ void __launch_bounds__(kRed) reduce_to_sums_kernel(const double* __restrict__ partials, int n,
                                                               double* __restrict__ sums_out) {
+    grid_begin();
     const int64_t* hdr = reinterpret_cast<const int64_t*>(partials);
     if (hdr[0] != kPartialsMagic || hdr[2] != n || hdr[1] < 1 || hdr[1] > (1 << 20)) {
         if (threadIdx.x == 0) sums_out[blockIdx.x] = CUDART_NAN;
@@ -126,7 +127,7 @@ extern "C" int dbw_aggregate_update_noalloc(const float* G, int64_t ld, int n, i
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_aggregate_update_noalloc: %s", cudaGetErrorString(e));
     e = launch_aggregate(G, ld, n, d, mask, lr, w, gbar, flags, partials, g, st);
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_aggregate_update_noalloc: %s", cudaGetErrorString(e));
-    reduce_to_sums_kernel<<<n + 2, kRed, 0, st>>>(partials, n, sums_out);
+    launch(reduce_to_sums_kernel, n + 2, kRed, 0, st, partials, n, sums_out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_aggregate_update_noalloc: %s", cudaGetErrorString(e));
     return call.done(DBW_OK);

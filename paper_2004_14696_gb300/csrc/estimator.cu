@@ -112,6 +112,7 @@ __global__ void __launch_bounds__(kRedThreads) grad_stats_kernel(
     double* __restrict__ partials, int n, const uint8_t* __restrict__ mask,
     const float* __restrict__ loss, const double* __restrict__ tsorted, double lr,
     dbw_state* __restrict__ st, double* __restrict__ stats_out, double* __restrict__ row_sqnorm) {
+    grid_begin();
     __shared__ double red[kRedThreads];
     const int tid = threadIdx.x;
     const int64_t* hdr = reinterpret_cast<const int64_t*>(partials);
@@ -254,6 +255,7 @@ __global__ void __launch_bounds__(1024) choose_b_kernel(dbw_state* __restrict__ 
                                                         int flags, int32_t* __restrict__ b_out,
                                                         double* __restrict__ ratio_out,
                                                         const double* __restrict__ T_ext) {
+    grid_begin();
     __shared__ double mean_s[3];
     __shared__ int ready_s;
     __shared__ double best_r[32];
@@ -351,6 +353,7 @@ __global__ void __launch_bounds__(1024) choose_b_kernel(dbw_state* __restrict__ 
 }
 
 __global__ void state_init_kernel(dbw_state* st, int n, int D) {
+    grid_begin();
     double* raw = reinterpret_cast<double*>(st);
     const int nwords = (int)(sizeof(dbw_state) / sizeof(double));
     for (int i = threadIdx.x; i < nwords; i += blockDim.x) raw[i] = 0.0;
@@ -369,14 +372,14 @@ __global__ void state_init_kernel(dbw_state* st, int n, int D) {
 }  // namespace
 
 cudaError_t launch_state_init(dbw_state* s, int n, int D, cudaStream_t st) {
-    state_init_kernel<<<1, 256, 0, st>>>(s, n, D);
+    launch(state_init_kernel, 1, 256, 0, st, s, n, D);
     return cudaGetLastError();
 }
 
 cudaError_t launch_grad_stats(const double* partials, int n, const uint8_t* mask, const float* loss,
                               const double* tsorted, double lr, dbw_state* s, double* stats_out,
                               double* row_sqnorm, cudaStream_t st) {
-    grad_stats_kernel<<<n + 1, kRedThreads, 0, st>>>(const_cast<double*>(partials), n, mask, loss, tsorted, lr, s,
+    launch(grad_stats_kernel, n + 1, kRedThreads, 0, st, const_cast<double*>(partials), n, mask, loss, tsorted, lr, s,
                                                      stats_out, row_sqnorm);
     return cudaGetLastError();
 }
@@ -384,7 +387,7 @@ cudaError_t launch_grad_stats(const double* partials, int n, const uint8_t* mask
 cudaError_t launch_choose_b(dbw_state* s, double lr, double beta, int flags, int32_t* b_out,
                             double* ratio_out, const double* T_ext, cudaStream_t st) {
     // a thread per candidate k; the launch does not know the state's n
-    choose_b_kernel<<<1, 1024, 0, st>>>(s, lr, beta, flags, b_out, ratio_out, T_ext);
+    launch(choose_b_kernel, 1, 1024, 0, st, s, lr, beta, flags, b_out, ratio_out, T_ext);
     return cudaGetLastError();
 }
 

@@ -102,6 +102,7 @@ __global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols
 template <int BN, int STAGES, int NMAIN, class Epi>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_kernel(const __grid_constant__ Operands op, int M, int N, int K, Epi epi, int* status) {
+    grid_begin();
     using C = Cfg<BN, STAGES, NMAIN>;
     using namespace tcx;
     extern __shared__ uint8_t smem_raw[];
@@ -261,7 +262,7 @@ cudaError_t run(int M, int N, int K, const float* A, int64_t lda, const float* B
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     dim3 grid((N + kBN - 1) / kBN, (M + BM - 1) / BM);
-    kern<<<grid, kThreads, C::SMEM, st>>>(op, M, N, K, epi, status);
+    launch(kern, grid, kThreads, C::SMEM, st, op, M, N, K, epi, status);
     return cudaGetLastError();
 }
 
@@ -331,6 +332,7 @@ template <bool kChunks>
 static __global__ void __launch_bounds__(dw::THREADS, 1)
     dw_kernel(const __grid_constant__ Operands op, int Mr, int Nr, int K, int batch, int* status,
               float* __restrict__ Gbase, int64_t ldrow, int64_t ldG) {
+    grid_begin();
     using namespace tcx;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -561,10 +563,10 @@ inline cudaError_t run_dw(int Mr, int Nr, int K, int batch, const float* dz, int
     {
         const int64_t ry = (rows + 31) / 32;
         dim3 g((Mr + 31) / 32, ry < 65535 ? static_cast<unsigned>(ry) : 65535u);
-        split_t_kernel<<<g, blk, 0, st>>>(dz, static_cast<int>(rows), Mr, ldz, K, pad, zt_hi, zt_lo, Mt);
+        launch(split_t_kernel, g, blk, 0, st, dz, static_cast<int>(rows), Mr, ldz, K, pad, zt_hi, zt_lo, Mt);
         if (!act_parts_ready) {
             dim3 g2((Nr + 31) / 32, g.y);
-            split_t_kernel<<<g2, blk, 0, st>>>(act, static_cast<int>(rows), Nr, lda, K, pad, at_hi, at_lo, Mt);
+            launch(split_t_kernel, g2, blk, 0, st, act, static_cast<int>(rows), Nr, lda, K, pad, at_hi, at_lo, Mt);
         }
     }
     Operands op;
@@ -578,7 +580,7 @@ inline cudaError_t run_dw(int Mr, int Nr, int K, int batch, const float* dz, int
     if (e != cudaSuccess) return e;
     const long long tiles = static_cast<long long>((Mr + BM - 1) / BM) * ((Nr + dw::BN - 1) / dw::BN) * batch;
     const int grid = static_cast<int>(tiles < sm_count() ? tiles : sm_count());
-    kern<<<grid, dw::THREADS, dw::SMEM, st>>>(op, Mr, Nr, K, batch, status, Gbase, ldrow, ldG);
+    launch(kern, grid, dw::THREADS, dw::SMEM, st, op, Mr, Nr, K, batch, status, Gbase, ldrow, ldG);
     return cudaGetLastError();
 }
 

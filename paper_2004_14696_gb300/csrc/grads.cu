@@ -27,6 +27,7 @@ namespace dbw {
 namespace tf32 {
 __global__ void split_kernel(const float* __restrict__ src, int rows, int cols, int64_t lds, float* __restrict__ hi,
                              float* __restrict__ lo, int64_t ldo) {
+    grid_begin();
     for (int r = blockIdx.y; r < rows; r += gridDim.y) {
         const float* s = src + (int64_t)r * lds;
         for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x) {
@@ -40,6 +41,7 @@ __global__ void split_kernel(const float* __restrict__ src, int rows, int cols, 
 
 __global__ void split4_kernel(const float* __restrict__ src, int rows, int cols, int64_t lds, float* __restrict__ hi,
                               float* __restrict__ lo, int64_t ldo) {
+    grid_begin();
     const int c4 = cols / 4;
     const int64_t total = (int64_t)rows * c4;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
@@ -60,15 +62,16 @@ void split(const float* src, int rows, int cols, int64_t lds, float* hi, float* 
     if (cols % 4 == 0 && lds % 4 == 0 && ldo % 4 == 0 && aligned16(src) && aligned16(hi) && aligned16(lo)) {
         const int64_t want = ((int64_t)rows * (cols / 4) + 255) / 256;
         const int blocks = static_cast<int>(want < 8 * sm_count() ? want : 8 * sm_count());
-        split4_kernel<<<blocks < 1 ? 1 : blocks, 256, 0, st>>>(src, rows, cols, lds, hi, lo, ldo);
+        launch(split4_kernel, blocks < 1 ? 1 : blocks, 256, 0, st, src, rows, cols, lds, hi, lo, ldo);
     } else {
         dim3 g((cols + 127) / 128, rows < 65535 ? rows : 65535);
-        split_kernel<<<g, 128, 0, st>>>(src, rows, cols, lds, hi, lo, ldo);
+        launch(split_kernel, g, 128, 0, st, src, rows, cols, lds, hi, lo, ldo);
     }
 }
 
 __global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols, int64_t lds, int B, int pad,
                                float* __restrict__ hiT, float* __restrict__ loT, int64_t ldt) {
+    grid_begin();
     __shared__ float tile[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int c0 = blockIdx.x * 32;
@@ -102,6 +105,7 @@ namespace {
 // reads row 0; the loss kernel poisons that worker.
 __global__ void gather_kernel(const float* __restrict__ pool, int64_t S, int in, const int32_t* __restrict__ idx,
                               int M, float* __restrict__ X) {
+    grid_begin();
     for (int m = blockIdx.y; m < M; m += gridDim.y) {
         int64_t r = idx[m];
         if (r < 0 || r >= S) r = 0;
@@ -122,6 +126,7 @@ __global__ void gather_parts_kernel(const float* __restrict__ pool, int64_t S, i
                                     const int32_t* __restrict__ idx, int M, float* __restrict__ X,
                                     float* __restrict__ hi, float* __restrict__ lo, int64_t ldo,
                                     float* __restrict__ hiT, float* __restrict__ loT, int64_t ldt, int B, int pad) {
+    grid_begin();
     __shared__ float tile[32][129];   // [row][column], padded: the transposed reads are conflict-free
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int c0 = blockIdx.x * 128;
@@ -183,6 +188,7 @@ template <bool A_K, bool B_K, class Epi, bool SPLIT>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
                                                         int64_t batchA, const float* __restrict__ B, int64_t ldb,
                                                         int64_t batchB, Epi epi, int kps, float* __restrict__ part) {
+    grid_begin();
     __shared__ __align__(16) float As[2][BK][BM];
     __shared__ __align__(16) float Bs[2][BK][BN];
     const int z = blockIdx.z;
@@ -281,6 +287,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, con
 // Sum of the splits of every output element, in split order, then the epilogue.
 template <class Epi>
 __global__ void splitk_reduce_kernel(int M, int N, int splits, const float* __restrict__ part, Epi epi) {
+    grid_begin();
     const int64_t total = (int64_t)M * N;
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
         float v = 0.f;
@@ -391,6 +398,7 @@ constexpr size_t kSkinnySmem = 48 * 1024;
 template <class Epi>
 __global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
                                                        const float* __restrict__ W, int64_t ldw, Epi epi) {
+    grid_begin();
     extern __shared__ float wsh[];   // W as [N, K] fp32
     fill_shared(wsh, N * K, [&](int e) { return (W[(int64_t)(e / K) * ldw + e % K]); });
     __syncthreads();
@@ -439,6 +447,7 @@ __global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, cons
 template <bool kTwo, class Epi>
 __global__ void __launch_bounds__(128) skinny_n4_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
                                                         const float* __restrict__ W, int64_t ldw, Epi epi) {
+    grid_begin();
     const int lane = threadIdx.x & 31;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < M; m += nwarps) {
@@ -518,6 +527,7 @@ __global__ void __launch_bounds__(128) skinny_n4_kernel(int M, int N, int K, con
 // computes the 16 rows' outputs.
 __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, const float* __restrict__ dZ, int64_t ldz,
                                                           const float* __restrict__ W, int64_t ldw, EpiDx epi) {
+    grid_begin();
     constexpr int R = 16;                               // rows per CTA
     extern __shared__ float wsh[];                      // W as [K, N] fp32, then the CTA's dZ rows [R, K]
     float* zsh = wsh + N * K;
@@ -562,6 +572,7 @@ template <int NO4>
 __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict__ dZ, const float* __restrict__ A,
                                                         int out, int in, int B, float* __restrict__ G, int64_t ldG,
                                                         int64_t offW, int64_t offb) {
+    grid_begin();
     constexpr int NO = 4 * NO4;
     __shared__ __align__(16) float zs[kDwRows][NO];
     __shared__ float red[8][NO][33];
@@ -633,7 +644,7 @@ cudaError_t launch_skinny_dw(const float* dZ, const float* A, int out, int in, i
                              int64_t offW, int64_t offb, cudaStream_t st) {
     const dim3 grid((in + 31) / 32, n);
     auto kern = out <= 4 ? skinny_dw_kernel<1> : out <= 8 ? skinny_dw_kernel<2> : skinny_dw_kernel<4>;
-    kern<<<grid, 256, 0, st>>>(dZ, A, out, in, B, G, ldG, offW, offb);
+    launch(kern, grid, 256, 0, st, dZ, A, out, in, B, G, ldG, offW, offb);
     return cudaGetLastError();
 }
 
@@ -650,15 +661,15 @@ cudaError_t run_gemm(int M, int N, int K, const float* A, int64_t lda, int64_t b
         const int kps = ((K + splits - 1) / splits + BK - 1) / BK * BK;
         splits = (K + kps - 1) / kps;
         dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, splits);
-        gemm_simt_kernel<A_K, B_K, Epi, true><<<grid, 256, 0, st>>>(M, N, K, A, lda, 0, B, ldb, 0, epi, kps,
+        launch(gemm_simt_kernel<A_K, B_K, Epi, true>, grid, 256, 0, st, M, N, K, A, lda, 0, B, ldb, 0, epi, kps,
                                                                        split_ws);
         const int64_t total = (int64_t)M * N;
         const int blocks = static_cast<int>((total + 255) / 256 < 4 * sm_count() ? (total + 255) / 256 : 4 * sm_count());
-        splitk_reduce_kernel<Epi><<<blocks, 256, 0, st>>>(M, N, splits, split_ws, epi);
+        launch(splitk_reduce_kernel<Epi>, blocks, 256, 0, st, M, N, splits, split_ws, epi);
         return cudaGetLastError();
     }
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch);
-    gemm_simt_kernel<A_K, B_K, Epi, false><<<grid, 256, 0, st>>>(M, N, K, A, lda, batchA, B, ldb, batchB, epi, K,
+    launch(gemm_simt_kernel<A_K, B_K, Epi, false>, grid, 256, 0, st, M, N, K, A, lda, batchA, B, ldb, batchB, epi, K,
                                                                     nullptr);
     return cudaGetLastError();
 }
@@ -683,7 +694,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
             // X itself only when one of them stays on SIMT
             const int ty = (M + 31) / 32;
             const bool need_x = !(P.tf32[0] && P.tf32_dw[0]);
-            gather_parts_kernel<<<dim3((in + 127) / 128, ty < 65535 ? ty : 65535), dim3(32, 8), 0, st>>>(
+            launch(gather_parts_kernel, dim3((in + 127) / 128, ty < 65535 ? ty : 65535), dim3(32, 8), 0, st, 
                 pool, S, in, idx, M, need_x ? X : nullptr,
                 P.tf32[0] ? reinterpret_cast<float*>(ws + P.off_ahi) : nullptr,
                 P.tf32[0] ? reinterpret_cast<float*>(ws + P.off_alo) : nullptr, (in + 3) / 4 * 4,
@@ -691,7 +702,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
                 P.tf32_dw[0] ? reinterpret_cast<float*>(ws + P.off_xtlo) : nullptr, P.n * tf32::padded_samples(B), B,
                 static_cast<int>(tf32::padded_samples(B) - B));
         } else {
-            gather_kernel<<<dim3((in + 1023) / 1024, M < 65535 ? M : 65535), 256, 0, st>>>(pool, S, in, idx, M, X);
+            launch(gather_kernel, dim3((in + 1023) / 1024, M < 65535 ? M : 65535), 256, 0, st, pool, S, in, idx, M, X);
         }
     }
     cudaError_t e = cudaGetLastError();
@@ -720,16 +731,16 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
                 const int want = (M + 3) / 4;   // 4 rows (warps) per CTA
                 const int grid = want < 8 * sm_count() ? want : 8 * sm_count();
                 if (fin > 256)
-                    skinny_n4_kernel<true><<<grid, 128, 0, st>>>(M, fout, fin, Ain, fin, W, fin, epi);
+                    launch(skinny_n4_kernel<true, decltype(epi)>, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
                 else
-                    skinny_n4_kernel<false><<<grid, 128, 0, st>>>(M, fout, fin, Ain, fin, W, fin, epi);
+                    launch(skinny_n4_kernel<false, decltype(epi)>, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
                 return cudaGetLastError();
             }
             if (skinny_n_ok(fout, fin)) {
                 const int rows_per_cta = 8;
                 const int want = (M + rows_per_cta - 1) / rows_per_cta;
                 const int grid = want < 2 * sm_count() ? want : 2 * sm_count();
-                skinny_n_kernel<<<grid, 256, (size_t)fout * fin * 4, st>>>(M, fout, fin, Ain, fin, W, fin, epi);
+                launch(skinny_n_kernel<decltype(epi)>, grid, 256, (size_t)fout * fin * 4, st, M, fout, fin, Ain, fin, W, fin, epi);
                 return cudaGetLastError();
             }
             return run_gemm<true, true>(M, fout, fin, Ain, fin, 0, W, fin, 0, 1, epi, st, split_ws, P.split_floats);
@@ -776,7 +787,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
             if (skinny_k_ok(fin, fout)) {
                 const int ry = (M + 15) / 16;
                 dim3 grid((fin + 255) / 256, ry < 65535 ? ry : 65535);
-                skinny_k_dx_kernel<<<grid, 256, ((size_t)fin + 16) * fout * 4, st>>>(M, fin, fout, dZl, fout,
+                launch(skinny_k_dx_kernel, grid, 256, ((size_t)fin + 16) * fout * 4, st, M, fin, fout, dZl, fout,
                                                                                   w + P.offW[l], fin,
                                                                                   EpiDx{Aprev, dnext, fin});
                 e = cudaGetLastError();

@@ -73,6 +73,7 @@ __device__ __forceinline__ void cast_row(const float* __restrict__ s, int cols, 
 template <class RowMap>
 __global__ void __launch_bounds__(256) cast_rows_kernel(const float* __restrict__ src, int64_t lds, int rows, int cols,
                                                         RowMap rowmap, __nv_bfloat16* __restrict__ out, int64_t ldo) {
+    grid_begin();
     const int live = rowmap.live(rows);
     const int warps = gridDim.x * (blockDim.x >> 5);
     for (int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < live; m += warps) {
@@ -99,6 +100,7 @@ struct WeightCasts {
 };
 
 __global__ void __launch_bounds__(256) cast_weights_kernel(WeightCasts a) {
+    grid_begin();
     const int warps = gridDim.x * (blockDim.x >> 5);
     for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < a.r0[a.L]; r += warps) {
         int l = 0;
@@ -144,6 +146,7 @@ __global__ void __launch_bounds__(1024) compact_received_kernel(const uint8_t* _
                                                                 int32_t* __restrict__ sel, int* __restrict__ kout,
                                                                 float* __restrict__ loss, int* __restrict__ zero,
                                                                 int nzero) {
+    grid_begin();
     __shared__ int warp_tot[32];
     const int j = threadIdx.x, lane = j & 31, warp = j >> 5;
     for (int q = j; q < nzero; q += blockDim.x) zero[q] = 0;
@@ -188,6 +191,7 @@ __device__ __forceinline__ int bias_layer(const BiasLayers& a, int blk) {
 // warps' sums are added in warp order into part[chunk][o].  Chunks past k B write
 // nothing.
 __global__ void __launch_bounds__(256) bias_rows_kernel(BiasLayers a, int B, const int* __restrict__ kdev) {
+    grid_begin();
     __shared__ float red[8][256];
     const int k = *kdev;
     const int rows = k > 0 ? k * B : 0;
@@ -229,6 +233,7 @@ __global__ void __launch_bounds__(256) bias_rows_kernel(BiasLayers a, int B, con
 // (fp64, fixed tree) into pieces[column block].
 __global__ void __launch_bounds__(256) bias_mean_update_kernel(BiasLayers a, int B, const int* __restrict__ kdev,
                                                                float lr) {
+    grid_begin();
     __shared__ double red[8];
     const int k = *kdev;
     const int chunks = k > 0 ? (k * B + 255) / 256 : 0;
@@ -277,6 +282,7 @@ constexpr int kFinishThreads = 1024;
 __global__ void __launch_bounds__(kFinishThreads) finish_received_kernel(FinishArgs a, const int32_t* __restrict__ sel,
                                                                          const int* __restrict__ kdev,
                                                                          double* __restrict__ partials) {
+    grid_begin();
     __shared__ double red[2][32];
     const int t = threadIdx.x, n = a.n, lane = t & 31, warp = t >> 5;
     const int k = *kdev;
@@ -358,7 +364,7 @@ static void launch_weight_casts(const TcPlan& P, const float* w, char* ws, cudaS
         a.wb[l] = reinterpret_cast<__nv_bfloat16*>(ws + P.off_wb[l]);
         a.ldw[l] = P.ldw[l];
     }
-    cast_weights_kernel<<<row_ctas(a.r0[g.L]), 256, 0, st>>>(a);
+    launch(cast_weights_kernel, row_ctas(a.r0[g.L]), 256, 0, st, a);
 }
 
 bool make_tc_plan(int L, const int32_t* widths, int n, int B, TcPlan* P) {
@@ -405,7 +411,7 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
 
     launch_weight_casts(P, w, ws, st);
-    cast_rows_kernel<<<row_ctas(M), 256, 0, st>>>(pool, g.widths[0], M, g.widths[0], GatherRows{idx, S},
+    launch(cast_rows_kernel<GatherRows>, row_ctas(M), 256, 0, st, pool, g.widths[0], M, g.widths[0], GatherRows{idx, S},
                                                   bf(P.off_act[0]), P.ldact[0]);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e));
@@ -536,9 +542,9 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
 
     int* gcnt = reinterpret_cast<int*>(ws + P.off_gcnt);
     float* gpart = reinterpret_cast<float*>(ws + P.off_gpart);
-    compact_received_kernel<<<1, 1024, 0, st>>>(mask, n, sel, kdev, loss, gcnt, P.ngcnt + P.npcnt);
+    launch(compact_received_kernel, 1, 1024, 0, st, mask, n, sel, kdev, loss, gcnt, P.ngcnt + P.npcnt);
     launch_weight_casts(T, w, ws, st);
-    cast_rows_kernel<<<row_ctas(M), 256, 0, st>>>(pool, g.widths[0], M, g.widths[0], ReceivedRows{idx, sel, kdev, B, S},
+    launch(cast_rows_kernel<ReceivedRows>, row_ctas(M), 256, 0, st, pool, g.widths[0], M, g.widths[0], ReceivedRows{idx, sel, kdev, B, S},
                                                   bf(T.off_act[0]), T.ldact[0]);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
@@ -616,8 +622,8 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
             bl.gb[l] = gbar ? gbar + g.offb[l] : nullptr;
             bl.pieces[l] = f64(P.off_pb[l]);
         }
-        bias_rows_kernel<<<dim3(bl.cb0[L], (M + 255) / 256), 256, 0, st>>>(bl, B, kdev);
-        bias_mean_update_kernel<<<bl.cb0[L], 256, 0, st>>>(bl, B, kdev, lr);
+        launch(bias_rows_kernel, dim3(bl.cb0[L], (M + 255) / 256), 256, 0, st, bl, B, kdev);
+        launch(bias_mean_update_kernel, bl.cb0[L], 256, 0, st, bl, B, kdev, lr);
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
     }
@@ -651,7 +657,7 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
         fa.npb[l] = P.npb[l];
         fa.pg[l] = f64(P.off_pg[l]);
     }
-    finish_received_kernel<<<1, kFinishThreads, 0, st>>>(fa, sel, kdev, partials);
+    launch(finish_received_kernel, 1, kFinishThreads, 0, st, fa, sel, kdev, partials);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
     return DBW_OK;

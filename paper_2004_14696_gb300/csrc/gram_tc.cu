@@ -58,6 +58,7 @@ struct GramLayers {
 __global__ void __launch_bounds__(GTHREADS, 1)
     tc_gram_kernel(const __grid_constant__ GramLayers G, int B, int CT, int target_ctas, const int* __restrict__ kdev,
                    float* __restrict__ part, int* __restrict__ cnt, int* status) {
+    grid_begin();
     const int k = *kdev;
     const long long live = static_cast<long long>(k > 0 ? k : 0) * B;   // received rows
     const int item = blockIdx.x / GSMAX, s_id = blockIdx.x % GSMAX;    // item over all layers
@@ -302,7 +303,7 @@ int tc_gram(int L, const __nv_bfloat16* const* act, const int64_t* ldA, const in
     cudaError_t e = cudaFuncSetAttribute(tc_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) {
         // ranges sized for two resident CTAs per SM
-        tc_gram_kernel<<<G.items * L * GSMAX, GTHREADS, smem, st>>>(G, B, CT, 2 * sm_count(), kdev, part, cnt,
+        launch(tc_gram_kernel, G.items * L * GSMAX, GTHREADS, smem, st, G, B, CT, 2 * sm_count(), kdev, part, cnt,
                                                                      status);
         e = cudaGetLastError();
     }

@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(kLossThreads) softmax_xent_kernel(
     const float* __restrict__ logits, int64_t ldl, int C, int B, int rows_cta, const int32_t* __restrict__ idx,
     int64_t S, const int32_t* __restrict__ labels, float* __restrict__ sample_loss, T* __restrict__ dZ, int64_t ldz,
     float* __restrict__ loss, int* __restrict__ cnt, const int32_t* __restrict__ sel, const int* __restrict__ kdev) {
+    grid_begin();
     constexpr int RW = loss_rows<NJ>();
     const int i = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kLossThreads / 32;
@@ -182,7 +183,7 @@ cudaError_t launch_softmax(const float* logits, int64_t ldl, int C, int n, int B
     const dim3 grid(n, (B + rows_cta - 1) / rows_cta);
     auto kern = C <= 32 ? softmax_xent_kernel<T, 1> : C <= 128 ? softmax_xent_kernel<T, 4>
               : C <= 1024 ? softmax_xent_kernel<T, 32> : softmax_xent_kernel<T, 0>;
-    kern<<<grid, kLossThreads, 0, st>>>(logits, ldl, C, B, rows_cta, idx, S, labels, sample_loss, dZ, ldz, loss, cnt,
+    launch(kern, grid, kLossThreads, 0, st, logits, ldl, C, B, rows_cta, idx, S, labels, sample_loss, dZ, ldz, loss, cnt,
                                         sel, kdev);
     return cudaGetLastError();
 }
@@ -209,6 +210,7 @@ template <typename T, int V>
 __global__ void __launch_bounds__(kBiasThreads) bias_grad_kernel(const T* __restrict__ dZ, int64_t ldz, int out, int B,
                                                                  int CG, float* __restrict__ G, int64_t ldG,
                                                                  int64_t offb) {
+    grid_begin();
     using Vec = typename BiasVec<T, V>::type;
     __shared__ float red[kBiasThreads * V];
     const int i = blockIdx.y;
@@ -255,7 +257,7 @@ cudaError_t launch_bias_v(const T* dZ, int64_t ldz, int out, int n, int B, float
     while (CG < 32 && CG * V < out) CG *= 2;
     const int line = 128 / (static_cast<int>(sizeof(T)) * V);
     while (CG > line && static_cast<int64_t>((out + CG * V - 1) / (CG * V)) * n < 2 * sm_count()) CG /= 2;
-    bias_grad_kernel<T, V><<<dim3((out + CG * V - 1) / (CG * V), n), kBiasThreads, 0, st>>>(dZ, ldz, out, B, CG, G, ldG,
+    launch(bias_grad_kernel<T, V>, dim3((out + CG * V - 1) / (CG * V), n), kBiasThreads, 0, st, dZ, ldz, out, B, CG, G, ldG,
                                                                                             offb);
     return cudaGetLastError();
 }

@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(1024) select_fastest_kernel(
     const double* times, int n, const int32_t* __restrict__ b_ptr,
     int32_t* __restrict__ order, uint8_t* __restrict__ mask, double* tsorted,
     int32_t* __restrict__ k_out) {
+    grid_begin();
     __shared__ double ts[DBW_NMAX];
     __shared__ unsigned long long key[DBW_NMAX];
     int b = *b_ptr;
@@ -63,9 +64,9 @@ __global__ void __launch_bounds__(1024) select_fastest_kernel(
 cudaError_t launch_select(const double* times, int n, const int32_t* b, int32_t* order,
                           uint8_t* mask, double* tsorted, int32_t* k_out, cudaStream_t st) {
     if (times < tsorted + n && tsorted < times + n)   // sorted in place: one CTA
-        select_fastest_kernel<<<1, 1024, 0, st>>>(times, n, b, order, mask, tsorted, k_out);
+        launch(select_fastest_kernel, 1, 1024, 0, st, times, n, b, order, mask, tsorted, k_out);
     else
-        select_fastest_kernel<<<(n + kSelectWarps - 1) / kSelectWarps, 32 * kSelectWarps, 0, st>>>(
+        launch(select_fastest_kernel, (n + kSelectWarps - 1) / kSelectWarps, 32 * kSelectWarps, 0, st, 
             times, n, b, order, mask, tsorted, k_out);
     return cudaGetLastError();
 }
