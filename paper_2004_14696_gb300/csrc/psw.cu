@@ -555,16 +555,692 @@ __device__ void record_sweep(float* X, float* P0, float* P1, float* P2, const fl
 
 constexpr int kFixRounds = 32;   // merging rounds of the exact block means
 
+// ------------------------------------------------------------ the fit in shared memory
+// The fit of a group table that fits in shared memory (about 27 rows at n = 256; the form
+// above serves larger ones).  A sweep is a chain of dependent accesses, so latency is its
+// time: there, with the table and the block stacks in the state buffer and chains split over
+// at most eight threads whose stacks one thread merges, a sweep of 23 rows x 256 columns took
+// 75-85 us and a whole fit of 19 / 43 / 61 sweeps 1.9 / 3.8 / 5.1 ms; here 15-18 us and
+// 0.45 / 0.96 / 1.20 ms.
+//
+// The observed cells of every chain are listed once.  A chain belongs to a group of g lanes of
+// a warp (g as large as the family's chains leave, at most 32).  Each lane pools its run of the
+// chain by pool-adjacent-violators; then neighbouring runs, pairs of runs, ... are joined at
+// their boundary in log2(g) steps: while the block before a boundary has a larger mean than the
+// one after it, they pool, and the pooled block pools on with its neighbours on both sides.  The
+// weighted isotonic regression is unique, so the blocks are those of the sequential scan.
+// A block [s, e] of chain positions keeps its sum and weight at s, LK[s] = e and LK[e] = s; any
+// other position p of it has LK[p] < p, so p starts a block iff LK[p] >= p.
+struct SharedFit {
+    int n, m, RS, MS, T;        // RS, MS: strides of a row's and a column's list
+    float *X, *P0, *P1, *W;     // fitted cells, duals of the row and column chains, weights; cell (a, i) at a RS + i + i / 32
+    float* P2;                  // [m] dual of the diagonal chain
+    float *SM, *SW;             // block sums and weights of the current family's chains
+    unsigned short* LK;
+    unsigned short *rl, *cl, *dl;   // listed cells of each row (by increasing k), column (decreasing h), diagonal
+    unsigned short *rc, *cc;    // their numbers
+    unsigned short* par;        // union-find parents
+    int *rows, *isrow;
+    double* mu;
+    int dc;
+};
+__host__ __device__ inline int fit_row_stride(int n) { return n + (n >> 5); }
+__host__ __device__ inline size_t fit_slots(int n, int m) {   // of SM, SW, LK: both families' lists
+    const size_t a = static_cast<size_t>(m) * fit_row_stride(n), b = static_cast<size_t>(n) * (m | 1);
+    return ((a > b ? a : b) + 3) / 4 * 4;
+}
+__host__ __device__ inline size_t fit_shared_fixed(int n) {
+    return (static_cast<size_t>(n) * (8 + 4 + 4 + 4 + 2 + 2 + 2) + 64) / 16 * 16;
+}
+// X, P0, P1, W, SM, SW; LK, par, the row and column lists
+__host__ __device__ inline size_t fit_shared_bytes(int n, int m) {
+    return fit_shared_fixed(n) + fit_slots(n, m) * (6 * 4 + 4 * 2);
+}
+inline int fit_shared_threads(int n) { return n < 32 ? 32 * ((n + 1) / 2 * 2) : 1024; }
+
+__device__ __forceinline__ int fit_cell(const SharedFit& s, int a, int i) { return a * s.RS + i + (i >> 5); }
+
+// Chain family F: 0 the rows (increasing in k), 1 the columns (decreasing in h), 2 the diagonal.
+// Where a chain's list (and its blocks) start, and position p of it.
+template <int F>
+__device__ __forceinline__ int fit_base(const SharedFit& s, int ch) { return F == 0 ? ch * s.RS : F == 1 ? ch * s.MS : 0; }
+template <int F>
+__device__ __forceinline__ int fit_at(int p) { return F == 0 ? p + (p >> 5) : p; }
+template <int F>
+__device__ __forceinline__ int fit_len(const SharedFit& s, int ch) { return F == 0 ? s.rc[ch] : F == 1 ? s.cc[ch] : s.dc; }
+
+// Pools a chain of len positions with values value(q, z, w) over a group of g lanes (this lane:
+// ``part``; every lane of the warp calls it, a group without a chain with len = 0), weighted
+// pool-adjacent-violators.  Position p's block entries are at at(p) of SM, SW and LK.
+template <class Real, class AtF, class ValueF>
+__device__ __forceinline__ void pool_chain(int part, int g, int len, Real* SM, Real* SW, unsigned short* LK, AtF at,
+                                           ValueF value) {
+    const int q0 = part * len / g, q1 = (part + 1) * len / g;
+    // 1) this lane's run; the open block [bs, q] in registers
+    {
+        int bs = q0;
+        Real ts = 0, tw = 0, nx = 0, nwt = 0;
+        if (q0 < q1) value(q0, nx, nwt);
+        for (int q = q0; q < q1; ++q) {
+            Real w = nwt, sm = nx * nwt;
+            if (q + 1 < q1) value(q + 1, nx, nwt);
+            LK[at(q)] = 0;   // inside a block unless it comes to start or end one
+            if (q > q0) {
+                if (ts * w > sm * tw) {   // earlier mean > this mean
+                    sm = ts + sm;
+                    w = tw + w;
+                    while (bs > q0) {
+                        const int ps = LK[at(bs - 1)];
+                        const Real psm = SM[at(ps)], psw = SW[at(ps)];
+                        if (!(psm * w > sm * psw)) break;
+                        sm = psm + sm;
+                        w = psw + w;
+                        bs = ps;
+                        LK[at(ps)] = 0;   // open again
+                    }
+                } else {   // close the open block
+                    SM[at(bs)] = ts;
+                    SW[at(bs)] = tw;
+                    LK[at(q - 1)] = static_cast<unsigned short>(bs);
+                    LK[at(bs)] = static_cast<unsigned short>(q - 1);
+                    bs = q;
+                }
+            }
+            ts = sm;
+            tw = w;
+        }
+        if (q0 < q1) {
+            SM[at(bs)] = ts;
+            SW[at(bs)] = tw;
+            LK[at(q1 - 1)] = static_cast<unsigned short>(bs);
+            LK[at(bs)] = static_cast<unsigned short>(q1 - 1);
+        }
+    }
+    __syncwarp();
+    // 2) join the runs of lanes [part - h, part) and [part, part + h)
+    for (int h = 1; h < g; h <<= 1) {
+        if ((part & (2 * h - 1)) == h) {
+            const int b0 = (part - h) * len / g, b1 = (part + h) * len / g;
+            if (b0 < q0 && q0 < b1) {
+                int S = LK[at(q0 - 1)], E = LK[at(q0)];
+                const Real lsm = SM[at(S)], lsw = SW[at(S)], rsm = SM[at(q0)], rsw = SW[at(q0)];
+                if (lsm * rsw > rsm * lsw) {
+                    Real sm = lsm + rsm, w = lsw + rsw;
+                    LK[at(q0)] = static_cast<unsigned short>(S);   // no longer a start
+                    for (;;) {
+                        if (E + 1 < b1) {
+                            const int s3 = E + 1, e3 = LK[at(s3)];
+                            const Real xsm = SM[at(s3)], xsw = SW[at(s3)];
+                            if (sm * xsw > xsm * w) {
+                                sm += xsm;
+                                w += xsw;
+                                LK[at(s3)] = static_cast<unsigned short>(S);
+                                E = e3;
+                                continue;
+                            }
+                        }
+                        if (S > b0) {
+                            const int s0 = LK[at(S - 1)];
+                            const Real xsm = SM[at(s0)], xsw = SW[at(s0)];
+                            if (xsm * w > sm * xsw) {
+                                sm += xsm;
+                                w += xsw;
+                                LK[at(S)] = static_cast<unsigned short>(s0);
+                                S = s0;
+                                continue;
+                            }
+                        }
+                        break;
+                    }
+                    SM[at(S)] = sm;
+                    SW[at(S)] = w;
+                    LK[at(E)] = static_cast<unsigned short>(S);
+                    LK[at(S)] = static_cast<unsigned short>(E);
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// Start of the block that covers this lane's first position when that is not a start itself
+// (the last start of the group's lanes before it).
+template <class AtF>
+__device__ __forceinline__ int covering_start(int part, int g, int q0, int q1, const unsigned short* LK, AtF at) {
+    int cover = -1;
+    for (int q = q0; q < q1; ++q)
+        if (LK[at(q)] >= q) cover = q;
+    for (int o = 1; o < g; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, cover, o, g);
+        if (part >= o) cover = max(cover, t);
+    }
+    return __shfl_up_sync(0xffffffffu, cover, 1, g);
+}
+
+// One Dykstra projection on family F; returns the thread's largest |change of x|.
+template <int F>
+__device__ float shared_phase(const SharedFit& s) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = s.T >> 5;
+    const int nch = F == 0 ? s.m : F == 1 ? s.n : 1, most = F == 0 ? s.n : s.m;
+    int g = 32;
+    while (g > 1 && (g * nch > s.T || g / 2 >= most)) g >>= 1;
+    const int per_warp = 32 / g, part = lane & (g - 1), sub = lane / g;
+    const unsigned short* list0 = F == 0 ? s.rl : F == 1 ? s.cl : s.dl;
+    float* pf = F == 0 ? s.P0 : F == 1 ? s.P1 : s.P2;
+    float moved = 0.f;
+    for (int c0 = warp * per_warp; c0 < nch; c0 += nw * per_warp) {
+        const int ch = c0 + sub;
+        const bool on = ch < nch;
+        const int len = on ? fit_len<F>(s, ch) : 0;
+        const int base = on ? fit_base<F>(s, ch) : 0;
+        const unsigned short* list = list0 + base;
+        float *SM = s.SM + base, *SW = s.SW + base;
+        unsigned short* LK = s.LK + base;
+        auto at = [](int p) { return fit_at<F>(p); };
+        const int q0 = part * len / g, q1 = (part + 1) * len / g;
+        // the dual of listed cell c at position q
+        auto dual = [&](int c, int q) -> float& { return F == 2 ? pf[q] : pf[c]; };
+        pool_chain(part, g, len, SM, SW, LK, at, [&](int q, float& z, float& w) {
+            const int c = list[at(q)];
+            z = s.X[c] + dual(c, q);
+            w = s.W[c];
+        });
+        // every lane assigns its run
+        const int cover = covering_start(part, g, q0, q1, LK, at);
+        bool single = false;
+        float val = 0.f;
+        for (int q = q0; q < q1; ++q) {
+            const int e = LK[at(q)];
+            const bool start = e >= q;
+            if (start || q == q0) {
+                const int b = start ? q : cover;
+                single = start && e == q;
+                val = SM[at(b)] / SW[at(b)];
+            }
+            const int c = list[at(q)];
+            float& pr = dual(c, q);
+            const float old = s.X[c], z = old + pr;
+            const float v = single ? z : val;
+            pr = z - v;
+            s.X[c] = v;
+            moved = fmaxf(moved, fabsf(v - old));
+        }
+        __syncwarp();   // the next chains of this warp reuse nothing of these, but keep the lanes together
+    }
+    return moved;
+}
+
+// f(prev, c) for every pair of consecutive listed cells of family F.
+template <int F, class EdgeF>
+__device__ void shared_edges(const SharedFit& s, EdgeF f) {
+    const int nch = F == 0 ? s.m : F == 1 ? s.n : 1, most = F == 0 ? s.n : s.m;
+    const unsigned short* list0 = F == 0 ? s.rl : F == 1 ? s.cl : s.dl;
+    for (int e = threadIdx.x; e < nch * most; e += s.T) {
+        const int ch = e / most, q = e - ch * most;
+        if (q < 1 || q >= fit_len<F>(s, ch)) continue;
+        const unsigned short* list = list0 + fit_base<F>(s, ch);
+        f(static_cast<int>(list[fit_at<F>(q - 1)]), static_cast<int>(list[fit_at<F>(q)]));
+    }
+}
+
+// uf_find / uf_union on 16-bit parents.
+__device__ __forceinline__ int uf_find16(volatile unsigned short* par, int x) {
+    for (;;) {
+        const int p = par[x];
+        if (p == x) return x;
+        const int gp = par[p];
+        if (gp != p) par[x] = static_cast<unsigned short>(gp);
+        x = p;
+    }
+}
+__device__ __forceinline__ void uf_union16(unsigned short* par, int a, int b) {
+    for (int guard = 0; guard < (1 << 22); ++guard) {
+        a = uf_find16(par, a);
+        b = uf_find16(par, b);
+        if (a == b) return;
+        if (a < b) {
+            const int t = a;
+            a = b;
+            b = t;
+        }
+        const unsigned short me = static_cast<unsigned short>(a);
+        if (atomicCAS(&par[a], me, static_cast<unsigned short>(b)) == me) return;
+    }
+}
+
+// The whole fit once the group rows are known (v.rows, v.isrow; m >= 1).
+__device__ void fit_in_shared(View& v, int n, int m, double tol, int max_sweeps, double* __restrict__ T_hat, char* smem,
+                              float* red) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, nw = T >> 5;
+    const size_t nn = static_cast<size_t>(n) * n;
+    const int32_t* cnt = v.cnt;
+    SharedFit s;
+    s.n = n;
+    s.m = m;
+    s.RS = fit_row_stride(n);
+    s.MS = m | 1;
+    s.T = T;
+    const int C = static_cast<int>(fit_slots(n, m));
+    char* at = smem;
+    auto take = [&](size_t bytes) {
+        char* r = at;
+        at += bytes;
+        return r;
+    };
+    const size_t N = static_cast<size_t>(n);
+    s.mu = reinterpret_cast<double*>(take(N * 8));
+    s.rows = reinterpret_cast<int*>(take(N * 4));
+    s.isrow = reinterpret_cast<int*>(take(N * 4));
+    s.P2 = reinterpret_cast<float*>(take(N * 4));
+    s.rc = reinterpret_cast<unsigned short*>(take(N * 2));
+    s.cc = reinterpret_cast<unsigned short*>(take(N * 2));
+    s.dl = reinterpret_cast<unsigned short*>(take(N * 2));
+    at = smem + fit_shared_fixed(n);
+    const size_t C4 = static_cast<size_t>(C) * 4, C2 = static_cast<size_t>(C) * 2;
+    s.P0 = reinterpret_cast<float*>(take(C4));   // P0 and P1 first: 8-byte words once the sweeps are over
+    s.P1 = reinterpret_cast<float*>(take(C4));
+    s.X = reinterpret_cast<float*>(take(C4));
+    s.W = reinterpret_cast<float*>(take(C4));
+    s.SM = reinterpret_cast<float*>(take(C4));
+    s.SW = reinterpret_cast<float*>(take(C4));
+    s.LK = reinterpret_cast<unsigned short*>(take(C2));
+    s.par = reinterpret_cast<unsigned short*>(take(C2));
+    s.rl = reinterpret_cast<unsigned short*>(take(C2));
+    s.cl = reinterpret_cast<unsigned short*>(take(C2));
+    s.dc = m;   // every group row's diagonal cell is observed
+    for (int i = tid; i < n; i += T) {
+        s.isrow[i] = v.isrow[i];
+        if (i < m) s.rows[i] = v.rows[i];
+    }
+    // pooled column means (exact sums, fp64) over the rows that have samples (listed in P2)
+    int* seen_rows = reinterpret_cast<int*>(s.P2);
+    for (int h = warp; h < n; h += nw) {
+        int any = 0;
+#pragma unroll 8
+        for (int i = lane; i < n; i += 32) any |= cnt[static_cast<size_t>(h) * n + i];
+        any = __any_sync(0xffffffffu, any != 0);
+        if (lane == 0) s.rc[h] = static_cast<unsigned short>(any);
+    }
+    __syncthreads();
+    int nseen = 0;
+    if (warp == 0) {
+        for (int h0 = 0; h0 < n; h0 += 32) {
+            const bool on = h0 + lane < n && s.rc[h0 + lane] != 0;
+            const unsigned bal = __ballot_sync(0xffffffffu, on);
+            if (on) seen_rows[nseen + __popc(bal & ((1u << lane) - 1u))] = h0 + lane;
+            nseen += __popc(bal);
+        }
+        if (lane == 0) s.cc[0] = static_cast<unsigned short>(nseen);
+    }
+    __syncthreads();
+    nseen = s.cc[0];
+    bool empty = false;
+    for (int i = tid; i < n; i += T) {
+        unsigned long long sm = 0;
+        long long c = 0;
+#pragma unroll 8
+        for (int q = 0; q < nseen; ++q) {
+            const size_t g = static_cast<size_t>(seen_rows[q]) * n + i;
+            sm += v.sum[g];
+            c += cnt[g];
+        }
+        s.mu[i] = c > 0 ? (static_cast<double>(sm) * kUnit) / static_cast<double>(c) : CUDART_NAN;
+        empty |= c == 0;
+    }
+    if (__syncthreads_or(empty) && tid == 0) {   // empty columns: the nearest earlier column, else the nearest later
+        int first = -1;
+        for (int i = 0; i < n; ++i) {
+            if (isnan(s.mu[i])) {
+                if (i > 0) s.mu[i] = s.mu[i - 1];
+            } else if (first < 0) {
+                first = i;
+            }
+        }
+        for (int i = 0; i < first; ++i) s.mu[i] = s.mu[first];
+    }
+    __syncthreads();   // seen_rows' memory is P2's from here
+    // targets, weights, warm start, as in the state-buffer form
+    float* lam0 = v.lam;
+    float* lam1 = v.lam + nn;
+    float* lam2 = v.lam + 2 * nn;
+    const int cells = m * n;
+    float ymax = 0.f;
+    for (int q = tid; q < cells; q += T) {
+        const int a = q / n, i = q - a * n;
+        const int c = fit_cell(s, a, i);
+        const size_t g = static_cast<size_t>(s.rows[a] - 1) * n + i;
+        const int k = cnt[g];
+        s.par[c] = static_cast<unsigned short>(c);
+        if (i == s.rows[a] - 1) s.P2[a] = 0.f;
+        if (k == 0) {
+            s.W[c] = 0.f;
+            continue;
+        }
+        const float w = static_cast<float>(k);
+        const float y = static_cast<float>((static_cast<double>(v.sum[g]) * kUnit) / static_cast<double>(k));
+        const float p0 = lam0[g] / w, p1 = lam1[g] / w, p2 = lam2[g] / w;
+        s.W[c] = w;
+        s.P0[c] = p0;
+        s.P1[c] = p1;
+        if (i == s.rows[a] - 1) s.P2[a] = p2;
+        s.X[c] = y - ((p0 + p1) + p2);
+        ymax = fmaxf(ymax, fabsf(y));
+    }
+    const float tol_abs = fmaxf(static_cast<float>(tol), kMinTol) * block_max(ymax, red);   // (its barriers end the set-up)
+    // the observed cells of each chain
+    for (int a = warp; a < m; a += nw) {
+        int count = 0;
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            const bool seen = i < n && s.W[fit_cell(s, a, i)] > 0.f;
+            const unsigned bal = __ballot_sync(0xffffffffu, seen);
+            if (seen)
+                s.rl[fit_base<0>(s, a) + fit_at<0>(count + __popc(bal & ((1u << lane) - 1u)))] =
+                    static_cast<unsigned short>(fit_cell(s, a, i));
+            count += __popc(bal);
+        }
+        if (lane == 0) {
+            s.rc[a] = static_cast<unsigned short>(count);
+            s.dl[a] = static_cast<unsigned short>(fit_cell(s, a, s.rows[a] - 1));
+        }
+    }
+    for (int i = tid; i < n; i += T) {
+        int count = 0;
+        for (int a = m - 1; a >= 0; --a) {
+            const int c = fit_cell(s, a, i);
+            if (s.W[c] > 0.f) s.cl[fit_base<1>(s, i) + count++] = static_cast<unsigned short>(c);
+        }
+        s.cc[i] = static_cast<unsigned short>(count);
+    }
+    __syncthreads();
+
+    int sweeps = 0;
+    bool converged = false;
+    while (sweeps < max_sweeps) {
+        ++sweeps;
+        float moved = shared_phase<0>(s);
+        __syncthreads();
+        moved = fmaxf(moved, shared_phase<1>(s));
+        __syncthreads();
+        moved = fmaxf(moved, shared_phase<2>(s));
+        if (block_max(moved, red) * 3.f <= tol_abs) {
+            converged = true;
+            break;
+        }
+    }
+    __syncthreads();
+    if (converged) {   // one more sweep, recording the blocks (record_sweep)
+        auto join = [&](int a, int b) {
+            if (s.X[a] == s.X[b]) uf_union16(s.par, a, b);
+        };
+        shared_phase<0>(s);
+        __syncthreads();
+        shared_edges<0>(s, join);
+        __syncthreads();
+        shared_phase<1>(s);
+        __syncthreads();
+        shared_edges<1>(s, join);
+        __syncthreads();
+        shared_phase<2>(s);
+        __syncthreads();
+        shared_edges<2>(s, join);
+        __syncthreads();
+    }
+    // keep the dual variables for the next fit; their shared memory is free after that
+    for (int q = tid; q < cells; q += T) {
+        const int a = q / n, i = q - a * n;
+        const int c = fit_cell(s, a, i);
+        const float w = s.W[c];
+        if (!(w > 0.f)) continue;
+        const size_t g = static_cast<size_t>(s.rows[a] - 1) * n + i;
+        lam0[g] = s.P0[c] * w;
+        lam1[g] = s.P1[c] * w;
+        if (i == s.rows[a] - 1) lam2[g] = s.P2[a] * w;
+        v.x[g] = s.X[c];
+    }
+    __syncthreads();
+    // exact block means (fp64 from the int64 cell sums)
+    unsigned long long* csum = reinterpret_cast<unsigned long long*>(s.P0);   // over P0 and P1
+    int* ccnt = reinterpret_cast<int*>(s.SM);
+    int* root = reinterpret_cast<int*>(s.SW);
+    bool polished = false;
+    if (converged) {
+        auto greater = [&](int a, int b) {
+            const int ra = root[a], rb = root[b];
+            if (ra == rb) return false;
+            const unsigned long long sa = csum[ra], sb = csum[rb];
+            const unsigned long long ca = static_cast<unsigned long long>(ccnt[ra]);
+            const unsigned long long cb = static_cast<unsigned long long>(ccnt[rb]);
+            const unsigned long long hi1 = __umul64hi(sa, cb), lo1 = sa * cb;
+            const unsigned long long hi2 = __umul64hi(sb, ca), lo2 = sb * ca;
+            return hi1 > hi2 || (hi1 == hi2 && lo1 > lo2);
+        };
+        int merged;
+        auto fix = [&](int a, int b) {   // pairs that break the order join one block
+            if (greater(a, b)) {
+                uf_union16(s.par, a, b);
+                merged = 1;
+            }
+        };
+        const int per = (cells + T - 1) / T;   // each thread owns a contiguous run of cells
+        const int r0 = tid * per < cells ? tid * per : cells, r1 = r0 + per < cells ? r0 + per : cells;
+        for (int round = 0; round < kFixRounds; ++round) {
+            for (int jump = 0; jump < 32; ++jump) {   // flatten the trees by pointer jumping
+                bool moved = false;
+                for (int q = r0; q < r1; ++q) {
+                    const int a = q / n, c = fit_cell(s, a, q - a * n);
+                    if (!(s.W[c] > 0.f)) continue;
+                    volatile unsigned short* par = s.par;
+                    const int pc = par[c], gp = par[pc];
+                    if (gp != pc) {
+                        par[c] = static_cast<unsigned short>(gp);
+                        moved = true;
+                    }
+                }
+                if (!__syncthreads_or(moved)) break;
+            }
+            for (int q = r0; q < r1; ++q) {
+                const int a = q / n, c = fit_cell(s, a, q - a * n);
+                if (!(s.W[c] > 0.f)) continue;
+                root[c] = uf_find16(s.par, c);
+                csum[c] = 0ull;
+                ccnt[c] = 0;
+            }
+            __syncthreads();
+            int cur = -1, cn = 0;   // exact sums per block: a run of cells with the same root adds once
+            unsigned long long sm = 0ull;
+            for (int q = r0; q < r1; ++q) {
+                const int a = q / n, i = q - a * n, c = fit_cell(s, a, i);
+                if (!(s.W[c] > 0.f)) continue;
+                const int r = root[c];
+                if (r != cur) {
+                    if (cur >= 0) {
+                        atomicAdd(csum + cur, sm);
+                        atomicAdd(ccnt + cur, cn);
+                    }
+                    cur = r;
+                    sm = 0ull;
+                    cn = 0;
+                }
+                const size_t g = static_cast<size_t>(s.rows[a] - 1) * n + i;
+                sm += v.sum[g];
+                cn += cnt[g];
+            }
+            if (cur >= 0) {
+                atomicAdd(csum + cur, sm);
+                atomicAdd(ccnt + cur, cn);
+            }
+            __syncthreads();
+            merged = 0;
+            shared_edges<0>(s, fix);
+            shared_edges<1>(s, fix);
+            shared_edges<2>(s, fix);
+            if (!__syncthreads_or(merged)) {
+                polished = true;
+                break;
+            }
+        }
+        if (polished) {   // each cell's exact block mean (fp64), and its fp32 copy
+            for (int q = tid; q < cells; q += T) {
+                const int a = q / n, i = q - a * n, c = fit_cell(s, a, i);
+                if (!(s.W[c] > 0.f)) continue;
+                const int r = root[c];
+                const double mc = (static_cast<double>(csum[r]) * kUnit) / static_cast<double>(ccnt[r]);
+                const size_t g = static_cast<size_t>(s.rows[a] - 1) * n + i;
+                v.xd[g] = mc;
+                v.x[g] = static_cast<float>(mc);
+            }
+        }
+    }
+    __syncthreads();
+    auto fitted = [&](size_t g) { return polished ? v.xd[g] : static_cast<double>(v.x[g]); };
+    // the observed ranks around each rank of a row: the last one <= i (plus 1, 0: none), the
+    // first one >= i (n: none)
+    unsigned short* before = reinterpret_cast<unsigned short*>(s.SM);
+    unsigned short* after = before + C;
+    for (int a = warp; a < m; a += nw) {
+        int carry = 0;
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            const unsigned seen = __ballot_sync(0xffffffffu, i < n && s.W[fit_cell(s, a, i < n ? i : 0)] > 0.f);
+            const unsigned upto = seen & (0xffffffffu >> (31 - lane));
+            if (i < n) before[fit_cell(s, a, i)] = static_cast<unsigned short>(upto ? i0 + 32 - __clz(upto) : carry);
+            if (seen) carry = i0 + 32 - __clz(seen);
+        }
+        carry = n;
+        for (int i0 = (n - 1) / 32 * 32; i0 >= 0; i0 -= 32) {
+            const int i = i0 + lane;
+            const unsigned seen = __ballot_sync(0xffffffffu, i < n && s.W[fit_cell(s, a, i < n ? i : 0)] > 0.f);
+            const unsigned from = seen & (0xffffffffu << lane);
+            if (i < n) after[fit_cell(s, a, i)] = static_cast<unsigned short>(from ? i0 + __ffs(from) - 1 : carry);
+            if (seen) carry = i0 + __ffs(seen) - 1;
+        }
+    }
+    // diagonal cells outside the group: pooled column means, nondecreasing (PAVA in fp64, unit
+    // weights), by one warp, over the block sums' and dual variables' memory (one thread took 140
+    // of the 250 us outside the sweeps at n = 256: a dependent fp64 operation is slow here)
+    if (warp == 0) {
+        double* bs = reinterpret_cast<double*>(s.P0);   // n - m entries each: see fit_shared_fits
+        double* bw = bs + (n - m);
+        unsigned short *LK = s.LK, *free_k = s.par;
+        int len = 0;
+        for (int k0 = 0; k0 < n; k0 += 32) {
+            const bool on = k0 + lane < n && s.isrow[k0 + lane] < 0;
+            const unsigned bal = __ballot_sync(0xffffffffu, on);
+            if (on) free_k[len + __popc(bal & ((1u << lane) - 1u))] = static_cast<unsigned short>(k0 + lane);
+            len += __popc(bal);
+        }
+        __syncwarp();
+        auto at = [](int p) { return p; };
+        pool_chain(lane, 32, len, bs, bw, LK, at, [&](int q, double& z, double& w) {
+            z = s.mu[free_k[q]];
+            w = 1.0;
+        });
+        const int q0 = lane * len / 32, q1 = (lane + 1) * len / 32;
+        const int cover = covering_start(lane, 32, q0, q1, LK, at);
+        int b = -1;
+        double val = 0.0;
+        for (int q = q0; q < q1; ++q) {
+            const int e = LK[q];
+            const bool start = e >= q;
+            if (start || q == q0) {
+                b = start ? q : cover;
+                val = bs[b] / bw[b];
+            }
+            if (!(start && e == q)) s.mu[free_k[q]] = val;   // a block of one keeps its mean as it is
+        }
+    }
+    if (tid == 0) {
+        v.hdr->sweeps = sweeps;
+        if (!converged) v.hdr->flags |= DBW_PSW_NOT_CONVERGED;
+        if (converged && !polished) v.hdr->flags |= DBW_PSW_UNPOLISHED;
+    }
+    __syncthreads();
+    // ... clipped to the bounds the fitted cells place on them: the largest of j <= min(h, k) is
+    // at the last observed one, the smallest of j >= max(h, k) at the first observed one
+    for (int k = tid; k < n; k += T) {
+        const int kk = k + 1;
+        if (s.isrow[k] >= 0) {
+            T_hat[k] = fitted(static_cast<size_t>(k) * (n + 1));
+        } else {
+            double lo = -CUDART_INF, hi = CUDART_INF;
+#pragma unroll 4
+            for (int a = 0; a < m; ++a) {
+                const int h = s.rows[a];
+                const size_t base = static_cast<size_t>(h - 1) * n;
+                const int below = before[fit_cell(s, a, min(h, kk) - 1)];
+                const int above = after[fit_cell(s, a, max(h, kk) - 1)];
+                if (below > 0) lo = fmax(lo, fitted(base + below - 1));
+                if (above < n) hi = fmin(hi, fitted(base + above));
+            }
+            T_hat[k] = fmin(fmax(s.mu[k], lo), hi);
+        }
+    }
+}
+
+constexpr size_t kFitSharedMax = 231000;   // dynamic shared memory of the fit (227 KB less its static part)
+// Whether the m x n table fits; the PAVA of the n - m free diagonal cells lies over P0 .. P1
+// (16 bytes each), LK and par (2 bytes each).
+__device__ __forceinline__ bool fit_shared_fits(int n, int m, size_t bytes) {
+    const size_t C = fit_slots(n, m), free_cells = static_cast<size_t>(n - m);
+    return fit_shared_bytes(n, m) <= bytes && C < 65536 && free_cells * 16 <= C * 8 && free_cells <= C;
+}
+
+// Group rows (diagonal cell has samples), in increasing h: v.rows, v.isrow; returns their
+// number.  The whole block calls it; ends in a barrier.
+__device__ int group_rows(View& v, int n, int* warp_tot) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int m = 0;
+    for (int h0 = 0; h0 < n; h0 += blockDim.x) {
+        const int h = h0 + tid;
+        const bool has = h < n && v.cnt[static_cast<size_t>(h) * (n + 1)] > 0;
+        const unsigned bal = __ballot_sync(0xffffffffu, has);
+        if (lane == 0) warp_tot[warp] = __popc(bal);
+        __syncthreads();
+        int pos = m + __popc(bal & ((1u << lane) - 1u));
+        for (int q = 0; q < static_cast<int>(blockDim.x >> 5); ++q) {
+            if (q < warp) pos += warp_tot[q];
+            m += warp_tot[q];
+        }
+        if (h < n) {
+            v.isrow[h] = has ? pos : -1;
+            if (has) v.rows[pos] = h + 1;
+        }
+        __syncthreads();
+    }
+    return m;
+}
+
+// The fit of a table that fits in shared memory; leaves the others to psw_estimate_kernel,
+// the next launch, which sees the same counts and so decides the same way.
+__global__ void __launch_bounds__(1024, 1) psw_fit_shared_kernel(char* base, Layout L, int n, double tol,
+                                                                  int max_sweeps, double* __restrict__ T_hat,
+                                                                  size_t shared_bytes) {
+    grid_begin();
+    extern __shared__ __align__(16) char fit_smem[];
+    __shared__ int warp_tot[32];
+    __shared__ float red[32];
+    View v = view(base, L);
+    const int m = group_rows(v, n, warp_tot);
+    if (m == 0) {
+        for (int k = threadIdx.x; k < n; k += blockDim.x) T_hat[k] = CUDART_NAN;
+        if (threadIdx.x == 0) v.hdr->sweeps = 0;
+        return;
+    }
+    if (fit_shared_fits(n, m, shared_bytes)) fit_in_shared(v, n, m, tol, max_sweeps, T_hat, fit_smem, red);
+}
+
 // The fit of Eq. (17) on the state buffer, one CTA of fit_threads(n) threads.
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) psw_estimate_kernel(char* base, Layout L, int n, double tol,
-                                                                int max_sweeps, double* __restrict__ T_hat) {
+                                                                int max_sweeps, double* __restrict__ T_hat,
+                                                                size_t shared_bytes) {
     grid_begin();
     __shared__ int warp_tot[32];
     __shared__ float red[32];
     __shared__ int fix_s, polished_s, jump_s;
     View v = view(base, L);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     const int T = blockDim.x;
     const size_t nn = static_cast<size_t>(n) * n;
     float* lam0 = v.lam;
@@ -572,19 +1248,8 @@ __global__ void __launch_bounds__(MAXT, 1) psw_estimate_kernel(char* base, Layou
     float* lam2 = v.lam + 2 * nn;
     const int32_t* cnt = v.cnt;
 
-    // group rows (diagonal cell has samples), in increasing h
-    const bool has = tid < n && cnt[static_cast<size_t>(tid) * (n + 1)] > 0;
-    const unsigned bal = __ballot_sync(0xffffffffu, has);
-    if (lane == 0) warp_tot[warp] = __popc(bal);
-    __syncthreads();
-    int m = 0;
-    for (int q = 0; q < (T >> 5); ++q) m += warp_tot[q];
-    if (tid < n) {
-        int pos = __popc(bal & ((1u << lane) - 1u));
-        for (int q = 0; q < warp; ++q) pos += warp_tot[q];
-        v.isrow[tid] = has ? pos : -1;
-        if (has) v.rows[pos] = tid + 1;
-    }
+    const int m = group_rows(v, n, warp_tot);
+    if (m == 0 || fit_shared_fits(n, m, shared_bytes)) return;   // psw_fit_shared_kernel did it
     // pooled column means (exact sums, fp64)
     if (tid < n) {
         unsigned long long sm = 0;
@@ -596,11 +1261,6 @@ __global__ void __launch_bounds__(MAXT, 1) psw_estimate_kernel(char* base, Layou
         v.mu[tid] = c > 0 ? (static_cast<double>(sm) * kUnit) / static_cast<double>(c) : CUDART_NAN;
     }
     __syncthreads();
-    if (m == 0) {
-        for (int k = tid; k < n; k += T) T_hat[k] = CUDART_NAN;
-        if (tid == 0) v.hdr->sweeps = 0;
-        return;
-    }
     if (tid == 0) {   // empty columns: the nearest earlier column with samples, else the nearest later
         int first = -1;
         for (int i = 0; i < n; ++i) {
@@ -865,14 +1525,18 @@ cudaError_t launch_psw_record(void* psw, int n, const int32_t* order, const doub
 }
 
 cudaError_t launch_psw_estimate(void* psw, int n, double tol, int max_sweeps, double* T_hat, cudaStream_t st) {
+    const Layout L = layout(n);
+    char* base = static_cast<char*>(psw);
+    // room for as many group rows as the table can have, within what a CTA can take
+    const size_t all = fit_shared_bytes(n, n), smem = all < kFitSharedMax ? all : kFitSharedMax;
+    cudaError_t e = cudaFuncSetAttribute(psw_fit_shared_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = launch(psw_fit_shared_kernel, 1, fit_shared_threads(n), smem, st, base, L, n, tol, max_sweeps, T_hat, smem);
+    if (e != cudaSuccess) return e;
     const int T = fit_threads(n);
+    auto kern = T <= 512 ? psw_estimate_kernel<512> : psw_estimate_kernel<kThreads>;   // fewer threads leave each more registers
     // not early: its tables live in L1, and a CTA set up beside other kernels finds its SM's L1
     // sized for those (n = 256: 5.0 ms, early 7.3)
-    if (T <= 512)   // fewer threads leave each one more registers
-        launch_when(false, psw_estimate_kernel<512>, 1, T, 0, st, static_cast<char*>(psw), layout(n), n, tol, max_sweeps, T_hat);
-    else
-        launch_when(false, psw_estimate_kernel<kThreads>, 1, T, 0, st, static_cast<char*>(psw), layout(n), n, tol, max_sweeps, T_hat);
-    return cudaGetLastError();
+    return launch_when(false, kern, 1, T, 0, st, base, L, n, tol, max_sweeps, T_hat, smem);
 }
 
 }  // namespace dbw

@@ -193,7 +193,8 @@ class Iteration:
         """Kernels libdbw launches per step (for the bench's launch count); the status-word
         memsets are copies, not kernels."""
         L = len(self.wl.widths) - 1
-        choose = (0 if self.static_b is not None else 1) + (3 if self.clock == "psw" else 0)   # + arrivals, record, fit
+        choose = (0 if self.static_b is not None else 1)
+        choose += 4 if self.clock == "psw" else 0   # arrivals, record, the fit's two forms
         if self.received:
             # select; compaction, the weight casts of all layers (1), X, L forward
             # GEMMs, loss + dZ_L, per layer the mean-gradient GEMM (with the dX GEMM in the same
