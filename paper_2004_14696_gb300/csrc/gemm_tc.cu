@@ -376,16 +376,18 @@ __global__ void __launch_bounds__(kThreads, MINB)
 // two thirds of what the single-CTA tile stages for the same work, so the ring
 // is deeper in the same shared memory and each SM pulls fewer bytes per flop.
 //
-// A GBAR problem may split each tile's K into ranges (choose_split): the ranges are
-// separate work items whose partial sums go through the workspace, and the epilogue warp
-// that finishes a block's last range adds them in range order, so the result does not
-// depend on which one came last.  (3072-1024-1024-10, k = 96 workers of 128 samples, K =
-// 12,288: 16 and 4 tiles of 192 K blocks beside 192 dX tiles of 16 and 1 took 180 us in two
-// launches, split 147.)
+// A GBAR problem may split the K of the tiles of its last, partial round into ranges
+// (choose_plan): the ranges are separate work items whose partial sums go to the workspace,
+// and a later kernel of the pass adds them in range order and takes the step.  (With the
+// sums in the epilogue warp that came last, a block's reads were one warp's chain of loads, and
+// the code cost the other epilogues registers: the 4096-wide launches took 429 -> 525 us.  The
+// launches of 4, 16 and 48 tiles at 3072-1024-1024-10, k = 96 workers of 128 samples, 192 K blocks
+// a tile, went from 62 + 86 + 90 us, split only up to one round and finished by the last warp, to
+// 37 + 59 + 54; the 4 rounds of 4096 x 4096 at 4096 samples, 28 tiles in the last, from 117 to 103.)
 //
-// One launch may carry two independent problems (nprob = 2, kinds KIND0 and
-// KIND1): their tiles form one list, those of problem 0 first, dealt to the pairs
-// in turn, so that the second problem fills the last partial wave of the first.
+// One launch may carry two independent problems (nprob = 2, kinds KIND0 and KIND1).  The
+// items of problem 0 are dealt to the pairs in turn; the pairs that come out one item short
+// first take ``extra`` tiles of problem 1 each, and the rest of those are dealt to all.
 // Shared memory: the ring of STAGES stages, then 256 bytes of barriers.
 //
 // Barriers (the same shared-memory offsets in both CTAs):
@@ -407,7 +409,7 @@ struct PairProblem {
 struct PairArgs {
     PairProblem p[2];
     int nprob;        // 1 or 2
-    int max_split;    // most K ranges of problem 0 (GBAR)
+    int max_items;    // most K ranges of problem 0 (GBAR) in all; 0: no scratch, no tile is split
     int* status;
 };
 
@@ -415,9 +417,7 @@ struct PairArgs {
 // K for GBAR) are not computed.
 struct PairShape {
     int Meff, Keff, live_k, mt_n, nt_n, msub_n, nk;
-    int split;          // K ranges per tile (1 unless GBAR)
-    long long tiles;    // output tiles
-    long long items;    // work items: range s of tile t is item s * tiles + t
+    int tiles;          // output tiles (each is 64 K elements of a matrix in memory: far below 2^31)
 };
 template <int KIND>
 __device__ __forceinline__ PairShape pair_shape(const PairProblem& P) {
@@ -437,54 +437,100 @@ __device__ __forceinline__ PairShape pair_shape(const PairProblem& P) {
     S.mt_n = (S.Meff + 2 * BM - 1) / (2 * BM);
     S.nt_n = (P.N + BN - 1) / BN;
     S.msub_n = (P.M + BM - 1) / BM;   // 128-row sub-tiles of the full row extent
-    S.tiles = S.live_k > 0 && S.Keff > 0 ? static_cast<long long>(S.mt_n) * S.nt_n : 0;
+    S.tiles = S.live_k > 0 && S.Keff > 0 ? S.mt_n * S.nt_n : 0;
     S.nk = (S.Keff + BK - 1) / BK;
-    S.split = 1;
-    S.items = S.tiles;
     return S;
 }
 
-// First K block of a tile's K range.
-__device__ __forceinline__ int range_begin(const PairShape& S, int range) {
-    return S.split == 1 ? range * S.nk : static_cast<int>(static_cast<long long>(range) * S.nk / S.split);
+// The order of the launch's work.  Items of problem 0: tiles 0 .. whole-1, then range r of tile
+// whole + j as item whole + r * cut + j (cut = tiles - whole tiles of ``split`` ranges each).
+struct PairPlan {
+    int split, cut;         // 1, 0: no tile is split
+    int whole, n0, n1;      // items of the two problems
+    int hi;                 // pairs below this one have an item of problem 0 more (0: all alike)
+    int extra;              // problem 1's tiles that each of the others takes first
+};
+
+// Item j of pair ``pair``: < n0 of problem 0, otherwise n0 + tile of problem 1; -1 past the end.
+__device__ __forceinline__ int pair_item(const PairPlan& L, int j, int pair, int npairs) {
+    const bool lo = L.hi > 0 && pair >= L.hi;
+    const int c0 = L.n0 / npairs + (pair < L.hi ? 1 : 0);
+    if (j < c0) return pair + j * npairs;
+    j -= c0;
+    const int nlo = npairs - L.hi;
+    int u;
+    if (lo && j < L.extra)
+        u = j * nlo + pair - L.hi;
+    else   // after the tiles that the pairs short of an item took first
+        u = L.extra * nlo + (lo ? j - L.extra : j) * npairs + pair;
+    return u < L.n1 ? L.n0 + u : -1;
+}
+// Tile and K range of an item of problem 0.
+__device__ __forceinline__ void item_tile(const PairPlan& L, int t, int* tile, int* range) {
+    *tile = t;
+    *range = 0;
+    if (t >= L.whole) {
+        *range = (t - L.whole) / L.cut;
+        *tile = L.whole + (t - L.whole) % L.cut;
+    }
+}
+__device__ __forceinline__ int range_begin(int nk, int split, int range) {
+    return split == 1 ? range * nk : static_cast<int>(static_cast<long long>(range) * nk / split);
 }
 
-// K ranges of the mean-gradient problem: its K is all received samples, so with few tiles a
-// tile's mainloop alone outlasts the rest of the launch.  The estimate, in K blocks: the
-// items of the two problems dealt to the pairs in turn, for the first pair and for the first
-// one with fewer of problem 0's items; a split item also writes its 128 KB per CTA of
-// partial sums (6), and the last range of a tile reads them all (8 + 3 per range, once).
-__device__ __forceinline__ int choose_split(const PairShape& S0, const PairShape& S1, int max_split, long long npairs) {
-    constexpr int kEpi = 8;   // a short tile lasts as long as its epilogue
-    int best = 1;
-    long long best_cost = 0;
-    for (int s = 1; s <= max_split; ++s) {
-        if (s > 1 && S0.nk < 8 * s) break;
-        const long long n0 = S0.tiles * s, n = n0 + S1.items;
-        const int len0 = (S0.nk + s - 1) / s + (s > 1 ? 6 : 0), len1 = S1.nk > kEpi ? S1.nk : kEpi;
-        long long cost = 0;
-        for (int side = 0; side < 2; ++side) {
-            const long long p = side ? n0 % npairs : 0;
-            const long long c0 = (n0 - p + npairs - 1) / npairs, c = (n - p + npairs - 1) / npairs;
-            const long long t = c0 * (len0 > kEpi ? len0 : kEpi) + (c - c0) * len1;
-            cost = t > cost ? t : cost;
-        }
-        if (s > 1) cost += 8 + 3 * s;
-        if (s == 1 || cost < best_cost) {
-            best = s;
-            best_cost = cost;
-        }
+// Chooses the split of the mean-gradient problem and ``extra``, one candidate (ranges s, extra)
+// per lane: its K is all received samples, so with few tiles, or a nearly empty last round, a
+// tile's mainloop outlasts the rest of the launch.  The estimate, in K blocks, is the later of
+// a pair with an item more and one without: a split item also writes its 128 KB per CTA of
+// partial sums (6), which are read back later (n / 12), and a tile
+// lasts at least as long as its epilogue.
+__device__ __forceinline__ PairPlan choose_plan(const PairShape& S0, const PairShape& S1, int max_items, int npairs) {
+    constexpr int kEpi = 10;
+    const int lane = threadIdx.x & 31;
+    const int s = 1 + lane / 4, e = lane % 4;
+    const int rest = S0.tiles % npairs;
+    const int len = (S0.nk + s - 1) / s;
+    const int item = s > 1 ? len + 6 : (len > kEpi ? len : kEpi);
+    const int whole = S0.nk > kEpi ? S0.nk : kEpi, len1 = S1.nk > kEpi ? S1.nk : kEpi;
+    const int n = rest * s, hi = n % npairs;
+    // 0, or as many of problem 1's tiles as an item lasts (one less, one more)
+    int extra = 0;
+    if (e > 0 && hi > 0) {
+        const int most = S1.tiles / (npairs - hi), x = item / len1 + e - 2;
+        extra = x < 0 ? 0 : x < most ? x : most;
     }
-    return best;
+    const int common = (S1.tiles - extra * (npairs - hi) + npairs - 1) / npairs;   // rounds of problem 1 over all pairs
+    const long long g0 = static_cast<long long>(S0.tiles / npairs) * whole + n / npairs * item;
+    const long long a = g0 + (hi > 0 ? item : 0) + static_cast<long long>(common) * len1;
+    const long long b = hi > 0 ? g0 + static_cast<long long>(extra + common) * len1 : 0;
+    long long cost = (a > b ? a : b) + (s > 1 ? 2 + n / 12 : 0);
+    if (s > 1 && (rest == 0 || n > max_items || S0.nk < 8 * s)) cost = 1ll << 40;
+    long long best = (cost << 8) | lane;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const long long x = __shfl_xor_sync(0xffffffffu, best, o);
+        best = x < best ? x : best;
+    }
+    const int win = static_cast<int>(best & 31);
+    PairPlan L;
+    L.split = 1 + win / 4;
+    L.extra = __shfl_sync(0xffffffffu, extra, win);
+    L.hi = __shfl_sync(0xffffffffu, hi, win);
+    L.cut = L.split > 1 ? rest : 0;
+    L.whole = S0.tiles - L.cut;
+    L.n0 = L.whole + L.cut * L.split;
+    L.n1 = S1.tiles;
+    return L;
 }
 
 // A split tile's partial sums: one block of 32 rows x 128 columns per (range, tile, CTA of
 // the pair, epilogue warp), as float4 [chunk][quad][lane] so that a warp moves 512
-// contiguous bytes per instruction.
-constexpr int kPartFloats = 32 * 128;
-__device__ __forceinline__ float* part_block(const TcEpi& e, const PairShape& S, int range, long long t, int rank,
+// contiguous bytes per instruction.  The block of range r of split tile j is number
+// (r * cut + j) * 16 + rank * 8 + warp.
+constexpr int kPartFloats = kTcPartFloats;
+__device__ __forceinline__ float* part_block(const TcEpi& e, const PairPlan& L, int range, int tile, int rank,
                                              int ew) {
-    return e.part + (((range * S.tiles + t) * 2 + rank) * 8 + ew) * kPartFloats;
+    return e.part + (((static_cast<long long>(range) * L.cut + tile - L.whole) * 2 + rank) * 8 + ew) * kPartFloats;
 }
 // The first ``chunks`` 32-column chunks of this warp's TMEM block -> its partial block.
 __device__ __forceinline__ void store_partial(float* dst, uint32_t taddr, int chunks, int lane) {
@@ -502,81 +548,16 @@ __device__ __forceinline__ void store_partial(float* dst, uint32_t taddr, int ch
 
 // Piece of ||g_t||^2 of one warp's block: fixed-shape warp tree, one piece per (128-row
 // sub-tile, column tile, half, quarter).
-__device__ __forceinline__ void store_piece(const TcEpi& e, const PairShape& S, long long t, int rank, int q, int h,
-                                            int lane, double sq) {
-    const int msub = static_cast<int>(t / S.nt_n) * 2 + rank, nt = static_cast<int>(t % S.nt_n);
+__device__ __forceinline__ void store_piece(const TcEpi& e, int msub, int nt, int nt_n, bool ok, int q, int h, int lane,
+                                            double sq) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if (lane == 0 && msub < S.msub_n) e.pieces[(static_cast<long long>(msub) * S.nt_n + nt) * 8 + h * 4 + q] = sq;
-}
-
-// The GBAR epilogue of one warp's block of a split tile: the ranges' partial sums added in
-// range order, then gbar_cols' arithmetic.  Not inlined: it would cost the unsplit path
-// registers (with it inlined both spilled, 429 -> 525 us on the 4096-wide launches).
-__device__ __noinline__ void finish_split(const PairProblem& P, const PairShape& S, long long tile, int rank, int q,
-                                          int h, int lane) {
-    const TcEpi& e = P.epi;
-    const int nb0 = static_cast<int>(tile % S.nt_n) * 256 + h * 128;
-    const int row = (static_cast<int>(tile / S.nt_n) * 2 + rank) * BM + q * 32 + lane;
-    const float inv_k = 1.0f / static_cast<float>(S.live_k);
-    const int64_t at0 = e.off + static_cast<int64_t>(row) * e.ldrow + nb0;
-    const bool wvec = ((reinterpret_cast<uintptr_t>(e.W) & 15u) == 0) &&
-                      ((reinterpret_cast<uintptr_t>(e.gbar) & 15u) == 0) && e.off % 4 == 0 && e.ldrow % 4 == 0;
-    const float4* src = reinterpret_cast<const float4*>(part_block(e, S, 0, tile, rank, h * 4 + (q + 2) % 4)) + lane;
-    const int64_t step = S.tiles * 16 * (kPartFloats / 4);   // float4 from one range to the next
-    double sq = 0.0;
-    for (int c = 0; c < 4 && nb0 + 32 * c < P.N; ++c) {
-        float part = 0.f;
-#pragma unroll 1
-        for (int g = 0; g < 2; ++g) {   // 16 columns at a time
-            float4 v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-            for (int s = 0; s < S.split; ++s) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float4 x = __ldcg(src + s * step + (c * 8 + g * 4 + i) * 32);
-                    v[i].x += x.x;
-                    v[i].y += x.y;
-                    v[i].z += x.z;
-                    v[i].w += x.w;
-                }
-            }
-            if (row < P.M) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int col = 32 * c + 16 * g + 4 * i;
-                    const float gr[4] = {v[i].x * inv_k, v[i].y * inv_k, v[i].z * inv_k, v[i].w * inv_k};
-                    float* wp = e.W + at0 + col;
-                    float* gp = e.gbar ? e.gbar + at0 + col : nullptr;
-                    if (wvec && nb0 + 32 * c + 32 <= P.N) {
-                        float4 w = *reinterpret_cast<const float4*>(wp);
-                        w.x = fmaf(-e.lr, gr[0], w.x);
-                        w.y = fmaf(-e.lr, gr[1], w.y);
-                        w.z = fmaf(-e.lr, gr[2], w.z);
-                        w.w = fmaf(-e.lr, gr[3], w.w);
-                        *reinterpret_cast<float4*>(wp) = w;
-                        if (gp) *reinterpret_cast<float4*>(gp) = make_float4(gr[0], gr[1], gr[2], gr[3]);
-                        part += gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2] + gr[3] * gr[3];
-                    } else {
-                        for (int j = 0; j < 4 && nb0 + col + j < P.N; ++j) {
-                            wp[j] = fmaf(-e.lr, gr[j], wp[j]);
-                            if (gp) gp[j] = gr[j];
-                            part += gr[j] * gr[j];
-                        }
-                    }
-                }
-            }
-        }
-        sq += part;
-    }
-    store_piece(e, S, tile, rank, q, h, lane, sq);
+    if (lane == 0 && ok) e.pieces[(static_cast<long long>(msub) * nt_n + nt) * 8 + h * 4 + q] = sq;
 }
 
 // Epilogue of one tile for problem kind KIND (one thread: one row, 128 columns).
 template <int KIND>
-__device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairShape& S, long long t, int rank, int q,
+__device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairShape& S, int t, int rank, int q,
                                               int h, int lane, uint32_t taddr) {
     constexpr int BN = 256;
     const TcEpi& epi = P.epi;
@@ -589,7 +570,7 @@ __device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairSh
                           ((reinterpret_cast<uintptr_t>(epi.gbar) & 15u) == 0) && epi.off % 4 == 0 &&
                           epi.ldrow % 4 == 0;
         double sq = gbar_cols(epi, row, nb0, P.M, P.N, 1.0f / static_cast<float>(S.live_k), taddr, wvec);
-        store_piece(epi, S, t, rank, q, h, lane, sq);
+        store_piece(epi, msub, nt, S.nt_n, msub < S.msub_n, q, h, lane, sq);
     } else if constexpr (KIND == TC_DX) {
         const bool avec = ((reinterpret_cast<uintptr_t>(epi.act) & 15u) == 0) && epi.ldact % 8 == 0;
         dx_cols(epi, row, nb0, P.M, P.N, taddr, avec);
@@ -637,6 +618,11 @@ __device__ __forceinline__ void pair_mma(uint32_t dcol, uint32_t a0, uint32_t b0
                 (!first || kk > 0) ? 1u : 0u);
 }
 
+struct PairWork {
+    PairShape shape[2];
+    PairPlan plan;
+};
+
 template <int KIND0, int KIND1, int STAGES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     tc_gemm_pair_kernel(const __grid_constant__ PairArgs args) {
@@ -658,17 +644,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
-    const long long pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+    const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     int* status = args.status;
-    PairShape S0 = pair_shape<KIND0>(args.p[0]);
-    PairShape S1 = S0;
-    S1.tiles = S1.items = 0;
-    if (args.nprob > 1) S1 = pair_shape<KIND1>(args.p[1]);
-    if constexpr (KIND0 == TC_GBAR) {
-        S0.split = choose_split(S0, S1, args.max_split, npairs);
-        S0.items = S0.tiles * S0.split;
+    // the shapes and the order of work stay in shared memory: in registers they crowd the epilogues
+    PairWork& work = *reinterpret_cast<PairWork*>(abort_flag + 1);
+    static_assert((2 * STAGES + 4) * 8 + 8 + sizeof(PairWork) <= 256, "barrier block");
+    if (warp == 2) {
+        const PairShape a = pair_shape<KIND0>(args.p[0]);
+        PairShape b{};
+        if (args.nprob > 1) b = pair_shape<KIND1>(args.p[1]);
+        PairPlan plan{1, 0, a.tiles, a.tiles, b.tiles, a.tiles % npairs, 0};
+        if (KIND0 == TC_GBAR) plan = choose_plan(a, b, args.max_items, npairs);
+        if (lane == 0) {
+            if (KIND0 == TC_GBAR && blockIdx.x == 0 && args.p[0].epi.plan) {
+                args.p[0].epi.plan[0] = plan.cut;
+                args.p[0].epi.plan[1] = plan.split;
+                args.p[0].epi.plan[2] = plan.whole;
+            }
+            work.shape[0] = a;
+            work.shape[1] = b;
+            work.plan = plan;
+        }
     }
-    const long long total = S0.items + S1.items;
+    const PairShape &S0 = work.shape[0], &S1 = work.shape[1];
+    const PairPlan& L = work.plan;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -696,12 +695,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer (both CTAs)
         long long g = 0;
-        for (long long t = pair; t < total && !*vabort; t += npairs) {
-            const bool second = t >= S0.items;
+        for (int j = 0, t; (t = pair_item(L, j, pair, npairs)) >= 0 && !*vabort; ++j) {
+            const bool second = t >= L.n0;
             const PairShape& S = second ? S1 : S0;
-            const int range = second ? 0 : static_cast<int>(t / S0.tiles);
-            const long long u = second ? t - S0.items : t - range * S0.tiles;
-            const int kb0 = range_begin(S, range), kb1 = range_begin(S, range + 1);
+            int u = t - L.n0;
+            int kb0 = 0, kb1 = S.nk;
+            if (!second) {
+                int range;
+                item_tile(L, t, &u, &range);
+                if (t >= L.whole) {
+                    kb0 = range_begin(S.nk, L.split, range);
+                    kb1 = range_begin(S.nk, L.split, range + 1);
+                }
+            }
             const int ma = static_cast<int>(u / S.nt_n) * (2 * BM) + static_cast<int>(rank) * BM;
             const int nb = static_cast<int>(u % S.nt_n) * BN + static_cast<int>(rank) * (BN / 2);
             for (int kb = kb0; kb < kb1; ++kb, ++g) {
@@ -735,10 +741,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         // ---------------- MMA issuer (even CTA)
         long long g = 0;
         int i = 0;
-        for (long long t = pair; t < total && !*vabort; t += npairs, ++i) {
-            const bool second = t >= S0.items;
-            const int range = second ? 0 : static_cast<int>(t / S0.tiles);
-            const int kb0 = second ? 0 : range_begin(S0, range), kb1 = second ? S1.nk : range_begin(S0, range + 1);
+        for (int t; (t = pair_item(L, i, pair, npairs)) >= 0 && !*vabort; ++i) {
+            const bool second = t >= L.n0;
+            int kb0 = 0, kb1 = second ? S1.nk : S0.nk;
+            if (!second && t >= L.whole) {
+                int u, range;
+                item_tile(L, t, &u, &range);
+                kb0 = range_begin(S0.nk, L.split, range);
+                kb1 = range_begin(S0.nk, L.split, range + 1);
+            }
             const int acc = i & 1;
             const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
             if (!mbar_wait(smem_u32(tempty_bar + acc), aph ^ 1)) {
@@ -774,7 +785,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         // ---------------- epilogue (both CTAs): 128-row sub-tile msub, lane quarter q, column half h
         const int q = warp & 3, h = (warp - 2) >> 2;
         int i = 0;
-        for (long long t = pair; t < total; t += npairs, ++i) {
+        for (int t; (t = pair_item(L, i, pair, npairs)) >= 0; ++i) {
             const int acc = i & 1;
             const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
             if (!mbar_wait(smem_u32(tfull_bar + acc), aph)) {
@@ -786,49 +797,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             tc_fence_after();
             const uint32_t taddr = tmem + static_cast<uint32_t>(acc * BN + h * (BN / 2)) +
                                    (static_cast<uint32_t>(q * 32) << 16);
-            bool partial = false;
-            if (t < S0.items) {
-                if (KIND0 == TC_GBAR && S0.split > 1) {
-                    const int range = static_cast<int>(t / S0.tiles);
-                    const long long tile = t - range * S0.tiles;
-                    const int cols = args.p[0].N - (static_cast<int>(tile % S0.nt_n) * BN + h * (BN / 2));
-                    const int row0 = (static_cast<int>(tile / S0.nt_n) * 2 + static_cast<int>(rank)) * BM + 32 * q;
-                    partial = cols > 0 && row0 < args.p[0].M;
-                    if (partial)
-                        store_partial(part_block(args.p[0].epi, S0, range, tile, static_cast<int>(rank), warp - 2),
+            if (t < L.n0) {
+                if (KIND0 == TC_GBAR && t >= L.whole) {
+                    int tile, range;
+                    item_tile(L, t, &tile, &range);
+                    const int cols = args.p[0].N - (tile % S0.nt_n * BN + h * (BN / 2));
+                    const int row0 = (tile / S0.nt_n * 2 + static_cast<int>(rank)) * BM + 32 * q;
+                    if (cols > 0 && row0 < args.p[0].M)
+                        store_partial(part_block(args.p[0].epi, L, range, tile, static_cast<int>(rank), warp - 2),
                                       taddr, cols >= BN / 2 ? 4 : (cols + 31) / 32, lane);
-                    else if (range == 0)   // a block outside the matrix only records its empty piece
-                        store_piece(args.p[0].epi, S0, tile, static_cast<int>(rank), q, h, lane, 0.0);
                 } else {
                     pair_epilogue<KIND0>(args.p[0], S0, t, static_cast<int>(rank), q, h, lane, taddr);
                 }
             } else {
-                pair_epilogue<KIND1>(args.p[1], S1, t - S0.items, static_cast<int>(rank), q, h, lane, taddr);
+                pair_epilogue<KIND1>(args.p[1], S1, t - L.n0, static_cast<int>(rank), q, h, lane, taddr);
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_remote(map_to_rank(smem_u32(tempty_bar + acc), 0));
-            if constexpr (KIND0 == TC_GBAR) {
-                // the warp that stores a block's last range adds the ranges in their order and
-                // runs the epilogue (the accumulator is already free)
-                if (partial) {
-                    const TcEpi& e = args.p[0].epi;
-                    const long long tile = t % S0.tiles;
-                    int* cnt = e.part_cnt + (tile * 2 + rank) * 8 + (warp - 2);
-                    __threadfence();
-                    __syncwarp();
-                    int last = 0;
-                    if (lane == 0) {
-                        last = atomicAdd(cnt, 1) == S0.split - 1;
-                        if (last) *cnt = 0;   // ready for the next launch
-                    }
-                    last = __shfl_sync(0xffffffffu, last, 0);
-                    if (last) {
-                        __threadfence();
-                        finish_split(args.p[0], S0, tile, static_cast<int>(rank), q, h, lane);
-                    }
-                }
-            }
         }
     }
     tc_fence_before();
@@ -1147,10 +1133,9 @@ cudaError_t launch_pair(const PairArgs& args, cudaStream_t st) {
     static int slots = 0;
     static std::once_flag once;
     std::call_once(once, [&] { slots = pair_slots(kern, SMEM); });
-    long long tiles = 0;   // upper bound on the items: the live extents and the split are read on the device
+    long long tiles = args.max_items;   // upper bound on the items: the live extents and the plan are read on the device
     for (int i = 0; i < args.nprob; ++i)
-        tiles += static_cast<long long>((args.p[i].M + 2 * BM - 1) / (2 * BM)) * ((args.p[i].N + 255) / 256) *
-                 (i == 0 ? args.max_split : 1);
+        tiles += static_cast<long long>((args.p[i].M + 2 * BM - 1) / (2 * BM)) * ((args.p[i].N + 255) / 256);
     const int pairs = static_cast<int>(tiles < slots ? tiles : slots);
     if (pairs < 1) return cudaSuccess;
     launch(kern, 2 * pairs, kPairThreads, SMEM, st, args);
@@ -1273,28 +1258,23 @@ static int pair_problem(PairProblem* P, int kind, const TcOperands& o, const TcE
     return DBW_OK;
 }
 
-// At most 8 ranges and at most 76 items, one round of the pairs (19 MB of partial sums): with
-// 48 tiles of 192 K blocks three ranges took 96 us, whole tiles 88.
+// A tile has at most 8 ranges, a launch at most 152 (two rounds of the pairs, 39 MB of partial
+// sums).
+constexpr int kSplitItems = 152;
 static long long gbar_tiles(int M, int N) {
     return static_cast<long long>((M + 2 * BM - 1) / (2 * BM)) * ((N + 255) / 256);
 }
-int tc_max_split(int M, int N) {
-    const long long s = 76 / gbar_tiles(M, N);
-    return static_cast<int>(s < 1 ? 1 : s > 8 ? 8 : s);
+int tc_split_items(int M, int N) {
+    const long long t = gbar_tiles(M, N) * 8;
+    return static_cast<int>(t < kSplitItems ? t : kSplitItems);
 }
-size_t tc_split_floats(int M, int N) {
-    const int s = tc_max_split(M, N);
-    return s > 1 ? static_cast<size_t>(gbar_tiles(M, N)) * s * 16 * kPartFloats : 0;
-}
-size_t tc_split_counters(int M, int N) {
-    return tc_max_split(M, N) > 1 ? static_cast<size_t>(gbar_tiles(M, N)) * 16 : 0;
-}
+size_t tc_split_floats(int M, int N) { return static_cast<size_t>(tc_split_items(M, N)) * 16 * kPartFloats; }
 
 int tc_gemm_mean_dx(const TcOperands& g, const TcEpi& ge, const TcOperands& x, const TcEpi& xe, int* status,
                     cudaStream_t st) {
     PairArgs args{};
     args.nprob = 2;
-    args.max_split = ge.part ? tc_max_split(g.M, g.N) : 1;
+    args.max_items = ge.part ? tc_split_items(g.M, g.N) : 0;
     args.status = status;
     int rc = pair_problem(&args.p[0], TC_GBAR, g, ge);
     if (rc) return rc;
@@ -1336,7 +1316,7 @@ int tc_dw(const TcOperands& o, int batch, const TcEpi& epi, int* status, cudaStr
 int tc_gemm(int kind, const TcOperands& o, const TcEpi& epi, int* status, cudaStream_t st) {
     PairArgs args{};
     args.nprob = 1;
-    args.max_split = kind == TC_GBAR && epi.part ? tc_max_split(o.M, o.N) : 1;
+    args.max_items = kind == TC_GBAR && epi.part ? tc_split_items(o.M, o.N) : 0;
     args.status = status;
     const int rc = pair_problem(&args.p[0], kind, o, epi);
     if (rc) return rc;

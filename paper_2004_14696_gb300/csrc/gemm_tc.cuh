@@ -31,11 +31,12 @@ struct TcEpi {
     float* gbar;
     float lr;
     double* pieces;
-    // GBAR, K split into ranges when the live K is long for the number of tiles (chosen on the
-    // device, at most max_split): part, tc_split_floats(M, N) floats of partial tiles; part_cnt,
-    // tc_split_counters(M, N) int32, zero on entry and left zero
+    // GBAR, K of the last round's tiles split into ranges when that ends the launch sooner
+    // (chosen on the device from the live K; never with part null): the partial sums go to
+    // part, tc_split_floats(M, N) floats, and {split tiles, ranges of each, first split tile}
+    // to plan[3].  W, gbar and pieces of those tiles are left to the caller.
     float* part;
-    int* part_cnt;
+    int* plan;
     // Live row count on the device: when non-null, only (*kdev) * kmul rows of the
     // row dimension are computed (M for HIDDEN / LOGITS / DX, K for GBAR, where k =
     // *kdev); *kdev <= 0 runs no tile.
@@ -43,10 +44,10 @@ struct TcEpi {
     int kmul;
 };
 
-// Most K ranges of a GBAR GEMM of M x N (1: never split), and its scratch.
-int tc_max_split(int M, int N);
+// Most K ranges of a GBAR GEMM of M x N over all its split tiles, and their scratch.
+int tc_split_items(int M, int N);
 size_t tc_split_floats(int M, int N);
-size_t tc_split_counters(int M, int N);
+constexpr int kTcPartFloats = 32 * 128;   // one block of partial sums
 
 // Operands of one GEMM, both row-major bf16 as their producers left them (ld multiples of
 // 8 elements, bases 16-byte aligned):

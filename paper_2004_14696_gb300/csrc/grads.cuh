@@ -76,9 +76,8 @@ struct RxPlan {
     size_t off_gpart;                  // fp32: partial Gram products of the K ranges (shared by the layers)
     size_t off_gcnt;                   // int32 [gram items]: per-item range counters, zeroed at the start of a call
     int ngcnt;
-    size_t off_part;                   // fp32: partial tiles of a split mean-gradient GEMM (shared by the layers)
-    size_t off_pcnt;                   // int32, right after the Gram counters and zeroed with them
-    int npcnt;
+    size_t off_split;                  // int32 [L][4]: the split of each layer's mean-gradient GEMM
+    size_t off_part[DBW_LMAX];         // fp32: its partial tiles
     size_t ws_bytes;
 };
 

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(1024) compact_received_kernel(const uint8_t* _
 }
 
 // Bias part of Eqs. (3)-(4), g[o] = (1/k) sum_{r < k B} dZ[r, o], for every layer,
-// in two launches.  The layers' blocks sit side by side in x; a block finds its
+// in two launches (bias_rows_kernel, mean_update_kernel).  The layers' blocks sit side by side in x; a block finds its
 // layer in the prefix table cb0 (blocks of 256 columns).
 struct BiasLayers {
     int L;
@@ -228,14 +228,21 @@ __global__ void __launch_bounds__(256) bias_rows_kernel(BiasLayers a, int B, con
     }
 }
 
-// bias_mean_update_kernel: one CTA per (layer, 256 columns): g[o] = (1/k) sum of the
-// chunks' sums (chunk order), wb[o] -= lr g, gb[o] = g (nullable); the CTA's sum of g^2
-// (fp64, fixed tree) into pieces[column block].
-__global__ void __launch_bounds__(256) bias_mean_update_kernel(BiasLayers a, int B, const int* __restrict__ kdev,
-                                                               float lr) {
-    grid_begin();
-    __shared__ double red[8];
-    const int k = *kdev;
+// The tiles of the mean-gradient GEMMs whose K was split (their partial sums are in part):
+// layer l's matrix is out x in, ``plan`` its {split tiles, ranges, first split tile}.
+struct SplitLayers {
+    int out[DBW_LMAX], in[DBW_LMAX];
+    const int* plan[DBW_LMAX];
+    const float* part[DBW_LMAX];
+    float* w[DBW_LMAX];        // W_l inside w
+    float* g[DBW_LMAX];        // W_l inside g_t (nullable)
+    double* pieces[DBW_LMAX];
+};
+
+// One CTA per (layer, 256 columns): g[o] = (1/k) sum of the chunks' sums (chunk order),
+// wb[o] -= lr g, gb[o] = g (nullable); the CTA's sum of g^2 (fp64, fixed tree) into
+// pieces[column block].
+__device__ __forceinline__ void bias_mean_update(const BiasLayers& a, int B, int k, float lr, double* red) {
     const int chunks = k > 0 ? (k * B + 255) / 256 : 0;
     const int l = bias_layer(a, blockIdx.x);
     const int cb = blockIdx.x - a.cb0[l], out = a.out[l];
@@ -257,6 +264,103 @@ __global__ void __launch_bounds__(256) bias_mean_update_kernel(BiasLayers a, int
         double t = 0.0;
         for (int w = 0; w < 8; ++w) t += red[w];
         a.pieces[l][cb] = t;
+    }
+}
+
+// One block (32 rows x 128 columns) of a split tile: the ranges' partial sums in range order,
+// then the GEMM epilogue's g = sum / k, W -= lr g, gbar = g and the sum of g^2.  The partial
+// sums hold a row per lane; the step runs along rows, through shared memory.
+__device__ __forceinline__ void finish_block(const SplitLayers& s, int l, int item, int k, float lr,
+                                             float (*tile)[132], double* red) {
+    const int cut = s.plan[l][0], split = s.plan[l][1], whole = s.plan[l][2];
+    const int M = s.out[l], N = s.in[l], nt_n = (N + 255) / 256;
+    const int j = item >> 4, rank = (item >> 3) & 1, ew = item & 7;
+    const int t = whole + j, msub = t / nt_n * 2 + rank, nt = t % nt_n;
+    const int q = (ew + 2) & 3, h = ew >> 2;
+    const int row0 = msub * 128 + 32 * q, col0 = nt * 256 + 128 * h;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double sq = 0.0;
+    if (row0 < M && col0 < N) {   // the same for the whole block
+        const float4* src = reinterpret_cast<const float4*>(s.part[l]) + static_cast<int64_t>(item) * (kTcPartFloats / 4) +
+                            warp * 32 + lane;
+        const int64_t step = static_cast<int64_t>(cut) * 16 * (kTcPartFloats / 4);
+        float4 v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+        for (int r = 0; r < split; ++r) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (col0 + 32 * c >= N) continue;
+                const float4 x = __ldcg(src + r * step + c * 256);
+                v[c].x += x.x;
+                v[c].y += x.y;
+                v[c].z += x.z;
+                v[c].w += x.w;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) *reinterpret_cast<float4*>(&tile[lane][32 * c + 4 * warp]) = v[c];
+        __syncthreads();
+        const float inv_k = 1.0f / static_cast<float>(k);
+        float* wl = s.w[l];
+        float* gl = s.g[l];
+        const bool vec = ((reinterpret_cast<uintptr_t>(wl) | reinterpret_cast<uintptr_t>(gl)) & 15u) == 0 && N % 4 == 0;
+        const int col = col0 + 4 * lane;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = warp + 8 * i, row = row0 + r;
+            if (row >= M || col >= N) continue;
+            const float4 x = *reinterpret_cast<const float4*>(&tile[r][4 * lane]);
+            const float g[4] = {x.x * inv_k, x.y * inv_k, x.z * inv_k, x.w * inv_k};
+            const int64_t at = static_cast<int64_t>(row) * N + col;
+            if (vec) {
+                float4 w = *reinterpret_cast<const float4*>(wl + at);
+                w.x = fmaf(-lr, g[0], w.x);
+                w.y = fmaf(-lr, g[1], w.y);
+                w.z = fmaf(-lr, g[2], w.z);
+                w.w = fmaf(-lr, g[3], w.w);
+                *reinterpret_cast<float4*>(wl + at) = w;
+                if (gl) *reinterpret_cast<float4*>(gl + at) = make_float4(g[0], g[1], g[2], g[3]);
+                sq += g[0] * g[0] + g[1] * g[1] + g[2] * g[2] + g[3] * g[3];
+            } else {
+                for (int e = 0; e < 4 && col + e < N; ++e) {
+                    wl[at + e] = fmaf(-lr, g[e], wl[at + e]);
+                    if (gl) gl[at + e] = g[e];
+                    sq += g[e] * g[e];
+                }
+            }
+        }
+    }
+    for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+    if (lane == 0) red[warp] = sq;
+    __syncthreads();
+    if (threadIdx.x == 0 && msub < (M + 127) / 128) {
+        double t8 = 0.0;
+        for (int w = 0; w < 8; ++w) t8 += red[w];
+        s.pieces[l][(static_cast<int64_t>(msub) * nt_n + nt) * 8 + h * 4 + q] = t8;
+    }
+    __syncthreads();   // tile and red are free again
+}
+
+// The bias part of g_t and its step (the first cb0[L] CTAs), and the split tiles of the
+// weight part (the others, a block at a time).
+__global__ void __launch_bounds__(256) mean_update_kernel(BiasLayers a, SplitLayers s, int B,
+                                                          const int* __restrict__ kdev, float lr) {
+    grid_begin();
+    __shared__ __align__(16) float tile[32][132];
+    __shared__ double red[8];
+    const int k = *kdev, nb = a.cb0[a.L];
+    if (static_cast<int>(blockIdx.x) < nb) {
+        bias_mean_update(a, B, k, lr, red);
+        return;
+    }
+    const int step = gridDim.x - nb;
+    int item = blockIdx.x - nb;   // counted through the layers
+    for (int l = 0; l < a.L; ++l) {
+        const int items = s.plan[l][0] * 16;
+        for (; item < items; item += step) finish_block(s, l, item, k, lr, tile, red);
+        item -= items;
     }
 }
 
@@ -510,16 +614,9 @@ bool make_rx_plan(int L, const int32_t* widths, int n, int B, RxPlan* P) {
     }
     P->off_gpart = take(tc_gram_partial_floats(g.M, B, L) * 4);
     P->ngcnt = static_cast<int>(tc_gram_items(g.M, B, L));
-    size_t part = 0, pcnt = 0;
-    for (int l = 0; l < L; ++l) {
-        const size_t f = tc_split_floats(g.widths[l + 1], g.widths[l]), c = tc_split_counters(g.widths[l + 1], g.widths[l]);
-        part = f > part ? f : part;
-        pcnt = c > pcnt ? c : pcnt;
-    }
-    P->npcnt = static_cast<int>(pcnt);
-    P->off_gcnt = take((static_cast<size_t>(P->ngcnt) + pcnt) * 4);
-    P->off_pcnt = P->off_gcnt + static_cast<size_t>(P->ngcnt) * 4;
-    P->off_part = take(part * 4);
+    P->off_gcnt = take(static_cast<size_t>(P->ngcnt) * 4);
+    P->off_split = take(static_cast<size_t>(L) * 16);
+    for (int l = 0; l < L; ++l) P->off_part[l] = take(tc_split_floats(g.widths[l + 1], g.widths[l]) * 4);
     P->ws_bytes = cur;
     return true;
 }
@@ -542,7 +639,7 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
 
     int* gcnt = reinterpret_cast<int*>(ws + P.off_gcnt);
     float* gpart = reinterpret_cast<float*>(ws + P.off_gpart);
-    launch(compact_received_kernel, 1, 1024, 0, st, mask, n, sel, kdev, loss, gcnt, P.ngcnt + P.npcnt);
+    launch(compact_received_kernel, 1, 1024, 0, st, mask, n, sel, kdev, loss, gcnt, P.ngcnt);
     launch_weight_casts(T, w, ws, st);
     launch(cast_rows_kernel<ReceivedRows>, row_ctas(M), 256, 0, st, pool, g.widths[0], M, g.widths[0], ReceivedRows{idx, sel, kdev, B, S},
                                                   bf(T.off_act[0]), T.ldact[0]);
@@ -586,8 +683,8 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
         gb.off = g.offW[l];
         gb.ldrow = fin;
         gb.pieces = f64(P.off_pw[l]);
-        gb.part = reinterpret_cast<float*>(ws + P.off_part);
-        gb.part_cnt = reinterpret_cast<int*>(ws + P.off_pcnt);
+        gb.part = reinterpret_cast<float*>(ws + P.off_part[l]);
+        gb.plan = reinterpret_cast<int*>(ws + P.off_split) + 4 * l;
         gb.kdev = kdev;
         gb.kmul = B;
         const TcOperands go{bf(P.off_dzl[l]), T.ldz, bf(T.off_act[l]), T.ldact[l], fout, fin, M};
@@ -607,9 +704,12 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
         }
         if (rc) return rc;
     }
-    // bias part of g_t and its step, every layer in two launches
+    // bias part of g_t and its step, every layer in two launches; the second one also finishes
+    // the split tiles of the mean-gradient GEMMs
     {
         BiasLayers bl{};
+        SplitLayers sl{};
+        int most = 0;
         bl.L = L;
         bl.ldz = T.ldz;
         bl.cb0[0] = 0;
@@ -621,9 +721,17 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
             bl.wb[l] = w + g.offb[l];
             bl.gb[l] = gbar ? gbar + g.offb[l] : nullptr;
             bl.pieces[l] = f64(P.off_pb[l]);
+            sl.out[l] = g.widths[l + 1];
+            sl.in[l] = g.widths[l];
+            sl.plan[l] = reinterpret_cast<const int*>(ws + P.off_split) + 4 * l;
+            sl.part[l] = reinterpret_cast<const float*>(ws + P.off_part[l]);
+            sl.w[l] = w + g.offW[l];
+            sl.g[l] = gbar ? gbar + g.offW[l] : nullptr;
+            sl.pieces[l] = f64(P.off_pw[l]);
+            most += tc_split_items(g.widths[l + 1], g.widths[l]) * 8;   // a split tile has 2 ranges or more
         }
         launch(bias_rows_kernel, dim3(bl.cb0[L], (M + 255) / 256), 256, 0, st, bl, B, kdev);
-        launch(bias_mean_update_kernel, bl.cb0[L], 256, 0, st, bl, B, kdev, lr);
+        launch(mean_update_kernel, bl.cb0[L] + (most < 608 ? most : 608), 256, 0, st, bl, sl, B, kdev, lr);
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
     }
