@@ -85,14 +85,23 @@ __device__ __forceinline__ void epilogue_chunk(const TcEpi& e, int z, int row, i
 
 // ------------------------------------------------------------------ epilogues of the pair kernel
 // One thread owns one output row and 128 columns of a tile (four 32-column chunks
-// read from TMEM at ``taddr``).  The global loads a chunk needs (w for the SGD
-// step, the layer input for the ReLU mask) are issued one chunk ahead, so that
-// their latency overlaps the previous chunk's work.
+// read from TMEM at ``taddr``).  GBAR's loads of w for the SGD step are issued one
+// chunk ahead, so that their latency overlaps the previous chunk's work.
 
-// bf16 activation chunk (32 columns of row ``row``) -> out.
-__device__ __forceinline__ void store_act_chunk(const TcEpi& e, int row, int nb, int N, const float (&x)[32]) {
+// bf16 activation chunk (32 columns of row ``row``) -> out.  ``wide``: rows of out start on 32
+// bytes, so that each store writes a whole sector per lane.
+__device__ __forceinline__ void store_act_chunk(const TcEpi& e, int row, int nb, int N, const float (&x)[32],
+                                                bool wide) {
     __nv_bfloat16* op = e.out + static_cast<int64_t>(row) * e.ldo + nb;
-    if (nb + 32 <= N && ((reinterpret_cast<uintptr_t>(op) & 15u) == 0)) {
+    if (nb + 32 <= N && wide) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            uint32_t w[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[j] = pack_bf16(x[16 * q + 2 * j], x[16 * q + 2 * j + 1]);
+            store_256(op + 16 * q, w);
+        }
+    } else if (nb + 32 <= N && ((reinterpret_cast<uintptr_t>(op) & 15u) == 0)) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             uint4 w;
@@ -108,9 +117,54 @@ __device__ __forceinline__ void store_act_chunk(const TcEpi& e, int row, int nb,
             if (nb + j < N) op[j] = __float2bfloat16_rn(x[j]);
     }
 }
+__device__ __forceinline__ bool out_wide(const TcEpi& e) {
+    return ((reinterpret_cast<uintptr_t>(e.out) & 31u) == 0) && e.ldo % 16 == 0;
+}
+
+// What a tile's epilogue needs from global memory is fetched before the tile's accumulator is
+// waited for, while its mainloop runs: the biases of the warp's 128 columns into its shared
+// row (HIDDEN), the ReLU mask of the thread's row as 128 bits (DX).  With biases
+// and mask loaded behind the accumulator and 16-byte stores, a tile's epilogue took longer than its
+// mainloop at K = 1024: the two dX launches of 16384 x 1024 outputs went from 32 + 43 us to 27 + 36,
+// the HIDDEN ones from 81 + 40 to 77 + 32 (wide stores, biases and mask gave 12, 10 and 2 us of
+// that pass).
+__device__ __forceinline__ void hidden_bias(const TcEpi& e, int nb0, int N, float* sb) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();   // the previous tile's reads
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int n = nb0 + 32 * c + lane;
+        sb[32 * c + lane] = n < N ? __ldg(e.bias + n) : 0.f;
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ void dx_mask(const TcEpi& e, int row, int nb0, int M, int N, bool avec, uint32_t (&mask)[4]) {
+    const __nv_bfloat16* ap = e.act + static_cast<int64_t>(row) * e.ldact + nb0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        mask[c] = 0;
+        if (row >= M || nb0 + 32 * c >= N) continue;
+        if (avec && nb0 + 32 * c + 32 <= N) {
+            uint4 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = *reinterpret_cast<const uint4*>(ap + 32 * c + 8 * q);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&v[q]);
+#pragma unroll
+                for (int t = 0; t < 8; ++t) mask[c] |= (__bfloat162float(h[t]) > 0.f ? 1u : 0u) << (8 * q + t);
+            }
+        } else {
+            for (int j = 0; j < 32 && nb0 + 32 * c + j < N; ++j)
+                mask[c] |= (__bfloat162float(ap[32 * c + j]) > 0.f ? 1u : 0u) << j;
+        }
+    }
+}
 
 // TC_HIDDEN: A_l = ReLU(Z_l + b_l) in bf16.
-__device__ __forceinline__ void hidden_cols(const TcEpi& e, int row, int nb0, int M, int N, uint32_t taddr) {
+__device__ __forceinline__ void hidden_cols(const TcEpi& e, int row, int nb0, int M, int N, uint32_t taddr,
+                                            const float* sb) {
+    const bool wide = out_wide(e);
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {
         const int nb = nb0 + 32 * c;
@@ -123,54 +177,35 @@ __device__ __forceinline__ void hidden_cols(const TcEpi& e, int row, int nb0, in
         float x[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
-            const float v = u2f(r[j]) + (nb + j < N ? __ldg(e.bias + nb + j) : 0.f);
+            const float v = u2f(r[j]) + sb[32 * c + j];
             x[j] = v > 0.f ? v : 0.f;
         }
-        store_act_chunk(e, row, nb, N, x);
+        store_act_chunk(e, row, nb, N, x, wide);
     }
 }
 
-// TC_DX: dZ_{l-1} = (dZ_l W_l) * 1[A_{l-1} > 0] in bf16; ``avec``: the act rows allow
-// 16-byte loads.
-__device__ __forceinline__ void dx_cols(const TcEpi& e, int row, int nb0, int M, int N, uint32_t taddr, bool avec) {
-    const bool rowok = row < M;
-    const __nv_bfloat16* ap = e.act + static_cast<int64_t>(row) * e.ldact + nb0;
-    uint4 nxt[4];
-    auto fetch = [&](int c) {
-        if (rowok && avec && nb0 + 32 * c + 32 <= N) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) nxt[j] = *reinterpret_cast<const uint4*>(ap + 32 * c + 8 * j);
-        }
-    };
-    fetch(0);
-#pragma unroll
+// TC_DX: dZ_{l-1} = (dZ_l W_l) * 1[A_{l-1} > 0] in bf16 (a product, so a NaN stays NaN).
+__device__ __forceinline__ void dx_cols(const TcEpi& e, int row, int nb0, int M, int N, uint32_t taddr,
+                                        const uint32_t (&mask)[4]) {
+    const bool wide = out_wide(e);
+    uint32_t m0 = mask[0], m1 = mask[1], m2 = mask[2], m3 = mask[3];
+#pragma unroll 1
     for (int c = 0; c < 4; ++c) {
         const int nb = nb0 + 32 * c;
         if (nb >= N) break;
-        uint4 cur[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
-        if (c + 1 < 4) fetch(c + 1);
         uint32_t r[32];
         __syncwarp();   // lanes past M skipped the previous chunk's stores
         tc_ld_32cols(taddr + 32 * c, r);
         tc_wait_ld();
-        if (!rowok) continue;
-        float x[32];
-        if (avec && nb + 32 <= N) {
+        if (row < M) {
+            float x[32];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const __nv_bfloat16* hv = reinterpret_cast<const __nv_bfloat16*>(&cur[q]);
-#pragma unroll
-                for (int t = 0; t < 8; ++t)
-                    x[8 * q + t] = u2f(r[8 * q + t]) * (__bfloat162float(hv[t]) > 0.f ? 1.f : 0.f);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                x[j] = (nb + j < N) ? u2f(r[j]) * (__bfloat162float(ap[32 * c + j]) > 0.f ? 1.f : 0.f) : 0.f;
+            for (int j = 0; j < 32; ++j) x[j] = u2f(r[j]) * ((m0 >> j) & 1u ? 1.f : 0.f);
+            store_act_chunk(e, row, nb, N, x, wide);
         }
-        store_act_chunk(e, row, nb, N, x);
+        m0 = m1;
+        m1 = m2;
+        m2 = m3;
     }
 }
 
@@ -388,7 +423,8 @@ __global__ void __launch_bounds__(kThreads, MINB)
 // One launch may carry two independent problems (nprob = 2, kinds KIND0 and KIND1).  The
 // items of problem 0 are dealt to the pairs in turn; the pairs that come out one item short
 // first take ``extra`` tiles of problem 1 each, and the rest of those are dealt to all.
-// Shared memory: the ring of STAGES stages, then 256 bytes of barriers.
+// Shared memory: the ring of STAGES stages, 256 bytes of barriers and the order of work, then
+// 128 biases per epilogue warp.
 //
 // Barriers (the same shared-memory offsets in both CTAs):
 //   full[s]    even CTA only: its producer arrives with the byte count of both
@@ -556,13 +592,25 @@ __device__ __forceinline__ void store_piece(const TcEpi& e, int msub, int nt, in
 }
 
 // Epilogue of one tile for problem kind KIND (one thread: one row, 128 columns).
+// Fetches what the epilogue of tile t needs besides the accumulator (before it is complete).
 template <int KIND>
-__device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairShape& S, int t, int rank, int q,
-                                              int h, int lane, uint32_t taddr) {
+__device__ __forceinline__ void pair_epilogue_fetch(const PairProblem& P, const PairShape& S, int t, int rank,
+                                                    int q, int h, int lane, float* sb, uint32_t (&mask)[4]) {
+    const int nb0 = t % S.nt_n * 256 + h * 128;
+    const int row = (t / S.nt_n * 2 + rank) * BM + q * 32 + lane;
+        if constexpr (KIND == TC_HIDDEN) hidden_bias(P.epi, nb0, P.N, sb);
+    if constexpr (KIND == TC_DX)
+        dx_mask(P.epi, row, nb0, P.M, P.N,
+                ((reinterpret_cast<uintptr_t>(P.epi.act) & 15u) == 0) && P.epi.ldact % 8 == 0, mask);
+}
+
+template <int KIND>
+__device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairShape& S, int t, int rank, int q, int h,
+                                              int lane, uint32_t taddr, const float* sb, const uint32_t (&mask)[4]) {
     constexpr int BN = 256;
     const TcEpi& epi = P.epi;
-    const int nt = static_cast<int>(t % S.nt_n);
-    const int msub = static_cast<int>(t / S.nt_n) * 2 + rank;
+    const int nt = t % S.nt_n;
+    const int msub = t / S.nt_n * 2 + rank;
     const int nb0 = nt * BN + h * (BN / 2);
     const int row = msub * BM + q * 32 + lane;
     if constexpr (KIND == TC_GBAR) {
@@ -572,17 +620,16 @@ __device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairSh
         double sq = gbar_cols(epi, row, nb0, P.M, P.N, 1.0f / static_cast<float>(S.live_k), taddr, wvec);
         store_piece(epi, msub, nt, S.nt_n, msub < S.msub_n, q, h, lane, sq);
     } else if constexpr (KIND == TC_DX) {
-        const bool avec = ((reinterpret_cast<uintptr_t>(epi.act) & 15u) == 0) && epi.ldact % 8 == 0;
-        dx_cols(epi, row, nb0, P.M, P.N, taddr, avec);
+        dx_cols(epi, row, nb0, P.M, P.N, taddr, mask);
     } else if constexpr (KIND == TC_HIDDEN) {
-        hidden_cols(epi, row, nb0, P.M, P.N, taddr);
+        hidden_cols(epi, row, nb0, P.M, P.N, taddr, sb);
     } else {
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
             if (nb0 + c * 32 >= P.N) break;
             uint32_t r[32];
             __syncwarp();
-            tc_ld_32cols(taddr + c * 32, r);
+            tc_ld_32cols(taddr + 32 * c, r);
             tc_wait_ld();
             epilogue_chunk<KIND>(epi, 0, row, nb0 + c * 32, P.M, P.N, r);
         }
@@ -708,8 +755,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                     kb1 = range_begin(S.nk, L.split, range + 1);
                 }
             }
-            const int ma = static_cast<int>(u / S.nt_n) * (2 * BM) + static_cast<int>(rank) * BM;
-            const int nb = static_cast<int>(u % S.nt_n) * BN + static_cast<int>(rank) * (BN / 2);
+            const int ma = u / S.nt_n * (2 * BM) + static_cast<int>(rank) * BM;
+            const int nb = u % S.nt_n * BN + static_cast<int>(rank) * (BN / 2);
             for (int kb = kb0; kb < kb1; ++kb, ++g) {
                 const int s = static_cast<int>(g % STAGES);
                 const uint32_t ph = static_cast<uint32_t>((g / STAGES) & 1);
@@ -784,10 +831,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     } else if (warp >= 2) {
         // ---------------- epilogue (both CTAs): 128-row sub-tile msub, lane quarter q, column half h
         const int q = warp & 3, h = (warp - 2) >> 2;
+        float* sb = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES + 256) + (warp - 2) * 128;   // HIDDEN: biases
         int i = 0;
         for (int t; (t = pair_item(L, i, pair, npairs)) >= 0; ++i) {
             const int acc = i & 1;
             const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
+            uint32_t mask[4];
+            if (t < L.n0)
+                pair_epilogue_fetch<KIND0>(args.p[0], S0, t, static_cast<int>(rank), q, h, lane, sb, mask);
+            else
+                pair_epilogue_fetch<KIND1>(args.p[1], S1, t - L.n0, static_cast<int>(rank), q, h, lane, sb, mask);
             if (!mbar_wait(smem_u32(tfull_bar + acc), aph)) {
                 atomicOr(status, 1);
                 *vabort = 1;
@@ -807,10 +860,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                         store_partial(part_block(args.p[0].epi, L, range, tile, static_cast<int>(rank), warp - 2),
                                       taddr, cols >= BN / 2 ? 4 : (cols + 31) / 32, lane);
                 } else {
-                    pair_epilogue<KIND0>(args.p[0], S0, t, static_cast<int>(rank), q, h, lane, taddr);
+                    pair_epilogue<KIND0>(args.p[0], S0, t, static_cast<int>(rank), q, h, lane, taddr, sb, mask);
                 }
             } else {
-                pair_epilogue<KIND1>(args.p[1], S1, t - L.n0, static_cast<int>(rank), q, h, lane, taddr);
+                pair_epilogue<KIND1>(args.p[1], S1, t - L.n0, static_cast<int>(rank), q, h, lane, taddr, sb, mask);
             }
             tc_fence_before();
             __syncwarp();
@@ -1125,7 +1178,7 @@ int pair_slots(Kern kern, int smem) {
 template <int KIND0, int KIND1>
 cudaError_t launch_pair(const PairArgs& args, cudaStream_t st) {
     constexpr int STAGES = DBW_PAIR_STAGES;
-    constexpr int SMEM = STAGES * (2 * BM * 64 * 2) + 256 + 1024;
+    constexpr int SMEM = STAGES * (2 * BM * 64 * 2) + 256 + 8 * 128 * 4 + 1024;
     static_assert(SMEM <= 227 * 1024, "pair ring does not fit in shared memory");
     auto kern = tc_gemm_pair_kernel<KIND0, KIND1, STAGES>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);

@@ -200,6 +200,13 @@ __device__ __forceinline__ void tc2_commit_multicast(uint32_t bar, uint16_t mask
                  : "memory");
 }
 
+// 32 bytes to global memory in one instruction (32-byte aligned).
+__device__ __forceinline__ void store_256(void* p, const uint32_t (&w)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
+                 "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);   // .x = a (low half), .y = b
     return *reinterpret_cast<const uint32_t*>(&h);
