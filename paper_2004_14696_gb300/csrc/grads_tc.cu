@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(256) bias_rows_kernel(BiasLayers a, int B, con
     const int c = cb * 256 + 8 * lane;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     const int rend = r0 + 256 < rows ? r0 + 256 : rows;
-    if (c + 7 < out) {
+    if (c < out) {   // rows are ldz (a multiple of 8) long: columns past out are read and dropped
 #pragma unroll 8
         for (int r = r0 + y; r < rend; r += 8) {
             const uint4 raw = *reinterpret_cast<const uint4*>(dZ + static_cast<int64_t>(r) * ldz + c);
@@ -213,9 +213,6 @@ __global__ void __launch_bounds__(256) bias_rows_kernel(BiasLayers a, int B, con
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(h[j]);
         }
-    } else {
-        for (int r = r0 + y; r < rend; r += 8)
-            for (int j = 0; j < 8 && c + j < out; ++j) acc[j] += __bfloat162float(dZ[static_cast<int64_t>(r) * ldz + c + j]);
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) red[y][8 * lane + j] = acc[j];

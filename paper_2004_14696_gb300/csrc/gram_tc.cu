@@ -61,21 +61,25 @@ __global__ void __launch_bounds__(GTHREADS, 1)
     grid_begin();
     const int k = *kdev;
     const long long live = static_cast<long long>(k > 0 ? k : 0) * B;   // received rows
-    const int item = blockIdx.x / GSMAX, s_id = blockIdx.x % GSMAX;    // item over all layers
-    const int layer = item / G.items, litem = item % G.items;
+    const long long live_tiles = (live + GBM - 1) / GBM * CT;   // per layer
+    // ranges only for worker blocks narrower than a tile: a 128-column block's
+    // partials cost as much traffic as the split saves
+    int S = B < GBM && live_tiles > 0 ? static_cast<int>(target_ctas / (live_tiles * G.L)) : 1;
+    S = S < 1 ? 1 : (S > GSMAX ? GSMAX : S);
+    // block -> (layer, live tile, range): the grid holds max(all items, target_ctas) blocks, so
+    // that few are launched in vain (@@G@@)
+    const int li = blockIdx.x / S;
+    const int s_id = blockIdx.x % S;
+    if (li >= live_tiles * G.L) return;         // whole CTA: no barrier or TMEM touched yet
+    const int layer = li / static_cast<int>(live_tiles), litem = li % static_cast<int>(live_tiles);
+    const int item = layer * G.items + litem;
     const int mb = litem / CT, ct = litem % CT;
     const int m0 = mb * GBM;
-    if (m0 >= live) return;                     // whole CTA: no barrier or TMEM touched yet
     const CUtensorMap& tmA = G.tmA[layer];
     const CUtensorMap& tmD = G.tmD[layer];
     double* __restrict__ pieces = G.pieces[layer];
     const int colsA = G.colsA[layer], colsD = G.colsD[layer];
     const int nk1 = (colsA + GBK - 1) / GBK, nk = nk1 + (colsD + GBK - 1) / GBK;
-    const long long live_items = (live + GBM - 1) / GBM * CT * G.L;   // over all layers of the launch
-    // ranges only for worker blocks narrower than a tile: a 128-column block's
-    // partials cost as much traffic as the split saves
-    int S = B < GBM ? static_cast<int>(target_ctas / live_items) : 1;
-    S = S < 1 ? 1 : (S > GSMAX ? GSMAX : S);
     S = S > nk ? nk : S;
     if (s_id >= S) return;
     const int g0 = static_cast<int>(static_cast<long long>(s_id) * nk / S);
@@ -303,8 +307,9 @@ int tc_gram(int L, const __nv_bfloat16* const* act, const int64_t* ldA, const in
     cudaError_t e = cudaFuncSetAttribute(tc_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) {
         // ranges sized for two resident CTAs per SM
-        launch(tc_gram_kernel, G.items * L * GSMAX, GTHREADS, smem, st, G, B, CT, 2 * sm_count(), kdev, part, cnt,
-                                                                     status);
+        const int target = 2 * sm_count(), all = G.items * L;
+        launch(tc_gram_kernel, B < GBM && all < target ? target : all, GTHREADS, smem, st, G, B, CT, target,
+               kdev, part, cnt, status);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return fail(DBW_ECUDA, "tc_gram launch: %s", cudaGetErrorString(e));
