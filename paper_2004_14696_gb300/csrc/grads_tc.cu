@@ -728,7 +728,8 @@ int received_grads_tc(const RxPlan& P, float* w, const float* pool, int64_t S, c
             most += tc_split_items(g.widths[l + 1], g.widths[l]) * 8;   // a split tile has 2 ranges or more
         }
         launch(bias_rows_kernel, dim3(bl.cb0[L], (M + 255) / 256), 256, 0, st, bl, B, kdev);
-        launch(mean_update_kernel, bl.cb0[L] + (most < 608 ? most : 608), 256, 0, st, bl, sl, B, kdev, lr);
+        const int ctas = 8 * sm_count();   // all at once: 373 -> 368 us a step over four per SM
+        launch(mean_update_kernel, bl.cb0[L] + (most < ctas ? most : ctas), 256, 0, st, bl, sl, B, kdev, lr);
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail(DBW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
     }
