@@ -272,15 +272,19 @@ cudaError_t run(int M, int N, int K, const float* A, int64_t lda, const float* B
 // in three tf32 passes: A = the hi / lo parts of dZ^T [Mr = out rows, z Kp + r], B = those
 // of act^T [Nr = in rows, z Kp + r], both K-major (the transposed parts are written by
 // split_t_kernel; Kp = K rounded up to 4 for the 16-byte strides, and the 3-D tensor maps
-// read zeros past a worker's K samples, so any K runs here).  A persistent grid walks 128 x 128 tiles (out x in) worker-major with
+// read zeros past a worker's K samples, so a ragged K runs here).  A persistent grid walks 128 x 128 tiles (out x in) worker-major with
 // the in-tiles fastest; each tile has a hi.hi accumulator and a correction accumulator
 // (256 TMEM columns), two tiles in flight (512 columns), so that the MMAs of tile i + 1
-// run while the epilogue drains tile i.  A K above 256 goes in chunks of 256 samples, each
-// into the next accumulator pair, which the epilogue warps add up in registers (rounding to
-// nearest), so a hi.hi accumulator takes at most 32 MMA additions.  (784-256-10, 16 workers
-// of 500 samples: both layers' weight gradients took 175 us on fp32 FFMA tiles, which
-// served B % 32 != 0 and B > 256; now 42 here, 7 for the parts of dZ, and 14 in the
-// few-output kernel.)  Eight epilogue warps, two per TMEM lane quarter (32 G rows),
+// run while the epilogue drains tile i.  A K above 256, or no multiple of 32, takes an
+// accumulator pair per 32 samples, which the epilogue warps add up in registers (rounding to
+// nearest): the fp32 FFMA tiles that serve such K otherwise round to nearest too, and this keeps
+// the error against 64 bits below theirs.  (Relative error of all of G, 784-256-10, 16 workers of
+// 500 / 260 / 130 samples, FFMA 4.07 / 3.74 / 3.22e-7; pairs of 256 samples 4.60 / 5.26 / 3.94e-7,
+// of 64 3.36 / 3.54 / 3.31e-7, of 32 3.29 / 3.41 / 3.13e-7, all in the same time.  At 70 and 50
+// samples 2.93 and 3.01 against 2.89 and 2.88: a ragged K up to 128 stays on FFMA.)
+// (784-256-10, 16 workers of 500 samples: both layers' weight gradients took 175 us on FFMA
+// tiles; now 42 here, 7 for the parts of dZ, and 14 in the few-output kernel.)
+// Eight epilogue warps, two per TMEM lane quarter (32 G rows),
 // each copy their 32 x 64 block TMEM -> registers (hi.hi + corrections, rounded to
 // nearest; its four TMEM loads in flight together) -> shared memory (16-byte pieces
 // XOR-swizzled by row) and then store it, 256 contiguous bytes of each of two G rows per
@@ -303,7 +307,7 @@ static_assert(WARP_COLS % 32 == 0 && EPI_WARPS % 4 == 0, "whole 32-column segmen
 constexpr int SMEM = STAGES * STAGE_BYTES + EPI_WARPS * WARP_STAGING + 256 + 1024;
 constexpr int TILE_COLS = 2 * BN;                         // hi.hi, then the corrections
 constexpr int TMEM_COLS = 2 * TILE_COLS;
-constexpr int CHUNK = 8;   // 32-deep K blocks of a chunk
+constexpr int WHOLE = 8;   // K blocks that one accumulator pair takes (more, or a ragged K: one each)
 }  // namespace dw
 
 // v = (or +=) main + corrections, 32 columns of one row.
@@ -327,7 +331,7 @@ static __device__ __forceinline__ void add_parts(float4 (&v)[8], const uint32_t 
     }
 }
 
-// kChunks: K spans several chunks.
+// kChunks: an accumulator pair per K block.
 template <bool kChunks>
 static __global__ void __launch_bounds__(dw::THREADS, 1)
     dw_kernel(const __grid_constant__ Operands op, int Mr, int Nr, int K, int batch, int* status,
@@ -352,7 +356,7 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
     const int mt_n = (Mr + BM - 1) / BM, nt_n = (Nr + dw::BN - 1) / dw::BN;
     const int tiles_per_z = mt_n * nt_n;
     const long long total = static_cast<long long>(tiles_per_z) * batch;
-    const int nk = (K + BK - 1) / BK;
+    const int nk = (K + BK - 1) / BK, chunk = kChunks ? 1 : nk;   // K blocks per accumulator pair
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < dw::STAGES; ++s) {
@@ -408,10 +412,10 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
         // ---------------- MMA issuer
         constexpr uint32_t idesc = instr_desc_tf32(BM, dw::BN);
         long long g = 0;
-        int i = 0;   // chunks so far
+        int i = 0;   // accumulator pairs so far
         bool ok = true;
         for (long long t = blockIdx.x; t < total && ok && !*vabort; t += gridDim.x) {
-            for (int k0 = 0; k0 < nk && ok; k0 += dw::CHUNK, ++i) {
+            for (int k0 = 0; k0 < nk && ok; k0 += chunk, ++i) {
                 const int acc = i & 1;
                 const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
                 if (!mbar_wait(smem_u32(tempty_bar + acc), aph ^ 1)) {
@@ -423,7 +427,7 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
                 tc_fence_after();
                 const uint32_t dmain = tmem + static_cast<uint32_t>(acc * dw::TILE_COLS);
                 const uint32_t dcorr = dmain + dw::BN;
-                const int k1 = k0 + dw::CHUNK < nk ? k0 + dw::CHUNK : nk;
+                const int k1 = k0 + chunk < nk ? k0 + chunk : nk;
                 for (int kb = k0; kb < k1; ++kb, ++g) {
                     const int s = static_cast<int>(g % dw::STAGES);
                     const uint32_t ph = static_cast<uint32_t>((g / dw::STAGES) & 1);
@@ -455,7 +459,7 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
         const int q = warp & 3;          // TMEM lanes 32 q .. 32 q + 31 = G rows m0 + 32 q ..
         const int h = (warp - 2) >> 2;   // columns [WARP_COLS h, WARP_COLS (h + 1)) of the tile
         uint8_t* buf = staging + (warp - 2) * dw::WARP_STAGING;
-        int i = 0;   // chunks so far
+        int i = 0;   // accumulator pairs so far
         bool ok = true;
         for (long long t = blockIdx.x; t < total && ok; t += gridDim.x) {
             const int z = static_cast<int>(t / tiles_per_z);
@@ -465,7 +469,7 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
             const int c0 = h * dw::WARP_COLS;   // this warp's first column of the tile
             const bool live = row0 < Mr && n0 + c0 < Nr;
             float4 v[dw::NSEG][8];   // this lane's row of the warp's block
-            for (int k0 = 0; k0 < nk; k0 += dw::CHUNK, ++i) {
+            for (int k0 = 0; k0 < nk; k0 += chunk, ++i) {
                 const int acc = i & 1;
                 const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
                 if (!mbar_wait(smem_u32(tfull_bar + acc), aph)) {
@@ -575,7 +579,7 @@ inline cudaError_t run_dw(int Mr, int Nr, int K, int batch, const float* dz, int
         !tc_make_batch_map_f32(&op.b_hi, at_hi, Nr, batch, K, Kp, dw::BN) ||
         !tc_make_batch_map_f32(&op.b_lo, at_lo, Nr, batch, K, Kp, dw::BN))
         return cudaErrorInvalidValue;
-    auto kern = K > BK * dw::CHUNK ? dw_kernel<true> : dw_kernel<false>;
+    auto kern = K % BK != 0 || K > BK * dw::WHOLE ? dw_kernel<true> : dw_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dw::SMEM);
     if (e != cudaSuccess) return e;
     const long long tiles = static_cast<long long>((Mr + BM - 1) / BM) * ((Nr + dw::BN - 1) / dw::BN) * batch;

@@ -562,8 +562,9 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
 // Weight gradient of a layer with few outputs (out <= kSkinnyN, the logits layer):
 // G[i, offW + o in + c] = sum_{r < B} dZ[i B + r, o] A[i B + r, c], and the bias part, its sum
 // over the rows of dZ alone.  CTA = 32 columns of one worker: the dZ rows sit in shared
-// memory kDwRows at a time (padded to 4 NO4 outputs), warp w takes rows w, w + 8, .. with its
-// 8 next activations loaded at a time, and the warps' sums are added in warp order; the first
+// memory kDwRows at a time (padded to 4 NO4 outputs), warp w of nw takes rows w, w + nw, .. with its
+// 8 next activations loaded at a time (nw = 8, fewer below 32 rows: at least four rows a warp, whose
+// products are not rounded apart), and the warps' sums are added in warp order; the first
 // column block also adds the bias part.  (On 128 x 128 FFMA tiles 118 of 128 rows were padding
 // and a CTA ran all B rows alone: 9.8 us for 64 workers of 64 samples, 256 x 10, and 5.4 for 16
 // of 32, 784 x 10, beside bias launches of 3.6 and 1.8; here 4.9 and under 3 with the bias.)
@@ -592,16 +593,17 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
             zs[r][o] = o < out ? z[(int64_t)(r0 + r) * out + o] : 0.f;
         }
         __syncthreads();
-        for (int q0 = warp; q0 < rows; q0 += 64) {
+        const int nw = rows >= 32 ? 8 : rows >= 8 ? rows / 4 : 1;
+        for (int q0 = warp < nw ? warp : rows; q0 < rows; q0 += 8 * nw) {
             float av[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int r = q0 + 8 * u;
+                const int r = q0 + nw * u;
                 av[u] = r < rows && c < in ? a[(int64_t)(r0 + r) * in] : 0.f;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int r = q0 + 8 * u;
+                const int r = q0 + nw * u;
                 if (r >= rows) break;
 #pragma unroll
                 for (int g = 0; g < NO4; ++g) {
@@ -870,13 +872,13 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
     P->off_whi = w_parts ? take(w_parts * 4) : 0;
     P->off_wlo = w_parts ? take(w_parts * 4) : 0;
     // weight gradients with at least 2^25 multiply-adds run in three tf32 passes when the G
-    // rows of the layer take 16-byte stores
+    // rows of the layer take 16-byte stores (a ragged B up to 128: less exact than FFMA, see dw_kernel)
     const size_t Mt = (size_t)n * tf32::padded_samples(B);   // columns of the transposed parts
     size_t zt = 0, at = 0;
     for (int l = 0; l < L; ++l) {
         const int fin = widths[l], fout = widths[l + 1];
-        P->tf32_dw[l] = prec == DBW_PREC_FP32 && fin % 4 == 0 && P->offW[l] % 4 == 0 && fout >= 32 &&
-                        (int64_t)n * fout * fin * B >= (int64_t(1) << 25);
+        P->tf32_dw[l] = prec == DBW_PREC_FP32 && (B % 32 == 0 || B > 128) && fin % 4 == 0 &&
+                        P->offW[l] % 4 == 0 && fout >= 32 && (int64_t)n * fout * fin * B >= (int64_t(1) << 25);
         if (!P->tf32_dw[l]) continue;
         zt = (size_t)fout * Mt > zt ? (size_t)fout * Mt : zt;
         if (l > 0) at = (size_t)fin * Mt > at ? (size_t)fin * Mt : at;

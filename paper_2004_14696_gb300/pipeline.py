@@ -237,7 +237,8 @@ class Iteration:
             fin, fout = wd[l], wd[l + 1]
             if fout <= 16:
                 extra -= 1                      # the bias gradient comes with the weight gradient
-            elif fin % 4 == 0 and off % 4 == 0 and fout >= 32 and n * fout * fin * B >= 1 << 25:
+            elif ((B % 32 == 0 or B > 128) and fin % 4 == 0 and off % 4 == 0 and fout >= 32
+                  and n * fout * fin * B >= 1 << 25):
                 extra += 1 if l == 0 else 2     # transposed parts of dZ_l (and of the input above layer 1)
             if fout >= 32 and M * fout * fin >= 1 << 27:
                 extra += 1 if l == 0 else 2     # the gather writes the first layer's input parts

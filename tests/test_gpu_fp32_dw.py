@@ -1,7 +1,7 @@
-"""GPU parity of the fp32 weight gradients at minibatches off the 32-sample blocks and the
-256-sample chunks of the three-tf32-pass kernel (a worker's samples past B must read as
-zero, and the chunks add up), and of the few-output kernel around its row blocks and
-output groups: every worker's row against the oracle."""
+"""GPU parity of the fp32 weight gradients at minibatches off the 32-sample blocks of the
+three-tf32-pass kernel, below and above the B where it takes ragged ones (a worker's samples
+past B must read as zero, and the blocks' sums add up), and of the few-output kernel around its
+row blocks and output groups: every worker's row against the oracle."""
 import pytest
 import torch
 
@@ -19,8 +19,10 @@ def built():
     torch.cuda.set_device(0)
 
 
-# n out in B >= 2^25 in the first layer: three tf32 passes there; the last layers have few outputs
-CASES = [((1028, 256, 10), n, B) for n, B in ((128, 1), (64, 3), (43, 7), (9, 31), (5, 33), (3, 255), (2, 257), (1, 513),
+# n out in B >= 2^25 in the first layer: three tf32 passes there at B % 32 == 0 or B > 128; the last
+# layers have few outputs
+CASES = [((1028, 256, 10), n, B) for n, B in ((128, 1), (64, 3), (43, 7), (9, 31), (5, 33), (2, 128), (2, 129),
+                                              (3, 255), (2, 257), (1, 513),
                                               (2, 500))]
 CASES += [((516, 200, 136, 12), 21, 90), ((40, 4), 3, 127), ((40, 5), 3, 128), ((33 * 4, 8), 2, 129),
           ((40, 16), 2, 300), ((64, 17), 2, 65), ((784, 10), 2, 1), ((24, 9, 3), 1, 1)]
