@@ -444,6 +444,76 @@ __global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, cons
 // order, then the butterfly.
 // kTwo: two groups per pass with all their loads issued first (fewer round trips for long
 // rows, at about 160 registers); else one group per pass (few registers, for K <= 256).
+template <bool kTwo>
+__device__ __forceinline__ float skinny_row(const float* __restrict__ a, const float* __restrict__ W, int64_t ldw, int N,
+                                            int K, int lane) {
+    float acc[kSkinnyN];
+#pragma unroll
+    for (int n = 0; n < kSkinnyN; ++n) acc[n] = 0.f;
+    if constexpr (kTwo) {
+        // two of the lane's 4-element groups per pass, all their loads issued before the
+        // products (which are added in group order, as below)
+        for (int k0 = 4 * lane; k0 < K; k0 += 256) {
+            const bool two = k0 + 128 < K;
+            const float4 av0 = __ldg(reinterpret_cast<const float4*>(a + k0));
+            const float4 av1 =
+                two ? __ldg(reinterpret_cast<const float4*>(a + k0 + 128)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 wv0[kSkinnyN], wv1[kSkinnyN];
+#pragma unroll
+            for (int n = 0; n < kSkinnyN; ++n) {
+                if (n < N) {
+                    wv0[n] = __ldg(reinterpret_cast<const float4*>(W + (int64_t)n * ldw + k0));
+                    if (two) wv1[n] = __ldg(reinterpret_cast<const float4*>(W + (int64_t)n * ldw + k0 + 128));
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < kSkinnyN; ++n) {
+                if (n < N) {
+                    float t = acc[n];
+                    t = fmaf(av0.x, wv0[n].x, t);
+                    t = fmaf(av0.y, wv0[n].y, t);
+                    t = fmaf(av0.z, wv0[n].z, t);
+                    t = fmaf(av0.w, wv0[n].w, t);
+                    if (two) {
+                        t = fmaf(av1.x, wv1[n].x, t);
+                        t = fmaf(av1.y, wv1[n].y, t);
+                        t = fmaf(av1.z, wv1[n].z, t);
+                        t = fmaf(av1.w, wv1[n].w, t);
+                    }
+                    acc[n] = t;
+                }
+            }
+        }
+    } else {
+        for (int k = 4 * lane; k < K; k += 128) {
+            const float4 av = __ldg(reinterpret_cast<const float4*>(a + k));
+#pragma unroll
+            for (int n = 0; n < kSkinnyN; ++n) {
+                if (n < N) {
+                    const float4 wv = __ldg(reinterpret_cast<const float4*>(W + (int64_t)n * ldw + k));
+                    float t = acc[n];
+                    t = fmaf(av.x, wv.x, t);
+                    t = fmaf(av.y, wv.y, t);
+                    t = fmaf(av.z, wv.z, t);
+                    t = fmaf(av.w, wv.w, t);
+                    acc[n] = t;
+                }
+            }
+        }
+    }
+    float mine = 0.f;
+#pragma unroll
+    for (int n = 0; n < kSkinnyN; ++n) {
+        if (n < N) {
+            float v = acc[n];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == n) mine = v;
+        }
+    }
+    return mine;
+}
+
 template <bool kTwo, class Epi>
 __global__ void __launch_bounds__(128) skinny_n4_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
                                                         const float* __restrict__ W, int64_t ldw, Epi epi) {
@@ -451,73 +521,54 @@ __global__ void __launch_bounds__(128) skinny_n4_kernel(int M, int N, int K, con
     const int lane = threadIdx.x & 31;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < M; m += nwarps) {
-        float acc[kSkinnyN];
-#pragma unroll
-        for (int n = 0; n < kSkinnyN; ++n) acc[n] = 0.f;
-        const float* a = A + (int64_t)m * lda;
-        if constexpr (kTwo) {
-            // two of the lane's 4-element groups per pass, all their loads issued before the
-            // products (which are added in group order, as below)
-            for (int k0 = 4 * lane; k0 < K; k0 += 256) {
-                const bool two = k0 + 128 < K;
-                const float4 av0 = __ldg(reinterpret_cast<const float4*>(a + k0));
-                const float4 av1 =
-                    two ? __ldg(reinterpret_cast<const float4*>(a + k0 + 128)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                float4 wv0[kSkinnyN], wv1[kSkinnyN];
-#pragma unroll
-                for (int n = 0; n < kSkinnyN; ++n) {
-                    if (n < N) {
-                        wv0[n] = __ldg(reinterpret_cast<const float4*>(W + (int64_t)n * ldw + k0));
-                        if (two) wv1[n] = __ldg(reinterpret_cast<const float4*>(W + (int64_t)n * ldw + k0 + 128));
-                    }
-                }
-#pragma unroll
-                for (int n = 0; n < kSkinnyN; ++n) {
-                    if (n < N) {
-                        float t = acc[n];
-                        t = fmaf(av0.x, wv0[n].x, t);
-                        t = fmaf(av0.y, wv0[n].y, t);
-                        t = fmaf(av0.z, wv0[n].z, t);
-                        t = fmaf(av0.w, wv0[n].w, t);
-                        if (two) {
-                            t = fmaf(av1.x, wv1[n].x, t);
-                            t = fmaf(av1.y, wv1[n].y, t);
-                            t = fmaf(av1.z, wv1[n].z, t);
-                            t = fmaf(av1.w, wv1[n].w, t);
-                        }
-                        acc[n] = t;
-                    }
-                }
-            }
-        } else {
-            for (int k = 4 * lane; k < K; k += 128) {
-                const float4 av = __ldg(reinterpret_cast<const float4*>(a + k));
-#pragma unroll
-                for (int n = 0; n < kSkinnyN; ++n) {
-                    if (n < N) {
-                        const float4 wv = __ldg(reinterpret_cast<const float4*>(W + (int64_t)n * ldw + k));
-                        float t = acc[n];
-                        t = fmaf(av.x, wv.x, t);
-                        t = fmaf(av.y, wv.y, t);
-                        t = fmaf(av.z, wv.z, t);
-                        t = fmaf(av.w, wv.w, t);
-                        acc[n] = t;
-                    }
-                }
-            }
-        }
-        float mine = 0.f;
-#pragma unroll
-        for (int n = 0; n < kSkinnyN; ++n) {
-            if (n < N) {
-                float v = acc[n];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == n) mine = v;
-            }
-        }
+        const float mine = skinny_row<kTwo>(A + (int64_t)m * lda, W, ldw, N, K, lane);
         if (lane < N) epi(0, m, lane, mine);
     }
+}
+
+// The last layer with few outputs and the loss in one launch: a warp forms its row's logits as
+// above and, lane c holding class c, the sample loss and the row of dZ_L as the loss kernel
+// does (the same exchanges, so the same bits).  CTA (x, i) takes rows x rows_cta .. of worker i.
+// Of a one-layer model the rows come straight from the pool (``pool`` non-null; an index
+// outside [0, S) reads row 0).  These passes are chains of launches of a few us each: with the
+// logits and the loss apart, and a gather before a single layer, 784-10 at 16 workers of 32
+// took 32.3 us an iteration in a graph, 784-256-10 at 64 of 64 125.8 and the gradients of 16 workers
+// of 500 181.5; now 28.9, 123.3 and 178.4.
+template <bool kTwo>
+__global__ void __launch_bounds__(128) logits_loss_kernel(int C, int K, int B, int rows_cta,
+                                                          const float* __restrict__ A, const float* __restrict__ pool,
+                                                          const int32_t* __restrict__ idx, int64_t S,
+                                                          const int32_t* __restrict__ labels,
+                                                          const float* __restrict__ W, const float* __restrict__ bias,
+                                                          float* __restrict__ sample_loss, float* __restrict__ dZ,
+                                                          float* __restrict__ loss, int* __restrict__ cnt) {
+    grid_begin();
+    const int i = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t row0 = (int64_t)i * B;
+    const int rbeg = blockIdx.x * rows_cta, rend = rbeg + rows_cta < B ? rbeg + rows_cta : B;
+    const float invB = 1.0f / static_cast<float>(B);
+    for (int r = rbeg + warp; r < rend; r += 4) {
+        const int64_t m = row0 + r, sidx = idx[m];
+        const bool in = sidx >= 0 && sidx < S;
+        const int y = in ? labels[sidx] : -1;
+        const bool bad = y < 0 || y >= C;
+        const float* a = pool ? pool + (in ? sidx : 0) * K : A + m * K;
+        const float dot = skinny_row<kTwo>(a, W, K, C, K, lane);
+        const float z = lane < C ? dot + bias[lane] : -INFINITY;
+        float mx = z;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const float ez = lane < C ? expf(z - mx) : 0.f;
+        float se = ez;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+        const float inv_se = 1.0f / se, zy = __shfl_sync(0xffffffffu, z, y & 31);
+        float g = ez * inv_se;
+        if (lane == y) g -= 1.0f;
+        if (lane < C) dZ[m * C + lane] = bad ? NAN : g * invB;
+        if (lane == 0) sample_loss[m] = bad ? NAN : (mx + logf(se)) - zy;
+    }
+    finish_worker_loss<128>(sample_loss + row0, B, gridDim.x, cnt + i, invB, loss + i);
 }
 
 // Input-gradient GEMM with a short inner dimension (K = out <= kSkinnyK):
@@ -562,7 +613,8 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
 // Weight gradient of a layer with few outputs (out <= kSkinnyN, the logits layer):
 // G[i, offW + o in + c] = sum_{r < B} dZ[i B + r, o] A[i B + r, c], and the bias part, its sum
 // over the rows of dZ alone.  CTA = 32 columns of one worker: the dZ rows sit in shared
-// memory kDwRows at a time (padded to 4 NO4 outputs), warp w of nw takes rows w, w + nw, .. with its
+// memory kDwRows at a time (padded to 4 NO4 outputs), A's row numbers beside them (the stacked
+// rows, or with ``idx`` the samples' rows of the pool; outside [0, S): row 0), warp w of nw takes rows w, w + nw, .. with its
 // 8 next activations loaded at a time (nw = 8, fewer below 32 rows: at least four rows a warp, whose
 // products are not rounded apart), and the warps' sums are added in warp order; the first
 // column block also adds the bias part.  (On 128 x 128 FFMA tiles 118 of 128 rows were padding
@@ -571,8 +623,9 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
 constexpr int kDwRows = 128;
 template <int NO4>
 __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict__ dZ, const float* __restrict__ A,
-                                                        int out, int in, int B, float* __restrict__ G, int64_t ldG,
-                                                        int64_t offW, int64_t offb) {
+                                                        const int32_t* __restrict__ idx, int64_t S, int out, int in,
+                                                        int B, float* __restrict__ G, int64_t ldG, int64_t offW,
+                                                        int64_t offb) {
     grid_begin();
     constexpr int NO = 4 * NO4;
     __shared__ __align__(16) float zs[kDwRows][NO];
@@ -580,7 +633,8 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
     const int i = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = blockIdx.x * 32 + lane;
     const float* z = dZ + (int64_t)i * B * out;
-    const float* a = A + (int64_t)i * B * in + c;
+    __shared__ int src[kDwRows];   // row of A of each of the rows
+    const float* a = A + c;
     float acc[NO];
 #pragma unroll
     for (int o = 0; o < NO; ++o) acc[o] = 0.f;
@@ -592,6 +646,14 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
             const int r = e / NO, o = e % NO;
             zs[r][o] = o < out ? z[(int64_t)(r0 + r) * out + o] : 0.f;
         }
+        for (int r = threadIdx.x; r < rows; r += 256) {
+            const int m = i * B + r0 + r;   // M = n B < 2^31
+            src[r] = m;
+            if (idx) {
+                const int64_t q = idx[m];
+                src[r] = q >= 0 && q < S ? static_cast<int>(q) : 0;
+            }
+        }
         __syncthreads();
         const int nw = rows >= 32 ? 8 : rows >= 8 ? rows / 4 : 1;
         for (int q0 = warp < nw ? warp : rows; q0 < rows; q0 += 8 * nw) {
@@ -599,7 +661,7 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int r = q0 + nw * u;
-                av[u] = r < rows && c < in ? a[(int64_t)(r0 + r) * in] : 0.f;
+                av[u] = r < rows && c < in ? a[(int64_t)src[r] * in] : 0.f;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -642,11 +704,11 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
     }
 }
 
-cudaError_t launch_skinny_dw(const float* dZ, const float* A, int out, int in, int n, int B, float* G, int64_t ldG,
-                             int64_t offW, int64_t offb, cudaStream_t st) {
+cudaError_t launch_skinny_dw(const float* dZ, const float* A, const int32_t* idx, int64_t S, int out, int in, int n,
+                             int B, float* G, int64_t ldG, int64_t offW, int64_t offb, cudaStream_t st) {
     const dim3 grid((in + 31) / 32, n);
     auto kern = out <= 4 ? skinny_dw_kernel<1> : out <= 8 ? skinny_dw_kernel<2> : skinny_dw_kernel<4>;
-    launch(kern, grid, 256, 0, st, dZ, A, out, in, B, G, ldG, offW, offb);
+    launch(kern, grid, 256, 0, st, dZ, A, idx, S, out, in, B, G, ldG, offW, offb);
     return cudaGetLastError();
 }
 
@@ -689,7 +751,10 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
     // the status word and the workers' loss counters
     cudaError_t e0 = cudaMemsetAsync(ws, 0, P.off_cnt + P.n * sizeof(int), st);
     if (e0 != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e0));
-    {
+    // the last layer's logits, loss and dZ_L in one launch; a single layer then needs no gather
+    const bool few = P.widths[L] <= kSkinnyN && P.widths[L - 1] % 4 == 0 && aligned16(w + P.offW[L - 1]);
+    const bool from_pool = few && L == 1;
+    if (!from_pool) {
         const int in = P.widths[0];
         if (P.tf32[0] || P.tf32_dw[0]) {
             // the first layer's GEMMs in three tf32 passes take their X parts from the gather;
@@ -752,13 +817,25 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
             e = fwd(EpiHidden{bias, Aout, fout});
             Ain = Aout;
         } else {
+            if (few) break;
             e = fwd(EpiLogits{bias, logits, fout});
         }
         if (e != cudaSuccess) return fail(DBW_ECUDA, "forward GEMM %d: %s", l, cudaGetErrorString(e));
     }
     const int C = P.widths[L];
-    e = launch_softmax(logits, C, C, P.n, B, idx, S, labels, sloss, dz[0], C, loss, reinterpret_cast<int*>(ws + P.off_cnt),
-                       st);
+    if (few) {
+        const int fin = P.widths[L - 1];
+        // 4 rows (a warp each) per CTA, or as many fours as bring the grid to 8 CTAs per SM
+        const int64_t most = 8 * sm_count();
+        const int rows_cta = static_cast<int>(4 * (((M + 3) / 4 + most - 1) / most));
+        const dim3 grid((B + rows_cta - 1) / rows_cta, P.n);
+        launch(fin > 256 ? logits_loss_kernel<true> : logits_loss_kernel<false>, grid, 128, 0, st, C, fin, B, rows_cta, Ain,
+               from_pool ? pool : nullptr, idx, S, labels, w + P.offW[L - 1], w + P.offb[L - 1], sloss, dz[0], loss,
+               reinterpret_cast<int*>(ws + P.off_cnt));
+        e = cudaGetLastError();
+    } else
+        e = launch_softmax(logits, C, C, P.n, B, idx, S, labels, sloss, dz[0], C, loss,
+                           reinterpret_cast<int*>(ws + P.off_cnt), st);
     if (e != cudaSuccess) return fail(DBW_ECUDA, "loss launch: %s", cudaGetErrorString(e));
 
     // backward
@@ -769,7 +846,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
         const float* dZl = dz[cur];
         // per-worker weight gradient: M' = fout, N' = fin, K = B; A(o, r) = dZ[r*fout + o], B(r, c) = A[r*fin + c]
         if (fout <= kSkinnyN) {
-            e = launch_skinny_dw(dZl, Aprev, fout, fin, P.n, B, G, ld, P.offW[l], P.offb[l], st);
+            e = launch_skinny_dw(dZl, from_pool ? pool : Aprev, from_pool ? idx : nullptr, S, fout, fin, P.n, B, G, ld, P.offW[l], P.offb[l], st);
         } else if (P.tf32_dw[l]) {
             const size_t ath = l == 0 ? P.off_xthi : P.off_athi, atl = l == 0 ? P.off_xtlo : P.off_atlo;
             e = tf32::run_dw(fout, fin, B, P.n, dZl, fout, Aprev, fin, reinterpret_cast<float*>(ws + P.off_zthi),

@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(GTHREADS, 1)
     int S = B < GBM && live_tiles > 0 ? static_cast<int>(target_ctas / (live_tiles * G.L)) : 1;
     S = S < 1 ? 1 : (S > GSMAX ? GSMAX : S);
     // block -> (layer, live tile, range): the grid holds max(all items, target_ctas) blocks, so
-    // that few are launched in vain (@@G@@)
+    // that few are launched in vain (eight for every item, most of them leaving at once, took 5.5 us
+    // more of a 4096-wide step of 1039, 128 workers of 32 samples)
     const int li = blockIdx.x / S;
     const int s_id = blockIdx.x % S;
     if (li >= live_tiles * G.L) return;         // whole CTA: no barrier or TMEM touched yet

@@ -32,14 +32,56 @@ __device__ __forceinline__ int live_rows(const int* kdev, int B, int M) {
 // CTA (i, y) takes rows y rows_cta .. of worker i, a warp kRows rows at a time: their
 // logits, sample indices and labels are all loaded before the first is reduced, and a lane
 // keeps its NJ logits of a row (classes lane, lane + 32, ..) in registers, so that each is
-// read once (NJ = 0, C > 1024: three passes over the row).  The CTA that finishes a worker
-// last (cnt[i], zero on entry) adds the sample losses in their order.  (One CTA per worker, a row at a time per warp, 32 masked
+// read once (NJ = 0, C > 1024: three passes over the row).  (One CTA per worker, a row at a time per warp, 32 masked
 // exponentials a row: 45 us for 16,384 rows of 10 classes in bf16, 49 for 16 workers of 500
 // in fp32; now 9 and 8.)
 //
 // With ``sel`` (received-workers pass): slot i is worker sel[i] (stacked rows i B .., samples
 // idx[sel[i] B + r], loss[sel[i]]); slots i >= k zero their dZ rows up to the live row count.
 constexpr int kLossThreads = 256;
+
+// The CTA that finishes a worker last of its ``parts`` (all T threads call it) adds the worker's
+// B sample losses in sample order (part of the loss's definition: F^ enters Eq. (12) as a
+// difference), from shared memory, into *loss.  *cnt is zero before the worker's first CTA.
+template <int T>
+__device__ __forceinline__ void finish_worker_loss(const float* __restrict__ sample_loss, int B, int parts,
+                                                   int* __restrict__ cnt, float invB, float* __restrict__ loss) {
+    __shared__ int last_s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last_s = 1;
+        if (parts > 1) {
+            __threadfence();
+            last_s = atomicAdd(cnt, 1) == parts - 1;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    if (!last_s) return;
+    constexpr int kStage = 1024;
+    __shared__ __align__(16) float ls[kStage];
+    float acc = 0.f;
+    for (int s0 = 0; s0 < B; s0 += kStage) {
+        const int len = B - s0 < kStage ? B - s0 : kStage;
+        for (int r = threadIdx.x; r < kStage; r += T)
+            if (r < len) ls[r] = __ldcg(sample_loss + s0 + r);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int r = 0;
+#pragma unroll 4
+            for (; r + 4 <= len; r += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(ls + r);
+                acc += v.x;
+                acc += v.y;
+                acc += v.z;
+                acc += v.w;
+            }
+            for (; r < len; ++r) acc += ls[r];
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = acc * invB;
+}
 
 template <int NJ>
 constexpr int loss_rows() { return NJ == 1 ? 4 : NJ == 4 ? 2 : 1; }   // rows a warp has in flight
@@ -133,43 +175,7 @@ __global__ void __launch_bounds__(kLossThreads) softmax_xent_kernel(
             if (lane == 0) sample_loss[row0 + r] = bad ? NAN : (mx + logf(se)) - zy;
         }
     }
-    __shared__ int last_s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        last_s = 1;
-        if (gridDim.y > 1) {
-            __threadfence();
-            last_s = atomicAdd(cnt + i, 1) == static_cast<int>(gridDim.y) - 1;
-            __threadfence();
-        }
-    }
-    __syncthreads();
-    if (!last_s) return;
-    // in sample order (part of the loss's definition: F^ enters Eq. (12) as a difference), from
-    // shared memory
-    constexpr int kStage = 1024;
-    __shared__ __align__(16) float ls[kStage];
-    float acc = 0.f;
-    for (int s0 = 0; s0 < B; s0 += kStage) {
-        const int len = B - s0 < kStage ? B - s0 : kStage;
-        for (int r = threadIdx.x; r < kStage; r += kLossThreads)
-            if (r < len) ls[r] = __ldcg(sample_loss + row0 + s0 + r);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int r = 0;
-#pragma unroll 4
-            for (; r + 4 <= len; r += 4) {
-                const float4 v = *reinterpret_cast<const float4*>(ls + r);
-                acc += v.x;
-                acc += v.y;
-                acc += v.z;
-                acc += v.w;
-            }
-            for (; r < len; ++r) acc += ls[r];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) loss[worker] = acc * invB;
+    finish_worker_loss<kLossThreads>(sample_loss + row0, B, gridDim.y, cnt + i, invB, loss + worker);
 }
 
 template <typename T>

@@ -233,6 +233,10 @@ class Iteration:
 
         B, n, off = self.wl.B, self.wl.n, 0
         extra = 0
+        last = sum(i * o + o for i, o in zip(wd[:-2], wd[1:-1]))   # offset of the last layer in w
+        if wd[-1] <= 16 and wd[-2] % 4 == 0 and last % 4 == 0:
+            # the last forward GEMM and the loss are one launch; a single layer needs no gather
+            extra -= 1 if len(wd) > 2 else 2
         for l in range(len(wd) - 1):
             fin, fout = wd[l], wd[l + 1]
             if fout <= 16:
