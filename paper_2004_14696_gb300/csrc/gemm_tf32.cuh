@@ -556,10 +556,12 @@ __host__ __device__ inline int64_t padded_samples(int64_t B) { return (B + 3) / 
 // layer's offset).  Needs Nr % 4 == 0, ldrow % 4 == 0, ldG % 4 == 0 and Gbase 16-byte
 // aligned (the caller checks).  zt_hi / zt_lo: [Mr, batch Kp] scratch, at_hi / at_lo: [Nr,
 // batch Kp] scratch, Kp = padded_samples(K).
-// act_parts_ready: at_hi / at_lo already hold act's transposed parts (act is not read).
+// act_parts_ready: at_hi / at_lo already hold act's transposed parts (act is not read);
+// dz_parts_ready: zt_hi / zt_lo those of dz.
 inline cudaError_t run_dw(int Mr, int Nr, int K, int batch, const float* dz, int64_t ldz, const float* act,
                           int64_t lda, float* zt_hi, float* zt_lo, float* at_hi, float* at_lo, float* Gbase,
-                          int64_t ldrow, int64_t ldG, int* status, cudaStream_t st, bool act_parts_ready = false) {
+                          int64_t ldrow, int64_t ldG, int* status, cudaStream_t st, bool act_parts_ready,
+                          bool dz_parts_ready) {
     const int64_t rows = static_cast<int64_t>(batch) * K;   // rows of dz / act
     const int64_t Kp = padded_samples(K), Mt = batch * Kp;  // columns of the transposes
     const int pad = static_cast<int>(Kp - K);
@@ -567,7 +569,8 @@ inline cudaError_t run_dw(int Mr, int Nr, int K, int batch, const float* dz, int
     {
         const int64_t ry = (rows + 31) / 32;
         dim3 g((Mr + 31) / 32, ry < 65535 ? static_cast<unsigned>(ry) : 65535u);
-        launch(split_t_kernel, g, blk, 0, st, dz, static_cast<int>(rows), Mr, ldz, K, pad, zt_hi, zt_lo, Mt);
+        if (!dz_parts_ready)
+            launch(split_t_kernel, g, blk, 0, st, dz, static_cast<int>(rows), Mr, ldz, K, pad, zt_hi, zt_lo, Mt);
         if (!act_parts_ready) {
             dim3 g2((Nr + 31) / 32, g.y);
             launch(split_t_kernel, g2, blk, 0, st, act, static_cast<int>(rows), Nr, lda, K, pad, at_hi, at_lo, Mt);

@@ -131,14 +131,26 @@ __global__ void gather_parts_kernel(const float* __restrict__ pool, int64_t S, i
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int c0 = blockIdx.x * 128;
     for (int64_t m0 = (int64_t)blockIdx.y * 32; m0 < M; m0 += (int64_t)gridDim.y * 32) {
-        for (int j = ty; j < 32; j += 8) {
+        // the four rows' indices, then their four loads in flight together
+        const int c = c0 + 4 * tx;
+        int64_t src[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t m = m0 + ty + 8 * u;
+            src[u] = m < M ? idx[m] : 0;
+            if (src[u] < 0 || src[u] >= S) src[u] = 0;
+        }
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            x[u] = m0 + ty + 8 * u < M && c < in ? *reinterpret_cast<const float4*>(pool + src[u] * in + c)
+                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = ty + 8 * u;
             const int64_t m = m0 + j;
-            const int c = c0 + 4 * tx;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 v = x[u];
             if (m < M && c < in) {
-                int64_t r = idx[m];
-                if (r < 0 || r >= S) r = 0;
-                v = *reinterpret_cast<const float4*>(pool + r * in + c);
                 if (X) *reinterpret_cast<float4*>(X + m * in + c) = v;
                 if (hi) {
                     float4 h, l;
@@ -575,9 +587,15 @@ __global__ void __launch_bounds__(128) logits_loss_kernel(int C, int K, int B, i
 // dZ_{l-1}[m, c] = (sum_{o < K} dZ_l[m, o] W[o, c]) * 1[act[m, c] > 0], the products
 // added in increasing o (EpiDx's arithmetic, with the 16 masks loaded before any
 // store).  W and the CTA's 16 rows of dZ_l sit in shared memory; a thread per column
-// computes the 16 rows' outputs.
+// computes the 16 rows' outputs.  With ``hiT`` it also writes their tf32 parts transposed, as
+// split_t_kernel would from dZ_{l-1} (hiT / loT [N, ldt], workers of B samples in blocks of
+// B + pad columns): with that pass apart, and the gather's rows loaded one after another,
+// 784-256-10 took 122.6 us an iteration at 64 workers of 64 samples and 179.4 for the gradients of
+// 16 of 500; now 118.4 and 173.7 (with 16-byte stores of the parts 120.1 and 176.4).
 __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, const float* __restrict__ dZ, int64_t ldz,
-                                                          const float* __restrict__ W, int64_t ldw, EpiDx epi) {
+                                                          const float* __restrict__ W, int64_t ldw, EpiDx epi,
+                                                          float* __restrict__ hiT, float* __restrict__ loT, int64_t ldt,
+                                                          int B, int pad) {
     grid_begin();
     constexpr int R = 16;                               // rows per CTA
     extern __shared__ float wsh[];                      // W as [K, N] fp32, then the CTA's dZ rows [R, K]
@@ -604,8 +622,37 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
 #pragma unroll
             for (int j = 0; j < R; ++j) a[j] = m0 + j < M ? (epi.act[(int64_t)(m0 + j) * epi.ldo + c]) : 0.f;
 #pragma unroll
-            for (int j = 0; j < R; ++j)
-                if (m0 + j < M) epi.out[(int64_t)(m0 + j) * epi.ldo + c] = (v[j] * (a[j] > 0.f ? 1.f : 0.f));
+            for (int j = 0; j < R; ++j) {
+                v[j] = v[j] * (a[j] > 0.f ? 1.f : 0.f);
+                if (m0 + j < M) epi.out[(int64_t)(m0 + j) * epi.ldo + c] = v[j];
+            }
+            if (hiT) {
+                float* hp = hiT + (int64_t)c * ldt;
+                float* lp = loT + (int64_t)c * ldt;
+                if (pad == 0 && ldt % 8 == 0 && m0 + R <= M) {   // whole 32-byte sectors
+#pragma unroll
+                    for (int j = 0; j < R; j += 8) {
+                        uint32_t h[8], l[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            float x, y;
+                            tf32::split_value(v[j + q], x, y);
+                            h[q] = __float_as_uint(x);
+                            l[q] = __float_as_uint(y);
+                        }
+                        tcx::store_256(hp + m0 + j, h);
+                        tcx::store_256(lp + m0 + j, l);
+                    }
+                } else {
+                    for (int j = 0; j < R && m0 + j < M; ++j) {
+                        const int t = m0 + j + (m0 + j) / B * pad;
+                        float h, l;
+                        tf32::split_value(v[j], h, l);
+                        hp[t] = h;
+                        lp[t] = l;
+                    }
+                }
+            }
         }
     }
 }
@@ -840,6 +887,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
 
     // backward
     int cur = 0;
+    bool dz_parts_ready = false;   // dZ_l's transposed parts are in the workspace
     for (int l = L - 1; l >= 0; --l) {
         const int fin = P.widths[l], fout = P.widths[l + 1];
         const float* Aprev = (l == 0) ? X : reinterpret_cast<const float*>(ws + P.off_act[l]);
@@ -852,12 +900,13 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
             e = tf32::run_dw(fout, fin, B, P.n, dZl, fout, Aprev, fin, reinterpret_cast<float*>(ws + P.off_zthi),
                              reinterpret_cast<float*>(ws + P.off_ztlo), reinterpret_cast<float*>(ws + ath),
                              reinterpret_cast<float*>(ws + atl), G + P.offW[l], fin, ld, reinterpret_cast<int*>(ws),
-                             st, /*act_parts_ready=*/l == 0);
+                             st, /*act_parts_ready=*/l == 0, dz_parts_ready);
         } else {
             e = run_gemm<false, false>(fout, fin, B, dZl, fout, (int64_t)B * fout, Aprev, fin, (int64_t)B * fin, P.n,
                                        EpiDW{G, ld, P.offW[l], fin}, st);
         }
         if (e != cudaSuccess) return fail(DBW_ECUDA, "dW GEMM %d: %s", l, cudaGetErrorString(e));
+        dz_parts_ready = false;
         if (fout > kSkinnyN) e = launch_bias_grad(dZl, fout, fout, P.n, B, G, ld, P.offb[l], st);
         if (e != cudaSuccess) return fail(DBW_ECUDA, "bias grad %d: %s", l, cudaGetErrorString(e));
         if (l > 0) {
@@ -866,9 +915,13 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
             if (skinny_k_ok(fin, fout)) {
                 const int ry = (M + 15) / 16;
                 dim3 grid((fin + 255) / 256, ry < 65535 ? ry : 65535);
+                const bool parts = P.tf32_dw[l - 1];   // the next weight gradient reads the transposed parts
+                const int Kp = static_cast<int>(tf32::padded_samples(B));
                 launch(skinny_k_dx_kernel, grid, 256, ((size_t)fin + 16) * fout * 4, st, M, fin, fout, dZl, fout,
-                                                                                  w + P.offW[l], fin,
-                                                                                  EpiDx{Aprev, dnext, fin});
+                       w + P.offW[l], fin, EpiDx{Aprev, dnext, fin},
+                       parts ? reinterpret_cast<float*>(ws + P.off_zthi) : nullptr,
+                       parts ? reinterpret_cast<float*>(ws + P.off_ztlo) : nullptr, (int64_t)P.n * Kp, B, Kp - B);
+                dz_parts_ready = parts;
                 e = cudaGetLastError();
             } else {
                 e = run_gemm<true, false>(M, fin, fout, dZl, fout, 0, w + P.offW[l], fin, 0, 1,

@@ -244,6 +244,8 @@ class Iteration:
             elif ((B % 32 == 0 or B > 128) and fin % 4 == 0 and off % 4 == 0 and fout >= 32
                   and n * fout * fin * B >= 1 << 25):
                 extra += 1 if l == 0 else 2     # transposed parts of dZ_l (and of the input above layer 1)
+                if l + 2 < len(wd) and skinny_k(fout, wd[l + 2]):
+                    extra -= 1                  # those of dZ_l come with the dX kernel that forms it
             if fout >= 32 and M * fout * fin >= 1 << 27:
                 extra += 1 if l == 0 else 2     # the gather writes the first layer's input parts
             elif not skinny_n(fout, fin, off):
