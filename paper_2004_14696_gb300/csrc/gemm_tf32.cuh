@@ -245,14 +245,16 @@ constexpr int kMain = 7;   // (7 + 1) x 64 = 512 TMEM columns
 // Splits both operands into ws buffers (a_hi, a_lo: [M, lda2]; b_hi, b_lo: [N, ldb2],
 // lda2 = ldb2 = K rounded up to 4) and runs C = A B^T into ``epi``.  A [M, K] (row
 // stride lda) and B [N, K] (row stride ldb) are fp32 row-major.
-// a_parts_ready: a_hi / a_lo already hold A's parts (written by the producer of A).
+// parts_ready: the buffers already hold both operands' parts (written by the producer of A).
 template <class Epi>
 cudaError_t run(int M, int N, int K, const float* A, int64_t lda, const float* B, int64_t ldb, float* a_hi,
                 float* a_lo, float* b_hi, float* b_lo, Epi epi, int* status, cudaStream_t st,
-                bool a_parts_ready = false) {
+                bool parts_ready) {
     const int64_t ld2 = (K + 3) / 4 * 4;
-    if (!a_parts_ready) split(A, M, K, lda, a_hi, a_lo, ld2, st);
-    split(B, N, K, ldb, b_hi, b_lo, ld2, st);
+    if (!parts_ready) {
+        split(A, M, K, lda, a_hi, a_lo, ld2, st);
+        split(B, N, K, ldb, b_hi, b_lo, ld2, st);
+    }
     Operands op;
     if (!tc_make_map_f32(&op.a_hi, a_hi, M, K, ld2, BM) || !tc_make_map_f32(&op.a_lo, a_lo, M, K, ld2, BM) ||
         !tc_make_map_f32(&op.b_hi, b_hi, N, K, ld2, kBN) || !tc_make_map_f32(&op.b_lo, b_lo, N, K, ld2, kBN))

@@ -247,7 +247,7 @@ class Iteration:
                 if l + 2 < len(wd) and skinny_k(fout, wd[l + 2]):
                     extra -= 1                  # those of dZ_l come with the dX kernel that forms it
             if fout >= 32 and M * fout * fin >= 1 << 27:
-                extra += 1 if l == 0 else 2     # the gather writes the first layer's input parts
+                extra += 0 if l == 0 else 2     # the gather writes the first layer's parts
             elif not skinny_n(fout, fin, off):
                 extra += split_launch(M, fout, fin)
             off += fin * fout + fout
