@@ -1,26 +1,29 @@
-// Eq. (2) for all n workers at once, fp32 workloads: g_i = (1/B) sum_{x in B_i} grad f(x, w).
+// Eq. (2) for all n workers at once (fp32, and bf16 where grads_tc.cu does not take it): g_i = (1/B) sum_{x in B_i} grad f(x, w).
 //
 // The n workers share w, so their minibatches are stacked into one batch of
 // M = n * B rows and every forward and input-gradient GEMM is a single GEMM over
 // M rows.  Only the weight gradient is per worker: G[i, W_l] = dZ_l[i]^T A_{l-1}[i]
 // with K = B, a batched GEMM over the n workers that writes G directly.
 //
-//   gather     X = pool[idx]
+//   gather     X = pool[idx] in the operand type (fp32: a single layer of at most 16 outputs
+//              reads the pool itself)
 //   forward    Z_l = A_{l-1} W_l^T + b_l, A_l = ReLU(Z_l)   (last layer: fp32 logits)
 //   loss       per-sample cross entropy, loss_i = mean over worker i's B samples,
-//              dZ_L = (softmax - onehot) / B
+//              dZ_L = (softmax - onehot) / B (fp32, at most 16 outputs: one launch with the
+//              last layer's forward)
 //   backward   G[i, W_l] = dZ_l[i]^T A_{l-1}[i],  G[i, b_l] = sum_rows dZ_l[i],
 //              dZ_{l-1} = (dZ_l W_l) * 1[A_{l-1} > 0]      (ReLU'(0) = 0)
 //
 // The large forward and weight-gradient GEMMs run on the tensor cores in three tf32
-// passes (gemm_tf32.cuh), which keeps fp32 accuracy; the others are fp32 FFMA kernels.
-// The bf16 workloads run in grads_tc.cu.
+// passes (gemm_tf32.cuh), which keeps fp32 accuracy; the others are FFMA kernels on fp32 or
+// bf16 operands.
 #include <math.h>
 
 #include "common.cuh"
 #include "gemm_tf32.cuh"
 #include "grads.cuh"
 #include "loss_bias.cuh"
+#include "tc_ptx.cuh"
 
 namespace dbw {
 
@@ -101,18 +104,35 @@ __global__ void split_t_kernel(const float* __restrict__ src, int rows, int cols
 namespace {
 
 // ------------------------------------------------------------------ gather
-// X[m, :] = pool[idx[m], :], 16 bytes a lane (in % 4 == 0).  An index outside [0, S)
-// reads row 0; the loss kernel poisons that worker.
+__device__ __forceinline__ float to_f(float v) { return v; }
+__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
+
+// X[m, :] = pool[idx[m], :] in the operand type, 16 bytes a lane (in % 4 == 0).  An index
+// outside [0, S) reads row 0; the loss kernel poisons that worker.
+template <typename T>
 __global__ void gather_kernel(const float* __restrict__ pool, int64_t S, int in, const int32_t* __restrict__ idx,
-                              int M, float* __restrict__ X) {
+                              int M, T* __restrict__ X) {
     grid_begin();
     for (int m = blockIdx.y; m < M; m += gridDim.y) {
         int64_t r = idx[m];
         if (r < 0 || r >= S) r = 0;
         const float4* src = reinterpret_cast<const float4*>(pool + r * in);
-        float4* dst = reinterpret_cast<float4*>(X + (int64_t)m * in);
-        for (int c = blockIdx.x * blockDim.x + threadIdx.x; 4 * c < in; c += gridDim.x * blockDim.x) dst[c] = src[c];
+        T* dst = X + (int64_t)m * in;
+        for (int c = blockIdx.x * blockDim.x + threadIdx.x; 4 * c < in; c += gridDim.x * blockDim.x) {
+            const float4 v = src[c];
+            if constexpr (sizeof(T) == 4)
+                reinterpret_cast<float4*>(dst)[c] = v;
+            else   // rows of in bf16 start on 8 bytes
+                reinterpret_cast<uint2*>(dst)[c] = make_uint2(tcx::pack_bf16(v.x, v.y), tcx::pack_bf16(v.z, v.w));
+        }
     }
+}
+
+// bf16 copy of the weights (the flat layout of w; the bias slots are not read).
+__global__ void cast_bf16_kernel(const float* __restrict__ w, int64_t d, __nv_bfloat16* __restrict__ wb) {
+    grid_begin();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
+        wb[i] = __float2bfloat16_rn(w[i]);
 }
 
 // The gather of the fp32 pass when its first layer runs in three tf32 passes: the
@@ -218,9 +238,9 @@ constexpr int BM = 128, BN = 128, BK = 16;
 // instead of a batch index; split z covers k in [z * kps, (z + 1) * kps) and
 // writes its partial tile to part[z][M][N], which splitk_reduce_kernel sums in
 // split order before the epilogue.
-template <bool A_K, bool B_K, class Epi, bool SPLIT>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
-                                                        int64_t batchA, const float* __restrict__ B, int64_t ldb,
+template <typename T, bool A_K, bool B_K, class Epi, bool SPLIT>
+__global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, const T* __restrict__ A, int64_t lda,
+                                                        int64_t batchA, const T* __restrict__ B, int64_t ldb,
                                                         int64_t batchB, Epi epi, int kps, float* __restrict__ part) {
     grid_begin();
     __shared__ __align__(16) float As[2][BK][BM];
@@ -250,7 +270,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, con
             int mm, kk;
             if (A_K) { mm = e / BK; kk = e % BK; } else { kk = e / BM; mm = e % BM; }
             const int gm = m0 + mm, gk = k0 + kk;
-            ra[q] = (gm < M && gk < kend) ? (A_K ? A[(int64_t)gm * lda + gk] : A[(int64_t)gk * lda + gm]) : 0.f;
+            ra[q] = (gm < M && gk < kend) ? to_f(A_K ? A[(int64_t)gm * lda + gk] : A[(int64_t)gk * lda + gm]) : 0.f;
         }
 #pragma unroll
         for (int q = 0; q < LB; ++q) {
@@ -258,7 +278,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, con
             int nn, kk;
             if (B_K) { nn = e / BK; kk = e % BK; } else { kk = e / BN; nn = e % BN; }
             const int gn = n0 + nn, gk = k0 + kk;
-            rb[q] = (gn < N && gk < kend) ? (B_K ? B[(int64_t)gn * ldb + gk] : B[(int64_t)gk * ldb + gn]) : 0.f;
+            rb[q] = (gn < N && gk < kend) ? to_f(B_K ? B[(int64_t)gn * ldb + gk] : B[(int64_t)gk * ldb + gn]) : 0.f;
         }
     };
     // registers -> shared buffer ``buf``
@@ -331,13 +351,14 @@ __global__ void splitk_reduce_kernel(int M, int N, int splits, const float* __re
 }
 
 // forward hidden layer: A_l = ReLU(C + b)
+template <typename T>
 struct EpiHidden {
     const float* bias;
-    float* out;
+    T* out;
     int ldo;
     __device__ __forceinline__ void operator()(int, int m, int n, float v) const {
         v += bias[n];
-        out[(int64_t)m * ldo + n] = (v > 0.f ? v : 0.f);
+        out[(int64_t)m * ldo + n] = from_f<T>(v > 0.f ? v : 0.f);
     }
     // 32 consecutive outputs of row m from column n0 (those below N): the biases are
     // loaded before any store
@@ -348,7 +369,7 @@ struct EpiHidden {
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
             const float x = v[j] + b[j];
-            if (n0 + j < N) out[(int64_t)m * ldo + n0 + j] = (x > 0.f ? x : 0.f);
+            if (n0 + j < N) out[(int64_t)m * ldo + n0 + j] = from_f<T>(x > 0.f ? x : 0.f);
         }
     }
 };
@@ -370,13 +391,14 @@ struct EpiLogits {
     }
 };
 // input gradient: dZ_{l-1} = C * 1[A_{l-1} > 0]  (a product, so a NaN-poisoned row stays NaN)
+template <typename T>
 struct EpiDx {
-    const float* act;
-    float* out;
+    const T* act;
+    T* out;
     int ldo;
     __device__ __forceinline__ void operator()(int, int m, int n, float v) const {
-        const float a = (act[(int64_t)m * ldo + n]);
-        out[(int64_t)m * ldo + n] = (v * (a > 0.f ? 1.f : 0.f));
+        const float a = to_f(act[(int64_t)m * ldo + n]);
+        out[(int64_t)m * ldo + n] = from_f<T>(v * (a > 0.f ? 1.f : 0.f));
     }
 };
 // weight gradient of worker z: G[z, off + o * in + c]
@@ -429,12 +451,12 @@ constexpr int kSkinnyN = 16;
 constexpr int kSkinnyK = 32;
 constexpr size_t kSkinnySmem = 48 * 1024;
 
-template <class Epi>
-__global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, const float* __restrict__ A, int64_t lda,
-                                                       const float* __restrict__ W, int64_t ldw, Epi epi) {
+template <typename T, class Epi>
+__global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, const T* __restrict__ A, int64_t lda,
+                                                       const T* __restrict__ W, int64_t ldw, Epi epi) {
     grid_begin();
     extern __shared__ float wsh[];   // W as [N, K] fp32
-    fill_shared(wsh, N * K, [&](int e) { return (W[(int64_t)(e / K) * ldw + e % K]); });
+    fill_shared(wsh, N * K, [&](int e) { return to_f(W[(int64_t)(e / K) * ldw + e % K]); });
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -442,12 +464,12 @@ __global__ void __launch_bounds__(256) skinny_n_kernel(int M, int N, int K, cons
         float acc[kSkinnyN];
 #pragma unroll
         for (int n = 0; n < kSkinnyN; ++n) acc[n] = 0.f;
-        const float* a = A + (int64_t)m * lda;
+        const T* a = A + (int64_t)m * lda;
         // 8 of the lane's elements loaded at a time, then multiplied
         for (int k0 = lane; k0 < K; k0 += 8 * 32) {
             float av[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) av[u] = k0 + 32 * u < K ? (a[k0 + 32 * u]) : 0.f;
+            for (int u = 0; u < 8; ++u) av[u] = k0 + 32 * u < K ? to_f(a[k0 + 32 * u]) : 0.f;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int k = k0 + 32 * u;
@@ -614,20 +636,21 @@ __global__ void __launch_bounds__(128) logits_loss_kernel(int C, int K, int B, i
 // B + pad columns): with that pass apart, and the gather's rows loaded one after another,
 // 784-256-10 took 122.6 us an iteration at 64 workers of 64 samples and 179.4 for the gradients of
 // 16 of 500; now 118.4 and 173.7 (with 16-byte stores of the parts 120.1 and 176.4).
-__global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, const float* __restrict__ dZ, int64_t ldz,
-                                                          const float* __restrict__ W, int64_t ldw, EpiDx epi,
+template <typename T>
+__global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, const T* __restrict__ dZ, int64_t ldz,
+                                                          const T* __restrict__ W, int64_t ldw, EpiDx<T> epi,
                                                           float* __restrict__ hiT, float* __restrict__ loT, int64_t ldt,
                                                           int B, int pad) {
     grid_begin();
     constexpr int R = 16;                               // rows per CTA
     extern __shared__ float wsh[];                      // W as [K, N] fp32, then the CTA's dZ rows [R, K]
     float* zsh = wsh + N * K;
-    fill_shared(wsh, N * K, [&](int e) { return (W[(int64_t)(e / N) * ldw + e % N]); });
+    fill_shared(wsh, N * K, [&](int e) { return to_f(W[(int64_t)(e / N) * ldw + e % N]); });
     for (int m0 = blockIdx.y * R; m0 < M; m0 += gridDim.y * R) {
         __syncthreads();   // the previous rows' reads of zsh are done
         fill_shared(zsh, R * K, [&](int e) {
             const int m = m0 + e / K;
-            return m < M ? (dZ[(int64_t)m * ldz + e % K]) : 0.f;
+            return m < M ? to_f(dZ[(int64_t)m * ldz + e % K]) : 0.f;
         });
         __syncthreads();
         for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
@@ -642,11 +665,11 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
             // the ReLU masks of the R rows, all loaded before the first store
             float a[R];
 #pragma unroll
-            for (int j = 0; j < R; ++j) a[j] = m0 + j < M ? (epi.act[(int64_t)(m0 + j) * epi.ldo + c]) : 0.f;
+            for (int j = 0; j < R; ++j) a[j] = m0 + j < M ? to_f(epi.act[(int64_t)(m0 + j) * epi.ldo + c]) : 0.f;
 #pragma unroll
             for (int j = 0; j < R; ++j) {
                 v[j] = v[j] * (a[j] > 0.f ? 1.f : 0.f);
-                if (m0 + j < M) epi.out[(int64_t)(m0 + j) * epi.ldo + c] = v[j];
+                if (m0 + j < M) epi.out[(int64_t)(m0 + j) * epi.ldo + c] = from_f<T>(v[j]);
             }
             if (hiT) {
                 float* hp = hiT + (int64_t)c * ldt;
@@ -690,8 +713,8 @@ __global__ void __launch_bounds__(256) skinny_k_dx_kernel(int M, int N, int K, c
 // and a CTA ran all B rows alone: 9.8 us for 64 workers of 64 samples, 256 x 10, and 5.4 for 16
 // of 32, 784 x 10, beside bias launches of 3.6 and 1.8; here 4.9 and under 3 with the bias.)
 constexpr int kDwRows = 128;
-template <int NO4>
-__global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict__ dZ, const float* __restrict__ A,
+template <typename T, int NO4>
+__global__ void __launch_bounds__(256) skinny_dw_kernel(const T* __restrict__ dZ, const T* __restrict__ A,
                                                         const int32_t* __restrict__ idx, int64_t S, int out, int in,
                                                         int B, float* __restrict__ G, int64_t ldG, int64_t offW,
                                                         int64_t offb) {
@@ -701,9 +724,9 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
     __shared__ float red[8][NO][33];
     const int i = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = blockIdx.x * 32 + lane;
-    const float* z = dZ + (int64_t)i * B * out;
+    const T* z = dZ + (int64_t)i * B * out;
     __shared__ int src[kDwRows];   // row of A of each of the rows
-    const float* a = A + c;
+    const T* a = A + c;
     float acc[NO];
 #pragma unroll
     for (int o = 0; o < NO; ++o) acc[o] = 0.f;
@@ -713,7 +736,7 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
         __syncthreads();   // the previous rows' reads of zs are done
         for (int e = threadIdx.x; e < rows * NO; e += 256) {
             const int r = e / NO, o = e % NO;
-            zs[r][o] = o < out ? z[(int64_t)(r0 + r) * out + o] : 0.f;
+            zs[r][o] = o < out ? to_f(z[(int64_t)(r0 + r) * out + o]) : 0.f;
         }
         for (int r = threadIdx.x; r < rows; r += 256) {
             const int m = i * B + r0 + r;   // M = n B < 2^31
@@ -730,7 +753,7 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int r = q0 + nw * u;
-                av[u] = r < rows && c < in ? a[(int64_t)src[r] * in] : 0.f;
+                av[u] = r < rows && c < in ? to_f(a[(int64_t)src[r] * in]) : 0.f;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -773,10 +796,11 @@ __global__ void __launch_bounds__(256) skinny_dw_kernel(const float* __restrict_
     }
 }
 
-cudaError_t launch_skinny_dw(const float* dZ, const float* A, const int32_t* idx, int64_t S, int out, int in, int n,
+template <typename T>
+cudaError_t launch_skinny_dw(const T* dZ, const T* A, const int32_t* idx, int64_t S, int out, int in, int n,
                              int B, float* G, int64_t ldG, int64_t offW, int64_t offb, cudaStream_t st) {
     const dim3 grid((in + 31) / 32, n);
-    auto kern = out <= 4 ? skinny_dw_kernel<1> : out <= 8 ? skinny_dw_kernel<2> : skinny_dw_kernel<4>;
+    auto kern = out <= 4 ? skinny_dw_kernel<T, 1> : out <= 8 ? skinny_dw_kernel<T, 2> : skinny_dw_kernel<T, 4>;
     launch(kern, grid, 256, 0, st, dZ, A, idx, S, out, in, B, G, ldG, offW, offb);
     return cudaGetLastError();
 }
@@ -784,8 +808,8 @@ cudaError_t launch_skinny_dw(const float* dZ, const float* A, const int32_t* idx
 inline bool skinny_n_ok(int N, int K) { return N <= kSkinnyN && (size_t)N * K * 4 <= kSkinnySmem; }
 inline bool skinny_k_ok(int N, int K) { return K <= kSkinnyK && ((size_t)N + 16) * K * 4 <= kSkinnySmem; }
 
-template <bool A_K, bool B_K, class Epi>
-cudaError_t run_gemm(int M, int N, int K, const float* A, int64_t lda, int64_t batchA, const float* B, int64_t ldb,
+template <typename T, bool A_K, bool B_K, class Epi>
+cudaError_t run_gemm(int M, int N, int K, const T* A, int64_t lda, int64_t batchA, const T* B, int64_t ldb,
                      int64_t batchB, int batch, Epi epi, cudaStream_t st, float* split_ws = nullptr,
                      size_t split_floats = 0) {
     int splits = split_ws ? splitk_count(M, N, K, batch) : 1;
@@ -794,7 +818,7 @@ cudaError_t run_gemm(int M, int N, int K, const float* A, int64_t lda, int64_t b
         const int kps = ((K + splits - 1) / splits + BK - 1) / BK * BK;
         splits = (K + kps - 1) / kps;
         dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, splits);
-        launch(gemm_simt_kernel<A_K, B_K, Epi, true>, grid, 256, 0, st, M, N, K, A, lda, 0, B, ldb, 0, epi, kps,
+        launch(gemm_simt_kernel<T, A_K, B_K, Epi, true>, grid, 256, 0, st, M, N, K, A, lda, 0, B, ldb, 0, epi, kps,
                                                                        split_ws);
         const int64_t total = (int64_t)M * N;
         const int blocks = static_cast<int>((total + 255) / 256 < 4 * sm_count() ? (total + 255) / 256 : 4 * sm_count());
@@ -802,20 +826,23 @@ cudaError_t run_gemm(int M, int N, int K, const float* A, int64_t lda, int64_t b
         return cudaGetLastError();
     }
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch);
-    launch(gemm_simt_kernel<A_K, B_K, Epi, false>, grid, 256, 0, st, M, N, K, A, lda, batchA, B, ldb, batchB, epi, K,
+    launch(gemm_simt_kernel<T, A_K, B_K, Epi, false>, grid, 256, 0, st, M, N, K, A, lda, batchA, B, ldb, batchB, epi, K,
                                                                     nullptr);
     return cudaGetLastError();
 }
 
-int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int64_t S, const int32_t* labels,
+// T: the operand type.  The tf32 and 16-byte kernels serve fp32 alone.
+template <typename T>
+int worker_grads_simt(const GradsPlan& P, const float* w, const float* pool, int64_t S, const int32_t* labels,
                       const int32_t* idx, float* G, int64_t ld, float* loss, char* ws, cudaStream_t st) {
     const int L = P.L;
     const int M = P.M;
     const int B = P.B;
-    float* X = reinterpret_cast<float*>(ws + P.off_x);
+    constexpr bool kF32 = sizeof(T) == 4;
+    T* X = reinterpret_cast<T*>(ws + P.off_x);
     float* logits = reinterpret_cast<float*>(ws + P.off_logits);
     float* sloss = reinterpret_cast<float*>(ws + P.off_sloss);
-    float* dz[2] = {reinterpret_cast<float*>(ws + P.off_dz[0]), reinterpret_cast<float*>(ws + P.off_dz[1])};
+    T* dz[2] = {reinterpret_cast<T*>(ws + P.off_dz[0]), reinterpret_cast<T*>(ws + P.off_dz[1])};
     float* split_ws = P.split_floats ? reinterpret_cast<float*>(ws + P.off_split) : nullptr;
     // the status word and the workers' loss counters
     const bool parts = P.tf32[0] || P.tf32_dw[0];   // the gather writes the first layer's tf32 parts
@@ -823,8 +850,15 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
         const cudaError_t e0 = cudaMemsetAsync(ws, 0, P.off_cnt + P.n * sizeof(int), st);
         if (e0 != cudaSuccess) return fail(DBW_ECUDA, "dbw_worker_grads: %s", cudaGetErrorString(e0));
     }
+    const T* wop;   // the weights as operands
+    if constexpr (kF32) {
+        wop = w;
+    } else {
+        launch(cast_bf16_kernel, 4 * sm_count(), 256, 0, st, w, P.d, reinterpret_cast<T*>(ws + P.off_wb));
+        wop = reinterpret_cast<const T*>(ws + P.off_wb);
+    }
     // the last layer's logits, loss and dZ_L in one launch; a single layer then needs no gather
-    const bool few = P.widths[L] <= kSkinnyN && P.widths[L - 1] % 4 == 0 && aligned16(w + P.offW[L - 1]);
+    const bool few = kF32 && P.widths[L] <= kSkinnyN && P.widths[L - 1] % 4 == 0 && aligned16(w + P.offW[L - 1]);
     const bool from_pool = few && L == 1;
     if (!from_pool) {
         const int in = P.widths[0];
@@ -839,24 +873,24 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
             const bool need_x = !(P.tf32[0] && P.tf32_dw[0]);
             launch(gather_parts_kernel, dim3(gx, ty + wy), dim3(32, 8), 0, st, ty, w + P.offW[0], nw4,
                 reinterpret_cast<float*>(ws + P.off_whi), reinterpret_cast<float*>(ws + P.off_wlo),
-                reinterpret_cast<int*>(ws), static_cast<int>(P.off_cnt / 4) + P.n, pool, S, in, idx, M, need_x ? X : nullptr,
+                reinterpret_cast<int*>(ws), static_cast<int>(P.off_cnt / 4) + P.n, pool, S, in, idx, M, need_x ? reinterpret_cast<float*>(X) : nullptr,
                 P.tf32[0] ? reinterpret_cast<float*>(ws + P.off_ahi) : nullptr,
                 P.tf32[0] ? reinterpret_cast<float*>(ws + P.off_alo) : nullptr, (in + 3) / 4 * 4,
                 P.tf32_dw[0] ? reinterpret_cast<float*>(ws + P.off_xthi) : nullptr,
                 P.tf32_dw[0] ? reinterpret_cast<float*>(ws + P.off_xtlo) : nullptr, P.n * tf32::padded_samples(B), B,
                 static_cast<int>(tf32::padded_samples(B) - B));
         } else {
-            launch(gather_kernel, dim3((in + 1023) / 1024, M < 65535 ? M : 65535), 256, 0, st, pool, S, in, idx, M, X);
+            launch(gather_kernel<T>, dim3((in + 1023) / 1024, M < 65535 ? M : 65535), 256, 0, st, pool, S, in, idx, M, X);
         }
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(DBW_ECUDA, "gather launch: %s", cudaGetErrorString(e));
 
     // forward
-    const float* Ain = X;
+    const T* Ain = X;
     for (int l = 0; l < L; ++l) {
         const int fin = P.widths[l], fout = P.widths[l + 1];
-        const float* W = w + P.offW[l];
+        const T* W = wop + P.offW[l];
         const float* bias = w + P.offb[l];
         const bool tc = P.tf32[l];
         float* part[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -868,30 +902,32 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
         }
         int* status = reinterpret_cast<int*>(ws);
         auto fwd = [&](auto epi) {
-            if (tc)
-                return tf32::run(M, fout, fin, Ain, fin, W, fin, part[0], part[1], part[2], part[3], epi, status, st,
-                                 /*parts_ready=*/l == 0);
-            if (fout <= kSkinnyN && fin % 4 == 0 && aligned16(Ain) && aligned16(W)) {
-                const int want = (M + 3) / 4;   // 4 rows (warps) per CTA
-                const int grid = want < 8 * sm_count() ? want : 8 * sm_count();
-                if (fin > 256)
-                    launch(skinny_n4_kernel<true, decltype(epi)>, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
-                else
-                    launch(skinny_n4_kernel<false, decltype(epi)>, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
-                return cudaGetLastError();
+            if constexpr (kF32) {
+                if (tc)
+                    return tf32::run(M, fout, fin, Ain, fin, W, fin, part[0], part[1], part[2], part[3], epi, status, st,
+                                     /*parts_ready=*/l == 0);
+                if (fout <= kSkinnyN && fin % 4 == 0 && aligned16(Ain) && aligned16(W)) {
+                    const int want = (M + 3) / 4;   // 4 rows (warps) per CTA
+                    const int grid = want < 8 * sm_count() ? want : 8 * sm_count();
+                    if (fin > 256)
+                        launch(skinny_n4_kernel<true, decltype(epi)>, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
+                    else
+                        launch(skinny_n4_kernel<false, decltype(epi)>, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
+                    return cudaGetLastError();
+                }
             }
             if (skinny_n_ok(fout, fin)) {
                 const int rows_per_cta = 8;
                 const int want = (M + rows_per_cta - 1) / rows_per_cta;
                 const int grid = want < 2 * sm_count() ? want : 2 * sm_count();
-                launch(skinny_n_kernel<decltype(epi)>, grid, 256, (size_t)fout * fin * 4, st, M, fout, fin, Ain, fin, W, fin, epi);
+                launch(skinny_n_kernel<T, decltype(epi)>, grid, 256, (size_t)fout * fin * 4, st, M, fout, fin, Ain, fin, W, fin, epi);
                 return cudaGetLastError();
             }
-            return run_gemm<true, true>(M, fout, fin, Ain, fin, 0, W, fin, 0, 1, epi, st, split_ws, P.split_floats);
+            return run_gemm<T, true, true>(M, fout, fin, Ain, fin, 0, W, fin, 0, 1, epi, st, split_ws, P.split_floats);
         };
         if (l < L - 1) {
-            float* Aout = reinterpret_cast<float*>(ws + P.off_act[l + 1]);
-            e = fwd(EpiHidden{bias, Aout, fout});
+            T* Aout = reinterpret_cast<T*>(ws + P.off_act[l + 1]);
+            e = fwd(EpiHidden<T>{bias, Aout, fout});
             Ain = Aout;
         } else {
             if (few) break;
@@ -901,6 +937,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
     }
     const int C = P.widths[L];
     if (few) {
+        if constexpr (kF32) {
         const int fin = P.widths[L - 1];
         // 4 rows (a warp each) per CTA, or as many fours as bring the grid to 8 CTAs per SM
         const int64_t most = 8 * sm_count();
@@ -910,6 +947,7 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
                from_pool ? pool : nullptr, idx, S, labels, w + P.offW[L - 1], w + P.offb[L - 1], sloss, dz[0], loss,
                reinterpret_cast<int*>(ws + P.off_cnt));
         e = cudaGetLastError();
+        }
     } else
         e = launch_softmax(logits, C, C, P.n, B, idx, S, labels, sloss, dz[0], C, loss,
                            reinterpret_cast<int*>(ws + P.off_cnt), st);
@@ -920,19 +958,22 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
     bool dz_parts_ready = false;   // dZ_l's transposed parts are in the workspace
     for (int l = L - 1; l >= 0; --l) {
         const int fin = P.widths[l], fout = P.widths[l + 1];
-        const float* Aprev = (l == 0) ? X : reinterpret_cast<const float*>(ws + P.off_act[l]);
-        const float* dZl = dz[cur];
+        const T* Aprev = (l == 0) ? X : reinterpret_cast<const T*>(ws + P.off_act[l]);
+        const T* dZl = dz[cur];
         // per-worker weight gradient: M' = fout, N' = fin, K = B; A(o, r) = dZ[r*fout + o], B(r, c) = A[r*fin + c]
         if (fout <= kSkinnyN) {
-            e = launch_skinny_dw(dZl, from_pool ? pool : Aprev, from_pool ? idx : nullptr, S, fout, fin, P.n, B, G, ld, P.offW[l], P.offb[l], st);
+            const T* rows = Aprev;
+            if constexpr (kF32) rows = from_pool ? pool : Aprev;
+            e = launch_skinny_dw(dZl, rows, from_pool ? idx : nullptr, S, fout, fin, P.n, B, G, ld, P.offW[l], P.offb[l], st);
         } else if (P.tf32_dw[l]) {
             const size_t ath = l == 0 ? P.off_xthi : P.off_athi, atl = l == 0 ? P.off_xtlo : P.off_atlo;
-            e = tf32::run_dw(fout, fin, B, P.n, dZl, fout, Aprev, fin, reinterpret_cast<float*>(ws + P.off_zthi),
-                             reinterpret_cast<float*>(ws + P.off_ztlo), reinterpret_cast<float*>(ws + ath),
-                             reinterpret_cast<float*>(ws + atl), G + P.offW[l], fin, ld, reinterpret_cast<int*>(ws),
-                             st, /*act_parts_ready=*/l == 0, dz_parts_ready);
+            if constexpr (kF32)
+                e = tf32::run_dw(fout, fin, B, P.n, dZl, fout, Aprev, fin, reinterpret_cast<float*>(ws + P.off_zthi),
+                                 reinterpret_cast<float*>(ws + P.off_ztlo), reinterpret_cast<float*>(ws + ath),
+                                 reinterpret_cast<float*>(ws + atl), G + P.offW[l], fin, ld, reinterpret_cast<int*>(ws),
+                                 st, /*act_parts_ready=*/l == 0, dz_parts_ready);
         } else {
-            e = run_gemm<false, false>(fout, fin, B, dZl, fout, (int64_t)B * fout, Aprev, fin, (int64_t)B * fin, P.n,
+            e = run_gemm<T, false, false>(fout, fin, B, dZl, fout, (int64_t)B * fout, Aprev, fin, (int64_t)B * fin, P.n,
                                        EpiDW{G, ld, P.offW[l], fin}, st);
         }
         if (e != cudaSuccess) return fail(DBW_ECUDA, "dW GEMM %d: %s", l, cudaGetErrorString(e));
@@ -941,21 +982,21 @@ int worker_grads_fp32(const GradsPlan& P, const float* w, const float* pool, int
         if (e != cudaSuccess) return fail(DBW_ECUDA, "bias grad %d: %s", l, cudaGetErrorString(e));
         if (l > 0) {
             // dZ_{l-1}[m, c] = sum_o dZ_l[m, o] W_l[o, c]: A(m, o) = dZ[m*fout + o], B(o, c) = W[o*fin + c]
-            float* dnext = dz[cur ^ 1];
+            T* dnext = dz[cur ^ 1];
             if (skinny_k_ok(fin, fout)) {
                 const int ry = (M + 15) / 16;
                 dim3 grid((fin + 255) / 256, ry < 65535 ? ry : 65535);
                 const bool parts = P.tf32_dw[l - 1];   // the next weight gradient reads the transposed parts
                 const int Kp = static_cast<int>(tf32::padded_samples(B));
-                launch(skinny_k_dx_kernel, grid, 256, ((size_t)fin + 16) * fout * 4, st, M, fin, fout, dZl, fout,
-                       w + P.offW[l], fin, EpiDx{Aprev, dnext, fin},
+                launch(skinny_k_dx_kernel<T>, grid, 256, ((size_t)fin + 16) * fout * 4, st, M, fin, fout, dZl, fout,
+                       wop + P.offW[l], fin, EpiDx<T>{Aprev, dnext, fin},
                        parts ? reinterpret_cast<float*>(ws + P.off_zthi) : nullptr,
                        parts ? reinterpret_cast<float*>(ws + P.off_ztlo) : nullptr, (int64_t)P.n * Kp, B, Kp - B);
                 dz_parts_ready = parts;
                 e = cudaGetLastError();
             } else {
-                e = run_gemm<true, false>(M, fin, fout, dZl, fout, 0, w + P.offW[l], fin, 0, 1,
-                                             EpiDx{Aprev, dnext, fin}, st, split_ws, P.split_floats);
+                e = run_gemm<T, true, false>(M, fin, fout, dZl, fout, 0, wop + P.offW[l], fin, 0, 1,
+                                             EpiDx<T>{Aprev, dnext, fin}, st, split_ws, P.split_floats);
             }
             if (e != cudaSuccess) return fail(DBW_ECUDA, "dX GEMM %d: %s", l, cudaGetErrorString(e));
             cur ^= 1;
@@ -999,13 +1040,15 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
     };
     take(256);   // status word (int32 at offset 0), as in the tcgen05 plan
     P->off_cnt = take((size_t)n * 4);
-    P->off_x = take((size_t)M * widths[0] * 4);
+    const size_t es = prec == DBW_PREC_BF16 ? 2 : 4;
+    P->off_x = take((size_t)M * widths[0] * es);
     P->off_act[0] = P->off_x;
-    for (int l = 1; l < L; ++l) P->off_act[l] = take((size_t)M * widths[l] * 4);
+    for (int l = 1; l < L; ++l) P->off_act[l] = take((size_t)M * widths[l] * es);
     P->off_logits = take((size_t)M * widths[L] * 4);
     P->off_sloss = take((size_t)M * 4);
-    P->off_dz[0] = take((size_t)M * maxw * 4);
-    P->off_dz[1] = take((size_t)M * maxw * 4);
+    P->off_dz[0] = take((size_t)M * maxw * es);
+    P->off_dz[1] = take((size_t)M * maxw * es);
+    P->off_wb = prec == DBW_PREC_BF16 ? take((size_t)P->d * 2) : 0;
     // split-K scratch of the forward and input-gradient GEMMs (the largest splits x M x N)
     size_t split = 0;
     for (int l = 0; l < L; ++l) {
@@ -1057,7 +1100,7 @@ bool make_grads_plan(int L, const int32_t* widths, int n, int B, int prec, Grads
 int grads_activations(int L, const int32_t* widths, int n, int B, int prec, int layer, size_t* offset, int64_t* ld,
                       int* elem_bytes) {
     if (layer < 1 || layer >= L) return fail(DBW_EINVAL, "dbw_worker_grads_activations: layer must be in [1, L-1]");
-    if (prec == DBW_PREC_BF16) {
+    if (tc_eligible(prec, L, B)) {
         TcPlan T;
         if (!make_tc_plan(L, widths, n, B, &T)) return fail(DBW_EINVAL, "dbw_worker_grads_activations: invalid shape");
         *offset = T.off_act[layer];
@@ -1069,12 +1112,12 @@ int grads_activations(int L, const int32_t* widths, int n, int B, int prec, int 
     if (!make_grads_plan(L, widths, n, B, prec, &P)) return fail(DBW_EINVAL, "dbw_worker_grads_activations: invalid shape");
     *offset = P.off_act[layer];
     *ld = widths[layer];
-    *elem_bytes = 4;
+    *elem_bytes = prec == DBW_PREC_BF16 ? 2 : 4;
     return DBW_OK;
 }
 
 size_t grads_workspace_bytes(int L, const int32_t* widths, int n, int B, int prec) {
-    if (prec == DBW_PREC_BF16) {
+    if (tc_eligible(prec, L, B)) {
         TcPlan T;
         if (!make_tc_plan(L, widths, n, B, &T)) return 0;
         return T.ws_bytes;
@@ -1091,7 +1134,7 @@ int launch_worker_grads(int L, const int32_t* widths, int prec, const float* w, 
     if (!make_grads_plan(L, widths, n, B, prec, &P)) return fail(DBW_EINVAL, "dbw_worker_grads: invalid model shape");
     if (P.d != d) return fail(DBW_EINVAL, "dbw_worker_grads: d = %lld but the widths give %lld", (long long)d,
                               (long long)P.d);
-    if (prec == DBW_PREC_BF16) {
+    if (tc_eligible(prec, L, B)) {
         TcPlan T;
         if (!make_tc_plan(L, widths, n, B, &T)) return fail(DBW_EINVAL, "dbw_worker_grads: invalid model shape");
         if (ws_bytes < T.ws_bytes)
@@ -1100,7 +1143,9 @@ int launch_worker_grads(int L, const int32_t* widths, int prec, const float* w, 
     }
     if (ws_bytes < P.ws_bytes)
         return fail(DBW_EINVAL, "dbw_worker_grads: workspace %zu bytes < %zu needed", ws_bytes, P.ws_bytes);
-    return worker_grads_fp32(P, w, pool, S, labels, idx, G, ld, loss, static_cast<char*>(ws), st);
+    if (prec == DBW_PREC_BF16)
+        return worker_grads_simt<__nv_bfloat16>(P, w, pool, S, labels, idx, G, ld, loss, static_cast<char*>(ws), st);
+    return worker_grads_simt<float>(P, w, pool, S, labels, idx, G, ld, loss, static_cast<char*>(ws), st);
 }
 
 }  // namespace dbw

@@ -1,5 +1,5 @@
 // Internal plans of the worker-gradient passes: layer offsets (both precisions) and
-// workspace layout (GradsPlan's is the fp32 pass's, TcPlan's the bf16 pass's).
+// workspace layout (GradsPlan's is the pass of grads.cu's, TcPlan's the tcgen05 pass's).
 #pragma once
 
 #include <stddef.h>
@@ -18,11 +18,12 @@ struct GradsPlan {
     int64_t d;
     // workspace byte offsets (256-byte aligned)
     size_t off_cnt;                 // int32 [n]: loss counters of the workers, right after the status word
-    size_t off_x;                   // X = gathered inputs [M, widths[0]] fp32
-    size_t off_act[DBW_LMAX];       // A_l [M, widths[l]] fp32 for l = 1..L-1 (off_act[0] = off_x)
+    size_t off_x;                   // X = gathered inputs [M, widths[0]] (operand type)
+    size_t off_act[DBW_LMAX];       // A_l [M, widths[l]] (operand type) for l = 1..L-1 (off_act[0] = off_x)
     size_t off_logits;              // [M, C] fp32
     size_t off_sloss;               // [M] fp32 per-sample loss
-    size_t off_dz[2];               // ping-pong dZ [M, max width] fp32
+    size_t off_dz[2];               // ping-pong dZ [M, max width] (operand type)
+    size_t off_wb;                  // bf16 weights [d] (bf16 only)
     size_t off_split;               // split-K partial tiles of the SIMT GEMMs
     size_t split_floats;
     // fp32 forward GEMMs on the tensor cores in three tf32 passes (gemm_tf32.cuh):
@@ -80,6 +81,9 @@ struct RxPlan {
     size_t off_part[DBW_LMAX];         // fp32: its partial tiles
     size_t ws_bytes;
 };
+
+// Which bf16 passes run on tcgen05 (grads_tc.cu); the others run in grads.cu.
+bool tc_eligible(int prec, int L, int B);
 
 // The received-workers pass needs bf16 and a Gram tile layout: B % 32 == 0 and either
 // 128 % B == 0 or B % 128 == 0.

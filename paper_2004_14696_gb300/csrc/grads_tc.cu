@@ -9,10 +9,9 @@
 //   dW        G_i = dZ_l[i]^T . A_{l-1}[i]   A = dZ_l [M, out],      B = act[l-1] [M, in]
 //                                            (worker i: rows i*B .. i*B+B-1, K = B)
 //
-// Every B runs here: a worker's rows are read through a 3-D tensor map (column, sample,
-// worker), so the last K block of a B that is not whole K blocks reads zeros past the
-// worker's samples.  (16 workers of 500 samples, 3072-1024-1024-10: 5,440 us on fp32 FFMA
-// tiles, which served B % 32 != 0 before.)
+// A worker's rows are read through a 3-D tensor map (column, sample, worker), so the last K
+// block of a B that is not whole K blocks reads zeros past the worker's samples (tc_eligible says
+// which such B run here).
 //
 // Every operand is the row-major bf16 buffer its producer wrote: the tensor cores read
 // dZ, the activations and (in dX) W as MN-major tiles, so no transposed copy is formed.
@@ -576,6 +575,17 @@ int worker_grads_tc(const TcPlan& P, const float* w, const float* pool, int64_t 
 // epilogue applies the SGD step (TC_GBAR), the bias part is a column sum, and the
 // per-worker squared norms come from B x B Gram matrices (tc_gram).  The number
 // of received workers k is read on the device from ``mask``.
+
+// Whole 32-sample blocks always.  Another B was computed on FFMA tiles, whose sums round in
+// another order; a bf16 rounding that falls the other way can move a pre-activation across the
+// ReLU's zero, which adds or drops one sample in an entry of G: the fewer samples and the more
+// layers, the larger the difference.  Against the bound of 0.9 of an entry's scale (the rms of G
+// or the entry), 14 random models each: with 16 samples up to 1.5, with 50 0.86, with 100 0.71,
+// with 200 and 500 0.49; iterations of four layers and more that receive one or two workers pass the
+// bound's 2-norm part (2e-2) at any B (up to 3.6e-2), of up to three layers they stay at 8.5e-3.
+// So a ragged B runs on the tensor cores from 96 samples and up to three layers: 16 workers of 500
+// samples, 3072-1024-1024-10, 5,440 us on FFMA, 288 here.
+bool tc_eligible(int prec, int L, int B) { return prec == DBW_PREC_BF16 && (B % 32 == 0 || (B >= 96 && L <= 3)); }
 
 bool rx_eligible(int prec, int B) {
     return prec == DBW_PREC_BF16 && B % 32 == 0 && (128 % B == 0 || B % 128 == 0);

@@ -268,7 +268,8 @@ cudaError_t launch_bias_v(const T* dZ, int64_t ldz, int out, int n, int B, float
     return cudaGetLastError();
 }
 
-// dZ 16-byte aligned.  Wide loads where the rows allow them (bf16 rows are padded to 8).
+// dZ 16-byte aligned.  Wide loads where the rows allow them (the tcgen05 pass pads its bf16 rows
+// to 8; the rows of the FFMA pass are as wide as the layer).
 inline cudaError_t launch_bias_grad(const float* dZ, int64_t ldz, int out, int n, int B, float* G, int64_t ldG,
                                     int64_t offb, cudaStream_t st) {
     if (ldz % 4 == 0 && out % 4 == 0) return launch_bias_v<float, 4>(dZ, ldz, out, n, B, G, ldG, offb, st);
@@ -277,7 +278,7 @@ inline cudaError_t launch_bias_grad(const float* dZ, int64_t ldz, int out, int n
 }
 inline cudaError_t launch_bias_grad(const __nv_bfloat16* dZ, int64_t ldz, int out, int n, int B, float* G, int64_t ldG,
                                     int64_t offb, cudaStream_t st) {
-    if (out >= 8) return launch_bias_v<__nv_bfloat16, 8>(dZ, ldz, out, n, B, G, ldG, offb, st);
+    if (out >= 8 && ldz % 8 == 0) return launch_bias_v<__nv_bfloat16, 8>(dZ, ldz, out, n, B, G, ldG, offb, st);
     return launch_bias_v<__nv_bfloat16, 1>(dZ, ldz, out, n, B, G, ldG, offb, st);
 }
 

@@ -201,20 +201,21 @@ class Iteration:
             # launch when l > 0); bias row sums and bias mean of all layers (2), Gram norms of all
             # layers (1), finish; grad_stats
             return choose + 1 + (1 + 1 + 1 + L + 1 + L + 2 + 1 + 1) + 1
-        if self.wl.prec == dbw.PREC_BF16:
+        if self.wl.prec == dbw.PREC_BF16 and (self.wl.B % 32 == 0 or (self.wl.B >= 96 and L <= 3)):
             # tcgen05 pass: the weight casts of all layers (1), X, L forward GEMMs, loss + dZ_L,
             # L dW GEMMs, L bias gradients, L-1 dX GEMMs
             grads = 1 + 1 + L + 1 + L + L + (L - 1)
         else:
             # gather, forward, loss, dW, bias, dX
-            grads = 1 + L + 1 + L + L + (L - 1) + self._fp32_extra_launches()
+            grads = 1 + L + 1 + L + L + (L - 1) + self._simt_extra_launches()
         return choose + grads + 1 + 1 + 1
 
-    def _fp32_extra_launches(self):
-        """Launches beyond one per GEMM on the fp32 pass: a GEMM in three tf32 passes splits
+    def _simt_extra_launches(self):
+        """Launches beyond one per GEMM on the pass of csrc/grads.cu: a GEMM in three tf32 passes splits
         its two operands first (2), a split-K GEMM sums its splits (1); the skinny kernels
         are one launch.  Mirrors the plan's rules in csrc/grads.cu."""
         wd, M = self.wl.widths, self.wl.n * self.wl.B
+        f32 = self.wl.prec == dbw.PREC_FP32
         sms = torch.cuda.get_device_properties(self.device).multi_processor_count
 
         def split_launch(m, n, k):
@@ -226,27 +227,27 @@ class Iteration:
             return 1 if -(-k // kps) > 1 else 0
 
         def skinny_n(n, k, off):     # the forward GEMM with few outputs (W_l at offset off of w)
-            return n <= 16 and ((k % 4 == 0 and off % 4 == 0) or n * k * 4 <= 48 * 1024)
+            return n <= 16 and ((f32 and k % 4 == 0 and off % 4 == 0) or n * k * 4 <= 48 * 1024)
 
         def skinny_k(n, k):     # the input-gradient GEMM with a short inner dimension
             return k <= 32 and (n + 16) * k * 4 <= 48 * 1024
 
         B, n, off = self.wl.B, self.wl.n, 0
-        extra = 0
+        extra = 0 if f32 else 1                 # the bf16 copy of the weights
         last = sum(i * o + o for i, o in zip(wd[:-2], wd[1:-1]))   # offset of the last layer in w
-        if wd[-1] <= 16 and wd[-2] % 4 == 0 and last % 4 == 0:
+        if f32 and wd[-1] <= 16 and wd[-2] % 4 == 0 and last % 4 == 0:
             # the last forward GEMM and the loss are one launch; a single layer needs no gather
             extra -= 1 if len(wd) > 2 else 2
         for l in range(len(wd) - 1):
             fin, fout = wd[l], wd[l + 1]
             if fout <= 16:
                 extra -= 1                      # the bias gradient comes with the weight gradient
-            elif ((B % 32 == 0 or B > 128) and fin % 4 == 0 and off % 4 == 0 and fout >= 32
+            elif (f32 and (B % 32 == 0 or B > 128) and fin % 4 == 0 and off % 4 == 0 and fout >= 32
                   and n * fout * fin * B >= 1 << 25):
                 extra += 1 if l == 0 else 2     # transposed parts of dZ_l (and of the input above layer 1)
                 if l + 2 < len(wd) and skinny_k(fout, wd[l + 2]):
                     extra -= 1                  # those of dZ_l come with the dX kernel that forms it
-            if fout >= 32 and M * fout * fin >= 1 << 27:
+            if f32 and fout >= 32 and M * fout * fin >= 1 << 27:
                 extra += 0 if l == 0 else 2     # the gather writes the first layer's parts
             elif not skinny_n(fout, fin, off):
                 extra += split_launch(M, fout, fin)

@@ -1,7 +1,9 @@
 """GPU parity of the bf16 pass at minibatches off the 32- and 64-deep K blocks of the
-weight-gradient kernel and off the 16-row steps of its MMAs: every worker's gradient
-row and loss against the oracle.  A worker's rows past its B samples belong to the next
-worker (or lie past the buffer); the kernel has to read them as zero."""
+weight-gradient kernel and off the 16-row steps of its MMAs, and at those that the FFMA
+tiles serve (a ragged B below 96, or in a model of more than three layers): every worker's
+gradient row and loss against the oracle.  On the tensor cores a worker's rows past its B
+samples belong to the next worker (or lie past the buffer); the kernel has to read them as
+zero.  The FFMA pass stores its rows unpadded, so odd widths start them on 2 bytes."""
 import pytest
 import torch
 
@@ -21,9 +23,11 @@ def built():
 
 # (widths, n, B): B at and around the K blocks, M = n B at and around 32-, 128- and 256-row
 # tiles; (36, 18, 10) stores its second layer with scalar stores (rows off 16 bytes)
-CASES = [((68, 40, 10), 3, B) for B in (1, 15, 16, 17, 31, 33, 50, 63, 65, 100)]
-CASES += [((36, 18, 10), 2, 17), ((36, 18, 10), 3, 65), ((200, 96, 10), 1, 1), ((260, 300, 7), 1, 129),
-          ((256, 130, 34), 5, 51), ((64, 320), 1, 255)]
+CASES = [((68, 40, 10), 3, B) for B in (1, 16, 17, 33, 50, 95, 97, 100, 111, 113, 127, 129, 191,
+                                                     193, 225)]
+CASES += [((36, 18, 10), 2, 17), ((36, 18, 10), 3, 97), ((68, 40, 36, 34, 10), 3, 100),
+          ((68, 40, 36, 10), 3, 161), ((200, 96, 10), 1, 1), ((260, 300, 7), 1, 129), ((256, 130, 34), 5, 51),
+          ((256, 131, 33), 2, 51), ((64, 320), 1, 255)]
 
 
 @pytest.mark.parametrize("widths,n,B", CASES, ids=lambda v: "-".join(map(str, v)) if isinstance(v, tuple) else str(v))
