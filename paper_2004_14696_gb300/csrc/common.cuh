@@ -54,6 +54,11 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 // dozen launches of 2-20 us.  A kernel that has nothing to wait for must wait all the same:
 // its successor relies on it.  (us per pass without and with: 784-256-10 at n = B = 64 142 and
 // 125, 784-10 at n = 16, B = 32 34.6 and 32.6, received 3072-1024-1024-10 at k = 96 501 and 477.)
+// The trigger follows the wait, so that one successor at a time waits on the SMs.  With the
+// trigger first, the kernels after it were set up one behind the other while the first still
+// ran, and the CTAs of a small grid shared the SMs that their slots had left: an iteration of
+// 400-300-200-20 at n = B = 10 in a graph took 151 us (122 now, 123 without early launches),
+// 784-256-10 at n = B = 64 116 (112); 784-10 29.7 (30.2).
 //
 // early = false: not before its predecessor has ended.
 template <class... Params, class... Args>
@@ -79,8 +84,8 @@ inline cudaError_t launch(void (*kern)(Params...), dim3 grid, dim3 block, size_t
 }
 
 __device__ __forceinline__ void grid_begin() {
-    cudaTriggerProgrammaticLaunchCompletion();   // the next kernel may be set up
     cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();   // the next kernel may be set up
 }
 
 // ----------------------------------------------------------------- launchers
