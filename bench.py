@@ -54,19 +54,19 @@ METRIC = "simulated PS iterations/sec at n workers"
 UNIT = "iter/s"
 
 # dram bytes (read + write) of one full-size aggregation launch from an ncu capture
-# (n = 256, d = 54,440,936, k = 142: 31.1411 GB read + 0.1717 GB written against
+# (n = 256, d = 54,440,936, k = 142: 31.1408 GB read + 0.2200 GB written against
 # 31.3580 GB algorithmic), as a ratio to the algorithmic bytes so that it scales to the
 # bench's launches (traffic grows with k d); reported as null once aggregate.cu
 # differs from the source the counters were taken on.
-AGG_TRAFFIC = {"ratio_to_algorithmic": (31.141070 + 0.171713) / 31.357979,
-               "source_sha256": "1d5f6bb0b751a7ad2fae28b88999146db77319f34bc6ba9bcc4d5be0abfcec09",
+AGG_TRAFFIC = {"ratio_to_algorithmic": (31.140790 + 0.219976) / 31.357979,
+               "source_sha256": "5ff9b7556686d6fadf831374be85769d08285d42c3a39b0fdeddd59fbe8492c9",
                "case": "n=256 d=54440936 k=142"}
 # dram bytes (read + write) of the per-worker weight-gradient launches of one
-# full-size pass (ncu on mlp4096x3-1000_n256_B32): 4.2158 + 17.2505 + 17.2508 +
-# 17.2520 GB against 4.2778 + 3 x 17.3141 GB algorithmic; keyed to the dW kernel's
+# full-size pass (ncu on mlp4096x3-1000_n256_B32): 4.2167 + 17.2496 + 17.2502 +
+# 17.2509 GB against 4.2778 + 3 x 17.3141 GB algorithmic; keyed to the dW kernel's
 # own source (dw_source_sha).
-DW_TRAFFIC = {"ratio_to_algorithmic": (4.2158 + 17.2505 + 17.2508 + 17.2520) / (4.2778 + 3 * 17.3141),
-              "source_sha256": "bafb8a813d2b51c8c7e1921e5fa40487cfd5f74fde82f3e96748fb7521c6d77b",
+DW_TRAFFIC = {"ratio_to_algorithmic": (4.2167 + 17.2496 + 17.2502 + 17.2509) / (4.2778 + 3 * 17.3141),
+              "source_sha256": "3c451b2893a4677646f80c9bfd5922d6c9015510b9ee8cd0f4353b16d8f29ca6",
               "case": "mlp4096x3-1000_n256_B32, one pass"}
 
 CASES = ("aggregate", "sweep", "grads", "received", "psw", "iterate")

@@ -19,7 +19,8 @@
 // softmax; a third of the casts' bytes and half of the epilogues' stores) the
 // 3072-1024-1024-10 pass of 128 x 128 samples took 822 us, without them 734.
 // Leading dimensions are padded to multiples of 8 elements (16 bytes, the TMA
-// stride rule); padding is never read (tensor maps carry the logical extents).
+// stride rule); tensor maps carry the logical extents, and the bias sums, whose 16-byte
+// loads reach into the padding, drop its columns.
 #include <math.h>
 
 #include "gemm_tc.cuh"
@@ -165,8 +166,8 @@ __global__ void __launch_bounds__(1024) compact_received_kernel(const uint8_t* _
 }
 
 // Bias part of Eqs. (3)-(4), g[o] = (1/k) sum_{r < k B} dZ[r, o], for every layer,
-// in two launches (bias_rows_kernel, mean_update_kernel).  The layers' blocks sit side by side in x; a block finds its
-// layer in the prefix table cb0 (blocks of 256 columns).
+// in two launches (bias_rows_kernel, mean_update_kernel).  The layers' blocks sit side by
+// side in x; a block finds its layer in the prefix table cb0 (blocks of 256 columns).
 struct BiasLayers {
     int L;
     const __nv_bfloat16* dz[DBW_LMAX];   // dZ_l [M, ldz]

@@ -32,8 +32,8 @@ __device__ __forceinline__ int live_rows(const int* kdev, int B, int M) {
 // CTA (i, y) takes rows y rows_cta .. of worker i, a warp kRows rows at a time: their
 // logits, sample indices and labels are all loaded before the first is reduced, and a lane
 // keeps its NJ logits of a row (classes lane, lane + 32, ..) in registers, so that each is
-// read once (NJ = 0, C > 1024: three passes over the row).  (One CTA per worker, a row at a time per warp, 32 masked
-// exponentials a row: 45 us for 16,384 rows of 10 classes in bf16, 49 for 16 workers of 500
+// read once (NJ = 0, C > 1024: three passes over the row).  (One CTA per worker, a row at a
+// time per warp, 32 masked exponentials a row: 45 us for 16,384 rows of 10 classes in bf16, 49 for 16 workers of 500
 // in fp32; now 9 and 8.)
 //
 // With ``sel`` (received-workers pass): slot i is worker sel[i] (stacked rows i B .., samples

@@ -11,8 +11,10 @@
 // over the rows whose diagonal cell has samples (group rows; a row's observed ranks
 // are a prefix, so the order of Eq. (17) among their observed cells is generated by
 // chains over observed cells only).  Each group row is a chain of the first family,
-// each column over the group rows one of the second, their diagonal cells the third;
-// a chain is split over up to eight threads whose block stacks are then merged.
+// each column over the group rows one of the second, their diagonal cells the third.
+// A group table that fits in shared memory is fitted there, a chain per group of lanes
+// (psw_fit_shared_kernel); a larger one in the state buffer, a chain split over up to
+// eight threads whose block stacks are then merged (psw_estimate_kernel).
 // Each projection is weighted pool-adjacent-violators with the sample counts as
 // weights; Dykstra's increments p_f are kept as dual variables lambda_f = w p_f
 // between calls (warm start).
@@ -561,7 +563,9 @@ constexpr int kFixRounds = 32;   // merging rounds of the exact block means
 // time: there, with the table and the block stacks in the state buffer and chains split over
 // at most eight threads whose stacks one thread merges, a sweep of 23 rows x 256 columns took
 // 75-85 us and a whole fit of 19 / 43 / 61 sweeps 1.9 / 3.8 / 5.1 ms; here 15-18 us and
-// 0.45 / 0.96 / 1.20 ms.
+// 0.45 / 0.96 / 1.20 ms.  (A cluster of 2 or 4 CTAs, each projecting its share of the rows and
+// columns into every CTA's copy of the table, took 0.94-1.02 and 0.90-1.02 of that: a phase is its
+// longest chain, not the number of them.)
 //
 // The observed cells of every chain are listed once.  A chain belongs to a group of g lanes of
 // a warp (g as large as the family's chains leave, at most 32).  Each lane pools its run of the
