@@ -218,11 +218,21 @@ __device__ __forceinline__ double gbar_cols(const TcEpi& e, int row, int nb0, in
     const int64_t at0 = e.off + static_cast<int64_t>(row) * e.ldrow + nb0;
     float* wp = e.W + at0;
     float* gp = e.gbar ? e.gbar + at0 : nullptr;
+    // a chunk's 32 weights, in flight together also where the rows do not allow 16-byte loads
+    // (one by one behind each other's stores they made a 1622 x 241 matrix's launch, k B = 32, 96 us; now 62)
     float4 nxt[8];
     auto fetch = [&](int c) {
-        if (rowok && wvec && nb0 + 32 * c + 32 <= N) {
+        if (!rowok) return;
+        if (wvec && nb0 + 32 * c + 32 <= N) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) nxt[j] = *reinterpret_cast<const float4*>(wp + 32 * c + 4 * j);
+        } else {
+            const int left = N - (nb0 + 32 * c);
+            const float* p = wp + 32 * c;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                nxt[j] = make_float4(4 * j < left ? p[4 * j] : 0.f, 4 * j + 1 < left ? p[4 * j + 1] : 0.f,
+                                     4 * j + 2 < left ? p[4 * j + 2] : 0.f, 4 * j + 3 < left ? p[4 * j + 3] : 0.f);
         }
     };
     fetch(0);
@@ -262,7 +272,9 @@ __device__ __forceinline__ double gbar_cols(const TcEpi& e, int row, int nb0, in
             for (int j = 0; j < 32; ++j) {
                 if (nb + j < N) {
                     const float g = u2f(r[j]) * inv_k;
-                    wp[32 * c + j] = fmaf(-e.lr, g, wp[32 * c + j]);
+                    const float4 q = cur[j / 4];
+                    const float w = j % 4 == 0 ? q.x : j % 4 == 1 ? q.y : j % 4 == 2 ? q.z : q.w;
+                    wp[32 * c + j] = fmaf(-e.lr, g, w);
                     if (gp) gp[32 * c + j] = g;
                     part += g * g;
                 }
