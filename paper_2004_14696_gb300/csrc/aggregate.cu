@@ -531,12 +531,21 @@ size_t wide_smem_bytes(int n) { return kWideRing + (size_t)kWarps * n * sizeof(d
 constexpr int64_t kWideMinCols = 8000000;
 bool use_wide(int64_t d) { return d >= kWideMinCols; }
 
+// The opt-in to shared memory belongs to the kernel and is shared by the host's threads: every
+// call sets it to the need of the largest n, so that none lowers it between another's set and launch.
+template <class Kern>
+cudaError_t allow_smem(Kern kern, bool wide) {
+    const size_t most = wide ? wide_smem_bytes(DBW_NMAX) : agg_smem_bytes(DBW_NMAX);
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Co-resident CTAs of a kernel per SM with its dynamic shared memory.
 template <class Kern>
-int ctas_per_sm(Kern kern, int threads, size_t smem) {
+int ctas_per_sm(Kern kern, bool wide, int n) {
     int per_sm = 0;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    allow_smem(kern, wide);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, wide ? kWideThreads : kThreads,
+                                                  wide ? wide_smem_bytes(n) : agg_smem_bytes(n));
     return per_sm < 1 ? 1 : per_sm;
 }
 
@@ -546,8 +555,7 @@ AggGeometry agg_geometry(int n, int64_t d) {
     AggGeometry g;
     // both instantiations of a kernel have the same launch shape; the default one sets the grid
     const bool wide = use_wide(d);
-    const int per_sm = wide ? ctas_per_sm(aggregate_wide_kernel<false>, kWideThreads, wide_smem_bytes(n))
-                            : ctas_per_sm(aggregate_kernel<false>, kThreads, agg_smem_bytes(n));
+    const int per_sm = wide ? ctas_per_sm(aggregate_wide_kernel<false>, true, n) : ctas_per_sm(aggregate_kernel<false>, false, n);
     const int64_t cols = wide ? kWideCols : kChunkCols * kWarps;   // columns of a CTA's chunks
     const int64_t need = (d + cols - 1) / cols;
     int64_t blocks = (int64_t)sm_count() * per_sm;
@@ -566,7 +574,7 @@ cudaError_t launch_aggregate_t(const float* G, int64_t ld, int n, int64_t d, con
     const bool wide = use_wide(d);
     const size_t smem = wide ? wide_smem_bytes(n) : agg_smem_bytes(n);
     auto kern = wide ? aggregate_wide_kernel<kAllRows> : aggregate_kernel<kAllRows>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, wide);
     if (e != cudaSuccess) return e;
     // A grid of several CTAs per SM must not be set up early: CTAs placed while other kernels
     // still hold an SM find its shared memory configured for those, fewer fit, and the rest of

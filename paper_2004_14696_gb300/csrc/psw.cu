@@ -1531,9 +1531,10 @@ cudaError_t launch_psw_record(void* psw, int n, const int32_t* order, const doub
 cudaError_t launch_psw_estimate(void* psw, int n, double tol, int max_sweeps, double* T_hat, cudaStream_t st) {
     const Layout L = layout(n);
     char* base = static_cast<char*>(psw);
-    // room for as many group rows as the table can have, within what a CTA can take
+    // room for as many group rows as the table can have, within what a CTA can take; the opt-in,
+    // which the host's threads share, is the same for every n
     const size_t all = fit_shared_bytes(n, n), smem = all < kFitSharedMax ? all : kFitSharedMax;
-    cudaError_t e = cudaFuncSetAttribute(psw_fit_shared_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(psw_fit_shared_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFitSharedMax);
     if (e == cudaSuccess) e = launch(psw_fit_shared_kernel, 1, fit_shared_threads(n), smem, st, base, L, n, tol, max_sweeps, T_hat, smem);
     if (e != cudaSuccess) return e;
     const int T = fit_threads(n);
