@@ -274,18 +274,22 @@ cudaError_t run(int M, int N, int K, const float* A, int64_t lda, const float* B
 // in three tf32 passes: A = the hi / lo parts of dZ^T [Mr = out rows, z Kp + r], B = those
 // of act^T [Nr = in rows, z Kp + r], both K-major (the transposed parts are written by
 // split_t_kernel; Kp = K rounded up to 4 for the 16-byte strides, and the 3-D tensor maps
-// read zeros past a worker's K samples, so a ragged K runs here).  A persistent grid walks 128 x 128 tiles (out x in) worker-major with
-// the in-tiles fastest; each tile has a hi.hi accumulator and a correction accumulator
-// (256 TMEM columns), two tiles in flight (512 columns), so that the MMAs of tile i + 1
-// run while the epilogue drains tile i.  A K above 256, or no multiple of 32, takes an
-// accumulator pair per 32 samples, which the epilogue warps add up in registers (rounding to
-// nearest): the fp32 FFMA tiles that serve such K otherwise round to nearest too, and this keeps
-// the error against 64 bits below theirs.  (Relative error of all of G, 784-256-10, 16 workers of
-// 500 / 260 / 130 samples, FFMA 4.07 / 3.74 / 3.22e-7; pairs of 256 samples 4.60 / 5.26 / 3.94e-7,
-// of 64 3.36 / 3.54 / 3.31e-7, of 32 3.29 / 3.41 / 3.13e-7, all in the same time.  At 70 and 50
-// samples 2.93 and 3.01 against 2.89 and 2.88: a ragged K up to 128 stays on FFMA.)
+// read zeros past a worker's K samples, so a ragged K runs here).
+// A persistent grid walks 128 x 128 tiles (out x in) worker-major with
+// the in-tiles fastest; hi.hi and correction accumulators are 128 TMEM columns each, two of
+// both, so that the MMAs of tile i + 1 run while the epilogue drains tile i.  A K above 256, or
+// no multiple of 32, takes a hi.hi accumulator per 8 samples (above 352: per 16), which the
+// epilogue warps add up in registers, rounding to nearest; the corrections, 2^-11 of the
+// products, stay in one accumulator.  The fp32 FFMA tiles that serve such K otherwise round to
+// nearest at every step, and a tensor core's addition is less exact than that: error of G
+// against 64 bits relative to theirs, 90 shapes of one and two hidden layers at B = 129 .. 507
+// (medians of 6 inputs): geometric mean 0.81, the worst 1.010 (2944-56-6 at B = 159), of a single
+// layer's weights 1.027.  With a pair per 32 samples single layers were up to 1.12 and all of G up
+// to 1.05 of FFMA's, with 16 samples at any K 1.07 and 1.02 (and 1 % to 8 % less time).  FFMA's
+// error grows with K, so that above 352 samples 16 do (worst 0.99); a ragged K up to 128 stays on
+// FFMA (2.89 against 2.93e-7 at 70 samples with a pair per 32).
 // (784-256-10, 16 workers of 500 samples: both layers' weight gradients took 175 us on FFMA
-// tiles; now 42 here, 7 for the parts of dZ, and 14 in the few-output kernel.)
+// tiles; now 47 here, 7 for the parts of dZ, and 14 in the few-output kernel.)
 // Eight epilogue warps, two per TMEM lane quarter (32 G rows),
 // each copy their 32 x 64 block TMEM -> registers (hi.hi + corrections, rounded to
 // nearest; its four TMEM loads in flight together) -> shared memory (16-byte pieces
@@ -309,32 +313,25 @@ static_assert(WARP_COLS % 32 == 0 && EPI_WARPS % 4 == 0, "whole 32-column segmen
 constexpr int SMEM = STAGES * STAGE_BYTES + EPI_WARPS * WARP_STAGING + 256 + 1024;
 constexpr int TILE_COLS = 2 * BN;                         // hi.hi, then the corrections
 constexpr int TMEM_COLS = 2 * TILE_COLS;
-constexpr int WHOLE = 8;   // K blocks that one accumulator pair takes (more, or a ragged K: one each)
+// Samples per main accumulator for K samples a worker (0: one accumulator for all of them).
+constexpr int kWhole = 256, kFine = 352;
+inline int chunk_samples(int K) { return K % BK == 0 && K <= kWhole ? 0 : K <= kFine ? 8 : 16; }
 }  // namespace dw
 
-// v = (or +=) main + corrections, 32 columns of one row.
-static __device__ __forceinline__ void add_parts(float4 (&v)[8], const uint32_t (&rm)[32], const uint32_t (&rc)[32],
-                                                 bool first) {
+// v = (or +=) 32 columns of one row.
+static __device__ __forceinline__ void add_part(float4 (&v)[8], const uint32_t (&r)[32], bool first) {
     using tcx::u2f;
 #pragma unroll
     for (int pc = 0; pc < 8; ++pc) {
-        float4 x;
-        x.x = u2f(rm[4 * pc]) + u2f(rc[4 * pc]);
-        x.y = u2f(rm[4 * pc + 1]) + u2f(rc[4 * pc + 1]);
-        x.z = u2f(rm[4 * pc + 2]) + u2f(rc[4 * pc + 2]);
-        x.w = u2f(rm[4 * pc + 3]) + u2f(rc[4 * pc + 3]);
-        if (!first) {
-            x.x += v[pc].x;
-            x.y += v[pc].y;
-            x.z += v[pc].z;
-            x.w += v[pc].w;
-        }
-        v[pc] = x;
+        v[pc].x = first ? u2f(r[4 * pc]) : v[pc].x + u2f(r[4 * pc]);
+        v[pc].y = first ? u2f(r[4 * pc + 1]) : v[pc].y + u2f(r[4 * pc + 1]);
+        v[pc].z = first ? u2f(r[4 * pc + 2]) : v[pc].z + u2f(r[4 * pc + 2]);
+        v[pc].w = first ? u2f(r[4 * pc + 3]) : v[pc].w + u2f(r[4 * pc + 3]);
     }
 }
 
-// kChunks: an accumulator pair per K block.
-template <bool kChunks>
+// kChunk: samples per main accumulator, several per tile (0: the whole K in one).
+template <int kChunk>
 static __global__ void __launch_bounds__(dw::THREADS, 1)
     dw_kernel(const __grid_constant__ Operands op, int Mr, int Nr, int K, int batch, int* status,
               float* __restrict__ Gbase, int64_t ldrow, int64_t ldG) {
@@ -358,7 +355,9 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
     const int mt_n = (Mr + BM - 1) / BM, nt_n = (Nr + dw::BN - 1) / dw::BN;
     const int tiles_per_z = mt_n * nt_n;
     const long long total = static_cast<long long>(tiles_per_z) * batch;
-    const int nk = (K + BK - 1) / BK, chunk = kChunks ? 1 : nk;   // K blocks per accumulator pair
+    constexpr int kSamples = kChunk ? kChunk : BK, kSteps = kSamples / 8;
+    static_assert(BK % kSamples == 0, "a chunk lies within a K block");
+    const int nk = (K + BK - 1) / BK, chunks = kChunk ? (K + kSamples - 1) / kSamples : 1;   // main accumulators per tile
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < dw::STAGES; ++s) {
@@ -414,64 +413,72 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
         // ---------------- MMA issuer
         constexpr uint32_t idesc = instr_desc_tf32(BM, dw::BN);
         long long g = 0;
-        int i = 0;   // accumulator pairs so far
+        int i = 0, tile = 0;   // main accumulators and tiles so far
         bool ok = true;
-        for (long long t = blockIdx.x; t < total && ok && !*vabort; t += gridDim.x) {
-            for (int k0 = 0; k0 < nk && ok; k0 += chunk, ++i) {
-                const int acc = i & 1;
-                const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
-                if (!mbar_wait(smem_u32(tempty_bar + acc), aph ^ 1)) {
+        // the next main accumulator, once the epilogue has drained it
+        auto next_main = [&] {
+            if (!mbar_wait(smem_u32(tempty_bar + (i & 1)), static_cast<uint32_t>((i >> 1) & 1) ^ 1)) {
+                atomicOr(status, 1);
+                *vabort = 1;
+                ok = false;
+            }
+            tc_fence_after();
+        };
+        for (long long t = blockIdx.x; t < total && ok && !*vabort; t += gridDim.x, ++tile) {
+            const uint32_t dcorr = tmem + static_cast<uint32_t>((tile & 1) * dw::TILE_COLS + dw::BN);
+            if (!kChunk) next_main();
+            for (int kb = 0; kb < nk && ok; ++kb, ++g) {
+                const int s = static_cast<int>(g % dw::STAGES);
+                const uint32_t ph = static_cast<uint32_t>((g / dw::STAGES) & 1);
+                if (!mbar_wait(smem_u32(full_bar + s), ph)) {
                     atomicOr(status, 1);
                     *vabort = 1;
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t dmain = tmem + static_cast<uint32_t>(acc * dw::TILE_COLS);
-                const uint32_t dcorr = dmain + dw::BN;
-                const int k1 = k0 + chunk < nk ? k0 + chunk : nk;
-                for (int kb = k0; kb < k1; ++kb, ++g) {
-                    const int s = static_cast<int>(g % dw::STAGES);
-                    const uint32_t ph = static_cast<uint32_t>((g / dw::STAGES) & 1);
-                    if (!mbar_wait(smem_u32(full_bar + s), ph)) {
-                        atomicOr(status, 1);
-                        *vabort = 1;
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t ah = smem_u32(part(s, 0)), al = smem_u32(part(s, 1));
-                    const uint32_t bh = smem_u32(part(s, 2)), bl = smem_u32(part(s, 3));
+                const uint32_t ah = smem_u32(part(s, 0)), al = smem_u32(part(s, 1));
+                const uint32_t bh = smem_u32(part(s, 2)), bl = smem_u32(part(s, 3));
 #pragma unroll
-                    for (int kk = 0; kk < BK / 8; ++kk) {
-                        if (kb * BK + 8 * kk >= K) break;   // samples past K are zero
-                        const uint32_t o = kk * 32;
-                        const uint32_t accum = (kb > k0 || kk > 0) ? 1u : 0u;
-                        tc_mma_tf32(dmain, smem_desc(ah + o, 128), smem_desc(bh + o, 128), idesc, accum);
-                        tc_mma_tf32(dcorr, smem_desc(ah + o, 128), smem_desc(bl + o, 128), idesc, accum);
-                        tc_mma_tf32(dcorr, smem_desc(al + o, 128), smem_desc(bh + o, 128), idesc, 1u);
+                for (int kk = 0; kk < BK / 8; ++kk) {
+                    if (kb * BK + 8 * kk >= K) break;   // samples past K are zero
+                    const bool fresh = kChunk ? kk % kSteps == 0 : kb == 0 && kk == 0;
+                    if (kChunk && fresh) {
+                        next_main();
+                        if (!ok) break;
                     }
-                    tc_commit(smem_u32(empty_bar + s));
+                    const uint32_t dmain = tmem + static_cast<uint32_t>((i & 1) * dw::TILE_COLS);
+                    const uint32_t o = kk * 32;
+                    tc_mma_tf32(dmain, smem_desc(ah + o, 128), smem_desc(bh + o, 128), idesc, fresh ? 0u : 1u);
+                    tc_mma_tf32(dcorr, smem_desc(ah + o, 128), smem_desc(bl + o, 128), idesc, kb > 0 || kk > 0 ? 1u : 0u);
+                    tc_mma_tf32(dcorr, smem_desc(al + o, 128), smem_desc(bh + o, 128), idesc, 1u);
+                    if (kChunk && (kk % kSteps == kSteps - 1 || kb * BK + 8 * (kk + 1) >= K))
+                        tc_commit(smem_u32(tfull_bar + (i++ & 1)));
                 }
-                tc_commit(smem_u32(tfull_bar + acc));
+                tc_commit(smem_u32(empty_bar + s));
             }
+            if (!kChunk) tc_commit(smem_u32(tfull_bar + (i++ & 1)));
         }
+        // after a wait that ran out the epilogue is woken once the MMAs issued have ended
+        if (kChunk && !ok) tc_commit(smem_u32(tfull_bar + (i & 1)));
     } else if (warp >= 2) {
         // ---------------- epilogue
         const int q = warp & 3;          // TMEM lanes 32 q .. 32 q + 31 = G rows m0 + 32 q ..
         const int h = (warp - 2) >> 2;   // columns [WARP_COLS h, WARP_COLS (h + 1)) of the tile
         uint8_t* buf = staging + (warp - 2) * dw::WARP_STAGING;
-        int i = 0;   // accumulator pairs so far
+        int i = 0, tile = 0;   // main accumulators and tiles so far
         bool ok = true;
-        for (long long t = blockIdx.x; t < total && ok; t += gridDim.x) {
+        for (long long t = blockIdx.x; t < total && ok; t += gridDim.x, ++tile) {
             const int z = static_cast<int>(t / tiles_per_z);
             const int rem = static_cast<int>(t % tiles_per_z);
             const int m0 = (rem / nt_n) * BM, n0 = (rem % nt_n) * dw::BN;
             const int row0 = m0 + q * 32;
             const int c0 = h * dw::WARP_COLS;   // this warp's first column of the tile
             const bool live = row0 < Mr && n0 + c0 < Nr;
+            const uint32_t tlane = tmem + (static_cast<uint32_t>(q * 32) << 16) + c0;
+            const uint32_t tcorr = tlane + static_cast<uint32_t>((tile & 1) * dw::TILE_COLS + dw::BN);
             float4 v[dw::NSEG][8];   // this lane's row of the warp's block
-            for (int k0 = 0; k0 < nk; k0 += chunk, ++i) {
+            for (int c = 0; c < chunks; ++c, ++i) {
                 const int acc = i & 1;
                 const uint32_t aph = static_cast<uint32_t>((i >> 1) & 1);
                 if (!mbar_wait(smem_u32(tfull_bar + acc), aph)) {
@@ -485,27 +492,33 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
                     break;
                 }
                 tc_fence_after();
-                const uint32_t tbase =
-                    tmem + static_cast<uint32_t>(acc * dw::TILE_COLS) + (static_cast<uint32_t>(q * 32) << 16);
+                const uint32_t tmain = tlane + static_cast<uint32_t>(acc * dw::TILE_COLS);
                 if (live) {
-                    if constexpr (!kChunks) {   // every segment's TMEM loads in flight together
+                    if constexpr (!kChunk) {   // every segment's TMEM loads in flight together
                         uint32_t rm[dw::NSEG][32], rc[dw::NSEG][32];
 #pragma unroll
                         for (int sg = 0; sg < dw::NSEG; ++sg) {
-                            tc_ld_32cols(tbase + c0 + 32 * sg, rm[sg]);
-                            tc_ld_32cols(tbase + dw::BN + c0 + 32 * sg, rc[sg]);
+                            tc_ld_32cols(tmain + 32 * sg, rm[sg]);
+                            tc_ld_32cols(tcorr + 32 * sg, rc[sg]);
                         }
                         tc_wait_ld();
 #pragma unroll
-                        for (int sg = 0; sg < dw::NSEG; ++sg) add_parts(v[sg], rm[sg], rc[sg], true);
+                        for (int sg = 0; sg < dw::NSEG; ++sg) {
+                            add_part(v[sg], rm[sg], true);
+                            add_part(v[sg], rc[sg], false);
+                        }
                     } else {
 #pragma unroll
                         for (int sg = 0; sg < dw::NSEG; ++sg) {
-                            uint32_t rm[32], rc[32];
-                            tc_ld_32cols(tbase + c0 + 32 * sg, rm);
-                            tc_ld_32cols(tbase + dw::BN + c0 + 32 * sg, rc);
+                            uint32_t r[32];
+                            tc_ld_32cols(tmain + 32 * sg, r);
                             tc_wait_ld();
-                            add_parts(v[sg], rm, rc, k0 == 0);
+                            add_part(v[sg], r, c == 0);
+                            if (c == chunks - 1) {   // the corrections of the whole K
+                                tc_ld_32cols(tcorr + 32 * sg, r);
+                                tc_wait_ld();
+                                add_part(v[sg], r, false);
+                            }
                         }
                     }
                 }
@@ -584,7 +597,8 @@ inline cudaError_t run_dw(int Mr, int Nr, int K, int batch, const float* dz, int
         !tc_make_batch_map_f32(&op.b_hi, at_hi, Nr, batch, K, Kp, dw::BN) ||
         !tc_make_batch_map_f32(&op.b_lo, at_lo, Nr, batch, K, Kp, dw::BN))
         return cudaErrorInvalidValue;
-    auto kern = K % BK != 0 || K > BK * dw::WHOLE ? dw_kernel<true> : dw_kernel<false>;
+    const int chunk = dw::chunk_samples(K);
+    auto kern = chunk == 0 ? dw_kernel<0> : chunk == 8 ? dw_kernel<8> : dw_kernel<16>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dw::SMEM);
     if (e != cudaSuccess) return e;
     const long long tiles = static_cast<long long>((Mr + BM - 1) / BM) * ((Nr + dw::BN - 1) / dw::BN) * batch;
