@@ -510,7 +510,8 @@ __global__ void __launch_bounds__(kWideThreads, 3) aggregate_wide_kernel(
 #pragma unroll
                         for (int v = 0; v < kWideVec; ++v) c[v] = x[v];
                     }
-                    add_row<kWideVec>(x, c, s1, s2, r, !kAllRows || p < k);
+                    // row 0 is the shift itself: left out of the sums, where an infinity would leave a NaN
+                    add_row<kWideVec>(x, c, s1, s2, r, p > 0 && (!kAllRows || p < k));
                 }
                 rn[h] = r;
             }

@@ -64,3 +64,36 @@ def test_aggregate_wide(n, d, k):
     # the received rows go through the same arithmetic with and without the others
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
     assert np.array_equal(got[0][2], got[1][2], equal_nan=True) and np.array_equal(got[0][3], got[1][3])
+
+
+@pytest.mark.parametrize("flags", [0, dbw.ALL_ROW_NORMS])
+@pytest.mark.parametrize("d", [7_999_999, 8_000_003])   # either side of the line
+def test_one_received_row_is_its_own_mean(d, flags):
+    """k = 1: g_t is the row, infinities and NaN included, and no entry deviates from it."""
+    n, ld, lr = 3, -(-d // 4) * 4, 0.05
+    g = torch.Generator(device="cuda").manual_seed(d)
+    G = torch.randn((n, ld), generator=g, device="cuda")
+    row = G[1]
+    row[0], row[d // 2], row[d // 2 + 1], row[d - 1] = float("inf"), -float("inf"), torch.finfo(torch.float32).min, float("inf")
+    mask = torch.tensor([0, 1, 0], dtype=torch.uint8, device="cuda")
+    for nan in (False, True):
+        if nan:
+            row[5] = float("nan")
+        w0 = torch.randn(d, generator=g, device="cuda")
+        w, gb = w0.clone(), torch.empty(d, device="cuda")
+        part = torch.empty(dbw.dbw_aggregate_partials_bytes(n, d), dtype=torch.uint8, device="cuda")
+        dbw.dbw_aggregate_update(G, n, d, mask, lr, w, part, gb, flags=flags)
+        state, stats = dbw.new_state(n, 5), torch.empty(dbw.STATS_LEN, dtype=torch.float64, device="cuda")
+        rows = torch.empty(n, dtype=torch.float64, device="cuda")
+        dbw.dbw_grad_stats(part, n, mask, torch.ones(n, device="cuda"),
+                           torch.arange(n, dtype=torch.float64, device="cuda"), lr, state, stats, rows)
+        torch.cuda.synchronize()
+        assert torch.equal(gb.nan_to_num(7.0, 8.0, 9.0), row[:d].nan_to_num(7.0, 8.0, 9.0))
+        step = torch.addcmul(w0.double(), row[:d].double(), torch.tensor(-np.float32(lr), device="cuda").double())
+        step = step.float()   # one rounding, as the kernel's fused multiply-add
+        assert torch.equal(w.nan_to_num(7.0, 8.0, 9.0), step.nan_to_num(7.0, 8.0, 9.0))
+        s, r = stats.cpu().numpy(), rows.cpu().numpy()
+        assert s[dbw.STAT_SS] == 0.0
+        assert np.isnan(s[dbw.STAT_GBAR_SQ]) if nan else np.isposinf(s[dbw.STAT_GBAR_SQ])
+        assert np.isnan(r[1]) if nan else np.isposinf(r[1])
+        assert np.isfinite(r[[0, 2]]).all() if flags else np.isnan(r[[0, 2]]).all()
