@@ -494,31 +494,30 @@ static __global__ void __launch_bounds__(dw::THREADS, 1)
                 tc_fence_after();
                 const uint32_t tmain = tlane + static_cast<uint32_t>(acc * dw::TILE_COLS);
                 if (live) {
-                    if constexpr (!kChunk) {   // every segment's TMEM loads in flight together
-                        uint32_t rm[dw::NSEG][32], rc[dw::NSEG][32];
+                    // every segment's TMEM loads in flight together
+                    uint32_t r[dw::NSEG][32];
 #pragma unroll
-                        for (int sg = 0; sg < dw::NSEG; ++sg) {
-                            tc_ld_32cols(tmain + 32 * sg, rm[sg]);
-                            tc_ld_32cols(tcorr + 32 * sg, rc[sg]);
-                        }
+                    for (int sg = 0; sg < dw::NSEG; ++sg) tc_ld_32cols(tmain + 32 * sg, r[sg]);
+                    if (!kChunk) {
+                        uint32_t rc[dw::NSEG][32];
+#pragma unroll
+                        for (int sg = 0; sg < dw::NSEG; ++sg) tc_ld_32cols(tcorr + 32 * sg, rc[sg]);
                         tc_wait_ld();
 #pragma unroll
                         for (int sg = 0; sg < dw::NSEG; ++sg) {
-                            add_part(v[sg], rm[sg], true);
+                            add_part(v[sg], r[sg], true);
                             add_part(v[sg], rc[sg], false);
                         }
                     } else {
+                        tc_wait_ld();
 #pragma unroll
-                        for (int sg = 0; sg < dw::NSEG; ++sg) {
-                            uint32_t r[32];
-                            tc_ld_32cols(tmain + 32 * sg, r);
+                        for (int sg = 0; sg < dw::NSEG; ++sg) add_part(v[sg], r[sg], c == 0);
+                        if (c == chunks - 1) {   // the corrections of the whole K
+#pragma unroll
+                            for (int sg = 0; sg < dw::NSEG; ++sg) tc_ld_32cols(tcorr + 32 * sg, r[sg]);
                             tc_wait_ld();
-                            add_part(v[sg], r, c == 0);
-                            if (c == chunks - 1) {   // the corrections of the whole K
-                                tc_ld_32cols(tcorr + 32 * sg, r);
-                                tc_wait_ld();
-                                add_part(v[sg], r, false);
-                            }
+#pragma unroll
+                            for (int sg = 0; sg < dw::NSEG; ++sg) add_part(v[sg], r[sg], false);
                         }
                     }
                 }
