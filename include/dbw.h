@@ -70,6 +70,7 @@ extern "C" {
 #define DBW_FLAG_L_SKIPPED (1 << 1) /* an Eq. (12) value had denominator <= 0 or was not finite */
 #define DBW_FLAG_EMPTY_MASK (1 << 2) /* dbw_grad_stats saw no received worker: nothing recorded */
 #define DBW_FLAG_BAD_STATE (1 << 3)  /* state->n disagrees with the call's n (or is out of range) */
+#define DBW_FLAG_WAIT_TIMEOUT (1 << 4) /* a bounded wait of the aggregation ran out: nothing recorded */
 
 /* indices into the stats_out vector of dbw_grad_stats (DBW_STATS_LEN doubles) */
 #define DBW_STAT_K 0       /* k_t, number of received gradients */
@@ -210,16 +211,17 @@ int dbw_profile_gemm_read(double* total_ms, int64_t* launches);
 
 /*
  * Test hook of the bounded waits (the paper has no counterpart; for tests of the
- * failure path).  Every wait of the tensor-core kernels on a pipeline barrier is
- * bounded (2 s); when one runs out the kernel sets bit 0 of the status word,
- * stops, waits (bounded) for its own copies still in flight, releases its tensor
- * memory and returns, so that the context stays usable.  This call arms the next
- * per-worker weight-gradient launch of dbw_worker_grads (one launch, then it
- * disarms itself): its waits are bounded by wait_ms, and its first CTA does not
- * issue the TMA load of pipeline stage ``stage`` (0 = its first), so that the
- * MMA's wait for that stage runs out, as a lost copy would make it.  That call's
- * G and loss are then undefined and its status word has bit 0 set.  stage < 0
- * disarms.  Host only; DBW_EINVAL unless 0 < wait_ms <= 2000.
+ * failure path).  Every wait of a kernel on a pipeline barrier is bounded (2 s);
+ * when one runs out the kernel records it, stops, waits (bounded) for its own
+ * copies still in flight, releases its tensor memory and returns, so that the
+ * context stays usable.  This call arms the next launch of the bf16 per-worker
+ * weight gradient (dbw_worker_grads) or of the aggregation for d >= 8,000,000,
+ * whichever comes first (one launch, then it disarms itself): its waits are
+ * bounded by wait_ms, and its first CTA does not issue the load of pipeline stage
+ * ``stage`` (0 = its first), so that the wait for that stage runs out, as a lost
+ * copy would make it.  A weight-gradient call's G and loss are then undefined and
+ * its status word has bit 0 set; an aggregation ends as dbw_aggregate_update says.
+ * stage < 0 disarms.  Host only; DBW_EINVAL unless 0 < wait_ms <= 2000.
  */
 int dbw_test_arm_wait_timeout(int stage, double wait_ms);
 
@@ -283,6 +285,10 @@ size_t dbw_aggregate_partials_bytes(int n, int64_t d);
  *           every row's norm in row_sqnorm.  Other bits: DBW_EINVAL.
  *  partials scratch of partials_bytes >= dbw_aggregate_partials_bytes(n, d),
  *           256-byte aligned; consumed by the next dbw_grad_stats.
+ * For large d the rows come through pipelines whose waits are bounded (2 s), never a
+ * hang.  If one runs out, the columns it concerns keep their w and gbar (the others
+ * have taken the step), and the sums say so: dbw_grad_stats sets
+ * DBW_FLAG_WAIT_TIMEOUT in state->flags, records nothing and gives NaN row norms.
  */
 #define DBW_ALL_ROW_NORMS 1
 int dbw_aggregate_update(const float* G, int64_t ld, int n, int64_t d,
@@ -316,7 +322,7 @@ int dbw_aggregate_update(const float* G, int64_t ld, int n, int64_t d,
  *  sums_out  [n + 2] fp64 device out: sums_out[j] = ||g_j||^2 for received rows
  *            (0 otherwise; every row with DBW_ALL_ROW_NORMS), sums_out[n] = the
  *            deviation sum of Eq. (10), sums_out[n + 1] = ||g_t||^2 -- the totals
- *            dbw_grad_stats would form.
+ *            dbw_grad_stats would form; NaN, but for rows not read, if a wait ran out.
  */
 #define DBW_NOALLOC_SCRATCH_BYTES ((size_t)4 << 20)
 int dbw_aggregate_update_noalloc(const float* G, int64_t ld, int n, int64_t d, const uint8_t* mask, float lr,

@@ -44,8 +44,6 @@
 // memory (each row slot is owned by one warp, so no atomics); the column
 // statistics are accumulated in fp64 per lane.  All reductions run in a fixed
 // order, so results are deterministic for a given device.
-#include <math_constants.h>
-
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -314,7 +312,8 @@ __device__ __forceinline__ void write_header(double* partials, int nblocks, int 
 template <bool kAllRows, class Bar>
 __device__ __forceinline__ void write_pieces(double* __restrict__ partials, int nblocks, int n, int nrows,
                                              const uint8_t* __restrict__ mask, const int* sel, const double* rowacc,
-                                             double ss_acc, double g2_acc, double (*red)[kWarps], Bar bar) {
+                                             double ss_acc, double g2_acc, double (*red)[kWarps], bool timed_out,
+                                             Bar bar) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     ss_acc = warp_sum_d(ss_acc);
     g2_acc = warp_sum_d(g2_acc);
@@ -327,11 +326,12 @@ __device__ __forceinline__ void write_pieces(double* __restrict__ partials, int 
         for (int q = tid; q < n; q += kThreads)
             if (!mask[q]) vals[(int64_t)q * nblocks + blockIdx.x] = 0.0;
     bar();
+    const double lost = __longlong_as_double(kPieceTimedOut);
     // rows are indexed by reading position in rowacc; scatter them to worker ids
     for (int p = tid; p < nrows; p += kThreads) {
         double t = 0.0;
         for (int wv = 0; wv < kWarps; ++wv) t += rowacc[(size_t)wv * n + p];
-        vals[(int64_t)sel[p] * nblocks + blockIdx.x] = t;
+        vals[(int64_t)sel[p] * nblocks + blockIdx.x] = timed_out ? lost : t;
     }
     if (tid == 0) {
         double x = 0.0, y = 0.0;
@@ -339,8 +339,8 @@ __device__ __forceinline__ void write_pieces(double* __restrict__ partials, int 
             x += red[0][wv];
             y += red[1][wv];
         }
-        vals[(int64_t)n * nblocks + blockIdx.x] = x;
-        vals[(int64_t)(n + 1) * nblocks + blockIdx.x] = y;
+        vals[(int64_t)n * nblocks + blockIdx.x] = timed_out ? lost : x;
+        vals[(int64_t)(n + 1) * nblocks + blockIdx.x] = timed_out ? lost : y;
         if (blockIdx.x == 0) write_header(partials, nblocks, n, kAllRows);
     }
 }
@@ -384,14 +384,16 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) aggregate_kernel(
         const int64_t col0 = chunk * kChunkCols + lane * 4;
         chunk_pass<kAllRows>(G, ld, d, col0, lane, k, nrows, inv_k, lr, sel, myrow, ring, w, gbar, ss_acc, g2_acc);
     }
-    write_pieces<kAllRows>(partials, nblocks, n, nrows, mask, sel, rowacc, ss_acc, g2_acc, red, bar);
+    write_pieces<kAllRows>(partials, nblocks, n, nrows, mask, sel, rowacc, ss_acc, g2_acc, red, false, bar);
 }
 
 // ------------------------------------------------------------------ wide form
 // Warps 0-7 reduce, warp 8's first lane produces.  A stage holds one row of the CTA's
 // chunk; full[s] completes when its bytes have landed, empty[s] when the eight warps have
-// read it.  Every wait is bounded (2 s): one that runs out raises a flag that stops the
-// producer and the other waits, and the block's deviation sum becomes NaN.
+// read it.  Every wait is bounded (2 s).  A warp one of whose waits ran out leaves w and g_t as
+// they are in that chunk and stops; it frees no further stage, so that the others either read
+// rows that have landed or run out in turn.  The block's pieces then all say so (kPieceTimedOut).
+// kTest: the instantiation of the tests of that path (see TestWaits).
 constexpr int kWideVec = 2;                                // float4 per lane and row
 constexpr int kWideCols = kWarps * 128 * kWideVec;
 constexpr int kWideStages = 4;                                   // one row of a chunk each
@@ -400,13 +402,14 @@ constexpr int kWideThreads = kThreads + 32;
 constexpr int kWideStageFloats = kWideCols;
 constexpr size_t kWideRing = (size_t)kWideStages * kWideStageFloats * 4;
 
-template <bool kAllRows>
+template <bool kAllRows, bool kTest = false>
 __global__ void __launch_bounds__(kWideThreads, 3) aggregate_wide_kernel(
     const float* __restrict__ G, int64_t ld, int n, int64_t d, const uint8_t* __restrict__ mask,
     float lr, float* __restrict__ w, float* __restrict__ gbar, double* __restrict__ partials,
-    int nblocks) {
+    int nblocks, TestWaits wt) {
     grid_begin();
     using namespace tcx;
+    const uint64_t wait_ns = kTest ? wt.limit_ns : kWaitLimitNs;
     extern __shared__ __align__(128) double smem_w[];
     float* ring = reinterpret_cast<float*>(smem_w);
     double* rowacc = smem_w + kWideRing / 8;
@@ -449,19 +452,19 @@ __global__ void __launch_bounds__(kWideThreads, 3) aggregate_wide_kernel(
                 const uint32_t bytes = left >= kWideCols ? kWideCols * 4u : (uint32_t)((left + 3) / 4) * 16u;
                 for (int p = 0; p < nrows; ++p, ++it) {
                     const int s = it % kWideStages;
-                    if (!mbar_wait(smem_u32(empty_bar + s), ((it / kWideStages) & 1) ^ 1)) {
+                    if (!mbar_wait(smem_u32(empty_bar + s), ((it / kWideStages) & 1) ^ 1, wait_ns)) {
                         *vabort = 1;
                         break;
                     }
+                    if (kTest && blockIdx.x == 0 && it == wt.skip_stage) continue;
                     const uint32_t fb = smem_u32(full_bar + s);
                     mbar_expect_tx(fb, bytes);
                     bulk_load(smem_u32(ring + s * kWideCols), G + (int64_t)sel[p] * ld + col0, bytes, fb);
                 }
             }
-            if (*vabort) {   // the copies still in flight land before the shared memory is given up
-                for (uint32_t q = it < kWideStages ? 0 : it - kWideStages; q < it; ++q)
-                    mbar_wait(smem_u32(full_bar + q % kWideStages), (q / kWideStages) & 1);
-            }
+            // the last copies land before the shared memory is given up, whatever the warps do
+            for (uint32_t q = it < kWideStages ? 0 : it - kWideStages; q < it; ++q)
+                mbar_wait(smem_u32(full_bar + q % kWideStages), (q / kWideStages) & 1, wait_ns);
         }
         return;
     }
@@ -485,8 +488,8 @@ __global__ void __launch_bounds__(kWideThreads, 3) aggregate_wide_kernel(
                 float r = 0.f;
                 if (p < nrows) {
                     const int s = it % kWideStages;
-                    if (!dead && !mbar_wait(smem_u32(full_bar + s), (it / kWideStages) & 1)) {
-                        dead = true;   // wait no further: the producer stops at the flag
+                    if (!dead && !mbar_wait(smem_u32(full_bar + s), (it / kWideStages) & 1, wait_ns)) {
+                        dead = true;
                         *vabort = 1;
                     }
                     ++it;
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__(kWideThreads, 3) aggregate_wide_kernel(
                     for (int v = 0; v < kWideVec; ++v)
                         x[v] = *reinterpret_cast<const float4*>(mine + s * kWideCols + v * 128);
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(empty_bar + s));
+                    if (lane == 0 && !dead) mbar_arrive(smem_u32(empty_bar + s));
                     if (!full) {   // columns >= d: row padding, or an earlier chunk's bytes
 #pragma unroll
                         for (int v = 0; v < kWideVec; ++v) {
@@ -519,11 +522,11 @@ __global__ void __launch_bounds__(kWideThreads, 3) aggregate_wide_kernel(
             const int p = p0 + lane / (32 / kWideGroup);
             if (lane % (32 / kWideGroup) == 0 && p < nrows) myrow[p] += (double)tot;
         }
+        if (__any_sync(0xffffffffu, dead)) break;   // rows not read: no step from them
         chunk_update<kWideVec>(c, s1, s2, col0, d, inv_k, lr, w, gbar, ss_acc, g2_acc);
     }
     bar();
-    if (*vabort) ss_acc = CUDART_NAN;
-    write_pieces<kAllRows>(partials, nblocks, n, nrows, mask, sel, rowacc, ss_acc, g2_acc, red, bar);
+    write_pieces<kAllRows>(partials, nblocks, n, nrows, mask, sel, rowacc, ss_acc, g2_acc, red, *vabort != 0, bar);
 }
 
 size_t agg_smem_bytes(int n) { return kRingBytes + (size_t)kWarps * n * sizeof(double) + (size_t)n * sizeof(int); }
@@ -573,14 +576,23 @@ template <bool kAllRows>
 cudaError_t launch_aggregate_t(const float* G, int64_t ld, int n, int64_t d, const uint8_t* mask, float lr,
                                float* w, float* gbar, double* partials, const AggGeometry& g, cudaStream_t st) {
     const bool wide = use_wide(d);
-    const size_t smem = wide ? wide_smem_bytes(n) : agg_smem_bytes(n);
-    auto kern = wide ? aggregate_wide_kernel<kAllRows> : aggregate_kernel<kAllRows>;
-    const cudaError_t e = allow_smem(kern, wide);
-    if (e != cudaSuccess) return e;
     // A grid of several CTAs per SM must not be set up early: CTAs placed while other kernels
     // still hold an SM find its shared memory configured for those, fewer fit, and the rest of
     // this grid becomes a second round (n = 64, d = 1e7 in a row: 395 us, early 523).
-    launch_when(g.blocks <= sm_count(), kern, g.blocks, wide ? kWideThreads : kThreads, smem, st, G, ld, n, d, mask, lr, w, gbar, partials, g.blocks);
+    const bool early = g.blocks <= sm_count();
+    if (!wide) {
+        const cudaError_t e = allow_smem(aggregate_kernel<kAllRows>, false);
+        if (e != cudaSuccess) return e;
+        launch_when(early, aggregate_kernel<kAllRows>, g.blocks, kThreads, agg_smem_bytes(n), st, G, ld, n, d, mask, lr, w,
+                    gbar, partials, g.blocks);
+        return cudaGetLastError();
+    }
+    const TestWaits wt = take_test_waits();
+    auto kern = wt.skip_stage >= 0 ? aggregate_wide_kernel<kAllRows, true> : aggregate_wide_kernel<kAllRows>;
+    const cudaError_t e = allow_smem(kern, true);
+    if (e != cudaSuccess) return e;
+    launch_when(early, kern, g.blocks, kWideThreads, wide_smem_bytes(n), st, G, ld, n, d, mask, lr, w, gbar, partials,
+                g.blocks, wt);
     return cudaGetLastError();
 }
 }  // namespace

@@ -131,10 +131,18 @@ int launch_worker_grads(int L, const int32_t* widths, int prec, const float* w, 
                         int n, int B, float* G, int64_t ld, float* loss, void* ws, size_t ws_bytes,
                         cudaStream_t st);
 
-// Tests of the bounded waits (gemm_tc.cu): the next weight-gradient launch bounds its
-// waits by limit_ns and its first CTA does not issue the load of pipeline stage
-// ``stage``; stage < 0 disarms.
-void arm_dw_wait_timeout(long long stage, unsigned long long limit_ns);
+// Tests of the bounded waits (gemm_tc.cu): the next launch of the bf16 weight gradient or of
+// the wide aggregation bounds its waits by limit_ns and its first CTA does not issue the load
+// of pipeline stage ``stage``; stage < 0 disarms.
+void arm_wait_timeout(long long stage, unsigned long long limit_ns);
+// What such a launch's kernel is given.  The production instantiations ignore it: their waits
+// are bounded by tcx::kWaitLimitNs.
+struct TestWaits {
+    unsigned long long limit_ns;   // every mbarrier wait of the launch
+    long long skip_stage;          // stage counter of block 0 left without its load; -1: none
+};
+// The armed test, which it disarms; skip_stage < 0 if none is.
+TestWaits take_test_waits();
 
 // Received-workers pass (grads_tc.cu)
 size_t received_workspace_bytes(int L, const int32_t* widths, int n, int B, int prec);
@@ -149,5 +157,8 @@ int launch_received_grads(int L, const int32_t* widths, int prec, float* w, int6
 //                                   q < n: ||g_q||^2, q = n: SS, q = n + 1: ||g_t||^2
 constexpr int64_t kPartialsMagic = DBW_PARTIALS_MAGIC;  // "DBWPART"
 constexpr int kPartialsHeader = 4;
+// The bits of every piece of a block of the aggregation one of whose waits ran out: a NaN that
+// no arithmetic gives, so that dbw_grad_stats tells it from a NaN in the gradients.
+constexpr long long kPieceTimedOut = 0x7ff8444257544f21ll;
 
 }  // namespace dbw

@@ -153,14 +153,22 @@ __global__ void __launch_bounds__(kRedThreads) grad_stats_kernel(
         span[0] = 255u;
         span[1] = 0u;
     }
-    const double ss_part = strided_sum(vals + (int64_t)n * blocks, blocks);
+    // a block of the aggregation whose wait ran out marks its pieces: w has not taken its whole step
+    int lost = 0;
+    double ss_part = 0.0;   // strided_sum's order
+    for (int i = tid; i < blocks; i += kRedThreads) {
+        const double piece = vals[(int64_t)n * blocks + i];
+        lost |= __double_as_longlong(piece) == kPieceTimedOut;
+        ss_part = ss_part + piece;
+    }
     const double g2_part = strided_sum(vals + (int64_t)(n + 1) * blocks, blocks);
     const dbw_state* sh = stage_head(st, head_s);   // (its barrier also orders mask_s, loss_s, span)
-    __shared__ int k_s;
-    if (tid == 0) k_s = 0;
+    __shared__ int k_s, lost_s;
+    if (tid == 0) k_s = lost_s = 0;
     const double SS0 = tree_sum(ss_part, red);      // (its barriers order k_s = 0)
     mine = __reduce_add_sync(0xffffffffu, mine);
     if ((tid & 31) == 0) atomicAdd(&k_s, mine);
+    if (lost) lost_s = 1;
     const double g20 = tree_sum(g2_part, red2);     // (its barriers complete k_s)
     const double SS = valid ? SS0 : CUDART_NAN, g2 = valid ? g20 : CUDART_NAN;
     if (tid == 0) {
@@ -168,9 +176,10 @@ __global__ void __launch_bounds__(kRedThreads) grad_stats_kernel(
         sums[n + 1] = g2;
     }
     const int k = k_s;
-    if (k == 0 || sh->n != n) {
+    if (k == 0 || sh->n != n || lost_s) {
         if (tid == 0)
-            st->flags = sh->flags | (k == 0 ? DBW_FLAG_EMPTY_MASK : 0) | (sh->n != n ? DBW_FLAG_BAD_STATE : 0);
+            st->flags = sh->flags | (k == 0 ? DBW_FLAG_EMPTY_MASK : 0) | (sh->n != n ? DBW_FLAG_BAD_STATE : 0) |
+                        (lost_s ? DBW_FLAG_WAIT_TIMEOUT : 0);
         return;
     }
     // Sect. 3.2: every arrival is observed, S[r] accumulates the r-th order statistic

@@ -930,19 +930,12 @@ struct DwCfg {
     static constexpr int SMEM = STAGES * STAGE_BYTES + STAGING + BAR_BYTES + 1024;
 };
 
-// Tests of the bounded-wait path (the kTest instantiation, launched only when armed):
-// the bound of the kernel's waits, and one pipeline stage whose TMA load the first CTA
-// does not issue, so that the MMA's wait for it runs out as a lost copy would make it.
-// The production instantiation ignores these: its waits are bounded by kWaitLimitNs.
-struct DwWaits {
-    unsigned long long limit_ns;   // every mbarrier wait of the launch
-    long long skip_stage;          // stage counter g of block 0 left without its load; -1: none
-};
-
+// kTest: the instantiation of the bounded-wait tests, whose MMA waits for a stage that was never
+// loaded as for a lost copy.
 template <int BK, int STAGES, bool kTest = false>
 __global__ void __launch_bounds__(DW_THREADS, 1)
     tc_dw_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int Mr, int Nr,
-                 int K, int batch, int* status, float* __restrict__ Gbase, int64_t ldrow, int64_t ldG, DwWaits wt) {
+                 int K, int batch, int* status, float* __restrict__ Gbase, int64_t ldrow, int64_t ldG, TestWaits wt) {
     grid_begin();
     const uint64_t wait_ns = kTest ? wt.limit_ns : kWaitLimitNs;
     using Cfg = DwCfg<BK, STAGES>;
@@ -1129,23 +1122,16 @@ __global__ void __launch_bounds__(DW_THREADS, 1)
 }
 
 // ------------------------------------------------------------------ host side
-// One-shot arming of a lost load in the next launch of tc_dw_kernel (tests of the
-// bounded-wait path; see dbw_test_arm_wait_timeout).
-std::atomic<long long> g_dw_skip_stage{-1};
-std::atomic<unsigned long long> g_dw_test_limit_ns{0};
+// One-shot arming of a lost load (tests of the bounded waits; see dbw_test_arm_wait_timeout).
+std::atomic<long long> g_test_skip_stage{-1};
+std::atomic<unsigned long long> g_test_limit_ns{0};
 
 template <int BK, int STAGES>
 cudaError_t launch_dw(const CUtensorMap& a, const CUtensorMap& b, int Mr, int Nr, int K, int batch, int* status,
                       float* gbase, int64_t ldrow, int64_t ldG, cudaStream_t st) {
     using Cfg = DwCfg<BK, STAGES>;
-    DwWaits wt{kWaitLimitNs, -1};
-    const long long skip = g_dw_skip_stage.exchange(-1);
-    const bool test = skip >= 0;
-    if (test) {
-        wt.skip_stage = skip;
-        wt.limit_ns = g_dw_test_limit_ns.load();
-    }
-    auto kern = test ? tc_dw_kernel<BK, STAGES, true> : tc_dw_kernel<BK, STAGES, false>;
+    const TestWaits wt = take_test_waits();
+    auto kern = wt.skip_stage >= 0 ? tc_dw_kernel<BK, STAGES, true> : tc_dw_kernel<BK, STAGES, false>;
     // each CTA holds all 512 TMEM columns: ask for enough shared memory that a
     // second CTA can never be resident on the same SM (it would wait in tcgen05.alloc)
     const int smem = Cfg::SMEM > 120 * 1024 ? Cfg::SMEM : 120 * 1024;
@@ -1222,9 +1208,14 @@ cudaError_t launch_cfg(const CUtensorMap& a, const CUtensorMap& b, int M, int N,
 
 }  // namespace
 
-void arm_dw_wait_timeout(long long stage, unsigned long long limit_ns) {
-    g_dw_test_limit_ns.store(limit_ns);
-    g_dw_skip_stage.store(stage);
+void arm_wait_timeout(long long stage, unsigned long long limit_ns) {
+    g_test_limit_ns.store(limit_ns);
+    g_test_skip_stage.store(stage);
+}
+TestWaits take_test_waits() {
+    TestWaits wt{tcx::kWaitLimitNs, g_test_skip_stage.exchange(-1)};
+    if (wt.skip_stage >= 0) wt.limit_ns = g_test_limit_ns.load();
+    return wt;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,

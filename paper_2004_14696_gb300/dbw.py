@@ -23,7 +23,7 @@ NMAX, DMAX, LMAX = 1024, 64, 8
 CHOOSE_BLIND = 1
 ALL_ROW_NORMS = 1
 NOALLOC_SCRATCH_BYTES = 4 << 20   # DBW_NOALLOC_SCRATCH_BYTES
-FLAG_K1, FLAG_L_SKIPPED, FLAG_EMPTY_MASK, FLAG_BAD_STATE = 1, 2, 4, 8
+FLAG_K1, FLAG_L_SKIPPED, FLAG_EMPTY_MASK, FLAG_BAD_STATE, FLAG_WAIT_TIMEOUT = 1, 2, 4, 8, 16
 PSW_NOT_CONVERGED, PSW_RANGE, PSW_UNPOLISHED = 1, 2, 4
 STAT_K, STAT_SS, STAT_GBAR_SQ, STAT_V, STAT_N, STAT_F, STAT_L, STAT_FLAGS, STAT_VCLOCK = range(9)
 STATS_LEN = 9
@@ -329,8 +329,8 @@ def dbw_choose_b(state, lr, beta, b_out, ratio_out=None, flags=0, stream=None):
 
 
 def dbw_test_arm_wait_timeout(stage, wait_ms):
-    """Arms the next weight-gradient launch to lose the load of one pipeline stage
-    (tests of the bounded-wait path); stage < 0 disarms."""
+    """Arms the next bf16 weight-gradient or wide aggregation launch to lose the load of one
+    pipeline stage (tests of the bounded-wait path); stage < 0 disarms."""
     _check("dbw_test_arm_wait_timeout", lib().dbw_test_arm_wait_timeout(int(stage), float(wait_ms)))
 
 
