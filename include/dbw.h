@@ -237,7 +237,8 @@ int dbw_test_arm_wait_timeout(int stage, double wait_ms);
  *  tsorted  [n] fp64 out: order statistics, tsorted[r] = times[order[r]];
  *           tsorted[k-1] is the iteration's duration for every candidate k.
  *  k_out    device int32 scalar out (nullable): the k actually used.
- *  n in [1, DBW_NMAX].
+ *  n in [1, DBW_NMAX].  tsorted may share memory with times, and k_out may be b; no
+ *  other output may share memory with an input or another output.
  */
 int dbw_select_fastest(const double* times, int n, const int32_t* b,
                        int32_t* order, uint8_t* mask, double* tsorted,

@@ -24,12 +24,12 @@ __device__ __forceinline__ unsigned long long order_key(double t) {
 
 constexpr int kSelectWarps = 8;
 
-// b (and times) may not be written by this launch; times may share memory with tsorted
-// only in a launch of one CTA (every time is staged before the first store).
+// Only a launch of one CTA, which stages every time and reads b before its first store, may have
+// times in tsorted's memory or b in k_out's.
 __global__ void __launch_bounds__(1024) select_fastest_kernel(
-    const double* times, int n, const int32_t* __restrict__ b_ptr,
+    const double* times, int n, const int32_t* b_ptr,
     int32_t* __restrict__ order, uint8_t* __restrict__ mask, double* tsorted,
-    int32_t* __restrict__ k_out) {
+    int32_t* k_out) {
     grid_begin();
     __shared__ double ts[DBW_NMAX];
     __shared__ unsigned long long key[DBW_NMAX];
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(1024) select_fastest_kernel(
 
 cudaError_t launch_select(const double* times, int n, const int32_t* b, int32_t* order,
                           uint8_t* mask, double* tsorted, int32_t* k_out, cudaStream_t st) {
-    if (times < tsorted + n && tsorted < times + n)   // sorted in place: one CTA
+    if ((times < tsorted + n && tsorted < times + n) || k_out == b)   // over its own inputs: one CTA
         launch(select_fastest_kernel, 1, 1024, 0, st, times, n, b, order, mask, tsorted, k_out);
     else
         launch(select_fastest_kernel, (n + kSelectWarps - 1) / kSelectWarps, 32 * kSelectWarps, 0, st, 

@@ -85,3 +85,17 @@ def test_select_may_sort_in_place():
     torch.cuda.synchronize()
     assert np.array_equal(t.cpu().numpy(), np.sort(times))
     assert np.array_equal(order.cpu().numpy(), np.argsort(times, kind="stable"))
+
+
+@pytest.mark.parametrize("n", [9, 1000])
+def test_select_may_leave_k_in_b(n):
+    times = np.random.default_rng(n).exponential(size=n)
+    b = torch.tensor([n // 3], dtype=torch.int32, device="cuda")
+    order = torch.empty(n, dtype=torch.int32, device="cuda")
+    mask = torch.empty(n, dtype=torch.uint8, device="cuda")
+    tsorted = torch.empty(n, dtype=torch.float64, device="cuda")
+    dbw.dbw_select_fastest(torch.from_numpy(times).cuda(), b, order, mask, tsorted, b)
+    torch.cuda.synchronize()
+    want = np.zeros(n, np.uint8)
+    want[np.argsort(times, kind="stable")[:n - n // 3]] = 1
+    assert int(b.item()) == n - n // 3 and np.array_equal(mask.cpu().numpy(), want)

@@ -1,9 +1,14 @@
-"""The opt-in to more than 48 KB of shared memory belongs to the kernel, not to a launch, and
+"""What the host code launches, checked without a GPU: the library's objects are linked
+against a stand-in for the CUDA runtime.
+
+The opt-in to more than 48 KB of shared memory belongs to the kernel, not to a launch, and
 host threads share it: a call that sets it to its own need would let a second thread, whose
 n is smaller, lower it between this thread's set and its launch, which the runtime then
-refuses.  Checked without a GPU: the library's objects are linked against a stand-in for
-the CUDA runtime that keeps the opt-in of each kernel, refuses a launch above it as the
-runtime does, and before each launch makes the call of the second thread."""
+refuses.  The stand-in keeps the opt-in of each kernel, refuses a launch above it as the
+runtime does, and before each launch makes the call of the second thread.
+
+The selection runs in several CTAs that share nothing; where an output lies over an input
+that each of them reads, it takes one."""
 import ctypes as C
 import os
 import subprocess
@@ -19,7 +24,7 @@ enum { kMost = 256, kDefault = 48 * 1024 };
 static const void* func[kMost];
 static int limit[kMost], used, inside;
 static cudaError_t last;
-int launches, refused;
+int launches, refused, grid;
 void (*other_thread)(void);
 
 static int* limit_of(const void* f) {
@@ -39,6 +44,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
         inside = 0;
     }
     ++launches;
+    grid = c->gridDim.x;
     if (c->dynamicSmemBytes > (size_t)*limit_of(f)) {
         ++refused;
         return last = cudaErrorInvalidValue;
@@ -132,3 +138,18 @@ def test_two_threads_fit(lib, n, other):
     def fit(n):
         return lib.dbw_psw_estimate(256, n, C.c_double(1e-4), 10, 256, None)
     assert with_other_thread(lib, lambda: fit(n), lambda: fit(other)) == dbw.DBW_OK
+
+
+@pytest.mark.parametrize("n", [1, 8, 9, 256, 1024])
+def test_selection_over_its_own_inputs_is_one_cta(lib, n):
+    times, b, order, mask, out, k = 1 << 20, 2 << 20, 3 << 20, 4 << 20, 5 << 20, 6 << 20   # addresses, not read here
+    grid = C.c_int.in_dll(lib, "grid")
+
+    def ctas(times, b, tsorted, k_out):
+        grid.value = 0
+        assert lib.dbw_select_fastest(times, n, b, order, mask, tsorted, k_out, None) == dbw.DBW_OK
+        return grid.value
+    assert ctas(times, b, out, k) == ctas(times, b, out, None) == -(-n // 8)
+    assert ctas(times, b, times, k) == 1          # sorted in place
+    assert ctas(times, b, times + 8 * n - 8, k) == 1 and ctas(times + 8 * n - 8, b, times, k) == 1
+    assert ctas(times, b, out, b) == 1            # k over b: a CTA could read b after another's k
