@@ -24,8 +24,12 @@
 // (k = 48, d = 1e7) / (64 rows read, d = 1e7) / (k = 192, d = 3e7): 297 / 384 / 3277, the
 // warp form 300 / 394 / 3404, the register form 331 / 428 / 3573; the last at 7.14 TB/s
 // (of measured copy bandwidth: 1.05).  Below kWideMinCols a CTA has few chunks and the last
-// round of them costs more (k = 12, d = 4e6: 45.9 against 43.3; k = 48, d = 203,530: 17.9
-// against 12.1).  Stages of two rows, 3 or 6 stages and 2 CTAs per SM were up to 4 % slower.
+// round of them costs more.  Wide over narrow, everything received, at d = 2, 4, 6, 7, 7.9, 9 and 12
+// million: k = 12 1.14, 1.06, 1.04, 1.04, 1.03, 1.06, 1.03; k = 48 1.06, 1.03, 1.01, 1.01, 1.005, 0.97,
+// 0.99; k = 192 1.06, 1.01, 1.00, 0.98, 0.98, 0.98, 0.96.  Those calls find part of few rows in L2;
+// with L2 flushed before each, d = 8.2e6 to 3e7, it is 0.87-1.01 at k = 1 .. 3, 0.91-1.07 at 4 .. 8 and
+// 0.93-0.99 above.  (The dearest corner: one row of 8.2e6 that stays in L2, 28.6 us against 24.5.)
+// Stages of two rows, 3 or 6 stages and 2 CTAs per SM were up to 4 % slower.
 //
 // Row norms.  The lanes' pieces of four rows are summed together: at each of the first two
 // exchange steps a lane gives away half of the rows it holds, so four rows cost 6 shuffles

@@ -603,19 +603,19 @@ __device__ __forceinline__ void store_piece(const TcEpi& e, int msub, int nt, in
     if (lane == 0 && ok) e.pieces[(static_cast<long long>(msub) * nt_n + nt) * 8 + h * 4 + q] = sq;
 }
 
-// Epilogue of one tile for problem kind KIND (one thread: one row, 128 columns).
 // Fetches what the epilogue of tile t needs besides the accumulator (before it is complete).
 template <int KIND>
 __device__ __forceinline__ void pair_epilogue_fetch(const PairProblem& P, const PairShape& S, int t, int rank,
                                                     int q, int h, int lane, float* sb, uint32_t (&mask)[4]) {
     const int nb0 = t % S.nt_n * 256 + h * 128;
     const int row = (t / S.nt_n * 2 + rank) * BM + q * 32 + lane;
-        if constexpr (KIND == TC_HIDDEN) hidden_bias(P.epi, nb0, P.N, sb);
+    if constexpr (KIND == TC_HIDDEN) hidden_bias(P.epi, nb0, P.N, sb);
     if constexpr (KIND == TC_DX)
         dx_mask(P.epi, row, nb0, P.M, P.N,
                 ((reinterpret_cast<uintptr_t>(P.epi.act) & 15u) == 0) && P.epi.ldact % 8 == 0, mask);
 }
 
+// Epilogue of one tile for problem kind KIND (one thread: one row, 128 columns).
 template <int KIND>
 __device__ __forceinline__ void pair_epilogue(const PairProblem& P, const PairShape& S, int t, int rank, int q, int h,
                                               int lane, uint32_t taddr, const float* sb, const uint32_t (&mask)[4]) {
@@ -1314,8 +1314,9 @@ static int pair_problem(PairProblem* P, int kind, const TcOperands& o, const TcE
     return DBW_OK;
 }
 
-// A tile has at most 8 ranges, a launch at most 152 (two rounds of the pairs, 39 MB of partial
-// sums).
+// A tile has at most 8 ranges, a launch at most 152: a cap on the scratch (39 MB of partial sums,
+// taken per layer when the workspace is sized) that two rounds of 76 pairs reach, not a limit of the
+// plan, which also holds with fewer pairs or more.
 constexpr int kSplitItems = 152;
 static long long gbar_tiles(int M, int N) {
     return static_cast<long long>((M + 2 * BM - 1) / (2 * BM)) * ((N + 255) / 256);

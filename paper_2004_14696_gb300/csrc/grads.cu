@@ -19,6 +19,8 @@
 // bf16 operands.
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "gemm_tf32.cuh"
 #include "grads.cuh"
@@ -906,14 +908,15 @@ int worker_grads_simt(const GradsPlan& P, const float* w, const float* pool, int
                 if (tc)
                     return tf32::run(M, fout, fin, Ain, fin, W, fin, part[0], part[1], part[2], part[3], epi, status, st,
                                      /*parts_ready=*/l == 0);
-                if (fout <= kSkinnyN && fin % 4 == 0 && aligned16(Ain) && aligned16(W)) {
-                    const int want = (M + 3) / 4;   // 4 rows (warps) per CTA
-                    const int grid = want < 8 * sm_count() ? want : 8 * sm_count();
-                    if (fin > 256)
-                        launch(skinny_n4_kernel<true, decltype(epi)>, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
-                    else
-                        launch(skinny_n4_kernel<false, decltype(epi)>, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
-                    return cudaGetLastError();
+                // (the last layer's go to logits_loss_kernel)
+                if constexpr (!std::is_same<decltype(epi), EpiLogits>::value) {
+                    if (fout <= kSkinnyN && fin % 4 == 0 && aligned16(Ain) && aligned16(W)) {
+                        const int want = (M + 3) / 4;   // 4 rows (warps) per CTA
+                        const int grid = want < 8 * sm_count() ? want : 8 * sm_count();
+                        auto kern = fin > 256 ? skinny_n4_kernel<true, decltype(epi)> : skinny_n4_kernel<false, decltype(epi)>;
+                        launch(kern, grid, 128, 0, st, M, fout, fin, Ain, fin, W, fin, epi);
+                        return cudaGetLastError();
+                    }
                 }
             }
             if (skinny_n_ok(fout, fin)) {
@@ -938,15 +941,15 @@ int worker_grads_simt(const GradsPlan& P, const float* w, const float* pool, int
     const int C = P.widths[L];
     if (few) {
         if constexpr (kF32) {
-        const int fin = P.widths[L - 1];
-        // 4 rows (a warp each) per CTA, or as many fours as bring the grid to 8 CTAs per SM
-        const int64_t most = 8 * sm_count();
-        const int rows_cta = static_cast<int>(4 * (((M + 3) / 4 + most - 1) / most));
-        const dim3 grid((B + rows_cta - 1) / rows_cta, P.n);
-        launch(fin > 256 ? logits_loss_kernel<true> : logits_loss_kernel<false>, grid, 128, 0, st, C, fin, B, rows_cta, Ain,
-               from_pool ? pool : nullptr, idx, S, labels, w + P.offW[L - 1], w + P.offb[L - 1], sloss, dz[0], loss,
-               reinterpret_cast<int*>(ws + P.off_cnt));
-        e = cudaGetLastError();
+            const int fin = P.widths[L - 1];
+            // 4 rows (a warp each) per CTA, or as many fours as bring the grid to 8 CTAs per SM
+            const int64_t most = 8 * sm_count();
+            const int rows_cta = static_cast<int>(4 * (((M + 3) / 4 + most - 1) / most));
+            const dim3 grid((B + rows_cta - 1) / rows_cta, P.n);
+            launch(fin > 256 ? logits_loss_kernel<true> : logits_loss_kernel<false>, grid, 128, 0, st, C, fin, B, rows_cta,
+                   Ain, from_pool ? pool : nullptr, idx, S, labels, w + P.offW[L - 1], w + P.offb[L - 1], sloss, dz[0], loss,
+                   reinterpret_cast<int*>(ws + P.off_cnt));
+            e = cudaGetLastError();
         }
     } else
         e = launch_softmax(logits, C, C, P.n, B, idx, S, labels, sloss, dz[0], C, loss,

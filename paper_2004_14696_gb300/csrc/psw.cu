@@ -558,8 +558,9 @@ __device__ void record_sweep(float* X, float* P0, float* P1, float* P2, const fl
 constexpr int kFixRounds = 32;   // merging rounds of the exact block means
 
 // ------------------------------------------------------------ the fit in shared memory
-// The fit of a group table that fits in shared memory (about 27 rows at n = 256; the form
-// above serves larger ones).  A sweep is a chain of dependent accesses, so latency is its
+// The fit of a group table that fits in shared memory (72 rows at n = 96, 26 at 256, 17 at 384, 12
+// at 512, 5 at 1024; the form above serves larger ones, at its own time: with 40 to 51 rows at
+// n = 256 1.7-7.5 ms).  A sweep is a chain of dependent accesses, so latency is its
 // time: there, with the table and the block stacks in the state buffer and chains split over
 // at most eight threads whose stacks one thread merges, a sweep of 23 rows x 256 columns took
 // 75-85 us and a whole fit of 19 / 43 / 61 sweeps 1.9 / 3.8 / 5.1 ms; here 15-18 us and

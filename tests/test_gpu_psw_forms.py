@@ -1,7 +1,8 @@
 """GPU parity of the two forms of the Eq. (17) fit (in shared memory; on the state buffer
 for larger tables) on planted cell tables: sizes around a warp, ranks without samples
-inside a row, and the last number of fitted rows that fits in shared memory at n = 96 (72)
-with the first that does not, against the oracle's fit of the same table."""
+inside a row, and the last number of fitted rows that fits in shared memory at n = 96 (72),
+256 (26) and 512 (12) with the first that does not, against the oracle's fit of the same
+table."""
 import numpy as np
 import pytest
 import torch
@@ -20,7 +21,7 @@ def built():
 
 
 @pytest.mark.parametrize("n,m", [(1, 1), (2, 2), (3, 1), (8, 8), (31, 20), (32, 32), (33, 33), (65, 40), (96, 1),
-                                 (96, 72), (96, 73)])
+                                 (96, 72), (96, 73), (256, 26), (256, 27), (512, 12), (512, 13)])
 def test_fit_forms_on_planted_tables(n, m):
     rng = np.random.default_rng(100 * n + m)
     unit = 2.0 ** -32
