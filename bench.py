@@ -54,19 +54,19 @@ METRIC = "simulated PS iterations/sec at n workers"
 UNIT = "iter/s"
 
 # dram bytes (read + write) of one full-size aggregation launch from an ncu capture
-# (n = 256, d = 54,440,936, k = 142: 31.1408 GB read + 0.2200 GB written against
+# (n = 256, d = 54,440,936, k = 142: 31.1409 GB read + 0.2195 GB written against
 # 31.3580 GB algorithmic), as a ratio to the algorithmic bytes so that it scales to the
 # bench's launches (traffic grows with k d); reported as null once aggregate.cu
 # differs from the source the counters were taken on.
-AGG_TRAFFIC = {"ratio_to_algorithmic": (31.140790 + 0.219976) / 31.357979,
-               "source_sha256": "5ff9b7556686d6fadf831374be85769d08285d42c3a39b0fdeddd59fbe8492c9",
+AGG_TRAFFIC = {"ratio_to_algorithmic": (31.140877 + 0.219537) / 31.357979,
+               "source_sha256": "5f6dace01162649f742f6174c40ecbbbffe1c312bc12893880cc25426f988d99",
                "case": "n=256 d=54440936 k=142"}
 # dram bytes (read + write) of the per-worker weight-gradient launches of one
-# full-size pass (ncu on mlp4096x3-1000_n256_B32): 4.2167 + 17.2496 + 17.2502 +
-# 17.2509 GB against 4.2778 + 3 x 17.3141 GB algorithmic; keyed to the dW kernel's
+# full-size pass (ncu on mlp4096x3-1000_n256_B32): 4.2163 + 17.2496 + 17.2499 +
+# 17.2498 GB against 4.2778 + 3 x 17.3141 GB algorithmic; keyed to the dW kernel's
 # own source (dw_source_sha).
-DW_TRAFFIC = {"ratio_to_algorithmic": (4.2167 + 17.2496 + 17.2502 + 17.2509) / (4.2778 + 3 * 17.3141),
-              "source_sha256": "3c451b2893a4677646f80c9bfd5922d6c9015510b9ee8cd0f4353b16d8f29ca6",
+DW_TRAFFIC = {"ratio_to_algorithmic": (4.2163 + 17.2496 + 17.2499 + 17.2498) / (4.2778 + 3 * 17.3141),
+              "source_sha256": "61b050ef04477d28af0a3c6fa1ce90f1807b4b8c3011bdb1a2b0ae9ee050e380",
               "case": "mlp4096x3-1000_n256_B32, one pass"}
 
 CASES = ("aggregate", "sweep", "grads", "received", "psw", "iterate")

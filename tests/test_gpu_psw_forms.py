@@ -30,7 +30,7 @@ def test_fit_forms_on_planted_tables(n, m):
         M = int(rng.integers(h, n + 1))
         i = np.arange(M)
         # increasing in the rank, decreasing in h, and noise that the projections pool
-        mean = 20.0 + 0.3 * i - 0.05 * h + rng.uniform(0.0, 2.0, size=M)
+        mean = max(20.0, 0.05 * n) + 0.3 * i - 0.05 * h + rng.uniform(0.0, 2.0, size=M)
         c = rng.integers(1, 5, size=M)
         c[(rng.random(M) < 0.1) & (i != h - 1)] = 0
         sums[h - 1, :M] = np.round(mean * c / unit).astype(np.uint64)
